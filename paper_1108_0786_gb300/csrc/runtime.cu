@@ -359,12 +359,15 @@ int ensure_device(lbm_t *h) {
     dv.omega_f = (float)dv.omega;
     dv.guo_f = (float)(1.0 - 0.5 * dv.omega);
     for (int i = 0; i < 3; ++i) dv.g_f[i] = (float)dv.g[i];
-    dv.om1_f = (float)(1.0 - dv.omega);
+    dv.om1 = 1.0 - dv.omega;
+    dv.om1_f = (float)dv.om1;
     {
         const double wc[3] = {1.0 / 3.0, 1.0 / 18.0, 1.0 / 36.0};
         for (int i = 0; i < 3; ++i) {
-            dv.ow_f[i] = (float)(dv.omega * wc[i]);
-            dv.gw_f[i] = (float)((1.0 - 0.5 * dv.omega) * wc[i]);
+            dv.ow[i] = dv.omega * wc[i];
+            dv.gw[i] = (1.0 - 0.5 * dv.omega) * wc[i];
+            dv.ow_f[i] = (float)dv.ow[i];
+            dv.gw_f[i] = (float)dv.gw[i];
         }
     }
     dv.forced = (h->g[0] != 0.0 || h->g[1] != 0.0 || h->g[2] != 0.0) ? 1 : 0;

@@ -107,27 +107,6 @@ __device__ __forceinline__ T shfl(T v, int delta, bool up) {
     return v;
 }
 
-// LBGK collision of one cell in place (deviation form):
-//   drho = sum delta, rho = 1 + drho, u = (sum e delta + g/2) / rho,
-//   delta_eq_b = w_b (drho + rho (3 e.u + 4.5 (e.u)^2 - 1.5 u.u)),
-//   delta~_b = delta_b + (delta_eq_b - delta_b) / tau
-//              + (1 - 1/(2 tau)) w_b (3 (e_b - u) . g + 9 (e_b . u)(e_b . g)).
-// In exact arithmetic the increments delta~_b - delta_b carry zero mass and
-// momentum exactly g.  With FP32 storage the rounded velocity that enters the
-// equilibrium would make each collision a small momentum source in every
-// cell, constant in a steady flow, and the slow viscous mode of a channel
-// integrates it into a ~1e-5 velocity error.  The FP32 update therefore sums
-// mass and momentum of the increments (small numbers, so the sums are
-// accurate) and moves the defect to the +-x, +-y, +-z pairs and the rest
-// population: only the value-dependent rounding of the final additions
-// remains.  FP64 keeps the plain update, as do the 16-bit formats, whose
-// storage rounding (2^-9 .. 2^-11 relative) dwarfs this effect.
-// CLOSE selects that closure.  PAIRED evaluates opposite directions (b, b + 1)
-// together: they share w, (e.u)^2 and e.g up to sign, so
-// deq = w (base + 4.5 rho (e.u)^2 +- 3 rho e.u) saves a fifth of the
-// arithmetic; otherwise one direction at a time.  Both forms compute the
-// same expression (FP32 takes the paired one; the 16-bit kernels schedule
-// the per-direction one better).
 // explicit fused multiply-adds: this file is compiled without implicit
 // contraction (-fmad=false), so every kernel that runs a cell's arithmetic --
 // any launch shape, the batched ensemble kernels, the boundary kernel --
@@ -148,9 +127,27 @@ __device__ __forceinline__ R edot(int b, R x, R y, R z) {
     return r;
 }
 
-template <typename Cd, bool CLOSE, bool PAIRED = CLOSE>
-__device__ __forceinline__ void collide(Cd (&f)[Q], const Device &dv) {
-    Cd s = 0, jx = 0, jy = 0, jz = 0;
+// LBGK collision of one cell in place (deviation form):
+//   drho = sum delta, rho = 1 + drho, u = (sum e delta + g/2) / rho,
+//   delta_eq_b = w_b (drho + rho (3 e.u + 4.5 (e.u)^2 - 1.5 u.u)),
+//   delta~_b = delta_b + (delta_eq_b - delta_b) / tau
+//              + (1 - 1/(2 tau)) w_b (3 (e_b - u) . g + 9 (e_b . u)(e_b . g)).
+// In exact arithmetic the increments delta~_b - delta_b carry zero mass and
+// momentum exactly g.  With FP32 storage the rounded velocity that enters the
+// equilibrium would make each collision a small momentum source in every
+// cell, constant in a steady flow, and the slow viscous mode of a channel
+// integrates it into a ~1e-5 velocity error.  The FP32 update therefore sums
+// mass and momentum of the increments (small numbers, so the sums are
+// accurate) and moves the defect to the +-x, +-y, +-z pairs and the rest
+// population: only the value-dependent rounding of the final additions
+// remains.  FP64 keeps the plain update (collide_f64), as do the 16-bit formats, whose
+// storage rounding (2^-9 .. 2^-11 relative) dwarfs this effect.
+// collide_f32 is that FP32 update.  It evaluates opposite directions (b, b + 1)
+// together: they share w, (e.u)^2 and e.g up to sign, so
+// deq = w (base + 4.5 rho (e.u)^2 +- 3 rho e.u) saves a fifth of the
+// arithmetic.
+__device__ __forceinline__ void collide_f32(float (&f)[Q], const Device &dv) {
+    float s = 0, jx = 0, jy = 0, jz = 0;
 #pragma unroll
     for (int b = 0; b < Q; ++b) {
         s += f[b];
@@ -158,77 +155,114 @@ __device__ __forceinline__ void collide(Cd (&f)[Q], const Device &dv) {
         if (ey(b)) jy += ey(b) > 0 ? f[b] : -f[b];
         if (ez(b)) jz += ez(b) > 0 ? f[b] : -f[b];
     }
-    const Cd rho = (Cd)1 + s;
-    const Cd inv = (Cd)1 / rho;
-    // FP32 takes the parameters rounded once on the host (no FP64 conversion per cell)
-    const bool f32 = sizeof(Cd) == 4;
-    const Cd gx = f32 ? (Cd)dv.g_f[0] : (Cd)dv.g[0], gy = f32 ? (Cd)dv.g_f[1] : (Cd)dv.g[1],
-             gz = f32 ? (Cd)dv.g_f[2] : (Cd)dv.g[2];
-    const Cd ux = mad((Cd)0.5, gx, jx) * inv, uy = mad((Cd)0.5, gy, jy) * inv, uz = mad((Cd)0.5, gz, jz) * inv;
-    const Cd usq = mad(ux, ux, mad(uy, uy, uz * uz));
-    const Cd om = f32 ? (Cd)dv.omega_f : (Cd)dv.omega;
-    const Cd guo = f32 ? (Cd)dv.guo_f : (Cd)(1.0 - 0.5 * dv.omega);
-    const Cd ug = mad(ux, gx, mad(uy, gy, uz * gz));
-    const Cd base = mad((Cd)(-1.5) * rho, usq, s);     // deviation of f_eq without the e.u terms, over w
-    Cd m = 0, px = 0, py = 0, pz = 0;
+    const float rho = 1.0f + s;
+    const float inv = 1.0f / rho;
+    // the parameters rounded once on the host (no FP64 conversion per cell)
+    const float gx = dv.g_f[0], gy = dv.g_f[1], gz = dv.g_f[2];
+    const float ux = mad(0.5f, gx, jx) * inv, uy = mad(0.5f, gy, jy) * inv, uz = mad(0.5f, gz, jz) * inv;
+    const float usq = mad(ux, ux, mad(uy, uy, uz * uz));
+    const float om = dv.omega_f, guo = dv.guo_f;
+    const float ug = mad(ux, gx, mad(uy, gy, uz * gz));
+    const float base = mad(-1.5f * rho, usq, s);       // deviation of f_eq without the e.u terms, over w
+    float m = 0, px = 0, py = 0, pz = 0;
     // one relaxation: the increment of direction b towards deq (+ Guo's term
-    // gt), kept for the conservation closure or applied directly
-    auto relax = [&](int b, Cd deq, Cd gt) {
-        if constexpr (CLOSE) {
-            const Cd d = dv.forced ? mad(om, deq - f[b], gt) : om * (deq - f[b]);
-            m += d;
-            if (ex(b)) px += ex(b) > 0 ? d : -d;
-            if (ey(b)) py += ey(b) > 0 ? d : -d;
-            if (ez(b)) pz += ez(b) > 0 ? d : -d;
-            f[b] += d;
-        } else {
-            Cd o = mad(-om, f[b] - deq, f[b]);
-            if (dv.forced) o += gt;
-            f[b] = o;
-        }
+    // gt), summed for the conservation closure
+    auto relax = [&](int b, float deq, float gt) {
+        const float d = dv.forced ? mad(om, deq - f[b], gt) : om * (deq - f[b]);
+        m += d;
+        if (ex(b)) px += ex(b) > 0 ? d : -d;
+        if (ey(b)) py += ey(b) > 0 ? d : -d;
+        if (ez(b)) pz += ez(b) > 0 ? d : -d;
+        f[b] += d;
     };
-    if constexpr (!PAIRED) {
-        // one direction at a time (the form the 16-bit kernels schedule best)
-#pragma unroll
-        for (int b = 0; b < Q; ++b) {
-            const Cd w = (Cd)wgt(b);
-            const Cd eu = edot(b, ux, uy, uz);
-            const Cd deq = w * mad(rho, mad((Cd)4.5 * eu, eu, mad((Cd)3, eu, (Cd)(-1.5) * usq)), s);
-            Cd gt = 0;
-            if (dv.forced) {
-                const Cd eg = edot(b, gx, gy, gz);
-                gt = guo * w * mad((Cd)9 * eu, eg, (Cd)3 * (eg - ug));
-            }
-            relax(b, deq, gt);
-        }
-    } else {
     {
-        const Cd w = (Cd)wgt(0);
-        relax(0, w * base, dv.forced ? guo * w * ((Cd)(-3) * ug) : (Cd)0);
+        const float w = (float)wgt(0);
+        relax(0, w * base, dv.forced ? guo * w * (-3.0f * ug) : 0.0f);
     }
 #pragma unroll
     for (int b = 1; b < Q; b += 2) {
-        const Cd w = (Cd)wgt(b);
-        const Cd eu = edot(b, ux, uy, uz);
-        const Cd a = mad((Cd)4.5 * rho * eu, eu, base);
-        const Cd c = (Cd)3 * rho * eu;
-        Cd g1 = 0, g2 = 0;
+        const float w = (float)wgt(b);
+        const float eu = edot(b, ux, uy, uz);
+        const float a = mad(4.5f * rho * eu, eu, base);
+        const float c = 3.0f * rho * eu;
+        float g1 = 0, g2 = 0;
         if (dv.forced) {
-            const Cd eg = edot(b, gx, gy, gz);
-            const Cd sym = mad((Cd)9 * eu, eg, (Cd)(-3) * ug), asym = (Cd)3 * eg;
+            const float eg = edot(b, gx, gy, gz);
+            const float sym = mad(9.0f * eu, eg, -3.0f * ug), asym = 3.0f * eg;
             g1 = guo * w * (sym + asym);
             g2 = guo * w * (sym - asym);
         }
         relax(b, w * (a + c), g1);
         relax(b + 1, w * (a - c), g2);
     }
+    const float hx = 0.5f * (gx - px), hy = 0.5f * (gy - py), hz = 0.5f * (gz - pz);
+    f[1] += hx; f[2] -= hx;
+    f[3] += hy; f[4] -= hy;
+    f[5] += hz; f[6] -= hz;
+    f[0] -= m;
+}
+
+// LBGK (+ Guo) of one cell for FP64 storage, the same update written for the
+// fewest FP64 instructions: an FP64 warp instruction occupies its
+// sub-partition for 64 cycles here, so the FP64 bulk kernel is bound by their
+// number and not by HBM.  Opposite directions share the moments' sums and
+// differences and the even part of the equilibrium, the weights and omega are
+// folded into per-cell factors of the two weight classes, and a population
+// takes two FMAs:
+//   f~ = ((1 - omega) f + a) +- C e.u,  a = omega w (drho - 1.5 rho u.u + 4.5 rho (e.u)^2),
+//   C = 3 omega w rho  (+ (1 - omega/2) w (9 (e.u)(e.g) - 3 u.g +- 3 e.g) with forcing).
+// 130 FP64 instructions a cell against 240 with each direction on its own: the
+// bulk kernel takes 1205 us a launch on 203 x 149 x 131 cells (1957 before),
+// its FP64 pipe 87 % busy.
+__device__ __forceinline__ void collide_f64(double (&f)[Q], const Device &dv) {
+    double d[Q / 2];
+    double s = f[0];
+#pragma unroll
+    for (int p = 0; p < Q / 2; ++p) {
+        d[p] = f[2 * p + 1] - f[2 * p + 2];
+        s += f[2 * p + 1] + f[2 * p + 2];
     }
-    if constexpr (CLOSE) {
-        const Cd hx = (Cd)0.5 * (gx - px), hy = (Cd)0.5 * (gy - py), hz = (Cd)0.5 * (gz - pz);
-        f[1] += hx; f[2] -= hx;
-        f[3] += hy; f[4] -= hy;
-        f[5] += hz; f[6] -= hz;
-        f[0] -= m;
+    double jx = d[0] + ((d[3] + d[4]) + (d[5] + d[6]));
+    double jy = d[1] + ((d[3] - d[4]) + (d[7] + d[8]));
+    double jz = d[2] + ((d[5] - d[6]) + (d[7] - d[8]));
+    const bool forced = dv.forced;
+    const double gx = dv.g[0], gy = dv.g[1], gz = dv.g[2];
+    if (forced) {
+        jx = mad(0.5, gx, jx);
+        jy = mad(0.5, gy, jy);
+        jz = mad(0.5, gz, jz);
+    }
+    const double rho = 1.0 + s;
+    const double inv = 1.0 / rho;
+    const double ux = jx * inv, uy = jy * inv, uz = jz * inv;
+    const double sq[3] = {ux * ux, uy * uy, uz * uz};
+    const double base = mad(-1.5 * rho, (sq[0] + sq[1]) + sq[2], s);
+    const double om1 = dv.om1;
+    const double ug3 = forced ? -3.0 * mad(ux, gx, mad(uy, gy, uz * gz)) : 0.0;
+    f[0] = mad(om1, f[0], dv.ow[0] * base);
+    if (forced) f[0] = mad(dv.gw[0], ug3, f[0]);
+    double b1 = dv.ow[1] * base, b2 = dv.ow[2] * base;
+    if (forced) {
+        b1 = mad(dv.gw[1], ug3, b1);
+        b2 = mad(dv.gw[2], ug3, b2);
+    }
+    const double r3[2] = {3.0 * dv.ow[1] * rho, 3.0 * dv.ow[2] * rho};
+    const double r45[2] = {1.5 * r3[0], 1.5 * r3[1]};
+#pragma unroll
+    for (int p = 0; p < Q / 2; ++p) {
+        const int b = 2 * p + 1, wc = p < 3 ? 0 : 1;
+        const double eu = edot(b, ux, uy, uz);
+        double a = mad(r45[wc], p < 3 ? sq[p] : eu * eu, wc ? b2 : b1);
+        if (forced) {
+            const double eg = edot(b, gx, gy, gz), gw = dv.gw[1 + wc];
+            a = mad(9.0 * gw * eu, eg, a);
+            const double c = mad(r3[wc], eu, 3.0 * gw * eg);
+            f[b] = mad(om1, f[b], a) + c;
+            f[b + 1] = mad(om1, f[b + 1], a) - c;
+        } else {
+            f[b] = mad(r3[wc], eu, mad(om1, f[b], a));
+            f[b + 1] = mad(-r3[wc], eu, mad(om1, f[b + 1], a));
+        }
     }
 }
 
@@ -288,6 +322,14 @@ __device__ __forceinline__ void collide_lean(float (&f)[Q], const Device &dv) {
         f[b] = fmaf(om1, f[b], r1);
         f[b + 1] = fmaf(om1, f[b + 1], r2);
     }
+}
+
+// the collision of storage type T on its deviations, unscaled
+template <typename T, typename Cd>
+__device__ __forceinline__ void collide(Cd (&f)[Q], const Device &dv) {
+    if constexpr (std::is_same<T, double>::value) collide_f64(f, dv);
+    else if constexpr (std::is_same<T, float>::value) collide_f32(f, dv);
+    else collide_lean<false>(f, dv);
 }
 
 // 16-bit storage without a per-population scale: FP16 keeps k delta, so the
@@ -445,7 +487,7 @@ __device__ __forceinline__ void bulk_body(const Device &dv, const StepPtrs &sp, 
 #pragma unroll
         for (int b = 0; b < Q; ++b) g[b] = f[b][i];
         if constexpr (raw16) collide_lean<std::is_same<T, __half>::value>(g, dv);
-        else collide<Cd, std::is_same<T, float>::value>(g, dv);
+        else collide<T>(g, dv);
         const bool solid = fl[i] & F_SOLID;
 #pragma unroll
         for (int b = 0; b < Q; ++b) f[b][i] = solid ? (Cd)0 : g[b];
@@ -896,7 +938,7 @@ __device__ __forceinline__ void boundary_body(const Device &dv, const StepPtrs &
             dv.rho_near[c] = (float)drho;
         }
     }
-    collide<Cd, std::is_same<T, float>::value>(f, dv);
+    collide<T>(f, dv);
     T *__restrict__ dst = static_cast<T *>(sp.dst);
     if constexpr (std::is_same<T, __nv_bfloat16>::value) {
         const Dither dz = bf16_dither(c, *sp.tstep);
@@ -1070,7 +1112,7 @@ __global__ void __launch_bounds__(TMA_THREADS, MINB) bulk_tma_kernel(const Devic
 #pragma unroll
                     for (int b = 0; b < Q; ++b) dst[(long long)b * C + c0 + x] = store16<T>(f[b], dz, b);
                 } else {
-                    collide<Cd, std::is_same<T, float>::value>(f, dv);
+                    collide<T>(f, dv);
 #pragma unroll
                     for (int b = 0; b < Q; ++b) dst[(long long)b * C + c0 + x] = Codec<T>::st(f[b], scale);
                 }
