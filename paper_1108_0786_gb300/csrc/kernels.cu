@@ -17,8 +17,11 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <cmath>
+#include <cstring>
 #include <type_traits>
 
+#include "../../include/lbm.h"
 #include "lbm_internal.cuh"
 
 namespace lbm {
@@ -1176,35 +1179,185 @@ __global__ void __launch_bounds__(256) integrate_kernel(const Device dv, const S
 
 // ---- field export / import -----------------------------------------------
 
-template <typename T, typename O>
-__global__ void export_kernel(const Device dv, const T *pop, const uint8_t *flags, const uint8_t *bid,
-                              int what, int mask_solid, O *out) {
-    const Domain d = dv.dom;
-    const long long C = d.C;
-    const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= C) return;
-    const float s = dv.f16_inv_scale;
-    const bool solid = mask_solid && (flags[c] & F_SOLID);
-    if (what == 2) {
-        reinterpret_cast<uint8_t *>(out)[c] = solid ? (uint8_t)(bid[c] + 1) : 0;
-        return;
+// The value of a float expansion hi + lo under additions: TwoSum (Knuth; Moller)
+// keeps each addition's rounding error in lo, so that a sum of 19 FP32 values
+// carries about 48 bits without the FP64 pipe (2 results a cycle an SM here,
+// against 128 FP32 ones).  Infinities and NaN do not survive it (inf - inf):
+// callers check the result.
+struct FloatSum {
+    float hi, lo;
+    __device__ __forceinline__ void add(float v) {
+        const float s = hi + v, t = s - hi;
+        lo += (hi - (s - t)) + (v - t);
+        hi = s;
     }
-    if (what == 3) {
-        for (int a = 0; a < Q; ++a) out[a * C + c] = (O)(wgt(a) + load_dev<T>(pop + a * C + c, s));
-        return;
-    }
-    double drho = 0.0, j[3] = {0.0, 0.0, 0.0};
-    for (int a = 0; a < Q; ++a) {
-        const double v = load_dev<T>(pop + a * C + c, s);
-        drho += v;
-        j[0] += ex(a) * v; j[1] += ey(a) * v; j[2] += ez(a) * v;
-    }
-    const double rho = 1.0 + drho;
-    if (what == 0) {
-        out[c] = (O)(solid ? 1.0 : rho);
+};
+
+// w_a + delta as stored in O.  FP32 output of 32/16-bit storage adds the two
+// parts of w_a (FP32 value and remainder) with one TwoSum: the FP64 sum rounded
+// to FP32, but for ties that the remainder's own rounding (2^-24 of an ulp)
+// decides.
+template <typename O, typename T>
+__device__ __forceinline__ O pop_value(double w, float wh, float wl, const T *v, float scale) {
+    if constexpr (sizeof(O) == 4 && sizeof(T) <= 4) {
+        const float x = load_dev_f<T>(v, scale);
+        const float s = wh + x, t = s - wh;
+        const float e = (wh - (s - t)) + (x - t);
+        return fabsf(s) < INFINITY ? s + (e + wl) : s;
     } else {
-        for (int i = 0; i < 3; ++i) out[i * C + c] = (O)(solid ? 0.0 : (j[i] - 0.5 * dv.g[i]) / rho);
+        return (O)(w + load_dev<T>(v, scale));
     }
+}
+
+// Populations: a plain stream of V-wide vectors, EXPORT_U of them a thread in
+// flight, direction blockIdx.y.  Bound by HBM: 33.5 M cells from FP32 to FP32
+// (5.1 GB) take 0.72 ms; a thread a cell with FP64 sums took 3.38 ms, bound by
+// the FP64 pipe's conversions and additions.
+constexpr int EXPORT_THREADS = 256;
+constexpr int EXPORT_U = 4;
+
+template <int BYTES> struct Chunk;
+template <> struct Chunk<2> { using type = unsigned short; };
+template <> struct Chunk<4> { using type = unsigned; };
+template <> struct Chunk<8> { using type = uint2; };
+template <> struct Chunk<16> { using type = uint4; };
+
+// V consecutive values to `p` in pieces of at most 16 bytes
+template <typename O, int V>
+__device__ __forceinline__ void put_values(O *p, const O (&o)[V]) {
+    constexpr int B = V * (int)sizeof(O) < 16 ? V * (int)sizeof(O) : 16, PER = B / (int)sizeof(O);
+    using R = typename Chunk<B>::type;
+#pragma unroll
+    for (int k = 0; k < V / PER; ++k) {
+        R r;
+        memcpy(&r, o + k * PER, B);
+        *reinterpret_cast<R *>(p + k * PER) = r;
+    }
+}
+
+template <typename T, typename O, int V>
+__global__ void __launch_bounds__(EXPORT_THREADS)
+export_pop_kernel(const T *__restrict__ pop, long long C, float scale, O *__restrict__ out) {
+    using R = typename Chunk<V * (int)sizeof(T)>::type;
+    const int a = blockIdx.y;
+    const double w = wgt(a);
+    const float wh = (float)w, wl = (float)(w - (double)wh);
+    const T *__restrict__ src = pop + a * C;
+    O *__restrict__ dst = out + a * C;
+    const long long groups = C / V, i0 = (long long)blockIdx.x * (EXPORT_THREADS * EXPORT_U) + threadIdx.x;
+    R r[EXPORT_U];
+#pragma unroll
+    for (int u = 0; u < EXPORT_U; ++u) {
+        const long long i = i0 + u * EXPORT_THREADS;
+        if (i < groups) r[u] = __ldg(reinterpret_cast<const R *>(src) + i);
+    }
+#pragma unroll
+    for (int u = 0; u < EXPORT_U; ++u) {
+        const long long i = i0 + u * EXPORT_THREADS;
+        if (i >= groups) break;
+        T v[V];
+        memcpy(&v, &r[u], sizeof(R));
+        O o[V];
+#pragma unroll
+        for (int k = 0; k < V; ++k) o[k] = pop_value<O, T>(w, wh, wl, v + k, scale);
+        put_values<O, V>(dst + i * V, o);
+    }
+}
+
+// density deviation and momentum of one cell's deviations, in FP64, in
+// direction order
+template <typename T>
+__device__ __forceinline__ void moments_f64(const T (&v)[Q], float scale, double &drho, double (&j)[3]) {
+    drho = j[0] = j[1] = j[2] = 0.0;
+#pragma unroll
+    for (int a = 0; a < Q; ++a) {
+        const double x = load_dev<T>(&v[a], scale);
+        drho += x;
+        if (ex(a)) j[0] += ex(a) > 0 ? x : -x;
+        if (ey(a)) j[1] += ey(a) > 0 ? x : -x;
+        if (ez(a)) j[2] += ez(a) > 0 ? x : -x;
+    }
+}
+
+// Density (U = false) or velocity (U = true) of each cell, one thread a cell,
+// all 19 loads issued before the sums.  FP32 output of 32/16-bit storage sums in
+// float expansions and divides with one correction step, so that the result is
+// rounded about once, as from FP64 sums; FP64 storage and FP64 output sum in
+// FP64.  A cell whose sums are not finite takes the FP64 path.
+template <typename T, typename O, bool U>
+__global__ void __launch_bounds__(EXPORT_THREADS)
+export_moments_kernel(const Device dv, const T *__restrict__ pop, const uint8_t *__restrict__ flags, int mask_solid,
+                      O *__restrict__ out) {
+    const long long C = dv.dom.C;
+    const long long c = (long long)blockIdx.x * EXPORT_THREADS + threadIdx.x;
+    if (c >= C) return;
+    const float scale = dv.f16_inv_scale;
+    const bool solid = mask_solid && (flags[c] & F_SOLID);
+    T v[Q];
+#pragma unroll
+    for (int a = 0; a < Q; ++a) v[a] = pop[a * C + c];
+    if (solid) {
+        if constexpr (U) {
+            for (int i = 0; i < 3; ++i) out[i * C + c] = (O)0;
+        } else {
+            out[c] = (O)1;
+        }
+        return;
+    }
+    if constexpr (sizeof(O) == 4 && sizeof(T) <= 4) {
+        FloatSum s{0.0f, 0.0f}, j[3] = {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}};
+#pragma unroll
+        for (int a = 0; a < Q; ++a) {
+            const float x = load_dev_f<T>(&v[a], scale);
+            s.add(x);
+            if constexpr (U) {
+                if (ex(a)) j[0].add(ex(a) > 0 ? x : -x);
+                if (ey(a)) j[1].add(ey(a) > 0 ? x : -x);
+                if (ez(a)) j[2].add(ez(a) > 0 ? x : -x);
+            }
+        }
+        FloatSum rho{1.0f, s.lo};
+        rho.add(s.hi);
+        if constexpr (!U) {
+            const float r = rho.hi + rho.lo;
+            if (fabsf(r) < INFINITY) {
+                out[c] = r;
+                return;
+            }
+        } else {
+            const float inv = 1.0f / rho.hi;
+            float q[3];
+            bool finite = true;
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                const float gh = dv.gh_f[i], gl = dv.gl_f[i];           // g / 2 in two parts
+                j[i].lo -= gl;
+                j[i].add(-gh);
+                const float n = j[i].hi + j[i].lo, nl = (j[i].hi - n) + j[i].lo;
+                const float q0 = n * inv;
+                const float r = fmaf(-q0, rho.hi, n) + fmaf(-q0, rho.lo, nl);
+                q[i] = fmaf(r, inv, q0);
+                finite = finite && fabsf(q[i]) < INFINITY;
+            }
+            if (finite) {
+                for (int i = 0; i < 3; ++i) out[i * C + c] = q[i];
+                return;
+            }
+        }
+    }
+    double drho, j[3];
+    moments_f64<T>(v, scale, drho, j);
+    const double rho = 1.0 + drho;
+    if constexpr (U) {
+        for (int i = 0; i < 3; ++i) out[i * C + c] = (O)((j[i] - 0.5 * dv.g[i]) / rho);
+    } else {
+        out[c] = (O)rho;
+    }
+}
+
+__global__ void export_flags_kernel(const uint8_t *flags, const uint8_t *bid, long long C, int mask_solid, uint8_t *out) {
+    const long long c = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (c < C) out[c] = mask_solid && (flags[c] & F_SOLID) ? (uint8_t)(bid[c] + 1) : 0;
 }
 
 // Running time average of the velocity (Sec. 6, the flow fields averaged
@@ -1353,22 +1506,56 @@ void launch_batch_small(int k, const Batch &bt, unsigned blocks, int precision, 
     }
 }
 
+template <typename T, typename O, int V>
+static void export_pop(const Device &dv, const T *pop, O *out, cudaStream_t s) {
+    const long long groups = dv.dom.C / V;
+    const dim3 grid(blocks_for(groups, EXPORT_THREADS * EXPORT_U), Q);
+    export_pop_kernel<T, O, V><<<grid, EXPORT_THREADS, 0, s>>>(pop, dv.dom.C, dv.f16_inv_scale, out);
+}
+
+template <typename T, typename O>
+static void export_typed(const Device &dv, const void *pop_, const uint8_t *flags, int what, int mask_solid, O *out,
+                         cudaStream_t s) {
+    const T *pop = static_cast<const T *>(pop_);
+    const unsigned bl = blocks_for(dv.dom.C, EXPORT_THREADS);
+    if (what == LBM_FIELD_RHO) {
+        export_moments_kernel<T, O, false><<<bl, EXPORT_THREADS, 0, s>>>(dv, pop, flags, mask_solid, out);
+    } else if (what == LBM_FIELD_U) {
+        export_moments_kernel<T, O, true><<<bl, EXPORT_THREADS, 0, s>>>(dv, pop, flags, mask_solid, out);
+    } else {
+        // 16-byte loads where every direction's run of cells and the caller's
+        // buffer allow them; the planes themselves are aligned (the handle's
+        // allocation), an odd cell count or an offset buffer takes single values
+        constexpr int V = 16 / (int)sizeof(T);
+        constexpr int A = V * (int)sizeof(O) < 16 ? V * (int)sizeof(O) : 16;
+        if (dv.dom.C % V == 0 && reinterpret_cast<uintptr_t>(out) % A == 0 &&
+            reinterpret_cast<uintptr_t>(pop_) % 16 == 0)
+            export_pop<T, O, V>(dv, pop, out, s);
+        else
+            export_pop<T, O, 1>(dv, pop, out, s);
+    }
+}
+
 template <typename O>
-static void export_typed(const Device &dv, const void *pop, const uint8_t *flags, const uint8_t *bid,
-                         int what, int mask_solid, O *out, cudaStream_t s) {
-    const unsigned bl = blocks_for(dv.dom.C, 256);
+static void export_as(const Device &dv, const void *pop, const uint8_t *flags, int what, int mask_solid, O *out,
+                      cudaStream_t s) {
     switch (dv.precision) {
-    case 0: export_kernel<double, O><<<bl, 256, 0, s>>>(dv, (const double *)pop, flags, bid, what, mask_solid, out); break;
-    case 1: export_kernel<float, O><<<bl, 256, 0, s>>>(dv, (const float *)pop, flags, bid, what, mask_solid, out); break;
-    case 2: export_kernel<__half, O><<<bl, 256, 0, s>>>(dv, (const __half *)pop, flags, bid, what, mask_solid, out); break;
-    default: export_kernel<__nv_bfloat16, O><<<bl, 256, 0, s>>>(dv, (const __nv_bfloat16 *)pop, flags, bid, what, mask_solid, out); break;
+    case 0: export_typed<double, O>(dv, pop, flags, what, mask_solid, out, s); break;
+    case 1: export_typed<float, O>(dv, pop, flags, what, mask_solid, out, s); break;
+    case 2: export_typed<__half, O>(dv, pop, flags, what, mask_solid, out, s); break;
+    default: export_typed<__nv_bfloat16, O>(dv, pop, flags, what, mask_solid, out, s); break;
     }
 }
 
 void launch_export(const Device &dv, const void *pop, const uint8_t *flags, const uint8_t *bid, int what,
                    int mask_solid, void *out, int dtype, cudaStream_t s) {
-    if (dtype == 1) export_typed<float>(dv, pop, flags, bid, what, mask_solid, static_cast<float *>(out), s);
-    else export_typed<double>(dv, pop, flags, bid, what, mask_solid, static_cast<double *>(out), s);
+    if (what == LBM_FIELD_FLAGS)
+        export_flags_kernel<<<blocks_for(dv.dom.C, 256), 256, 0, s>>>(flags, bid, dv.dom.C, mask_solid,
+                                                                      static_cast<uint8_t *>(out));
+    else if (dtype == LBM_DTYPE_F32)
+        export_as<float>(dv, pop, flags, what, mask_solid, static_cast<float *>(out), s);
+    else
+        export_as<double>(dv, pop, flags, what, mask_solid, static_cast<double *>(out), s);
 }
 
 void launch_average(const Device &dv, const StepPtrs &sp, cudaStream_t s) {

@@ -358,7 +358,11 @@ int ensure_device(lbm_t *h) {
     for (int i = 0; i < 3; ++i) dv.g[i] = h->g[i];
     dv.omega_f = (float)dv.omega;
     dv.guo_f = (float)(1.0 - 0.5 * dv.omega);
-    for (int i = 0; i < 3; ++i) dv.g_f[i] = (float)dv.g[i];
+    for (int i = 0; i < 3; ++i) {
+        dv.g_f[i] = (float)dv.g[i];
+        dv.gh_f[i] = (float)(0.5 * dv.g[i]);
+        dv.gl_f[i] = (float)(0.5 * dv.g[i] - (double)dv.gh_f[i]);
+    }
     dv.om1 = 1.0 - dv.omega;
     dv.om1_f = (float)dv.om1;
     {
