@@ -104,8 +104,8 @@ extern "C" {
 
 /* kernel slots reported by lbm_time_kernels */
 #define LBM_KERNEL_REMAP          0   /* body geometry and remap candidates, then map bodies to the lattice */
-#define LBM_KERNEL_STREAM_COLLIDE 1   /* bulk pull + LBGK over all cells */
-#define LBM_KERNEL_BOUNDARY       2   /* refill / bounce-back cells near bodies and walls */
+#define LBM_KERNEL_STREAM_COLLIDE 1   /* bulk pull + LBGK over all cells, walls included */
+#define LBM_KERNEL_BOUNDARY       2   /* refill / bounce-back cells near bodies */
 #define LBM_KERNEL_LINKS          3   /* per-body link lists, then the step's drive and spring loads */
 #define LBM_KERNEL_FORCE          4   /* momentum exchange; with fluid it also runs the rigid-body step */
 #define LBM_KERNEL_INTEGRATE      5   /* drive, springs, rigid-body step when there is no fluid */
@@ -434,9 +434,8 @@ int lbm_ensemble_destroy(lbm_ensemble_t *e);
 const char *lbm_ensemble_last_error(lbm_ensemble_t *e);
 
 /* Kernel launches one step makes (for launch accounting): with bodies and
- * fluid, remap, bulk stream-collide, boundary cells (one more launch with
- * walls), link lists, drive and spring loads, and the momentum exchange
- * with the rigid-body step.  A body preparation kernel (geometry records of
+ * fluid, remap, bulk stream-collide, boundary cells, link lists, drive and
+ * spring loads, and the momentum exchange with the rigid-body step.  A body preparation kernel (geometry records of
  * states the rigid-body step did not make) runs once before the first step
  * after the host wrote a body state, and in every overlapped step. */
 int lbm_kernels_per_step(lbm_t *h);

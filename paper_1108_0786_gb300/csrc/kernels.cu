@@ -481,7 +481,7 @@ __device__ __forceinline__ void remap_body(const Device &dv, const StepPtrs &sp,
                 }
                 // the boundary kernel's cells: a shared-memory atomic per warp
                 // (past the buffer, a global one)
-                const bool mine = live && !init_mode && !(flags & F_SOLID) && (flags & (F_NEAR | F_SOLID_PREV));
+                const bool mine = live && !init_mode && !(flags & F_SOLID) && (flags & F_LISTED);
                 const unsigned mb = __ballot_sync(0xffffffffu, mine);
                 if (mb) {
                     const int leader = __ffs(mb) - 1;
@@ -994,8 +994,7 @@ __device__ __forceinline__ void force_body(const Device &dv, const StepPtrs &sp,
             // less than a cell a step), else the FP32 sum of the stored
             // deviations (the bulk kernel's cells a body has just reached)
             float drho;
-            const uint8_t fc = sp.flags_cur[c];
-            if (fc != 0 && !(fc & F_SOLID)) {
+            if (sp.flags_cur[c] & F_LISTED) {
                 drho = __ldcg(dv.rho_near + c);
             } else {
                 drho = 0.0f;

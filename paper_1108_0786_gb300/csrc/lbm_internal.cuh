@@ -51,6 +51,7 @@ constexpr uint8_t F_SOLID = 1;      // solid at n
 constexpr uint8_t F_SOLID_PREV = 2; // solid at n-1 (uncovered if F_SOLID is clear)
 constexpr uint8_t F_NEAR = 4;       // some neighbour x - e_b was solid at n-1
 constexpr uint8_t F_WALL = 8;       // some neighbour lies beyond a no-slip wall
+constexpr uint8_t F_LISTED = F_NEAR | F_SOLID_PREV;     // fluid with one of these: the boundary kernel's cell
 constexpr uint8_t NO_BODY = 0xFF;
 
 // device status word bits
@@ -195,7 +196,13 @@ struct StepPtrs {
     const unsigned *far_skip;
     const long long *tstep;                 // step index n (the BF16 rounding bits' counter)
     int parity;
+    unsigned row_recip;                     // row_recip of the V-cell groups in an x-row (the bulk launch's)
 };
+
+// 2^32 / n rounded down (2^32 - 1 for n = 1): for q < 2^31 the high word of
+// q row_recip(n) is q / n or one less (a block's loads wait for the row index,
+// and a 32-bit division is a chain of some 25 instructions)
+inline unsigned row_recip(int n) { return n > 1 ? (unsigned)((1ULL << 32) / (unsigned)n) : 0xffffffffu; }
 
 // Overlapped steps.  The bulk kernel of step n needs only the populations of
 // step n-1 where no body is near: outside the remap cubes flags are static
@@ -362,7 +369,7 @@ __device__ inline void batch_member(const Batch &bt, Device &sdv, StepPtrs &ssp,
 }
 
 // the per-step kernels a batched step launches, in step order
-enum BatchKernel { BK_PREP, BK_REMAP, BK_BOUNDARY, BK_WALLS, BK_LINKS, BK_LOADS, BK_BULK, BK_FORCE, BK_COUNT };
+enum BatchKernel { BK_PREP, BK_REMAP, BK_BOUNDARY, BK_LINKS, BK_LOADS, BK_BULK, BK_FORCE, BK_COUNT };
 
 // the start of a batched kernel: sdv, ssp and sbk are this block's member
 // record, step pointers and block coordinates
@@ -467,7 +474,8 @@ void launch_average(const Device &dv, const StepPtrs &sp, cudaStream_t s);
 void batch_grid_small(const Device &dv, int k, int g[3]);                     // kernels.cu
 void launch_batch_small(int k, const Batch &bt, unsigned blocks, int precision, cudaStream_t s);
 void batch_grid_cells(const Device &dv, int k, int variant, int g[3]);        // stream_collide.cu
-void launch_batch_cells(int k, int variant, const Batch &bt, unsigned blocks, int precision, cudaStream_t s);
+void launch_batch_cells(int k, int variant, const Batch &bt, unsigned blocks, int precision, bool walls,
+                        cudaStream_t s);     // walls: some member has a non-periodic axis
 // batched bulk shape i of a precision: its cells per thread, or 0 past the list
 int batch_bulk_shape(int precision, int i);
 int adjoint_part_stride(const Device &dv);

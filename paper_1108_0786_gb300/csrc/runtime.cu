@@ -286,12 +286,10 @@ bool overlapped(const lbm_t *h) {
 
 int kernels_per_step(const lbm_t *h) {
     const bool bodies = nb(h) > 0, fl = fluid(h);
-    const bool walls = (h->bc & 7) != 7;
     int n = 0;
     if (bodies && fl) n += overlapped(h) ? 2 : 1;           // (body preparation,) remap
-    if (fl) n += 1;                                         // bulk stream-collide
-    if (fl) n += (bodies ? 1 : 0) + (walls ? 1 : 0);        // boundary cells
-    if (bodies && fl) n += 3;                               // links, drive and spring loads, force + rigid-body step
+    if (fl) n += 1;                                         // bulk stream-collide (no-slip walls with it)
+    if (bodies && fl) n += 4;                               // boundary cells, links, drive and spring loads, force + rigid-body step
     if (bodies && !fl) n += 1;                              // rigid-body step alone
     if (!bodies && fl) n += 1;                              // step counter
     if (fl && h->dv.avg_u) n += 1;                          // running velocity average
@@ -1839,6 +1837,7 @@ int lbm_adjoint_backward(lbm_t *h, const double *seed, double *grad_state, doubl
 // kernel the members' flattened block ranges and grids)
 struct EnsGroup {
     int precision = 1;
+    bool walls = false;                     // some member has a non-periodic axis
     int lane = 0;                           // batched mode: the chain of launches the group is in
     std::vector<int> members;               // ensemble indices
     void *mem = nullptr;                    // the tables, one allocation (first member's allocator)
@@ -1945,8 +1944,10 @@ int ens_group_tables(lbm_ensemble_t *e, EnsGroup &g) {
     for (int j = 0; j < M; ++j) {
         lbm_t *h = e->members[g.members[j]];
         dvs[j] = h->dv;
+        g.walls = g.walls || (h->bc & 7) != 7;
         sps[j] = step_ptrs(h, 0);
         sps[M + j] = step_ptrs(h, 1);
+        sps[j].row_recip = sps[M + j].row_recip = lbm::row_recip(h->nx / lbm::batch_bulk_shape(g.precision, variant));
     }
     if (M > 65535) return ens_fail(e, LBM_E_ARG, "more than 65535 members of one precision");
     std::vector<int> tab;                   // per kernel: first[M + 1], grid[3 M]
@@ -1960,7 +1961,7 @@ int ens_group_tables(lbm_ensemble_t *e, EnsGroup &g) {
         long long total = 0;
         for (int j = 0; j < M; ++j) {
             int gd[3];
-            if (k == lbm::BK_BOUNDARY || k == lbm::BK_WALLS || k == lbm::BK_BULK)
+            if (k == lbm::BK_BOUNDARY || k == lbm::BK_BULK)
                 lbm::batch_grid_cells(dvs[j], k, variant, gd);
             else
                 lbm::batch_grid_small(dvs[j], k, gd);
@@ -2023,7 +2024,7 @@ void ens_enqueue_batched(lbm_ensemble_t *e, std::vector<EnsGroup> &groups, int l
             if (g.lane != lane) continue;
             lbm::Batch b = g.bt[k];
             b.parity = p;
-            lbm::launch_batch_cells(k, e->variant[g.precision], b, g.blocks[k], g.precision, st);
+            lbm::launch_batch_cells(k, e->variant[g.precision], b, g.blocks[k], g.precision, g.walls, st);
         }
     };
     // the batched remap takes its candidates from the body preparation
@@ -2033,7 +2034,6 @@ void ens_enqueue_batched(lbm_ensemble_t *e, std::vector<EnsGroup> &groups, int l
     cudaEventRecord(fork, main);
     cudaStreamWaitEvent(side, fork, 0);
     cells(lbm::BK_BOUNDARY, side);
-    cells(lbm::BK_WALLS, side);
     small(lbm::BK_LINKS, side);
     small(lbm::BK_LOADS, side);
     cudaEventRecord(join, side);
@@ -2352,10 +2352,10 @@ int lbm_ensemble_autotune(lbm_ensemble_t *e, int trials, int *cells_per_thread) 
             // the populations of every member's next step, which that step rewrites in full
             lbm::Batch b = g.bt[lbm::BK_BULK];
             b.parity = p;
-            lbm::launch_batch_cells(lbm::BK_BULK, v, b, g.blocks[lbm::BK_BULK], prec, e->stream);
+            lbm::launch_batch_cells(lbm::BK_BULK, v, b, g.blocks[lbm::BK_BULK], prec, g.walls, e->stream);
             cudaEventRecord(e0, e->stream);
             for (int t = 0; t < trials; ++t)
-                lbm::launch_batch_cells(lbm::BK_BULK, v, b, g.blocks[lbm::BK_BULK], prec, e->stream);
+                lbm::launch_batch_cells(lbm::BK_BULK, v, b, g.blocks[lbm::BK_BULK], prec, g.walls, e->stream);
             cudaEventRecord(e1, e->stream);
             cudaError_t err = cudaEventSynchronize(e1);
             float ms = 0.0f;

@@ -8,13 +8,13 @@
 // Two kernels write the populations of step n (pull scheme, two grids: src =
 // step n-1, dst = step n):
 //
-//  bulk      every cell with a zero flag byte: f_b(x) = f~_b(x - e_b) for
-//            all 19 b, LBGK relaxation to the second-order equilibrium with
-//            Guo's forcing, store; solid cells store deviation 0.  No
-//            data-dependent paths, so the kernel stays small and light.
-//  boundary  only the fluid cells whose flag byte is non-zero (they lie in
-//            the cubes around the bodies or on wall faces; the bulk kernel
-//            leaves them alone, so the two kernels may run concurrently):
+//  bulk      every cell the remap did not list: f_b(x) = f~_b(x - e_b) for
+//            all 19 b (f~_{-b}(x) where x - e_b lies beyond a no-slip wall,
+//            Eq. 4), LBGK relaxation to the second-order equilibrium with
+//            Guo's forcing, store; solid cells store deviation 0.
+//  boundary  only the listed fluid cells (F_NEAR or F_SOLID_PREV: they lie in
+//            the cubes around the bodies; the bulk kernel leaves them alone,
+//            so the two kernels may run concurrently):
 //              - x was solid at n-1 (uncovered): f_b = f_eq(rho_avg, u_w(x)),
 //                rho_avg the mean density of the D3Q19 neighbours that are
 //                fluid in both epochs (1 if none), u_w at the state of step n;
@@ -411,29 +411,69 @@ template <typename T> __device__ __forceinline__ Dither dither_for(long long c, 
     else return Dither{};
 }
 
-template <typename T, int V, int BX, int BY, bool FLAT = false>
+// The thread's V-cell group of a z-plane: the groups in row order, BULK_THREADS
+// a block, so that no lane idles at the end of a row whatever nx is.  A warp's
+// lanes may cross a row end, where the loads of a row's first and last cell
+// take over from the shuffles.  (Blocks of 32 or 128 groups of one row left 21 %
+// of the FP64 kernel's lanes idle at nx = 203: 1205 -> 955 us a launch on
+// 203 x 149 x 131 cells; 22 % of the FP32 kernel's at nx = 100.)
+constexpr int BULK_THREADS = 256;
+
+__device__ __forceinline__ void plane_group(const Blk &bk, int nxq, int ny, unsigned recip, int &xq, int &y,
+                                            bool &active) {
+    const unsigned per_plane = (unsigned)nxq * ny;
+    unsigned q = bk.x * BULK_THREADS + threadIdx.x;
+    active = q < per_plane;
+    q = min(q, per_plane - 1);          // inactive lanes still join the shuffles
+    // q / nxq by row_recip: the truncated reciprocal loses less than q / 2^32
+    // < 1, which the comparison restores
+    unsigned r = __umulhi(q, recip), x = q - r * nxq;
+    if (x >= (unsigned)nxq) {
+        x -= nxq;
+        ++r;
+    }
+    xq = (int)x;
+    y = (int)r;
+}
+
+// No-slip walls (Eq. 4) in the bulk kernels (WALLS instances, for lattices with
+// a non-periodic axis): where the source of direction b lies beyond a wall, the
+// cell takes its own reversed population of step n-1, so a row on a y or z wall
+// reads the reversed direction's plane at its own place, unshifted, and the
+// first and last cell of a row do so on x walls.  A kernel of their own over the
+// wall faces, a thread a cell, took 15 us on a 128 x 64 x 64 channel and 36 us on
+// 100 x 100 x 200 cells (x walls: one 4-byte value a sector), in series with the
+// boundary kernel.
+struct WallRows {
+    bool y0, y1, z0, z1, x;         // this row lies on that wall; the x axis has walls
+    __device__ __forceinline__ bool beyond(int b) const {
+        return (ey(b) > 0 && y0) || (ey(b) < 0 && y1) || (ez(b) > 0 && z0) || (ez(b) < 0 && z1);
+    }
+};
+
+__device__ __forceinline__ WallRows wall_rows(const Domain &d, int y, int z) {
+    return WallRows{!d.py && y == 0, !d.py && y == d.ny - 1, !d.pz && z == 0, !d.pz && z == d.nz - 1, !d.px};
+}
+
+// cells the bulk kernels write: all but the fluid cells the remap listed for
+// the boundary kernel
+__device__ __forceinline__ bool bulk_cell(uint8_t f) { return (f & F_SOLID) || !(f & F_LISTED); }
+
+template <typename T, int V, bool WALLS, bool TILE = false>
 __device__ __forceinline__ void bulk_body(const Device &dv, const StepPtrs &sp, const Blk &bk) {
     using Cd = typename Codec<T>::C;
     const Domain d = dv.dom;
     const int nxq = d.nx / V;
     int xq, y;
     bool active;
-    if constexpr (FLAT) {
-        // the z-plane's V-cell groups in row order, BX * BY a block: a warp's
-        // lanes may cross a row end, where the x-neighbour fallbacks below
-        // (first and last cell of a row) take over from the shuffles
-        const int per_plane = nxq * d.ny;
-        int q = bk.x * (BX * BY) + threadIdx.y * BX + threadIdx.x;
-        active = q < per_plane;
-        q = min(q, per_plane - 1);
-        xq = q % nxq;
-        y = q / nxq;
-    } else {
-        xq = bk.x * BX + threadIdx.x;
-        y = bk.y * BY + threadIdx.y;
-        active = xq < nxq && y < d.ny;
+    if constexpr (TILE) {
+        // one TILE_X-cell tile of a row a block (the near kernel)
+        xq = bk.x * TILE_X + threadIdx.x;
+        y = bk.y;
+        active = xq < nxq;
         xq = min(xq, nxq - 1);          // inactive lanes still join the shuffles
-        y = min(y, d.ny - 1);
+    } else {
+        plane_group(bk, nxq, d.ny, sp.row_recip, xq, y, active);
     }
     const int z = bk.z;
     const int lane = threadIdx.x & 31;
@@ -455,12 +495,15 @@ __device__ __forceinline__ void bulk_body(const Device &dv, const StepPtrs &sp, 
         else return Codec<T>::ld(v, inv_scale);
     };
 
+    const WallRows wr = wall_rows(d, y, z);
     Cd f[Q][V];
 #pragma unroll
     for (int b = 0; b < Q; ++b) {
         const int ys = ey(b) > 0 ? ym : (ey(b) < 0 ? yp : y);
         const int zs = ez(b) > 0 ? zm : (ez(b) < 0 ? zp : z);
-        const T *row = src + (long long)b * C + ((long long)zs * d.ny + ys) * d.nx;
+        const bool own = WALLS && wr.beyond(b);
+        const T *row = own ? src + (long long)opp(b) * C + (c0 - x0)
+                           : src + (long long)b * C + ((long long)zs * d.ny + ys) * d.nx;
         T A[V];
         load_vec<T, V>(row + x0, A);
         if (ex(b) == 0) {
@@ -468,16 +511,22 @@ __device__ __forceinline__ void bulk_body(const Device &dv, const StepPtrs &sp, 
             for (int i = 0; i < V; ++i) f[b][i] = ld(A[i]);
         } else if (ex(b) > 0) {          // pull from x - 1
             T left = shfl(A[V - 1], 1, true);
-            if (lane == 0 || x0 == 0) left = row[x0 == 0 ? d.nx - 1 : x0 - 1];
-            f[b][0] = ld(left);
+            if (lane == 0 || x0 == 0) {
+                if (WALLS && wr.x && x0 == 0) left = src[(long long)opp(b) * C + c0];
+                else left = row[x0 == 0 ? d.nx - 1 : x0 - 1];
+            }
+            f[b][0] = ld(own ? A[0] : left);
 #pragma unroll
-            for (int i = 1; i < V; ++i) f[b][i] = ld(A[i - 1]);
+            for (int i = 1; i < V; ++i) f[b][i] = ld(own ? A[i] : A[i - 1]);
         } else {                          // pull from x + 1
             T right = shfl(A[0], 1, false);
-            if (lane == 31 || x0 + V == d.nx) right = row[x0 + V == d.nx ? 0 : x0 + V];
+            if (lane == 31 || x0 + V == d.nx) {
+                if (WALLS && wr.x && x0 + V == d.nx) right = src[(long long)opp(b) * C + c0 + V - 1];
+                else right = row[x0 + V == d.nx ? 0 : x0 + V];
+            }
 #pragma unroll
-            for (int i = 0; i < V - 1; ++i) f[b][i] = ld(A[i + 1]);
-            f[b][V - 1] = ld(right);
+            for (int i = 0; i < V - 1; ++i) f[b][i] = ld(own ? A[i] : A[i + 1]);
+            f[b][V - 1] = ld(own ? A[V - 1] : right);
         }
     }
 
@@ -504,11 +553,11 @@ __device__ __forceinline__ void bulk_body(const Device &dv, const StepPtrs &sp, 
         if constexpr (raw16) return store16<T>(v, dz, b);
         else return Codec<T>::st(v, scale);
     };
-    // fluid cells with a non-zero flag byte belong to the boundary kernel,
-    // which may run concurrently: leave them alone
+    // listed fluid cells belong to the boundary kernel, which may run
+    // concurrently: leave them alone
     bool all_mine = true;
 #pragma unroll
-    for (int i = 0; i < V; ++i) all_mine = all_mine && (fl[i] == 0 || (fl[i] & F_SOLID));
+    for (int i = 0; i < V; ++i) all_mine = all_mine && bulk_cell(fl[i]);
     if (all_mine) {
 #pragma unroll
         for (int b = 0; b < Q; ++b) {
@@ -523,16 +572,16 @@ __device__ __forceinline__ void bulk_body(const Device &dv, const StepPtrs &sp, 
     for (int b = 0; b < Q; ++b)
 #pragma unroll
         for (int i = 0; i < V; ++i)
-            if (fl[i] == 0 || (fl[i] & F_SOLID)) dst[(long long)b * C + c0 + i] = st(f[b][i], b);
+            if (bulk_cell(fl[i])) dst[(long long)b * C + c0 + i] = st(f[b][i], b);
 }
 
 // MINB == 1 leaves the register budget to the compiler (an explicit minimum
 // of one block lets it spend far more registers than it needs)
-template <typename T, int V, int BX, int BY, int MINB>
-__global__ void __launch_bounds__(BX * BY, MINB == 1 ? 0 : MINB)
+template <typename T, int V, int MINB, bool WALLS>
+__global__ void __launch_bounds__(BULK_THREADS, MINB == 1 ? 0 : MINB)
 bulk_kernel(const Device dv, const StepPtrs sp) {
     pdl_enter();
-    bulk_body<T, V, BX, BY>(dv, sp, launch_blk());
+    bulk_body<T, V, WALLS>(dv, sp, launch_blk());
 }
 
 // a batched bulk block takes BATCH_PZ consecutive z-planes of its member:
@@ -540,14 +589,14 @@ bulk_kernel(const Device dv, const StepPtrs sp) {
 // no population traffic in flight) is paid once for all of them
 constexpr int BATCH_PZ = 4;
 
-template <typename T, int V, int BX, int BY, int MINB>
-__global__ void __launch_bounds__(BX * BY, MINB == 1 ? 0 : MINB) bulk_batch(const Batch bt) {
+template <typename T, int V, int MINB, bool WALLS>
+__global__ void __launch_bounds__(BULK_THREADS, MINB == 1 ? 0 : MINB) bulk_batch(const Batch bt) {
     LBM_BATCH_MEMBER(bt);
     const int z0 = sbk.z * BATCH_PZ, z1 = min(z0 + BATCH_PZ, sdv.dom.nz);
     for (int z = z0; z < z1; ++z) {
         Blk pb = sbk;
         pb.z = z;
-        bulk_body<T, V, BX, BY, true>(sdv, ssp, pb);
+        bulk_body<T, V, WALLS>(sdv, ssp, pb);
     }
 }
 
@@ -583,7 +632,7 @@ template <typename T> __device__ __forceinline__ unsigned store_bits(float v, co
 // shuffled from the neighbouring lane); a cell's 19 values are widened to
 // FP32 just before its collision (collide_lean, the row-staged kernel's
 // arithmetic) and narrowed back into their half-words after it.
-template <typename T, int V, int BX, int BY, bool FLAT = false>
+template <typename T, int V, bool WALLS>
 __device__ __forceinline__ void bulk16_body(const Device &dv, const StepPtrs &sp, const Blk &bk) {
     static_assert(sizeof(T) == 2 && V % 2 == 0, "two 16-bit cells a word");
     constexpr int W = V / 2;
@@ -592,23 +641,7 @@ __device__ __forceinline__ void bulk16_body(const Device &dv, const StepPtrs &sp
     const int nxq = d.nx / V;
     int xq, y;
     bool active;
-    if constexpr (FLAT) {
-        // the z-plane's V-cell groups in row order, BX * BY a block: a warp's
-        // lanes may cross a row end, where the x-neighbour fallbacks below
-        // (first and last cell of a row) take over from the shuffles
-        const int per_plane = nxq * d.ny;
-        int q = bk.x * (BX * BY) + threadIdx.y * BX + threadIdx.x;
-        active = q < per_plane;
-        q = min(q, per_plane - 1);
-        xq = q % nxq;
-        y = q / nxq;
-    } else {
-        xq = bk.x * BX + threadIdx.x;
-        y = bk.y * BY + threadIdx.y;
-        active = xq < nxq && y < d.ny;
-        xq = min(xq, nxq - 1);          // inactive lanes still join the shuffles
-        y = min(y, d.ny - 1);
-    }
+    plane_group(bk, nxq, d.ny, sp.row_recip, xq, y, active);
     const int z = bk.z;
     const int lane = threadIdx.x & 31;
     const int x0 = xq * V;
@@ -622,12 +655,15 @@ __device__ __forceinline__ void bulk16_body(const Device &dv, const StepPtrs &sp
     uint8_t fl[V];
     load_vec<uint8_t, V>(sp.flags_cur + c0, fl);
 
+    const WallRows wr = wall_rows(d, y, z);
     unsigned w[Q][W];
 #pragma unroll
     for (int b = 0; b < Q; ++b) {
         const int ys = ey(b) > 0 ? ym : (ey(b) < 0 ? yp : y);
         const int zs = ez(b) > 0 ? zm : (ez(b) < 0 ? zp : z);
-        const unsigned short *row = src + (long long)b * C + ((long long)zs * d.ny + ys) * d.nx;
+        const bool own = WALLS && wr.beyond(b);
+        const unsigned short *row = own ? src + (long long)opp(b) * C + (c0 - x0)
+                                        : src + (long long)b * C + ((long long)zs * d.ny + ys) * d.nx;
         unsigned R[W];
         {
             const RawV r = __ldg(reinterpret_cast<const RawV *>(row + x0));
@@ -638,16 +674,22 @@ __device__ __forceinline__ void bulk16_body(const Device &dv, const StepPtrs &sp
             for (int j = 0; j < W; ++j) w[b][j] = R[j];
         } else if (ex(b) > 0) {          // pull from x - 1: the left neighbour's last half-word first
             unsigned lw = __shfl_up_sync(0xffffffffu, R[W - 1], 1);
-            if (lane == 0 || x0 == 0) lw = (unsigned)row[x0 == 0 ? d.nx - 1 : x0 - 1] << 16;
-            w[b][0] = __byte_perm(lw, R[0], 0x5432);
+            if (lane == 0 || x0 == 0) {
+                if (WALLS && wr.x && x0 == 0) lw = (unsigned)src[(long long)opp(b) * C + c0] << 16;
+                else lw = (unsigned)row[x0 == 0 ? d.nx - 1 : x0 - 1] << 16;
+            }
+            w[b][0] = own ? R[0] : __byte_perm(lw, R[0], 0x5432);
 #pragma unroll
-            for (int j = 1; j < W; ++j) w[b][j] = __byte_perm(R[j - 1], R[j], 0x5432);
+            for (int j = 1; j < W; ++j) w[b][j] = own ? R[j] : __byte_perm(R[j - 1], R[j], 0x5432);
         } else {                          // pull from x + 1: the right neighbour's first half-word last
             unsigned rw = __shfl_down_sync(0xffffffffu, R[0], 1);
-            if (lane == 31 || x0 + V == d.nx) rw = (unsigned)row[x0 + V == d.nx ? 0 : x0 + V];
+            if (lane == 31 || x0 + V == d.nx) {
+                if (WALLS && wr.x && x0 + V == d.nx) rw = (unsigned)src[(long long)opp(b) * C + c0 + V - 1];
+                else rw = (unsigned)row[x0 + V == d.nx ? 0 : x0 + V];
+            }
 #pragma unroll
-            for (int j = 0; j < W - 1; ++j) w[b][j] = __byte_perm(R[j], R[j + 1], 0x5432);
-            w[b][W - 1] = __byte_perm(R[W - 1], rw, 0x5432);
+            for (int j = 0; j < W - 1; ++j) w[b][j] = own ? R[j] : __byte_perm(R[j], R[j + 1], 0x5432);
+            w[b][W - 1] = own ? R[W - 1] : __byte_perm(R[W - 1], rw, 0x5432);
         }
     }
 
@@ -678,11 +720,11 @@ __device__ __forceinline__ void bulk16_body(const Device &dv, const StepPtrs &sp
     const bool far = !sp.far_skip || sp.far_skip[((long long)z * d.ny + y) * ((d.nx + TILE_X - 1) / TILE_X) +
                                                  x0 / TILE_X] == 0u;
     if (!active || !far) return;
-    // fluid cells with a non-zero flag byte belong to the boundary kernel,
-    // which may run concurrently: leave them alone
+    // listed fluid cells belong to the boundary kernel, which may run
+    // concurrently: leave them alone
     bool all_mine = true;
 #pragma unroll
-    for (int i = 0; i < V; ++i) all_mine = all_mine && (fl[i] == 0 || (fl[i] & F_SOLID));
+    for (int i = 0; i < V; ++i) all_mine = all_mine && bulk_cell(fl[i]);
     if (all_mine) {
 #pragma unroll
         for (int b = 0; b < Q; ++b) {
@@ -696,25 +738,25 @@ __device__ __forceinline__ void bulk16_body(const Device &dv, const StepPtrs &sp
     for (int b = 0; b < Q; ++b)
 #pragma unroll
         for (int i = 0; i < V; ++i)
-            if (fl[i] == 0 || (fl[i] & F_SOLID))
+            if (bulk_cell(fl[i]))
                 dst[(long long)b * C + c0 + i] = (unsigned short)((i & 1) ? w[b][i >> 1] >> 16 : w[b][i >> 1] & 0xffffu);
 }
 
-template <typename T, int V, int BX, int BY, int MINB>
-__global__ void __launch_bounds__(BX * BY, MINB == 1 ? 0 : MINB)
+template <typename T, int V, int MINB, bool WALLS>
+__global__ void __launch_bounds__(BULK_THREADS, MINB == 1 ? 0 : MINB)
 bulk16_kernel(const Device dv, const StepPtrs sp) {
     pdl_enter();
-    bulk16_body<T, V, BX, BY>(dv, sp, launch_blk());
+    bulk16_body<T, V, WALLS>(dv, sp, launch_blk());
 }
 
-template <typename T, int V, int BX, int BY, int MINB>
-__global__ void __launch_bounds__(BX * BY, MINB == 1 ? 0 : MINB) bulk16_batch(const Batch bt) {
+template <typename T, int V, int MINB, bool WALLS>
+__global__ void __launch_bounds__(BULK_THREADS, MINB == 1 ? 0 : MINB) bulk16_batch(const Batch bt) {
     LBM_BATCH_MEMBER(bt);
     const int z0 = sbk.z * BATCH_PZ, z1 = min(z0 + BATCH_PZ, sdv.dom.nz);
     for (int z = z0; z < z1; ++z) {
         Blk pb = sbk;
         pb.z = z;
-        bulk16_body<T, V, BX, BY, true>(sdv, ssp, pb);
+        bulk16_body<T, V, WALLS>(sdv, ssp, pb);
     }
 }
 
@@ -776,16 +818,14 @@ __device__ inline void wall_velocity_wrapped(const Domain &d, const WallBody &b,
     u[2] = b.v[2] + (b.w[0] * o1 - b.w[1] * o0);
 }
 
-// Cells with a non-zero flag byte: refill, bounce-back at walls and moving
-// obstacles, then LBGK.  mode 0: the cells the remap listed (fluid with
-// F_NEAR or F_SOLID_PREV), one a thread, on a grid sized for the longest
-// possible list; mode 1: block row y = wall face (axis * 2 + side), the
-// face's cells.  A cell in
-// both sets, or listed twice, is computed more than once with the same
-// result.  Every load a cell needs is issued before any of them is used, so
-// a thread waits for memory about twice instead of once per direction.
+// The cells the remap listed (fluid with F_NEAR or F_SOLID_PREV): refill,
+// bounce-back at walls and moving obstacles, then LBGK, one cell a thread on a
+// grid sized for the longest possible list.  A cell listed twice (it lies in
+// two bodies' cubes) is computed twice with the same result.  Every load a cell
+// needs is issued before any of them is used, so a thread waits for memory
+// about twice instead of once per direction.
 template <typename T>
-__device__ __forceinline__ void boundary_body(const Device &dv, const StepPtrs &sp, const Blk &bk, int mode) {
+__device__ __forceinline__ void boundary_body(const Device &dv, const StepPtrs &sp, const Blk &bk) {
     using Cd = typename Codec<T>::C;
     const Domain d = dv.dom;
     // 32/16-bit storage: the bodies of step n-1 with their centres wrapped
@@ -794,36 +834,19 @@ __device__ __forceinline__ void boundary_body(const Device &dv, const StepPtrs &
     __shared__ WallBody wb[sizeof(T) == 8 ? 1 : LBM_MAX_BODIES_DEV];
     const int l = bk.x * blockDim.x + threadIdx.x;
     // the count may pass the capacity after an overflow (reported as an error): never read past it
-    const int listed = mode == 0 ? (int)min((long long)*dv.bcount, dv.blist_cap) : 0;
-    if (mode == 0 && (int)(bk.x * blockDim.x) >= listed) return;      // the whole block is past the list
+    const int listed = (int)min((long long)*dv.bcount, dv.blist_cap);
+    if ((int)(bk.x * blockDim.x) >= listed) return;      // the whole block is past the list
     if constexpr (sizeof(T) != 8) {
         for (int k = threadIdx.x; k < dv.nb; k += blockDim.x) wb[k] = wall_body(dv.geom[(sp.parity ^ 1) * dv.nb + k]);
         __syncthreads();
     }
-    int x, y, z;
-    if (mode == 0) {
-        if (l >= listed) return;
-        const unsigned cl = dv.blist[l];          // C < 2^31: 32-bit division
-        const unsigned nxu = (unsigned)d.nx, nyu = (unsigned)d.ny;
-        x = (int)(cl % nxu);
-        y = (int)((cl / nxu) % nyu);
-        z = (int)(cl / (nxu * nyu));
-    } else {
-        const int axis = bk.y >> 1, hi = bk.y & 1;
-        const int n3[3] = {d.nx, d.ny, d.nz}, per[3] = {d.px, d.py, d.pz};
-        if (per[axis]) return;
-        const int ua = axis == 0 ? 1 : 0, va = axis == 2 ? 1 : 2;
-        if (l >= n3[ua] * n3[va]) return;
-        int p[3];
-        p[axis] = hi ? n3[axis] - 1 : 0;
-        p[ua] = l % n3[ua];
-        p[va] = l / n3[ua];
-        x = p[0]; y = p[1]; z = p[2];
-    }
+    if (l >= listed) return;
+    const unsigned cl = dv.blist[l];          // C < 2^31: 32-bit division
+    const unsigned nxu = (unsigned)d.nx, nyu = (unsigned)d.ny;
+    const int x = (int)(cl % nxu), y = (int)((cl / nxu) % nyu), z = (int)(cl / (nxu * nyu));
     const long long C = d.C;
     const long long c = ((long long)z * d.ny + y) * d.nx + x;
     const uint8_t fc = sp.flags_cur[c];
-    if (fc == 0 || (fc & F_SOLID)) return;
     const T *__restrict__ src = static_cast<const T *>(sp.src);
     const float s = dv.f16_inv_scale;
     Cd f[Q];
@@ -928,15 +951,11 @@ __device__ __forceinline__ void boundary_body(const Device &dv, const StepPtrs &
         }
     }
     if constexpr (sizeof(T) != 8) {
-        // rho - 1 of the cell for the momentum exchange (the collision keeps
-        // it); a lattice without bodies has no momentum exchange and no
-        // record (a wall-face cell is listed here all the same)
-        if (dv.nb > 0) {
-            Cd drho = 0;
+        // rho - 1 of the cell for the momentum exchange (the collision keeps it)
+        Cd drho = 0;
 #pragma unroll
-            for (int b = 0; b < Q; ++b) drho += f[b];
-            dv.rho_near[c] = (float)drho;
-        }
+        for (int b = 0; b < Q; ++b) drho += f[b];
+        dv.rho_near[c] = (float)drho;
     }
     collide<T>(f, dv);
     T *__restrict__ dst = static_cast<T *>(sp.dst);
@@ -951,15 +970,14 @@ __device__ __forceinline__ void boundary_body(const Device &dv, const StepPtrs &
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) boundary_kernel(const Device dv, const StepPtrs sp, int mode) {
-    boundary_body<T>(dv, sp, launch_blk(), mode);
+__global__ void __launch_bounds__(256) boundary_kernel(const Device dv, const StepPtrs sp) {
+    boundary_body<T>(dv, sp, launch_blk());
 }
 
-// a batched launch of one mode over the members
 template <typename T>
-__global__ void __launch_bounds__(256) boundary_batch(const Batch bt, int mode) {
+__global__ void __launch_bounds__(256) boundary_batch(const Batch bt) {
     LBM_BATCH_MEMBER(bt);
-    boundary_body<T>(sdv, ssp, sbk, mode);
+    boundary_body<T>(sdv, ssp, sbk);
 }
 
 // ---- TMA row-staged variant ---------------------------------------------------
@@ -1057,8 +1075,10 @@ __global__ void __launch_bounds__(TMA_THREADS, MINB) bulk_tma_kernel(const Devic
 #pragma unroll
             for (int b = 0; b < Q; ++b) {
                 const int ys = wrap_axis(y - ey(b), d.ny), zs = wrap_axis(z - ez(b), d.nz);
-                bulk_copy(buf + b * row_bytes, src + (long long)b * C + ((long long)zs * d.ny + ys) * nx,
-                          row_bytes, &bar[st]);
+                const T *from = wall_rows(d, y, z).beyond(b)      // Eq. 4: the row's own reversed populations
+                                    ? src + (long long)opp(b) * C + r * nx
+                                    : src + (long long)b * C + ((long long)zs * d.ny + ys) * nx;
+                bulk_copy(buf + b * row_bytes, from, row_bytes, &bar[st]);
             }
             bulk_copy(buf + flag_off, sp.flags_cur + r * nx, (unsigned)nx, &bar[st]);
         }
@@ -1089,9 +1109,10 @@ __global__ void __launch_bounds__(TMA_THREADS, MINB) bulk_tma_kernel(const Devic
             const uint8_t *fl = buf + flag_off;
             const long long r = first + (g * ROWS + rr) * gridDim.x;
             const long long c0 = r * nx;
+            const WallRows wr = wall_rows(d, (int)(r % d.ny), (int)(r / d.ny));
             for (int x = threadIdx.x; x < nx; x += TMA_THREADS) {
                 const uint8_t f8 = fl[x];
-                if (f8 != 0 && !(f8 & F_SOLID)) continue;      // the boundary kernel's cell
+                if (!bulk_cell(f8)) continue;                  // the boundary kernel's cell
                 if (sp.far_skip && sp.far_skip[r * ntx + x / TILE_X]) continue;    // the near kernel's
                 if (f8 & F_SOLID) {
 #pragma unroll
@@ -1102,9 +1123,13 @@ __global__ void __launch_bounds__(TMA_THREADS, MINB) bulk_tma_kernel(const Devic
 #pragma unroll
                 for (int b = 0; b < Q; ++b) {
                     int xs = x - ex(b);
+                    const bool out = xs < 0 || xs >= nx;
                     xs = xs < 0 ? xs + nx : (xs >= nx ? xs - nx : xs);
-                    if constexpr (sizeof(T) == 2) f[b] = raw_ld<T>(rowb[b * nx + xs]);
-                    else f[b] = Codec<T>::ld(rowb[b * nx + xs], inv_scale);
+                    if (wr.beyond(b)) xs = x;
+                    T v = rowb[b * nx + xs];
+                    if (out && wr.x) v = src[(long long)opp(b) * C + c0 + x];
+                    if constexpr (sizeof(T) == 2) f[b] = raw_ld<T>(v);
+                    else f[b] = Codec<T>::ld(v, inv_scale);
                 }
                 if constexpr (sizeof(T) == 2) {
                     collide_lean<std::is_same<T, __half>::value>(f, dv);
@@ -1170,34 +1195,23 @@ void tma_prepare() {
                          227 * 1024);
 }
 
-template <typename T, int V, int BX, int BY, int MINB>
-void launch_bulk(const Device &dv, const StepPtrs &sp, cudaStream_t s) {
-    const int nxq = dv.dom.nx / V;
-    dim3 grid((nxq + BX - 1) / BX, (dv.dom.ny + BY - 1) / BY, dv.dom.nz);
-    launch_kernel(dv.pdl != 0, bulk_kernel<T, V, BX, BY, MINB>, grid, dim3(BX, BY), 0, s, dv, sp);
-}
-
-template <typename T, int V, int BX, int BY, int MINB>
-void launch_bulk16(const Device &dv, const StepPtrs &sp, cudaStream_t s) {
-    const int nxq = dv.dom.nx / V;
-    dim3 grid((nxq + BX - 1) / BX, (dv.dom.ny + BY - 1) / BY, dv.dom.nz);
-    launch_kernel(dv.pdl != 0, bulk16_kernel<T, V, BX, BY, MINB>, grid, dim3(BX, BY), 0, s, dv, sp);
-}
-
+// launch shapes: V cells per thread in blocks of BULK_THREADS; MINB > 1 caps
+// the registers so that MINB blocks fit an SM.  16-bit storage with an even V
+// takes the packed kernel.
 template <typename T, int V, int MINB>
-void launch_shape16(const Device &dv, const StepPtrs &sp, cudaStream_t s) {
-    const int nxq = dv.dom.nx / V;
-    if (nxq >= 128) launch_bulk16<T, V, 128, 2, MINB>(dv, sp, s);
-    else launch_bulk16<T, V, 32, 8, MINB>(dv, sp, s);
-}
-
-// launch shapes: V cells per thread in blocks of 256 threads (BX a multiple
-// of 32 along x); MINB > 1 caps the registers so that MINB blocks fit an SM
-template <typename T, int V, int MINB>
-void launch_shape(const Device &dv, const StepPtrs &sp, cudaStream_t s) {
-    const int nxq = dv.dom.nx / V;
-    if (nxq >= 128) launch_bulk<T, V, 128, 2, MINB>(dv, sp, s);
-    else launch_bulk<T, V, 32, 8, MINB>(dv, sp, s);
+void launch_shape(const Device &dv, const StepPtrs &ptrs, cudaStream_t s) {
+    const Domain &d = dv.dom;
+    StepPtrs sp = ptrs;
+    sp.row_recip = row_recip(d.nx / V);
+    const long long per_plane = (long long)(d.nx / V) * d.ny;
+    const dim3 grid((unsigned)((per_plane + BULK_THREADS - 1) / BULK_THREADS), 1, d.nz);
+    const bool walls = !(d.px && d.py && d.pz);
+    if constexpr (sizeof(T) == 2 && V % 2 == 0)
+        launch_kernel(dv.pdl != 0, walls ? bulk16_kernel<T, V, MINB, true> : bulk16_kernel<T, V, MINB, false>, grid,
+                      dim3(BULK_THREADS), 0, s, dv, sp);
+    else
+        launch_kernel(dv.pdl != 0, walls ? bulk_kernel<T, V, MINB, true> : bulk_kernel<T, V, MINB, false>, grid,
+                      dim3(BULK_THREADS), 0, s, dv, sp);
 }
 
 using Launcher = void (*)(const Device &, const StepPtrs &, cudaStream_t);
@@ -1216,21 +1230,21 @@ const Variant kVariants[] = {
     {1, 2, 4, launch_shape<float, 2, 4>},
     {1, 1, 1, launch_shape<float, 1, 1>},
     {1, 4, 1, launch_shape<float, 4, 1>},
-    {2, 4, 1, launch_shape16<__half, 4, 1>},
-    {2, 4, 2, launch_shape16<__half, 4, 2>},
-    {2, 4, 3, launch_shape16<__half, 4, 3>},
-    {2, 8, 1, launch_shape16<__half, 8, 1>},
-    {2, 8, 2, launch_shape16<__half, 8, 2>},
-    {2, 2, 1, launch_shape16<__half, 2, 1>},
-    {2, 2, 4, launch_shape16<__half, 2, 4>},
+    {2, 4, 1, launch_shape<__half, 4, 1>},
+    {2, 4, 2, launch_shape<__half, 4, 2>},
+    {2, 4, 3, launch_shape<__half, 4, 3>},
+    {2, 8, 1, launch_shape<__half, 8, 1>},
+    {2, 8, 2, launch_shape<__half, 8, 2>},
+    {2, 2, 1, launch_shape<__half, 2, 1>},
+    {2, 2, 4, launch_shape<__half, 2, 4>},
     {2, 1, 1, launch_shape<__half, 1, 1>},
-    {3, 4, 1, launch_shape16<__nv_bfloat16, 4, 1>},
-    {3, 4, 2, launch_shape16<__nv_bfloat16, 4, 2>},
-    {3, 4, 3, launch_shape16<__nv_bfloat16, 4, 3>},
-    {3, 8, 1, launch_shape16<__nv_bfloat16, 8, 1>},
-    {3, 8, 2, launch_shape16<__nv_bfloat16, 8, 2>},
-    {3, 2, 1, launch_shape16<__nv_bfloat16, 2, 1>},
-    {3, 2, 4, launch_shape16<__nv_bfloat16, 2, 4>},
+    {3, 4, 1, launch_shape<__nv_bfloat16, 4, 1>},
+    {3, 4, 2, launch_shape<__nv_bfloat16, 4, 2>},
+    {3, 4, 3, launch_shape<__nv_bfloat16, 4, 3>},
+    {3, 8, 1, launch_shape<__nv_bfloat16, 8, 1>},
+    {3, 8, 2, launch_shape<__nv_bfloat16, 8, 2>},
+    {3, 2, 1, launch_shape<__nv_bfloat16, 2, 1>},
+    {3, 2, 4, launch_shape<__nv_bfloat16, 2, 4>},
     {3, 1, 1, launch_shape<__nv_bfloat16, 1, 1>},
     {0, -1, 1, launch_tma<double, 2, 1>, tma_fits<double, 2, 1>},
     {1, -1, 1, launch_tma<float, 4, 1>, tma_fits<float, 4, 1>},
@@ -1254,18 +1268,10 @@ const Variant *find_variant(int precision, int vec, int minb) {
 
 template <typename T>
 void launch_boundary(const Device &dv, const StepPtrs &sp, cudaStream_t s) {
-    if (dv.nb > 0) {
-        // the list's length is on the device: blocks past it return at once
-        const long long side = dv.remap_side;
-        const long long most = (long long)dv.nb * side * side * side;
-        const unsigned bx = (unsigned)((most + 255) / 256);
-        boundary_kernel<T><<<bx, 256, 0, s>>>(dv, sp, 0);
-    }
-    if (!(dv.dom.px && dv.dom.py && dv.dom.pz)) {
-        const long long nx = dv.dom.nx, ny = dv.dom.ny, nz = dv.dom.nz;
-        const long long area = std::max(ny * nz, std::max(nx * nz, nx * ny));
-        boundary_kernel<T><<<dim3((unsigned)((area + 255) / 256), 6), 256, 0, s>>>(dv, sp, 1);
-    }
+    // the list's length is on the device: blocks past it return at once
+    const long long side = dv.remap_side;
+    const long long most = (long long)dv.nb * side * side * side;
+    boundary_kernel<T><<<(unsigned)((most + 255) / 256), 256, 0, s>>>(dv, sp);
 }
 
 }  // namespace
@@ -1337,7 +1343,7 @@ void launch_boundary_fix(const Device &dv, const StepPtrs &sp, cudaStream_t s) {
 namespace {
 
 // one listed near tile of the step a block (TILE_X threads, one cell each):
-// the bulk kernel's arithmetic on the cells whose flag byte is zero or solid
+// the bulk kernel's arithmetic on the cells that are not listed
 // (the same bits as any launch shape of it)
 template <typename T>
 __global__ void __launch_bounds__(TILE_X) near_bulk_kernel(const Device dv, const StepPtrs sp) {
@@ -1348,7 +1354,7 @@ __global__ void __launch_bounds__(TILE_X) near_bulk_kernel(const Device dv, cons
     const Blk bk{t % ntx, row % dv.dom.ny, row / dv.dom.ny, ntx, dv.dom.ny, dv.dom.nz};
     StepPtrs own = sp;
     own.far_skip = nullptr;
-    bulk_body<T, 1, TILE_X, 1>(dv, own, bk);
+    bulk_body<T, 1, true, true>(dv, own, bk);
 }
 
 }  // namespace
@@ -1367,19 +1373,20 @@ void launch_near_bulk(const Device &dv, const StepPtrs &sp, cudaStream_t s) {
 
 namespace {
 
-constexpr int BATCH_BX = 32, BATCH_BY = 8;      // 256 threads a block, a plane's cells in row order
-
 template <typename T, int V, int MINB = 1>
-void bulk_batch_launch(const Batch &bt, unsigned blocks, cudaStream_t s) {
-    if constexpr (sizeof(T) == 2 && V % 2 == 0)
-        bulk16_batch<T, V, BATCH_BX, BATCH_BY, MINB><<<blocks, dim3(BATCH_BX, BATCH_BY), 0, s>>>(bt);
-    else
-        bulk_batch<T, V, BATCH_BX, BATCH_BY, MINB><<<blocks, dim3(BATCH_BX, BATCH_BY), 0, s>>>(bt);
+void bulk_batch_launch(const Batch &bt, unsigned blocks, bool walls, cudaStream_t s) {
+    if constexpr (sizeof(T) == 2 && V % 2 == 0) {
+        if (walls) bulk16_batch<T, V, MINB, true><<<blocks, BULK_THREADS, 0, s>>>(bt);
+        else bulk16_batch<T, V, MINB, false><<<blocks, BULK_THREADS, 0, s>>>(bt);
+    } else {
+        if (walls) bulk_batch<T, V, MINB, true><<<blocks, BULK_THREADS, 0, s>>>(bt);
+        else bulk_batch<T, V, MINB, false><<<blocks, BULK_THREADS, 0, s>>>(bt);
+    }
 }
 
 struct BatchShape {
     int precision, vec;
-    void (*fn)(const Batch &, unsigned, cudaStream_t);
+    void (*fn)(const Batch &, unsigned, bool, cudaStream_t);
 };
 
 // per precision, index 0 and 1 are one and two cells a thread (the
@@ -1419,41 +1426,35 @@ void batch_grid_cells(const Device &dv, int k, int variant, int g[3]) {
         const long long side = dv.remap_side;
         g[0] = (int)((dv.nb * side * side * side + 255) / 256);
         g[1] = g[2] = 1;
-    } else if (k == BK_WALLS && !(d.px && d.py && d.pz)) {
-        const long long nx = d.nx, ny = d.ny, nz = d.nz;
-        const long long area = std::max(ny * nz, std::max(nx * nz, nx * ny));
-        g[0] = (int)((area + 255) / 256);
-        g[1] = 6;
-        g[2] = 1;
     } else if (k == BK_BULK) {
         const BatchShape *b = batch_shape(dv.precision, variant);
         if (!b || d.nx % b->vec) return;
         // a z-plane's V-cell groups in row order (no lanes idle at row ends),
         // BATCH_PZ planes a block
-        g[0] = (int)(((long long)(d.nx / b->vec) * d.ny + BATCH_BX * BATCH_BY - 1) / (BATCH_BX * BATCH_BY));
+        g[0] = (int)(((long long)(d.nx / b->vec) * d.ny + BULK_THREADS - 1) / BULK_THREADS);
         g[1] = 1;
         g[2] = (d.nz + BATCH_PZ - 1) / BATCH_PZ;
     }
 }
 
-void launch_batch_cells(int k, int variant, const Batch &bt, unsigned blocks, int precision, cudaStream_t s) {
+void launch_batch_cells(int k, int variant, const Batch &bt, unsigned blocks, int precision, bool walls,
+                        cudaStream_t s) {
     if (blocks == 0) return;
     if (k == BK_BULK) {
         const BatchShape *b = batch_shape(precision, variant);
-        if (b) b->fn(bt, blocks, s);
+        if (b) b->fn(bt, blocks, walls, s);
         return;
     }
-    const int mode = k == BK_WALLS ? 1 : 0;
     switch (precision) {
-    case 0: boundary_batch<double><<<blocks, 256, 0, s>>>(bt, mode); break;
-    case 1: boundary_batch<float><<<blocks, 256, 0, s>>>(bt, mode); break;
-    case 2: boundary_batch<__half><<<blocks, 256, 0, s>>>(bt, mode); break;
-    default: boundary_batch<__nv_bfloat16><<<blocks, 256, 0, s>>>(bt, mode); break;
+    case 0: boundary_batch<double><<<blocks, 256, 0, s>>>(bt); break;
+    case 1: boundary_batch<float><<<blocks, 256, 0, s>>>(bt); break;
+    case 2: boundary_batch<__half><<<blocks, 256, 0, s>>>(bt); break;
+    default: boundary_batch<__nv_bfloat16><<<blocks, 256, 0, s>>>(bt); break;
     }
 }
 
 bool needs_boundary_fix(const Device &dv) {
-    return dv.nb > 0 || !(dv.dom.px && dv.dom.py && dv.dom.pz);
+    return dv.nb > 0;
 }
 
 }  // namespace lbm
