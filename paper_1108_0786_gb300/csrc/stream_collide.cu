@@ -266,62 +266,165 @@ __device__ __forceinline__ void collide_f64(double (&f)[Q], const Device &dv) {
     }
 }
 
-// LBGK (+ Guo) of one cell for 16-bit storage, the form with the fewest
-// instructions (these kernels are bound by instruction issue, not by HBM):
-// opposite directions (b, b + 1) are paired, the moments come from pair
-// sums and differences, and each relaxation is one FMA,
-//   f~_b = (1 - omega) f_b + (omega w_b) (a +- c) [+ (1 - omega/2) w_b (s +- t)],
-//   a = drho - 1.5 rho u.u + 4.5 rho (e.u)^2,  c = 3 rho e.u,
-//   s = 9 (e.u)(e.g) - 3 u.g,  t = 3 e.g,
-// the same expression as collide<> (other roundings).  SCALED: f holds
-// k delta (k = f16_scale, a power of two) on entry and exit, so the scale
-// enters only rho, u and the per-cell constants, never a population.
+// Two FP32 values in one 64-bit register pair and the packed FP32 operations of
+// sm_100 and later on them (PTX add / mul / fma .f32x2, each half rounded to
+// nearest like the scalar operation): one issue slot for two cells' arithmetic.
+struct F2 {
+    unsigned long long v;
+};
+__device__ __forceinline__ F2 pack2(float lo, float hi) {
+    F2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ float lo2(F2 a) { return __uint_as_float((unsigned)a.v); }
+__device__ __forceinline__ float hi2(F2 a) { return __uint_as_float((unsigned)(a.v >> 32)); }
+
+// the operations the lean collision is written in, for one cell or two
+__device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float vsub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float vfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ F2 vadd(F2 a, F2 b) {
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 vsub(F2 a, F2 b) {
+    F2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 vmul(F2 a, F2 b) {
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 vfma(F2 a, F2 b, F2 c) {
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+template <typename R> __device__ __forceinline__ R splat(float x);
+template <> __device__ __forceinline__ float splat<float>(float x) { return x; }
+template <> __device__ __forceinline__ F2 splat<F2>(float x) { return pack2(x, x); }
+// a times, or times and plus, a launch constant: two scalar operations on its
+// place in the constant bank, which a packed one would first copy to registers
+__device__ __forceinline__ float vscale(float a, float c) { return __fmul_rn(a, c); }
+__device__ __forceinline__ F2 vscale(F2 a, float c) { return pack2(__fmul_rn(lo2(a), c), __fmul_rn(hi2(a), c)); }
+__device__ __forceinline__ float vscale_add(float a, float c, float b) { return __fmaf_rn(a, c, b); }
+__device__ __forceinline__ F2 vscale_add(F2 a, float c, F2 b) {
+    return pack2(__fmaf_rn(lo2(a), c, lo2(b)), __fmaf_rn(hi2(a), c, hi2(b)));
+}
+__device__ __forceinline__ float vplus(float a, float c) { return __fadd_rn(a, c); }
+__device__ __forceinline__ F2 vplus(F2 a, float c) { return pack2(__fadd_rn(lo2(a), c), __fadd_rn(hi2(a), c)); }
+__device__ __forceinline__ float vrcp(float a) { return __frcp_rn(a); }
+__device__ __forceinline__ F2 vrcp(F2 a) { return pack2(__frcp_rn(lo2(a)), __frcp_rn(hi2(a))); }
+
+// e_b . (x, y, z) for odd b, whose first non-zero component is +1
+template <typename R>
+__device__ __forceinline__ R vdot(int b, R x, R y, R z) {
+    const R first = ex(b) ? x : (ey(b) ? y : z);
+    if (b < 7) return first;
+    const R second = ez(b) ? z : y;
+    return (ez(b) ? ez(b) : ey(b)) > 0 ? vadd(first, second) : vsub(first, second);
+}
+
+// LBGK (+ Guo) for 16-bit storage in the form with the fewest instructions
+// (these kernels are bound by instruction issue before HBM), for one cell
+// (R = float) or two (R = F2) with the same bits.  Opposite directions
+// (b, b + 1) are paired: the moments come from pair sums and differences, and
+//   f~_b = ((1 - omega) f_b + a) +- C e.u,
+//   a = omega w (drho - 1.5 rho u.u + 4.5 rho (e.u)^2),  C = 3 omega w rho
+//   (+ (1 - omega/2) w (9 (e.u)(e.g) - 3 u.g +- 3 e.g) with forcing).
+// SCALED: the populations are k delta (k = f16_scale, a power of two) on entry
+// and exit, so the scale enters only rho, u and the per-cell constants, never a
+// population.  Use: rest(f_0), pair(f_b, f_b+1) for the nine pairs in order,
+// solve(), then relax0 and relax for the populations.
+template <typename R, bool SCALED>
+struct Lean {
+    R s, jx, jy, jz;        // sum of delta, momentum; after solve(): u in jx, jy, jz
+    R base;                 // k (drho - 1.5 rho u.u)
+    R kr;                   // k rho
+    R ug3;                  // -3 k u.g (forcing)
+    R b, A, C, N;           // a = A (e.u)^2 + b, C and -C of the weight class at hand
+
+    __device__ __forceinline__ void rest(R f0) { s = f0; }
+    __device__ __forceinline__ void pair(int p, R f1, R f2) {
+        const int b = 2 * p + 1;
+        s = vadd(s, vadd(f1, f2));
+        const R d = vsub(f1, f2);
+        if (ex(b)) jx = p == 0 ? d : vadd(jx, d);
+        if (ey(b)) jy = p == 1 ? d : (ey(b) > 0 ? vadd(jy, d) : vsub(jy, d));
+        if (ez(b)) jz = p == 2 ? d : (ez(b) > 0 ? vadd(jz, d) : vsub(jz, d));
+    }
+    __device__ __forceinline__ void solve(const Device &dv) {
+        const float k = SCALED ? dv.f16_scale : 1.0f, ik = SCALED ? dv.f16_inv_scale : 1.0f;
+        const bool forced = dv.forced;
+        if (forced) {
+            const float kh = 0.5f * k;
+            jx = vplus(jx, kh * dv.g_f[0]);
+            jy = vplus(jy, kh * dv.g_f[1]);
+            jz = vplus(jz, kh * dv.g_f[2]);
+        }
+        const R rho = vplus(SCALED ? vscale(s, ik) : s, 1.0f);
+        R inv = vrcp(rho);
+        if (SCALED) inv = vscale(inv, ik);
+        jx = vmul(jx, inv);
+        jy = vmul(jy, inv);
+        jz = vmul(jz, inv);
+        const R usq = vfma(jx, jx, vfma(jy, jy, vmul(jz, jz)));
+        kr = SCALED ? vscale(rho, k) : rho;
+        base = vfma(vscale(kr, -1.5f), usq, s);
+        if (forced)
+            ug3 = vscale_add(jx, -3.0f * k * dv.g_f[0],
+                             vscale_add(jy, -3.0f * k * dv.g_f[1], vscale(jz, -3.0f * k * dv.g_f[2])));
+    }
+    // the factors of weight class wc (1: axes, 2: diagonals)
+    __device__ __forceinline__ void weights(int wc, const Device &dv) {
+        const float ow = dv.ow_f[wc];
+        b = vscale(base, ow);
+        if (dv.forced) b = vscale_add(ug3, dv.gw_f[wc], b);
+        A = vscale(kr, 4.5f * ow);
+        C = vscale(kr, 3.0f * ow);
+        N = vscale(kr, -3.0f * ow);
+    }
+    __device__ __forceinline__ R relax0(R f0, const Device &dv) const {
+        R r = vscale_add(f0, dv.om1_f, vscale(base, dv.ow_f[0]));
+        if (dv.forced) r = vscale_add(ug3, dv.gw_f[0], r);
+        return r;
+    }
+    // pair p; the weights of its class are set before the class's first pair
+    __device__ __forceinline__ void relax(int p, R &f1, R &f2, const Device &dv) {
+        if (p == 0) weights(1, dv);
+        if (p == 3) weights(2, dv);
+        const int i = 2 * p + 1;
+        const R eu = vdot(i, jx, jy, jz), om1 = splat<R>(dv.om1_f);
+        R a = vfma(A, vmul(eu, eu), b);
+        if (dv.forced) {
+            const float k = SCALED ? dv.f16_scale : 1.0f;
+            const float eg = edot(i, dv.g_f[0], dv.g_f[1], dv.g_f[2]), gw = dv.gw_f[p < 3 ? 1 : 2];
+            a = vscale_add(eu, 9.0f * k * gw * eg, a);
+            const float c = 3.0f * k * gw * eg;
+            f1 = vplus(vfma(C, eu, vfma(f1, om1, a)), c);
+            f2 = vplus(vfma(N, eu, vfma(f2, om1, a)), -c);
+        } else {
+            f1 = vfma(C, eu, vfma(f1, om1, a));
+            f2 = vfma(N, eu, vfma(f2, om1, a));
+        }
+    }
+};
+
 template <bool SCALED>
 __device__ __forceinline__ void collide_lean(float (&f)[Q], const Device &dv) {
-    const float k = SCALED ? dv.f16_scale : 1.0f, ik = SCALED ? dv.f16_inv_scale : 1.0f;
-    float s = f[0], jx = 0.0f, jy = 0.0f, jz = 0.0f;
-    float del[Q / 2];
+    Lean<float, SCALED> c;
+    c.rest(f[0]);
 #pragma unroll
-    for (int p = 0; p < Q / 2; ++p) {
-        const int b = 2 * p + 1;
-        s += f[b] + f[b + 1];
-        del[p] = f[b] - f[b + 1];
-        if (ex(b)) jx += ex(b) > 0 ? del[p] : -del[p];
-        if (ey(b)) jy += ey(b) > 0 ? del[p] : -del[p];
-        if (ez(b)) jz += ez(b) > 0 ? del[p] : -del[p];
-    }
-    const float rho = fmaf(s, ik, 1.0f);
-    const float inv = ik / rho;
-    const float kh = 0.5f * k;
-    const float gx = dv.g_f[0], gy = dv.g_f[1], gz = dv.g_f[2];
-    const float ux = fmaf(kh, gx, jx) * inv, uy = fmaf(kh, gy, jy) * inv, uz = fmaf(kh, gz, jz) * inv;
-    const float usq = fmaf(ux, ux, fmaf(uy, uy, uz * uz));
-    const float kr = k * rho;
-    const float base = fmaf(-1.5f * kr, usq, s);       // k (drho - 1.5 rho u.u)
-    const float A = 4.5f * kr, Cc = 3.0f * kr;
-    const float om1 = dv.om1_f;
-    const bool forced = dv.forced;
-    const float ug3 = forced ? -3.0f * k * fmaf(ux, gx, fmaf(uy, gy, uz * gz)) : 0.0f;
-    f[0] = fmaf(om1, f[0], forced ? fmaf(dv.gw_f[0], ug3, dv.ow_f[0] * base) : dv.ow_f[0] * base);
+    for (int p = 0; p < Q / 2; ++p) c.pair(p, f[2 * p + 1], f[2 * p + 2]);
+    c.solve(dv);
+    f[0] = c.relax0(f[0], dv);
 #pragma unroll
-    for (int p = 0; p < Q / 2; ++p) {
-        const int b = 2 * p + 1;
-        const int wc = b < 7 ? 1 : 2;
-        const float eu = edot(b, ux, uy, uz);
-        const float a = fmaf(A, eu * eu, base);
-        const float c = Cc * eu;
-        const float ow = dv.ow_f[wc];
-        float r1 = ow * (a + c), r2 = ow * (a - c);
-        if (forced) {
-            const float eg = edot(b, gx, gy, gz);
-            const float sym = fmaf(9.0f * k * eu, eg, ug3), asym = 3.0f * k * eg;
-            const float gw = dv.gw_f[wc];
-            r1 = fmaf(gw, sym + asym, r1);
-            r2 = fmaf(gw, sym - asym, r2);
-        }
-        f[b] = fmaf(om1, f[b], r1);
-        f[b + 1] = fmaf(om1, f[b + 1], r2);
-    }
+    for (int p = 0; p < Q / 2; ++p) c.relax(p, f[2 * p + 1], f[2 * p + 2], dv);
 }
 
 // the collision of storage type T on its deviations, unscaled
@@ -496,16 +599,20 @@ __device__ __forceinline__ void bulk_body(const Device &dv, const StepPtrs &sp, 
     };
 
     const WallRows wr = wall_rows(d, y, z);
+    // offsets of the rows within a direction's plane (C < 2^31): the planes'
+    // addresses are the same for all threads
+    const unsigned nxu = (unsigned)d.nx;
+    const unsigned rows[3][3] = {{(zm * d.ny + ym) * nxu, (zm * d.ny + y) * nxu, (zm * d.ny + yp) * nxu},
+                                 {(z * d.ny + ym) * nxu, (z * d.ny + y) * nxu, (z * d.ny + yp) * nxu},
+                                 {(zp * d.ny + ym) * nxu, (zp * d.ny + y) * nxu, (zp * d.ny + yp) * nxu}};
     Cd f[Q][V];
 #pragma unroll
     for (int b = 0; b < Q; ++b) {
-        const int ys = ey(b) > 0 ? ym : (ey(b) < 0 ? yp : y);
-        const int zs = ez(b) > 0 ? zm : (ez(b) < 0 ? zp : z);
         const bool own = WALLS && wr.beyond(b);
-        const T *row = own ? src + (long long)opp(b) * C + (c0 - x0)
-                           : src + (long long)b * C + ((long long)zs * d.ny + ys) * d.nx;
+        const T *row = src + (long long)b * C + rows[1 - ez(b)][1 - ey(b)];
+        if (own) row = src + (long long)opp(b) * C + rows[1][1];
         T A[V];
-        load_vec<T, V>(row + x0, A);
+        load_vec<T, V>(row + (unsigned)x0, A);
         if (ex(b) == 0) {
 #pragma unroll
             for (int i = 0; i < V; ++i) f[b][i] = ld(A[i]);
@@ -564,7 +671,7 @@ __device__ __forceinline__ void bulk_body(const Device &dv, const StepPtrs &sp, 
             T out[V];
 #pragma unroll
             for (int i = 0; i < V; ++i) out[i] = st(f[b][i], b);
-            store_vec<T, V>(dst + (long long)b * C + c0, out);
+            store_vec<T, V>(dst + (long long)b * C + (unsigned)c0, out);
         }
         return;
     }
@@ -600,28 +707,91 @@ __global__ void __launch_bounds__(BULK_THREADS, MINB == 1 ? 0 : MINB) bulk_batch
     }
 }
 
-// 16-bit values packed two to a 32-bit word (the lower address in the low
-// half): widening to FP32 and narrowing back (round to nearest even)
-template <typename T> __device__ __forceinline__ float half_lo(unsigned w);
-template <typename T> __device__ __forceinline__ float half_hi(unsigned w);
-template <typename T> __device__ __forceinline__ unsigned half_bits(float v);
-template <> __device__ __forceinline__ float half_lo<__half>(unsigned w) {
-    return __half2float(__ushort_as_half((unsigned short)(w & 0xffffu)));
+// the two cells of a 32-bit word of 16-bit populations (the lower address in
+// the low half), widened to FP32
+template <typename T> __device__ __forceinline__ F2 widen(unsigned w);
+template <> __device__ __forceinline__ F2 widen<__half>(unsigned w) {
+    const __half2 h = *reinterpret_cast<const __half2 *>(&w);
+    const float2 f = __half22float2(h);
+    return pack2(f.x, f.y);
 }
-template <> __device__ __forceinline__ float half_hi<__half>(unsigned w) {
-    return __half2float(__ushort_as_half((unsigned short)(w >> 16)));
+template <> __device__ __forceinline__ F2 widen<__nv_bfloat16>(unsigned w) {
+    return pack2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
 }
-template <> __device__ __forceinline__ unsigned half_bits<__half>(float v) {
-    return __half_as_ushort(__float2half_rn(v));
+
+// population a of two cells as a stored word: FP16 to nearest, BF16
+// stochastically (the rounded bits are the upper halves of the sums)
+template <typename T> __device__ __forceinline__ unsigned narrow(F2 v, const Dither &d0, const Dither &d1, int a);
+template <> __device__ __forceinline__ unsigned narrow<__half>(F2 v, const Dither &, const Dither &, int) {
+    const __half2 h = __floats2half2_rn(lo2(v), hi2(v));
+    return *reinterpret_cast<const unsigned *>(&h);
 }
-template <> __device__ __forceinline__ float half_lo<__nv_bfloat16>(unsigned w) { return __uint_as_float(w << 16); }
-template <> __device__ __forceinline__ float half_hi<__nv_bfloat16>(unsigned w) {
-    return __uint_as_float(w & 0xffff0000u);
+template <> __device__ __forceinline__ unsigned narrow<__nv_bfloat16>(F2 v, const Dither &d0, const Dither &d1, int a) {
+    return __byte_perm(bf16_sr_word(lo2(v), d0, a), bf16_sr_word(hi2(v), d1, a), 0x7632);
 }
-// the stored bits of population a of a cell: FP16 to nearest, BF16 stochastically
-template <typename T> __device__ __forceinline__ unsigned store_bits(float v, const Dither &d, int a) {
-    if constexpr (std::is_same<T, __nv_bfloat16>::value) return bf16_sr_bits(v, d, a);
-    else return half_bits<T>(v);
+
+// collide the V cells in the words w of a thread (pairs 2j, 2j + 1 in word j)
+template <typename T, int V>
+__device__ __forceinline__ void collide_words(unsigned (&w)[Q][V / 2], const uint8_t (&fl)[V], long long c0,
+                                              const Device &dv, const StepPtrs &sp) {
+#pragma unroll
+    for (int j = 0; j < V / 2; ++j) {
+        Lean<F2, std::is_same<T, __half>::value> c;
+        c.rest(widen<T>(w[0][j]));
+#pragma unroll
+        for (int p = 0; p < Q / 2; ++p) c.pair(p, widen<T>(w[2 * p + 1][j]), widen<T>(w[2 * p + 2][j]));
+        c.solve(dv);
+        // the words are opaque from here, so that the compiler widens them anew
+        // instead of keeping 38 FP32 values
+#pragma unroll
+        for (int b = 0; b < Q; ++b) asm volatile("" : "+r"(w[b][j]));
+        const Dither d0 = dither_for<T>(c0 + 2 * j, sp.tstep), d1 = dither_for<T>(c0 + 2 * j + 1, sp.tstep);
+        // solid cells store 0
+        const unsigned keep = (fl[2 * j] & F_SOLID ? 0u : 0xffffu) | (fl[2 * j + 1] & F_SOLID ? 0u : 0xffff0000u);
+        w[0][j] = narrow<T>(c.relax0(widen<T>(w[0][j]), dv), d0, d1, 0) & keep;
+#pragma unroll
+        for (int p = 0; p < Q / 2; ++p) {
+            F2 f1 = widen<T>(w[2 * p + 1][j]), f2 = widen<T>(w[2 * p + 2][j]);
+            c.relax(p, f1, f2, dv);
+            w[2 * p + 1][j] = narrow<T>(f1, d0, d1, 2 * p + 1) & keep;
+            w[2 * p + 2][j] = narrow<T>(f2, d0, d1, 2 * p + 2) & keep;
+        }
+    }
+}
+
+// store them, but for the cells of a near tile and listed ones
+template <int V>
+__device__ __forceinline__ void store_words(const unsigned (&w)[Q][V / 2], const uint8_t (&fl)[V], bool active, int x0,
+                                            int y, int z, long long c0, const Device &dv, const StepPtrs &sp) {
+    using RawV = typename Raw<2 * V>::type;
+    const Domain &d = dv.dom;
+    const long long C = d.C;
+    unsigned short *__restrict__ dst = static_cast<unsigned short *>(sp.dst);
+    // overlapped steps: a tile near a body is the near kernel's
+    static_assert(TILE_X % V == 0, "a thread's cells lie in one tile");
+    const bool far = !sp.far_skip || sp.far_skip[((long long)z * d.ny + y) * ((d.nx + TILE_X - 1) / TILE_X) +
+                                                 x0 / TILE_X] == 0u;
+    if (!active || !far) return;
+    // listed fluid cells belong to the boundary kernel, which may run
+    // concurrently: leave them alone
+    bool all_mine = true;
+#pragma unroll
+    for (int i = 0; i < V; ++i) all_mine = all_mine && bulk_cell(fl[i]);
+    if (all_mine) {
+#pragma unroll
+        for (int b = 0; b < Q; ++b) {
+            RawV r;
+            memcpy(&r, &w[b], sizeof(r));
+            *reinterpret_cast<RawV *>(reinterpret_cast<char *>(dst + (long long)b * C) + 2u * (unsigned)c0) = r;
+        }
+        return;
+    }
+#pragma unroll
+    for (int b = 0; b < Q; ++b)
+#pragma unroll
+        for (int i = 0; i < V; ++i)
+            if (bulk_cell(fl[i]))
+                dst[(long long)b * C + c0 + i] = (unsigned short)((i & 1) ? w[b][i >> 1] >> 16 : w[b][i >> 1] & 0xffffu);
 }
 
 // The bulk kernel for 16-bit storage, V (even) cells per thread.  The
@@ -629,9 +799,15 @@ template <typename T> __device__ __forceinline__ unsigned store_bits(float v, co
 // in word j) from load to store, half the registers of widened values, so
 // that more warps -- or more bytes per warp -- keep HBM requests in flight.
 // A shift along x is a byte permute of adjacent words (and of one word
-// shuffled from the neighbouring lane); a cell's 19 values are widened to
-// FP32 just before its collision (collide_lean, the row-staged kernel's
-// arithmetic) and narrowed back into their half-words after it.
+// shuffled from the neighbouring lane).  The two cells of a word collide
+// together in packed FP32 arithmetic (Lean<F2>); the words are widened once for
+// the moments and again for the relaxation, so that only one pair's populations
+// are held in FP32 at a time.  Bound by instruction issue and, at 24 warps an SM,
+// by the bytes in flight: 512 x 256 x 256 cells take 428 us in FP16 (6.0 TB/s)
+// and 482 us in BF16 against 449 and 542 us with a cell at a time in scalar
+// arithmetic.  (Copying the sources ahead into shared memory with cp.async, two
+// stages at 16 warps an SM, took 525 and 549 us: the issue-bound part needs the
+// warps.)
 template <typename T, int V, bool WALLS>
 __device__ __forceinline__ void bulk16_body(const Device &dv, const StepPtrs &sp, const Blk &bk) {
     static_assert(sizeof(T) == 2 && V % 2 == 0, "two 16-bit cells a word");
@@ -650,23 +826,33 @@ __device__ __forceinline__ void bulk16_body(const Device &dv, const StepPtrs &sp
     const long long C = d.C;
     const long long c0 = ((long long)z * d.ny + y) * d.nx + x0;
     const unsigned short *__restrict__ src = static_cast<const unsigned short *>(sp.src);
-    unsigned short *__restrict__ dst = static_cast<unsigned short *>(sp.dst);
 
     uint8_t fl[V];
     load_vec<uint8_t, V>(sp.flags_cur + c0, fl);
 
     const WallRows wr = wall_rows(d, y, z);
+    // byte offsets of the rows within a direction's plane (2 C < 2^32): the
+    // planes' addresses are the same for all threads, so an access is a uniform
+    // base and a 32-bit offset
+    const unsigned cy = (unsigned)z * d.ny;
+    const unsigned pitch = 2u * (unsigned)d.nx;
+    const unsigned rows[3][3] = {{(zm * d.ny + ym) * pitch, (zm * d.ny + y) * pitch, (zm * d.ny + yp) * pitch},
+                                 {(cy + ym) * pitch, (cy + y) * pitch, (cy + yp) * pitch},
+                                 {(zp * d.ny + ym) * pitch, (zp * d.ny + y) * pitch, (zp * d.ny + yp) * pitch}};
+    const unsigned xl = 2u * (x0 == 0 ? d.nx - 1 : x0 - 1), xr = 2u * (x0 + V == d.nx ? 0 : x0 + V);
     unsigned w[Q][W];
 #pragma unroll
     for (int b = 0; b < Q; ++b) {
-        const int ys = ey(b) > 0 ? ym : (ey(b) < 0 ? yp : y);
-        const int zs = ez(b) > 0 ? zm : (ez(b) < 0 ? zp : z);
         const bool own = WALLS && wr.beyond(b);
-        const unsigned short *row = own ? src + (long long)opp(b) * C + (c0 - x0)
-                                        : src + (long long)b * C + ((long long)zs * d.ny + ys) * d.nx;
+        const char *plane = reinterpret_cast<const char *>(src + (long long)b * C);
+        unsigned row = rows[1 - ez(b)][1 - ey(b)];
+        if (own) {
+            plane = reinterpret_cast<const char *>(src + (long long)opp(b) * C);
+            row = rows[1][1];
+        }
         unsigned R[W];
         {
-            const RawV r = __ldg(reinterpret_cast<const RawV *>(row + x0));
+            const RawV r = __ldg(reinterpret_cast<const RawV *>(plane + (row + 2u * x0)));
             memcpy(&R, &r, sizeof(R));
         }
         if (ex(b) == 0) {
@@ -676,7 +862,7 @@ __device__ __forceinline__ void bulk16_body(const Device &dv, const StepPtrs &sp
             unsigned lw = __shfl_up_sync(0xffffffffu, R[W - 1], 1);
             if (lane == 0 || x0 == 0) {
                 if (WALLS && wr.x && x0 == 0) lw = (unsigned)src[(long long)opp(b) * C + c0] << 16;
-                else lw = (unsigned)row[x0 == 0 ? d.nx - 1 : x0 - 1] << 16;
+                else lw = (unsigned)__ldg(reinterpret_cast<const unsigned short *>(plane + (row + xl))) << 16;
             }
             w[b][0] = own ? R[0] : __byte_perm(lw, R[0], 0x5432);
 #pragma unroll
@@ -685,7 +871,7 @@ __device__ __forceinline__ void bulk16_body(const Device &dv, const StepPtrs &sp
             unsigned rw = __shfl_down_sync(0xffffffffu, R[0], 1);
             if (lane == 31 || x0 + V == d.nx) {
                 if (WALLS && wr.x && x0 + V == d.nx) rw = (unsigned)src[(long long)opp(b) * C + c0 + V - 1];
-                else rw = (unsigned)row[x0 + V == d.nx ? 0 : x0 + V];
+                else rw = (unsigned)__ldg(reinterpret_cast<const unsigned short *>(plane + (row + xr)));
             }
 #pragma unroll
             for (int j = 0; j < W - 1; ++j) w[b][j] = own ? R[j] : __byte_perm(R[j], R[j + 1], 0x5432);
@@ -693,53 +879,8 @@ __device__ __forceinline__ void bulk16_body(const Device &dv, const StepPtrs &sp
         }
     }
 
-#pragma unroll
-    for (int i = 0; i < V; ++i) {
-        const int j = i >> 1;
-        const bool hi = i & 1;
-        float g[Q];
-#pragma unroll
-        for (int b = 0; b < Q; ++b) g[b] = hi ? half_hi<T>(w[b][j]) : half_lo<T>(w[b][j]);
-        collide_lean<std::is_same<T, __half>::value>(g, dv);
-        const bool solid = fl[i] & F_SOLID;
-        const Dither dz = dither_for<T>(c0 + i, sp.tstep);
-#pragma unroll
-        for (int b = 0; b < Q; ++b) {
-            if constexpr (std::is_same<T, __nv_bfloat16>::value) {
-                // the rounded bits are the upper half of the sum: select them
-                const unsigned h = solid ? 0u : bf16_sr_word(g[b], dz, b);
-                w[b][j] = hi ? __byte_perm(w[b][j], h, 0x7610) : __byte_perm(h, w[b][j], 0x7632);
-            } else {
-                const unsigned h = solid ? 0u : store_bits<T>(g[b], dz, b);
-                w[b][j] = hi ? __byte_perm(w[b][j], h, 0x5410) : __byte_perm(h, w[b][j], 0x7610);
-            }
-        }
-    }
-    // overlapped steps: a tile near a body is the near kernel's
-    static_assert(TILE_X % V == 0, "a thread's cells lie in one tile");
-    const bool far = !sp.far_skip || sp.far_skip[((long long)z * d.ny + y) * ((d.nx + TILE_X - 1) / TILE_X) +
-                                                 x0 / TILE_X] == 0u;
-    if (!active || !far) return;
-    // listed fluid cells belong to the boundary kernel, which may run
-    // concurrently: leave them alone
-    bool all_mine = true;
-#pragma unroll
-    for (int i = 0; i < V; ++i) all_mine = all_mine && bulk_cell(fl[i]);
-    if (all_mine) {
-#pragma unroll
-        for (int b = 0; b < Q; ++b) {
-            RawV r;
-            memcpy(&r, &w[b], sizeof(r));
-            *reinterpret_cast<RawV *>(dst + (long long)b * C + c0) = r;
-        }
-        return;
-    }
-#pragma unroll
-    for (int b = 0; b < Q; ++b)
-#pragma unroll
-        for (int i = 0; i < V; ++i)
-            if (bulk_cell(fl[i]))
-                dst[(long long)b * C + c0 + i] = (unsigned short)((i & 1) ? w[b][i >> 1] >> 16 : w[b][i >> 1] & 0xffffu);
+    collide_words<T, V>(w, fl, c0, dv, sp);
+    store_words<V>(w, fl, active, x0, y, z, c0, dv, sp);
 }
 
 template <typename T, int V, int MINB, bool WALLS>
@@ -1032,7 +1173,7 @@ constexpr int TMA_HEADER = 128;                      // mbarriers, ahead of the 
 
 __host__ __device__ constexpr size_t tma_stage_bytes(int nx, int elem) { return (size_t)Q * nx * elem + (size_t)nx; }
 
-template <typename T, int NSTAGE, int MINB, int ROWS>
+template <typename T, int NSTAGE, int MINB, int ROWS, bool WALLS>
 __global__ void __launch_bounds__(TMA_THREADS, MINB) bulk_tma_kernel(const Device dv, const StepPtrs sp) {
     pdl_enter();
     using Cd = typename Codec<T>::C;
@@ -1075,7 +1216,7 @@ __global__ void __launch_bounds__(TMA_THREADS, MINB) bulk_tma_kernel(const Devic
 #pragma unroll
             for (int b = 0; b < Q; ++b) {
                 const int ys = wrap_axis(y - ey(b), d.ny), zs = wrap_axis(z - ez(b), d.nz);
-                const T *from = wall_rows(d, y, z).beyond(b)      // Eq. 4: the row's own reversed populations
+                const T *from = WALLS && wall_rows(d, y, z).beyond(b)      // Eq. 4: the row's own reversed populations
                                     ? src + (long long)opp(b) * C + r * nx
                                     : src + (long long)b * C + ((long long)zs * d.ny + ys) * nx;
                 bulk_copy(buf + b * row_bytes, from, row_bytes, &bar[st]);
@@ -1125,9 +1266,9 @@ __global__ void __launch_bounds__(TMA_THREADS, MINB) bulk_tma_kernel(const Devic
                     int xs = x - ex(b);
                     const bool out = xs < 0 || xs >= nx;
                     xs = xs < 0 ? xs + nx : (xs >= nx ? xs - nx : xs);
-                    if (wr.beyond(b)) xs = x;
+                    if (WALLS && wr.beyond(b)) xs = x;
                     T v = rowb[b * nx + xs];
-                    if (out && wr.x) v = src[(long long)opp(b) * C + c0 + x];
+                    if (WALLS && out && wr.x) v = src[(long long)opp(b) * C + c0 + x];
                     if constexpr (sizeof(T) == 2) f[b] = raw_ld<T>(v);
                     else f[b] = Codec<T>::ld(v, inv_scale);
                 }
@@ -1180,8 +1321,10 @@ void launch_tma(const Device &dv, const StepPtrs &sp, cudaStream_t s) {
     const size_t bytes = tma_smem_bytes<T, NSTAGE, PER_SM, ROWS>(dv.dom.nx);
     const long long rows = (long long)dv.dom.ny * dv.dom.nz;
     const long long grid = std::min<long long>(rows, (long long)sm_count() * PER_SM);
-    launch_kernel(dv.pdl != 0, bulk_tma_kernel<T, NSTAGE, PER_SM, ROWS>, dim3((unsigned)grid), dim3(TMA_THREADS), bytes,
-                  s, dv, sp);
+    const bool walls = !(dv.dom.px && dv.dom.py && dv.dom.pz);
+    launch_kernel(dv.pdl != 0, walls ? bulk_tma_kernel<T, NSTAGE, PER_SM, ROWS, true>
+                                     : bulk_tma_kernel<T, NSTAGE, PER_SM, ROWS, false>,
+                  dim3((unsigned)grid), dim3(TMA_THREADS), bytes, s, dv, sp);
 }
 
 template <typename T, int NSTAGE, int PER_SM, int ROWS = 1>
@@ -1191,8 +1334,8 @@ bool tma_fits(int nx) {
 
 template <typename T, int NSTAGE, int PER_SM, int ROWS = 1>
 void tma_prepare() {
-    cudaFuncSetAttribute(bulk_tma_kernel<T, NSTAGE, PER_SM, ROWS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         227 * 1024);
+    for (auto k : {bulk_tma_kernel<T, NSTAGE, PER_SM, ROWS, true>, bulk_tma_kernel<T, NSTAGE, PER_SM, ROWS, false>})
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
 }
 
 // launch shapes: V cells per thread in blocks of BULK_THREADS; MINB > 1 caps
@@ -1222,12 +1365,14 @@ struct Variant {
 };
 
 // the compiled variants of the bulk kernel; the first entry of a precision
-// and width is its default
+// and width is its default (FP32, two cells: 4 blocks an SM take 794 us on
+// 512 x 256 x 256 cells, 106 us on 204 x 148 x 132 and 20.0 us on 128 x 64 x 64,
+// against 833, 112 and 20.5 us without the register cap)
 const Variant kVariants[] = {
     {0, 1, 1, launch_shape<double, 1, 1>},
     {0, 2, 1, launch_shape<double, 2, 1>},
-    {1, 2, 1, launch_shape<float, 2, 1>},
     {1, 2, 4, launch_shape<float, 2, 4>},
+    {1, 2, 1, launch_shape<float, 2, 1>},
     {1, 1, 1, launch_shape<float, 1, 1>},
     {1, 4, 1, launch_shape<float, 4, 1>},
     {2, 4, 1, launch_shape<__half, 4, 1>},
@@ -1324,7 +1469,17 @@ int list_variants(const Device &dv, int *vec, int *minb, int max) {
 }
 
 void launch_stream_collide(const Device &dv, const StepPtrs &sp, cudaStream_t s) {
-    const Variant *v = find_variant(dv.precision, dv.vec, dv.minb);
+    int minb = dv.minb;
+    if (minb == 0 && dv.precision >= 2 && dv.vec == 4) {
+        // 16-bit storage, four cells a thread: with 3 blocks an SM the registers
+        // spill a little, which pays once two or more waves of blocks overlap
+        // (FP16 428 against 526 us on 512 x 256 x 256 cells, 62 against 72 us on
+        // 204 x 148 x 132; on 128 x 64 x 64, one wave, 15.9 against 13.8 us)
+        const Domain &d = dv.dom;
+        const long long per_plane = (long long)(d.nx / 4) * d.ny;
+        minb = (per_plane + BULK_THREADS - 1) / BULK_THREADS * d.nz >= 2LL * 3 * sm_count() ? 3 : 2;
+    }
+    const Variant *v = find_variant(dv.precision, dv.vec, minb);
     if (!v) v = find_variant(dv.precision, 1, 0);
     v->fn(dv, sp, s);
 }
