@@ -484,14 +484,23 @@ __device__ __forceinline__ Dither bf16_dither(long long c, long long t) {
     return d;
 }
 
+// word k of bf16_dither alone
+__device__ __forceinline__ unsigned bf16_dither_word(long long c, long long t, int k) {
+    unsigned x = fmix32((unsigned)c * 0x9E3779B1u ^ ((unsigned)t * 0x85EBCA77u + (unsigned)(t >> 32)));
+    if (k == 0) return x;
+    for (int i = 0; i < k; ++i) x = x * 1664525u + 1013904223u;
+    return x ^ (x >> 15);
+}
+
 // v rounded stochastically to BF16 with byte a % 4 of word a / 4 of d, its
 // bits in the upper half of the result: adding 8 random bits and half a
 // step of them below the kept bits, then truncating, rounds the magnitude
 // up with the probability of the dropped fraction (to 2^-9 of an ulp)
-__device__ __forceinline__ unsigned bf16_sr_word(float v, const Dither &d, int a) {
-    const unsigned r = __byte_perm(d.h[a >> 2], 0x80u, 0x5504u | ((unsigned)(a & 3) << 4));   // byte << 8 | 0x80
+__device__ __forceinline__ unsigned bf16_sr_add(float v, unsigned word, int a) {
+    const unsigned r = __byte_perm(word, 0x80u, 0x5504u | ((unsigned)(a & 3) << 4));          // byte << 8 | 0x80
     return __float_as_uint(v) + r;
 }
+__device__ __forceinline__ unsigned bf16_sr_word(float v, const Dither &d, int a) { return bf16_sr_add(v, d.h[a >> 2], a); }
 
 // the same BF16 bits in the low half
 __device__ __forceinline__ unsigned bf16_sr_bits(float v, const Dither &d, int a) {
@@ -901,222 +910,230 @@ __global__ void __launch_bounds__(BULK_THREADS, MINB == 1 ? 0 : MINB) bulk16_bat
     }
 }
 
-// Velocity of body b's surface at lattice point p in the compute type R:
-// FP64 throughout for FP64 storage; otherwise the minimum-image offset in
-// FP64 and V + W x offset in R (the moving-wall term is ~1e-4 and its R
-// rounding sits below the storage's)
-template <typename R>
-__device__ inline void wall_velocity(const Domain &d, const BodyState &b, int px, int py, int pz, R (&u)[3]) {
-    if constexpr (sizeof(R) == 8) {
-        double w[3];
-        surface_velocity(d, b, px, py, pz, w);
-        u[0] = w[0]; u[1] = w[1]; u[2] = w[2];
-    } else {
-        double od[3];
-        offset_from(d, b, (double)px, (double)py, (double)pz, od);
-        const R o0 = (R)od[0], o1 = (R)od[1], o2 = (R)od[2];
-        const R w0 = (R)b.W[0], w1 = (R)b.W[1], w2 = (R)b.W[2];
-        u[0] = (R)b.V[0] + (w1 * o2 - w2 * o1);
-        u[1] = (R)b.V[1] + (w2 * o0 - w0 * o2);
-        u[2] = (R)b.V[2] + (w0 * o1 - w1 * o0);
-    }
-}
-
-// a body for the moving-wall term: the centre wrapped into the domain and
-// split into its cell (int) and the offset within it (FP32), velocity and
-// angular velocity in FP32 (copied from the step's geometry record)
-struct WallBody {
-    int ic[3];
-    float frac[3], v[3], w[3];
-};
-
-__device__ inline WallBody wall_body(const BodyGeom &g) {
-    WallBody r;
-    for (int i = 0; i < 3; ++i) {
-        r.ic[i] = g.ci[i];
-        r.frac[i] = g.cf[i];
-        r.v[i] = g.v[i];
-        r.w[i] = g.w[i];
-    }
-    return r;
-}
-
-__device__ inline int near_cell(int o, int n, int periodic) {
+// Minimum image of a cell difference by integer compares
+__device__ __forceinline__ int near_cell(int o, int n, int periodic) {
     if (!periodic) return o;
     return 2 * o > n ? o - n : (2 * o < -n ? o + n : o);
 }
 
-// V + W x (p - X) in FP32; the minimum-image offset is an integer difference
-// of cells wrapped by compares minus the centre's fraction (exact to FP32
-// rounding of a few-cell offset)
-__device__ inline void wall_velocity_wrapped(const Domain &d, const WallBody &b, int px, int py, int pz,
-                                             float (&u)[3]) {
-    const float o0 = (float)near_cell(px - b.ic[0], d.nx, d.px) - b.frac[0];
-    const float o1 = (float)near_cell(py - b.ic[1], d.ny, d.py) - b.frac[1];
-    const float o2 = (float)near_cell(pz - b.ic[2], d.nz, d.pz) - b.frac[2];
-    u[0] = b.v[0] + (b.w[1] * o2 - b.w[2] * o1);
-    u[1] = b.v[1] + (b.w[2] * o0 - b.w[0] * o2);
-    u[2] = b.v[2] + (b.w[0] * o1 - b.w[1] * o0);
+// V + W x (p - X) of body k's surface at lattice point p: the minimum-image
+// offset is an integer difference of cells wrapped by compares minus the centre's
+// position within its cell (FP32: exact to the rounding of a few-cell offset).
+// g: the geometry record of the state, st: the state itself (FP64).
+__device__ __forceinline__ void wall_velocity(const Domain &d, const BodyGeom &g, const BodyState &, int px, int py,
+                                              int pz, float (&u)[3]) {
+    const float o0 = (float)near_cell(px - g.ci[0], d.nx, d.px) - g.cf[0];
+    const float o1 = (float)near_cell(py - g.ci[1], d.ny, d.py) - g.cf[1];
+    const float o2 = (float)near_cell(pz - g.ci[2], d.nz, d.pz) - g.cf[2];
+    u[0] = g.v[0] + (g.w[1] * o2 - g.w[2] * o1);
+    u[1] = g.v[1] + (g.w[2] * o0 - g.w[0] * o2);
+    u[2] = g.v[2] + (g.w[0] * o1 - g.w[1] * o0);
+}
+__device__ __forceinline__ void wall_velocity(const Domain &d, const BodyGeom &g, const BodyState &st, int px, int py,
+                                              int pz, double (&u)[3]) {
+    const double o0 = near_cell(px - g.ci[0], d.nx, d.px) - g.cfd[0];
+    const double o1 = near_cell(py - g.ci[1], d.ny, d.py) - g.cfd[1];
+    const double o2 = near_cell(pz - g.ci[2], d.nz, d.pz) - g.cfd[2];
+    u[0] = st.V[0] + mad(st.W[1], o2, -(st.W[2] * o1));
+    u[1] = st.V[1] + mad(st.W[2], o0, -(st.W[0] * o2));
+    u[2] = st.V[2] + mad(st.W[0], o1, -(st.W[1] * o0));
+}
+
+// direction components by lane, from bit masks of the directions with + and -
+constexpr unsigned component_mask(int axis, int sign) {
+    unsigned m = 0;
+    for (int b = 0; b < Q; ++b)
+        if ((axis == 0 ? ex(b) : (axis == 1 ? ey(b) : ez(b))) == sign) m |= 1u << b;
+    return m;
+}
+__device__ __forceinline__ int lane_component(int axis, int b) {
+    constexpr unsigned P[3] = {component_mask(0, 1), component_mask(1, 1), component_mask(2, 1)};
+    constexpr unsigned N[3] = {component_mask(0, -1), component_mask(1, -1), component_mask(2, -1)};
+    const unsigned p = axis == 0 ? P[0] : (axis == 1 ? P[1] : P[2]), n = axis == 0 ? N[0] : (axis == 1 ? N[1] : N[2]);
+    return (int)((p >> b) & 1u) - (int)((n >> b) & 1u);
+}
+template <typename R> __device__ __forceinline__ R signed_by(int e, R v) { return e > 0 ? v : (e < 0 ? -v : (R)0); }
+
+// Sum and momentum of a cell whose population b lane b holds (0 on the lanes
+// past the last direction): 8 lanes form each of the four sums, three values a
+// lane and three butterfly steps, so that all four take five additions (FP64: a
+// warp's addition costs the same whatever the lanes do).  sg: the lane's three
+// factors (lane_factors).
+template <typename R> struct Moments { R s, x, y, z; };
+struct LaneFactors { int a, b, c; };
+__device__ __forceinline__ LaneFactors lane_factors(int lane) {
+    const int i = lane & 7, q = lane >> 3;
+    if (q == 0) return LaneFactors{1, 1, 1};
+    return LaneFactors{lane_component(q - 1, i), lane_component(q - 1, i + 8), lane_component(q - 1, i + 16)};
+}
+template <typename R>
+__device__ __forceinline__ Moments<R> lane_moments(R f, int lane, const LaneFactors &sg) {
+    constexpr unsigned FULL = 0xffffffffu;
+    const int i = lane & 7;
+    const R a = __shfl_sync(FULL, f, i), b = __shfl_sync(FULL, f, i + 8), c = __shfl_sync(FULL, f, i + 16);
+    R v = (signed_by(sg.a, a) + signed_by(sg.b, b)) + signed_by(sg.c, c);
+    v += __shfl_xor_sync(FULL, v, 1);
+    v += __shfl_xor_sync(FULL, v, 2);
+    v += __shfl_xor_sync(FULL, v, 4);
+    return Moments<R>{__shfl_sync(FULL, v, 0), __shfl_sync(FULL, v, 8), __shfl_sync(FULL, v, 16), __shfl_sync(FULL, v, 24)};
+}
+template <typename R> __device__ __forceinline__ R lane_sum(R v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
 }
 
 // The cells the remap listed (fluid with F_NEAR or F_SOLID_PREV): refill,
-// bounce-back at walls and moving obstacles, then LBGK, one cell a thread on a
-// grid sized for the longest possible list.  A cell listed twice (it lies in
-// two bodies' cubes) is computed twice with the same result.  Every load a cell
-// needs is issued before any of them is used, so a thread waits for memory
-// about twice instead of once per direction.
+// bounce-back at walls and moving obstacles, then LBGK, a warp a cell with lane b
+// the direction b: the 19 pulls, wall velocities and relaxations run side by side
+// and the cell's sums by shuffles.  Latency-bound (some hundred cells a body): a
+// thread a cell walked ~250 dependent operations, in FP64 at 64 issue cycles
+// each.  (32^3 swimmer in FP64, a step: 93 -> 50 us, the kernel 70 us of it
+// before; 48^3 in FP32 with the body read: 69 -> 62 us a step.)  A cell listed twice (it lies in two bodies' cubes) is
+// computed twice with the same result.
+constexpr int BOUNDARY_WARPS = 8;
+
 template <typename T>
 __device__ __forceinline__ void boundary_body(const Device &dv, const StepPtrs &sp, const Blk &bk) {
     using Cd = typename Codec<T>::C;
-    const Domain d = dv.dom;
-    // 32/16-bit storage: the bodies of step n-1 with their centres wrapped
-    // into the domain, so that a link's minimum-image offset is an integer
-    // difference, two compares and the FP32 position within the cell
-    __shared__ WallBody wb[sizeof(T) == 8 ? 1 : LBM_MAX_BODIES_DEV];
-    const int l = bk.x * blockDim.x + threadIdx.x;
+    constexpr unsigned FULL = 0xffffffffu;
+    const Domain &d = dv.dom;
+    const int lane = threadIdx.x & 31;
+    int l = bk.x * BOUNDARY_WARPS + (threadIdx.x >> 5);
     // the count may pass the capacity after an overflow (reported as an error): never read past it
     const int listed = (int)min((long long)*dv.bcount, dv.blist_cap);
-    if ((int)(bk.x * blockDim.x) >= listed) return;      // the whole block is past the list
-    if constexpr (sizeof(T) != 8) {
-        for (int k = threadIdx.x; k < dv.nb; k += blockDim.x) wb[k] = wall_body(dv.geom[(sp.parity ^ 1) * dv.nb + k]);
-        __syncthreads();
-    }
     if (l >= listed) return;
-    const unsigned cl = dv.blist[l];          // C < 2^31: 32-bit division
-    const unsigned nxu = (unsigned)d.nx, nyu = (unsigned)d.ny;
-    const int x = (int)(cl % nxu), y = (int)((cl / nxu) % nyu), z = (int)(cl / (nxu * nyu));
+    const bool act = lane < Q;
+    const int b = act ? lane : 0;
+    const int bx = lane_component(0, b), by = lane_component(1, b), bz = lane_component(2, b);
+    const int ob = b == 0 ? 0 : ((b & 1) ? b + 1 : b - 1);
+    const Cd w = b == 0 ? (Cd)wgt(0) : (b < 7 ? (Cd)wgt(1) : (Cd)wgt(7));
+    const LaneFactors sg = lane_factors(lane);
     const long long C = d.C;
-    const long long c = ((long long)z * d.ny + y) * d.nx + x;
-    const uint8_t fc = sp.flags_cur[c];
     const T *__restrict__ src = static_cast<const T *>(sp.src);
+    T *__restrict__ dst = static_cast<T *>(sp.dst);
     const float s = dv.f16_inv_scale;
-    Cd f[Q];
-    if (fc & F_SOLID_PREV) {
-        // uncovered cell: f = f_eq(rho_avg, u_w(x)) with the state of step n;
-        // rho_avg over the D3Q19 neighbours fluid in both epochs (1 if none)
-        long long nc[Q];
-        bool ok[Q];
+    const bool f32 = sizeof(Cd) == 4;
+    const Cd gx = f32 ? (Cd)dv.g_f[0] : (Cd)dv.g[0], gy = f32 ? (Cd)dv.g_f[1] : (Cd)dv.g[1],
+             gz = f32 ? (Cd)dv.g_f[2] : (Cd)dv.g[2];
+    for (; l < listed; l += bk.gx * BOUNDARY_WARPS) {
+        const unsigned cl = dv.blist[l];          // C < 2^31: 32-bit division
+        const unsigned nxu = (unsigned)d.nx, nyu = (unsigned)d.ny;
+        const unsigned row = cl / nxu, zu = row / nyu;
+        const int x = (int)(cl - row * nxu), y = (int)(row - zu * nyu), z = (int)zu;
+        const uint8_t fc = sp.flags_cur[cl];
+        Cd f = 0;
+        if (fc & F_SOLID_PREV) {
+            // uncovered cell: f = f_eq(rho_avg, u_w(x)) with the state of step n;
+            // rho_avg over the D3Q19 neighbours fluid in both epochs (1 if none),
+            // as deviations (small numbers: no 1 + drho is rounded), lane a the
+            // neighbour x + e_a
+            const int nx_ = x + bx, ny_ = y + by, nz_ = z + bz;
+            const bool in = act && b > 0 &&
+                            !((!d.px && (nx_ < 0 || nx_ >= d.nx)) || (!d.py && (ny_ < 0 || ny_ >= d.ny)) ||
+                              (!d.pz && (nz_ < 0 || nz_ >= d.nz)));
+            const long long nc = ((long long)wrap_axis(nz_, d.nz) * d.ny + wrap_axis(ny_, d.ny)) * d.nx +
+                                 wrap_axis(nx_, d.nx);
+            Cd drho = 0;
 #pragma unroll
-        for (int a = 1; a < Q; ++a) {
-            const int nx_ = x + ex(a), ny_ = y + ey(a), nz_ = z + ez(a);
-            ok[a] = !((!d.px && (nx_ < 0 || nx_ >= d.nx)) || (!d.py && (ny_ < 0 || ny_ >= d.ny)) ||
-                      (!d.pz && (nz_ < 0 || nz_ >= d.nz)));
-            nc[a] = ((long long)wrap_axis(nz_, d.nz) * d.ny + wrap_axis(ny_, d.ny)) * d.nx + wrap_axis(nx_, d.nx);
-        }
-#pragma unroll
-        for (int a = 1; a < Q; ++a) ok[a] = ok[a] && !(sp.flags_cur[nc[a]] & (F_SOLID | F_SOLID_PREV));
-        const int k = sp.bid_prev[c];
-        if constexpr (sizeof(T) == 8) {
-            double sum = 0.0;
-            int cnt = 0;
-#pragma unroll
-            for (int a = 1; a < Q; ++a) {
-                Cd drho = 0;
-#pragma unroll
-                for (int bb = 0; bb < Q; ++bb) drho += Codec<T>::ld(src[bb * C + nc[a]], s);
-                if (ok[a]) {
-                    sum += 1.0 + (double)drho;
-                    ++cnt;
-                }
-            }
-            const double rho = cnt ? sum / cnt : 1.0;
-            double u[3] = {0.0, 0.0, 0.0};
-            if (k != NO_BODY) surface_velocity(d, sp.body_cur[k], x, y, z, u);
-            const double uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-#pragma unroll
-            for (int b = 0; b < Q; ++b) {
-                const double eu = ex(b) * u[0] + ey(b) * u[1] + ez(b) * u[2];
-                f[b] = (Cd)(wgt(b) * (rho - 1.0) + wgt(b) * rho * (3.0 * eu + 4.5 * eu * eu - 1.5 * uu));
-            }
+            for (int q = 0; q < Q; ++q) drho += Codec<T>::ld(src[q * C + nc], s);
+            const bool ok = in && !(sp.flags_cur[nc] & (F_SOLID | F_SOLID_PREV));
+            const int cnt = __popc(__ballot_sync(FULL, ok));
+            const Cd sum = lane_sum(ok ? drho : (Cd)0);
+            drho = cnt ? sum / (Cd)cnt : (Cd)0;
+            const Cd rho = (Cd)1 + drho;
+            const int k = sp.bid_prev[cl];
+            Cd u[3] = {0, 0, 0};
+            if (k != NO_BODY) wall_velocity(d, dv.geom[sp.parity * dv.nb + k], sp.body_cur[k], x, y, z, u);
+            const Cd uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+            const Cd eu = signed_by(bx, u[0]) + signed_by(by, u[1]) + signed_by(bz, u[2]);
+            f = w * drho + w * rho * ((Cd)3 * eu + (Cd)4.5 * eu * eu - (Cd)1.5 * uu);
+            if (!act) f = 0;
         } else {
-            // FP32: the mean of the neighbours' density deviations (small
-            // numbers: no 1 + drho is ever rounded), u_w of state n
-            float dsum = 0.0f;
-            int cnt = 0;
-#pragma unroll
-            for (int a = 1; a < Q; ++a) {
-                float drho = 0.0f;
-#pragma unroll
-                for (int bb = 0; bb < Q; ++bb) drho += Codec<T>::ld(src[bb * C + nc[a]], s);
-                if (ok[a]) {
-                    dsum += drho;
-                    ++cnt;
-                }
-            }
-            const float drho = cnt ? dsum / (float)cnt : 0.0f;
-            const float rho = 1.0f + drho;
-            float u[3] = {0.0f, 0.0f, 0.0f};
-            if (k != NO_BODY) wall_velocity_wrapped(d, wall_body(dv.geom[sp.parity * dv.nb + k]), x, y, z, u);
-            const float uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-#pragma unroll
-            for (int b = 0; b < Q; ++b) {
-                const float w = (float)wgt(b);
-                const float eu = ex(b) * u[0] + ey(b) * u[1] + ez(b) * u[2];
-                f[b] = w * drho + w * rho * (3.0f * eu + 4.5f * eu * eu - 1.5f * uu);
-            }
-        }
-    } else {
-        // bounce-back at walls (Eq. 4) and at obstacles of step n-1
-        Cd own[Q];
-        Cd drho = 0;
-#pragma unroll
-        for (int a = 0; a < Q; ++a) {
-            own[a] = Codec<T>::ld(src[(long long)a * C + c], s);
-            drho += own[a];
-        }
-        const Cd rho_x = (Cd)1 + drho;
-        f[0] = own[0];
-#pragma unroll
-        for (int b = 1; b < Q; ++b) {
-            const int sx = x - ex(b), sy = y - ey(b), sz = z - ez(b);
+            // bounce-back at walls (Eq. 4) and at obstacles of step n-1
+            const int sx = x - bx, sy = y - by, sz = z - bz;
             const bool wall = (!d.px && (sx < 0 || sx >= d.nx)) || (!d.py && (sy < 0 || sy >= d.ny)) ||
                               (!d.pz && (sz < 0 || sz >= d.nz));
             const long long sc = ((long long)wrap_axis(sz, d.nz) * d.ny + wrap_axis(sy, d.ny)) * d.nx +
                                  wrap_axis(sx, d.nx);
             const uint8_t fp = sp.flags_prev[sc];
+            const int k = sp.bid_prev[sc];
+            const Cd own = act ? Codec<T>::ld(src[(long long)b * C + cl], s) : (Cd)0;
             const Cd pulled = Codec<T>::ld(src[(long long)b * C + sc], s);
-            Cd v = pulled;
+            const Cd rho_x = (Cd)1 + lane_sum(own);
+            const Cd own_opp = __shfl_sync(FULL, own, ob);
+            f = pulled;
             if (wall) {
-                v = own[opp(b)];                                             // Eq. 4
+                f = own_opp;                                                 // Eq. 4
             } else if (fp & F_SOLID) {
-                const int k = sp.bid_prev[sc];
                 Cd u[3] = {0, 0, 0};
-                if (k != NO_BODY) {
-                    if constexpr (sizeof(T) == 8) wall_velocity<Cd>(d, sp.body_prev[k], sx, sy, sz, u);
-                    else wall_velocity_wrapped(d, wb[k], sx, sy, sz, u);
-                }
-                const Cd eu = (Cd)ex(b) * u[0] + (Cd)ey(b) * u[1] + (Cd)ez(b) * u[2];
-                v = own[opp(b)] + (Cd)(6.0 * wgt(b)) * rho_x * eu;          // moving wall
+                if (k != NO_BODY) wall_velocity(d, dv.geom[(sp.parity ^ 1) * dv.nb + k], sp.body_prev[k], sx, sy, sz, u);
+                const Cd eu = signed_by(bx, u[0]) + signed_by(by, u[1]) + signed_by(bz, u[2]);
+                f = own_opp + (Cd)6 * w * rho_x * eu;                        // moving wall
             }
-            f[b] = v;
+            if (!act) f = 0;
         }
-    }
-    if constexpr (sizeof(T) != 8) {
-        // rho - 1 of the cell for the momentum exchange (the collision keeps it)
-        Cd drho = 0;
-#pragma unroll
-        for (int b = 0; b < Q; ++b) drho += f[b];
-        dv.rho_near[c] = (float)drho;
-    }
-    collide<T>(f, dv);
-    T *__restrict__ dst = static_cast<T *>(sp.dst);
-    if constexpr (std::is_same<T, __nv_bfloat16>::value) {
-        const Dither dz = bf16_dither(c, *sp.tstep);
-#pragma unroll
-        for (int b = 0; b < Q; ++b) dst[(long long)b * C + c] = store16<T>(f[b], dz, b);
-    } else {
-#pragma unroll
-        for (int b = 0; b < Q; ++b) dst[(long long)b * C + c] = Codec<T>::st(f[b], dv.f16_scale);
+        // LBGK (+ Guo), the bulk kernels' update with the sums over the lanes
+        const Moments<Cd> mo = lane_moments(f, lane, sg);
+        if constexpr (sizeof(T) != 8)
+            if (lane == 0) dv.rho_near[cl] = mo.s;      // rho - 1 for the momentum exchange
+        const Cd rho = (Cd)1 + mo.s;
+        const Cd inv = (Cd)1 / rho;
+        const Cd ux = mad((Cd)0.5, gx, mo.x) * inv, uy = mad((Cd)0.5, gy, mo.y) * inv, uz = mad((Cd)0.5, gz, mo.z) * inv;
+        const Cd usq = mad(ux, ux, mad(uy, uy, uz * uz));
+        const Cd base = mad((Cd)(-1.5) * rho, usq, mo.s);
+        const Cd eu = signed_by(bx, ux) + signed_by(by, uy) + signed_by(bz, uz);
+        const Cd deq = w * mad(rho, mad((Cd)4.5 * eu, eu, (Cd)3 * eu), base);
+        Cd gt = 0;
+        if (dv.forced) {
+            const Cd eg = signed_by(bx, gx) + signed_by(by, gy) + signed_by(bz, gz);
+            const Cd ug = mad(ux, gx, mad(uy, gy, uz * gz));
+            gt = (f32 ? (Cd)dv.guo_f : (Cd)(1.0 - 0.5 * dv.omega)) * w * mad((Cd)9 * eu, eg, (Cd)3 * (eg - ug));
+        }
+        const Cd om = f32 ? (Cd)dv.omega_f : (Cd)dv.omega;
+        if constexpr (std::is_same<T, float>::value) {
+            // the increments' mass and momentum are moved to 0 and g (collide_f32)
+            const Cd inc = act ? mad(om, deq - f, gt) : (Cd)0;
+            const Moments<Cd> dm = lane_moments(inc, lane, sg);
+            f += inc;
+            if (b == 0) f -= dm.s;
+            else if (b < 7) f += (Cd)0.5 * (signed_by(bx, gx - dm.x) + signed_by(by, gy - dm.y) + signed_by(bz, gz - dm.z));
+        } else {
+            f = mad(om, deq - f, f) + gt;
+        }
+        if (act) {
+            T out;
+            if constexpr (std::is_same<T, __nv_bfloat16>::value) {
+                out = __ushort_as_bfloat16((unsigned short)(bf16_sr_add(f, bf16_dither_word(cl, *sp.tstep, b >> 2), b) >> 16));
+            } else {
+                out = Codec<T>::st(f, dv.f16_scale);
+            }
+            dst[(long long)b * C + cl] = out;
+        }
     }
 }
 
+// grid of the boundary kernel: `turns` cells a warp for the cells a body of
+// half-width E usually lists (within ~1.2 cells of its surface: about 15 E^2 for
+// the bodies of the workloads), at most what the SMs hold at once; longer lists
+// take more turns.  A batched block pays its member lookup before its first cell
+// and runs beside other members' blocks (48 boxes, 32 steps: 23.4 ms with 4 cells a
+// warp, 24.2 ms with one).
+int sm_count();
+constexpr int BOUNDARY_BATCH_TURNS = 4;
+int boundary_blocks(const Device &dv, int turns) {
+    const long long E = (dv.remap_side - 1) / 2 - REMAP_MARGIN, per = BOUNDARY_WARPS * turns;
+    const long long blocks = ((long long)dv.nb * 15 * E * E + per - 1) / per;
+    return (int)std::min<long long>(std::max<long long>(blocks, 1), 4LL * sm_count());
+}
+
 template <typename T>
-__global__ void __launch_bounds__(256) boundary_kernel(const Device dv, const StepPtrs sp) {
+__global__ void __launch_bounds__(32 * BOUNDARY_WARPS) boundary_kernel(const Device dv, const StepPtrs sp) {
     boundary_body<T>(dv, sp, launch_blk());
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) boundary_batch(const Batch bt) {
+__global__ void __launch_bounds__(32 * BOUNDARY_WARPS) boundary_batch(const Batch bt) {
     LBM_BATCH_MEMBER(bt);
     boundary_body<T>(sdv, ssp, sbk);
 }
@@ -1414,9 +1431,7 @@ const Variant *find_variant(int precision, int vec, int minb) {
 template <typename T>
 void launch_boundary(const Device &dv, const StepPtrs &sp, cudaStream_t s) {
     // the list's length is on the device: blocks past it return at once
-    const long long side = dv.remap_side;
-    const long long most = (long long)dv.nb * side * side * side;
-    boundary_kernel<T><<<(unsigned)((most + 255) / 256), 256, 0, s>>>(dv, sp);
+    boundary_kernel<T><<<boundary_blocks(dv, 1), 32 * BOUNDARY_WARPS, 0, s>>>(dv, sp);
 }
 
 }  // namespace
@@ -1578,8 +1593,7 @@ void batch_grid_cells(const Device &dv, int k, int variant, int g[3]) {
     g[0] = g[1] = g[2] = 0;
     const Domain &d = dv.dom;
     if (k == BK_BOUNDARY && dv.nb > 0) {
-        const long long side = dv.remap_side;
-        g[0] = (int)((dv.nb * side * side * side + 255) / 256);
+        g[0] = boundary_blocks(dv, BOUNDARY_BATCH_TURNS);
         g[1] = g[2] = 1;
     } else if (k == BK_BULK) {
         const BatchShape *b = batch_shape(dv.precision, variant);
@@ -1601,10 +1615,10 @@ void launch_batch_cells(int k, int variant, const Batch &bt, unsigned blocks, in
         return;
     }
     switch (precision) {
-    case 0: boundary_batch<double><<<blocks, 256, 0, s>>>(bt); break;
-    case 1: boundary_batch<float><<<blocks, 256, 0, s>>>(bt); break;
-    case 2: boundary_batch<__half><<<blocks, 256, 0, s>>>(bt); break;
-    default: boundary_batch<__nv_bfloat16><<<blocks, 256, 0, s>>>(bt); break;
+    case 0: boundary_batch<double><<<blocks, 32 * BOUNDARY_WARPS, 0, s>>>(bt); break;
+    case 1: boundary_batch<float><<<blocks, 32 * BOUNDARY_WARPS, 0, s>>>(bt); break;
+    case 2: boundary_batch<__half><<<blocks, 32 * BOUNDARY_WARPS, 0, s>>>(bt); break;
+    default: boundary_batch<__nv_bfloat16><<<blocks, 32 * BOUNDARY_WARPS, 0, s>>>(bt); break;
     }
 }
 
