@@ -32,6 +32,10 @@ constexpr int ADJ_THREADS = 256;
 // the work, and small blocks spread them over more SMs
 constexpr int ADJ_BOUNDARY_THREADS = 64;
 
+// flags of epoch n+1 that call for the full rule (a cell that is only F_LINK has
+// no neighbour solid at n)
+constexpr uint8_t F_FULL_RULE = F_SOLID | F_SOLID_PREV | F_NEAR | F_WALL;
+
 // density and velocity of step n from the post-collision deviations:
 // rho = 1 + sum delta; the collision adds g to the momentum (Guo), so
 // rho u = sum e delta - g / 2
@@ -111,7 +115,7 @@ __global__ void __launch_bounds__(ADJ_THREADS) adj_bulk_kernel(const Device dv, 
     if (x >= d.nx || y >= d.ny) return;
     const long long C = d.C;
     const long long c = ((long long)z * d.ny + y) * d.nx + x;
-    if (ap.flags_next[c] != 0 || (ap.flags_cur[c] & F_SOLID_PREV)) return;   // a boundary cell
+    if ((ap.flags_next[c] & F_FULL_RULE) || (ap.flags_cur[c] & F_SOLID_PREV)) return;   // a boundary cell
     const A *__restrict__ ain = static_cast<const A *>(ap.ain);
     A a[Q];
 #pragma unroll
@@ -157,7 +161,7 @@ __global__ void __launch_bounds__(ADJ_BOUNDARY_THREADS) adj_wall_kernel(const De
     const long long c = ((long long)z * d.ny + y) * d.nx + x;
     if (live) {
         const uint8_t fcur = ap.flags_cur[c], fnext = ap.flags_next[c];
-        if (fnext == 0 && !(fcur & F_SOLID_PREV)) live = false;     // a bulk cell
+        if (!(fnext & F_FULL_RULE) && !(fcur & F_SOLID_PREV)) live = false;     // a bulk cell
         else if (fcur & F_SOLID) {                                    // obstacle at n: no adjoint
             A *aout = static_cast<A *>(ap.aout);
 #pragma unroll
@@ -327,7 +331,7 @@ __global__ void __launch_bounds__(32 * ADJ_CUBE_WARPS) adj_cube_kernel(const Dev
         if (cube_cell(l, x, y, z)) {
             const long long c = ((long long)z * d.ny + y) * d.nx + x;
             const uint8_t fcur = ap.flags_cur[c], fnext = ap.flags_next[c];
-            if (fnext == 0 && !(fcur & F_SOLID_PREV)) {
+            if (!(fnext & F_FULL_RULE) && !(fcur & F_SOLID_PREV)) {
                 // a bulk cell: adj_bulk's
             } else if (fcur & F_SOLID) {            // obstacle at n: no adjoint
 #pragma unroll

@@ -51,7 +51,7 @@ __device__ inline bool cell_inside(const Domain &d, const BodyProps &p, const Bo
 // outside the margin max(1e-3 max(r^2, 1), 2e-6 l max(r, 1)) of r^2 it
 // returns 1 (inside) or 0 (outside), within it -1 and the FP64 test
 // decides: the map is the FP64 map bit for bit.
-__device__ inline int inside_screen(const Domain &d, const BodyGeom *__restrict__ g, int x, int y, int z) {
+__device__ inline float body_distance2(const Domain &d, const BodyGeom *__restrict__ g, int x, int y, int z) {
     const int n3[3] = {d.nx, d.ny, d.nz}, per[3] = {d.px, d.py, d.pz}, q3[3] = {x, y, z};
     float o[3];
 #pragma unroll
@@ -61,16 +61,14 @@ __device__ inline int inside_screen(const Domain &d, const BodyGeom *__restrict_
         o[i] = (float)io - g->cf[i];
     }
     const float o0 = o[0], o1 = o[1], o2 = o[2];
-    float d2;
-    if (g->shape == 0) {
-        d2 = o0 * o0 + o1 * o1 + o2 * o2;
-    } else {
-        const float h = g->h;
-        float sp = o0 * g->ax[0] + o1 * g->ax[1] + o2 * g->ax[2];
-        sp = sp > h ? h : (sp < -h ? -h : sp);
-        const float e0 = o0 - sp * g->ax[0], e1 = o1 - sp * g->ax[1], e2 = o2 - sp * g->ax[2];
-        d2 = e0 * e0 + e1 * e1 + e2 * e2;
-    }
+    if (g->shape == 0) return o0 * o0 + o1 * o1 + o2 * o2;
+    const float h = g->h;
+    float sp = o0 * g->ax[0] + o1 * g->ax[1] + o2 * g->ax[2];
+    sp = sp > h ? h : (sp < -h ? -h : sp);
+    const float e0 = o0 - sp * g->ax[0], e1 = o1 - sp * g->ax[1], e2 = o2 - sp * g->ax[2];
+    return e0 * e0 + e1 * e1 + e2 * e2;
+}
+__device__ inline int inside_screen(const BodyGeom *__restrict__ g, float d2) {
     const float r2 = g->r2, margin = g->margin;
     return d2 < r2 - margin ? 1 : (d2 > r2 + margin ? 0 : -1);
 }
@@ -142,6 +140,7 @@ __device__ inline void geom_scalars(const BodyProps &p, BodyGeom &g) {
     g.r2 = p.r2f;
     g.h = p.hf;
     g.margin = p.marginf;
+    g.link2 = p.link2f;
     g.shape = p.shape;
     g.side = 2 * (p.E + REMAP_MARGIN) + 1;
 }
@@ -305,7 +304,7 @@ __device__ inline int wrap_up(int v, int n) { return v < n ? v : (v - n < n ? v 
 // overlapping cubes write identical values.  A cell tests only body b's
 // candidates, in body order (integer boxes, the FP32 screen, and the FP64
 // inside test only within the screen's margin).  Fluid cells flagged F_NEAR
-// or F_SOLID_PREV are appended to the boundary kernel's list.
+// F_SOLID_PREV or F_LINK are appended to the boundary kernel's list.
 constexpr int REMAP_THREADS = 256;
 constexpr int REMAP_R = 2;
 constexpr int REMAP_CELLS = REMAP_THREADS * REMAP_R;    // cube cells a block covers
@@ -334,6 +333,12 @@ __device__ __forceinline__ void remap_body(const Device &dv, const StepPtrs &sp,
     const int side2 = side * side, cells = side2 * side;
     const int i0 = bk.x * REMAP_CELLS;
     if (i0 >= cells) return;                  // the grid covers the largest body's cube
+    // the step's index by parity (the force kernel advances the clock while the
+    // bulk kernel may still read it); an overlapped step's is there already
+    if (threadIdx.x == 0 && bk.x == 0 && b == 0 && !init_mode) {
+        const long long t = *dv.t_dev;
+        if (dv.tstep[sp.parity] != t) dv.tstep[sp.parity] = t;
+    }
     // this block's share of the boundary kernel's list, gathered in shared
     // memory and appended with one atomic at the end
     __shared__ uint32_t lbuf[REMAP_LIST_BUF];
@@ -379,6 +384,7 @@ __device__ __forceinline__ void remap_body(const Device &dv, const StepPtrs &sp,
     // every lane runs each of its cells, so the ballots below see whole warps
         {
             int xr[REMAP_R], yr[REMAP_R], zr[REMAP_R], idr[REMAP_R];
+            bool linkr[REMAP_R];
             long long cr[REMAP_R];
             bool liver[REMAP_R];
 #pragma unroll
@@ -394,6 +400,7 @@ __device__ __forceinline__ void remap_body(const Device &dv, const StepPtrs &sp,
                 const int p3[3] = {x, y, z};
                 int id = NO_BODY;
                 bool reached = false;           // within STATIC_REACH cells of some body's box
+                bool link = false;
                 for (int i = 0; i < ncand && live; ++i) {
                     const int kb = cid[i];
                     const BodyGeom *g = i < REMAP_STAGED ? cg + i : geo + kb;
@@ -405,14 +412,12 @@ __device__ __forceinline__ void remap_body(const Device &dv, const StepPtrs &sp,
                     }
                     if (!in) continue;
                     reached = true;
-                    for (int a = 0; a < 3 && in; ++a) {
-                        int o = p3[a] - g->box[a];
-                        if (per[a] && o < 0) o += n3[a];
-                        in = o >= 0 && o < g->box[3 + a];
-                    }
-                    if (!in) continue;
-                    // FP32 screen; cells within its margin of the surface take the FP64 test
-                    const int screen = inside_screen(d, g, x, y, z);
+                    // the squared distance to the centre or axis in FP32: cells
+                    // that may hold links, and the inside screen (cells within
+                    // its margin of the surface take the FP64 test)
+                    const float d2 = body_distance2(d, g, x, y, z);
+                    link = link || d2 < g->link2;
+                    const int screen = inside_screen(g, d2);
                     if (screen == 0 || (screen < 0 && !cell_inside(d, dv.props[kb], sp.body_cur[kb], x, y, z)))
                         continue;
                     if (id != NO_BODY) atomicOr(dv.status, ST_OVERLAP);
@@ -426,6 +431,7 @@ __device__ __forceinline__ void remap_body(const Device &dv, const StepPtrs &sp,
                 yr[r] = y;
                 zr[r] = z;
                 idr[r] = id;
+                linkr[r] = link;
                 cr[r] = ((long long)z * d.ny + y) * d.nx + x;
                 liver[r] = live && reached;
             }
@@ -471,6 +477,7 @@ __device__ __forceinline__ void remap_body(const Device &dv, const StepPtrs &sp,
                     const uint8_t solid = id != NO_BODY ? F_SOLID : 0;
                     flags = solid | wall_bit(d, xr[r], yr[r], zr[r]);
                     if (!init_mode) {
+                        if (linkr[r]) flags |= F_LINK;
                         const uint8_t prev = prevr[r] & F_SOLID;
                         if (prev) flags |= F_SOLID_PREV;
                         if (nearr[r] & F_SOLID) flags |= F_NEAR;
@@ -989,17 +996,9 @@ __device__ __forceinline__ void force_body(const Device &dv, const StepPtrs &sp,
             const int a = (int)lk.dir;
             const unsigned cu = lk.cell, nxu = (unsigned)d.nx, nyu = (unsigned)d.ny;
             const int x = (int)(cu % nxu), y = (int)((cu / nxu) % nyu), z = (int)(cu / (nxu * nyu));
-            // rho - 1 of the fluid cell: the boundary kernel's record when it
-            // collided the cell (nearly every link cell: bodies move far
-            // less than a cell a step), else the FP32 sum of the stored
-            // deviations (the bulk kernel's cells a body has just reached)
-            float drho;
-            if (sp.flags_cur[c] & F_LISTED) {
-                drho = __ldcg(dv.rho_near + c);
-            } else {
-                drho = 0.0f;
-                for (int q = 0; q < Q; ++q) drho += load_dev_f<T>(pop + q * C + c, s);
-            }
+            // rho - 1 of the fluid cell: the boundary kernel's record (every
+            // link cell is listed, F_LINK)
+            const float drho = __ldcg(dv.rho_near + c);
             const float rho = 1.0f + drho;
             const float da = load_dev_f<T>(pop + a * C + c, s);
             const int i0 = near_cell_k(x - ci[0], d.nx, d.px);

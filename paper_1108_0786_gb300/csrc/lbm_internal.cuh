@@ -51,7 +51,11 @@ constexpr uint8_t F_SOLID = 1;      // solid at n
 constexpr uint8_t F_SOLID_PREV = 2; // solid at n-1 (uncovered if F_SOLID is clear)
 constexpr uint8_t F_NEAR = 4;       // some neighbour x - e_b was solid at n-1
 constexpr uint8_t F_WALL = 8;       // some neighbour lies beyond a no-slip wall
-constexpr uint8_t F_LISTED = F_NEAR | F_SOLID_PREV;     // fluid with one of these: the boundary kernel's cell
+constexpr uint8_t F_LINK = 16;      // within sqrt(2) cells of a body at n (a little more): may hold links of n
+// fluid with one of these: the boundary kernel's cell.  F_LINK puts every cell
+// the momentum exchange of step n reads into that kernel's list, so the force
+// sums need not wait for the bulk kernel.
+constexpr uint8_t F_LISTED = F_NEAR | F_SOLID_PREV | F_LINK;
 constexpr uint8_t NO_BODY = 0xFF;
 
 // device status word bits
@@ -68,6 +72,10 @@ constexpr int ST_OVERLAP = 1, ST_OUTSIDE = 2, ST_NAN = 4, ST_UNSTABLE = 8, ST_LI
 // cell more is kept as a spare.
 constexpr int REMAP_MARGIN = 3;
 constexpr double MAX_STEP = 0.5;
+// a cell with a link to a body lies within sqrt(2) of its surface; the margin to
+// 1.5 covers the FP32 distance's rounding.  Cells flagged F_LINK in epoch n-2
+// lie within reach + 1.5 + 1 of X_n, inside the cube as above.
+constexpr double LINK_REACH = 1.5;
 constexpr int FORCE_BLOCKS = 8;     // blocks per body in the momentum-exchange sum
 constexpr int LBM_MAX_BODIES_DEV = 254;
 
@@ -75,6 +83,7 @@ struct BodyProps {
     int shape;          // 0 sphere, 1 capsule
     int E;              // ceil(r + l/2) + 1: half-width of the box that holds every solid cell
     float r2f, hf, marginf;     // r^2, l / 2 and the FP32 inside test's margin, in FP32
+    float link2f;       // (r + LINK_REACH)^2 in FP32
     double r, l, m, volume;
     double reach;       // r + l / 2
     double inertia[3];      // body-frame principal moments of inertia
@@ -115,6 +124,7 @@ struct BodyGeom {
     float ax[3];            // body x axis (a capsule's axis)
     float v[3], w[3];       // velocity and angular velocity
     float r2, h, margin;    // r^2, l / 2 and the margin of the FP32 inside test
+    float link2;            // (r + LINK_REACH)^2
     int shape;
     int side;               // edge of the remap cube, 2 (E + REMAP_MARGIN) + 1
     int ncand;              // state n: bodies whose grown box meets this body's remap cube (cand list; the batched remap's)
@@ -194,7 +204,8 @@ struct StepPtrs {
     // overlapped steps: the tiles of step n near a body, which the bulk
     // kernel leaves to the near kernel (null: the bulk kernel does every cell)
     const unsigned *far_skip;
-    const long long *tstep;                 // step index n (the BF16 rounding bits' counter)
+    const long long *tstep;                 // step index n (the BF16 rounding bits' counter), kept by parity: the
+                                            // clock t_dev advances while the bulk kernel of step n still runs
     int parity;
     unsigned row_recip;                     // row_recip of the V-cell groups in an x-row (the bulk launch's)
 };
@@ -445,7 +456,6 @@ void launch_remap(const Device &dv, const StepPtrs &sp, int init_mode, cudaStrea
 void launch_prep(const Device &dv, const StepPtrs &sp, cudaStream_t s);
 void launch_stream_collide(const Device &dv, const StepPtrs &sp, cudaStream_t s);
 void launch_boundary_fix(const Device &dv, const StepPtrs &sp, cudaStream_t s);
-bool needs_boundary_fix(const Device &dv);
 bool valid_vector_width(const Device &dv, int v);
 bool valid_variant(const Device &dv, int v, int minb);
 int list_variants(const Device &dv, int *vec, int *minb, int max);

@@ -65,6 +65,7 @@ struct lbm_s {
     // boundary kernel (a small lattice's bulk kernel is shorter than both)
     cudaStream_t side2 = nullptr;
     cudaEvent_t join2_ev = nullptr;
+    cudaEvent_t bulk_ev[2] = {nullptr, nullptr};    // by step parity: bulk kernel (and average) of step n done
     // overlapped steps: the far bulk kernels' stream, and by step parity the
     // events "far bulk of step n done" and "near cells of step n done"
     cudaStream_t far = nullptr;
@@ -162,7 +163,9 @@ lbm::StepPtrs step_ptrs(lbm_t *h, int p, bool overlap = false) {
     lbm::StepPtrs sp{};
     overlap = overlap && h->dv.overlap;
     sp.far_skip = overlap ? h->dv.near_mask[p] : nullptr;
-    sp.tstep = overlap ? h->dv.tstep + p : h->dv.t_dev;
+    // with bodies the remap (overlapped steps: the near-tile kernel) keeps the
+    // step's index by parity; a lattice without bodies advances its clock last
+    sp.tstep = nb(h) > 0 && fluid(h) ? h->dv.tstep + p : h->dv.t_dev;
     sp.src = h->pop[q];
     sp.dst = h->pop[p];
     sp.flags_prev = h->flags[q];
@@ -177,15 +180,31 @@ lbm::StepPtrs step_ptrs(lbm_t *h, int p, bool overlap = false) {
 }
 
 // the kernels of one step of parity p, in Algorithm 2's order; `ev`
-// (optional) brackets each kernel slot with a pair of events.  With `fork`
-// the boundary-cell kernel, then the link lists and the drive and spring
-// loads, run on a second stream concurrently with the bulk kernel (they
-// touch no data the bulk kernel reads or writes) and join before the force
-// sums.
+// (optional) brackets each kernel slot with a pair of events.
+//
+// With `fork` (a capture) the step takes three streams.  The chain s runs remap,
+// boundary cells and force + rigid-body step; the next step's chain follows at
+// once.  The bulk kernel runs on h->side beside it: the force sums read only
+// cells of the boundary kernel (F_LINK), so the chain of step n+1 needs nothing
+// of step n's bulk kernel until its boundary kernel.  The link lists and the
+// drive and spring loads run on h->side2 beside the boundary kernel.  What
+// orders the shared buffers:
+//   bulk(n)      after remap(n) (flags n; the chain before it ends with
+//                boundary(n-1), the other writer of its sources) and, on its
+//                stream, bulk(n-1), which reads the buffer it writes;
+//   boundary(n)  after bulk(n-1): its sources, and the reader of its buffer;
+//   remap(n+1)   rewrites flags n-1, read by bulk(n-1) (done before boundary(n))
+//                and boundary(n).
+// `first`: the first step of a capture (what ran before it has completed).
+// join_bulk brings the bulk stream back at the end.  The chain has the greater
+// node priority: without it its blocks queue behind the bulk kernel's (a step of
+// the 100 x 100 x 200 study takes 66 us with, 89 us without; one after the other
+// it was 92 us; 128 x 64 x 64 channel 39, 43, 45 us; 512 x 256 x 256 swarm 820,
+// 846, 845 us).
 void enqueue_overlapped(lbm_t *h, int p, cudaStream_t s, bool first);
 
 void enqueue_step(lbm_t *h, int p, cudaStream_t s, cudaEvent_t *ev = nullptr, bool *ran = nullptr,
-                  bool fork = false, bool prep = true) {
+                  bool fork = false, bool first = true) {
     const lbm::StepPtrs sp = step_ptrs(h, p);
     const bool bodies = nb(h) > 0, fl = fluid(h);
     auto run = [&](int slot, cudaStream_t st, auto &&fn) {
@@ -194,33 +213,34 @@ void enqueue_step(lbm_t *h, int p, cudaStream_t s, cudaEvent_t *ev = nullptr, bo
         if (ev) cudaEventRecord(ev[2 * slot + 1], st);
         if (ran) ran[slot] = true;
     };
-    if (bodies && fl) run(LBM_KERNEL_REMAP, s, [&] { lbm::launch_remap(h->dv, sp, 0, s, prep); });
-    const bool boundary = fl && lbm::needs_boundary_fix(h->dv);
-    const bool forked = boundary && fork;
-    if (forked) {
+    // captured steps leave the body preparation out (lbm_step runs it where needed)
+    if (bodies && fl) run(LBM_KERNEL_REMAP, s, [&] { lbm::launch_remap(h->dv, sp, 0, s, !fork); });
+    if (fork && bodies && fl) {
         cudaEventRecord(h->fork_ev, s);
+        cudaStreamWaitEvent(h->side2, h->fork_ev, 0);
+        lbm::launch_links(h->dv, sp, h->side2);
+        cudaEventRecord(h->join2_ev, h->side2);
+        if (!first) cudaStreamWaitEvent(s, h->bulk_ev[p ^ 1], 0);
+        lbm::launch_boundary_fix(h->dv, sp, s);
         cudaStreamWaitEvent(h->side, h->fork_ev, 0);
-        lbm::launch_boundary_fix(h->dv, sp, h->side);
-        cudaEventRecord(h->join_ev, h->side);
-        if (bodies) {
-            cudaStreamWaitEvent(h->side2, h->fork_ev, 0);
-            lbm::launch_links(h->dv, sp, h->side2);
-            cudaEventRecord(h->join2_ev, h->side2);
-        }
-    }
-    if (fl) run(LBM_KERNEL_STREAM_COLLIDE, s, [&] {
-        // the bulk kernel waits for the remap in full: launched before the
-        // remap ends, its blocks would hold every SM ahead of the boundary
-        // branch, which is launched when the remap ends
         lbm::Device dvb = h->dv;
         dvb.pdl = 0;
-        lbm::launch_stream_collide(dvb, sp, s);
-    });
-    if (boundary && !forked) run(LBM_KERNEL_BOUNDARY, s, [&] { lbm::launch_boundary_fix(h->dv, sp, s); });
-    if (bodies && fl && !forked) run(LBM_KERNEL_LINKS, s, [&] { lbm::launch_links(h->dv, sp, s); });
-    if (forked) {
-        cudaStreamWaitEvent(s, h->join_ev, 0);
-        if (bodies) cudaStreamWaitEvent(s, h->join2_ev, 0);
+        lbm::launch_stream_collide(dvb, sp, h->side);
+        if (h->dv.avg_u) {
+            // the running velocity average reads the populations both kernels wrote
+            cudaEventRecord(h->join_ev, s);
+            cudaStreamWaitEvent(h->side, h->join_ev, 0);
+            lbm::launch_average(h->dv, sp, h->side);
+        }
+        cudaEventRecord(h->bulk_ev[p], h->side);
+        cudaStreamWaitEvent(s, h->join2_ev, 0);
+        lbm::launch_force(h->dv, sp, s);
+        return;
+    }
+    if (fl) run(LBM_KERNEL_STREAM_COLLIDE, s, [&] { lbm::launch_stream_collide(h->dv, sp, s); });
+    if (bodies && fl) {
+        run(LBM_KERNEL_BOUNDARY, s, [&] { lbm::launch_boundary_fix(h->dv, sp, s); });
+        run(LBM_KERNEL_LINKS, s, [&] { lbm::launch_links(h->dv, sp, s); });
     }
     if (bodies && fl) {
         // momentum exchange; the last block of each body runs its rigid-body step
@@ -232,6 +252,11 @@ void enqueue_step(lbm_t *h, int p, cudaStream_t s, cudaEvent_t *ev = nullptr, bo
     }
     // the running velocity average reads the populations this step wrote
     if (fl && h->dv.avg_u) lbm::launch_average(h->dv, sp, s);
+}
+
+// the end of a capture whose last step had parity p: the bulk stream joins the chain
+void join_bulk(lbm_t *h, int p, cudaStream_t s) {
+    if (nb(h) > 0 && fluid(h)) cudaStreamWaitEvent(s, h->bulk_ev[p], 0);
 }
 
 // One overlapped step n of parity p (lattices with bodies and fluid).  Two
@@ -517,17 +542,19 @@ int ensure_device(lbm_t *h) {
 
 int build_graphs(lbm_t *h) {
     if (h->graphs_ready) return LBM_OK;
-    // overlapped steps: the chain (captured on cap) takes precedence over the
-    // far bulk kernel, so that its short kernels start as soon as SMs free
-    const bool ov = h->dv.overlap != 0;
+    // the chain (captured on cap) takes precedence over the bulk kernel beside
+    // it, so that its short kernels start as soon as SMs free
+    const bool ov = h->dv.overlap != 0, chain = nb(h) > 0 && fluid(h);
     int least = 0, greatest = 0;
     CK(cudaDeviceGetStreamPriorityRange(&least, &greatest));
-    if (!h->cap) CK(cudaStreamCreateWithPriority(&h->cap, cudaStreamNonBlocking, ov ? greatest : 0));
-    if (!h->side) CK(cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking));
+    if (!h->cap) CK(cudaStreamCreateWithPriority(&h->cap, cudaStreamNonBlocking, chain ? greatest : 0));
+    if (!h->side) CK(cudaStreamCreateWithPriority(&h->side, cudaStreamNonBlocking, least));
     if (!h->fork_ev) CK(cudaEventCreateWithFlags(&h->fork_ev, cudaEventDisableTiming));
     if (!h->join_ev) CK(cudaEventCreateWithFlags(&h->join_ev, cudaEventDisableTiming));
-    if (!h->side2) CK(cudaStreamCreateWithFlags(&h->side2, cudaStreamNonBlocking));
+    if (!h->side2) CK(cudaStreamCreateWithPriority(&h->side2, cudaStreamNonBlocking, chain ? greatest : 0));
     if (!h->join2_ev) CK(cudaEventCreateWithFlags(&h->join2_ev, cudaEventDisableTiming));
+    for (cudaEvent_t &ev : h->bulk_ev)
+        if (!ev) CK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
     if (ov) {
         if (!h->far) CK(cudaStreamCreateWithPriority(&h->far, cudaStreamNonBlocking, least));
         for (int i = 0; i < 2; ++i) {
@@ -540,8 +567,9 @@ int build_graphs(lbm_t *h) {
         for (int i = 0; i < n; ++i) {
             const int p = (p0 + i) & 1;
             if (ov) enqueue_overlapped(h, p, h->cap, i == 0);
-            else enqueue_step(h, p, h->cap, nullptr, nullptr, true, false);
+            else enqueue_step(h, p, h->cap, nullptr, nullptr, true, i == 0);
         }
+        if (!ov) join_bulk(h, (p0 + n - 1) & 1, h->cap);
         if (ov) cudaStreamWaitEvent(h->cap, h->far_ev[(p0 + n - 1) & 1], 0);
     };
     // one graph of n steps from parity p0
@@ -551,7 +579,7 @@ int build_graphs(lbm_t *h) {
         if (e != cudaSuccess) return e;
         steps(p0, n);
         e = cudaStreamEndCapture(h->cap, &g);
-        if (e == cudaSuccess) e = cudaGraphInstantiate(x, g, ov ? cudaGraphInstantiateFlagUseNodePriority : 0);
+        if (e == cudaSuccess) e = cudaGraphInstantiate(x, g, chain ? cudaGraphInstantiateFlagUseNodePriority : 0);
         if (g) cudaGraphDestroy(g);
         return e;
     };
@@ -626,6 +654,8 @@ void release_device(lbm_t *h) {
     if (h->join_ev) cudaEventDestroy(h->join_ev);
     if (h->side2) cudaStreamDestroy(h->side2);
     if (h->join2_ev) cudaEventDestroy(h->join2_ev);
+    for (cudaEvent_t ev : h->bulk_ev)
+        if (ev) cudaEventDestroy(ev);
     if (h->far) cudaStreamDestroy(h->far);
     for (int i = 0; i < 2; ++i) {
         if (h->far_ev[i]) cudaEventDestroy(h->far_ev[i]);
@@ -789,6 +819,7 @@ int lbm_add_body(lbm_t *h, int shape, double radius, double length, double mass,
     p.reach = radius + 0.5 * length;
     p.r2f = (float)(radius * radius);
     p.hf = (float)(0.5 * length);
+    p.link2f = (float)((radius + lbm::LINK_REACH) * (radius + lbm::LINK_REACH));
     // the FP32 inside test's margin: its error stays near 1e-5 max(r^2, 1)
     // and grows like 1.3e-7 l r for long thin capsules
     p.marginf = (float)std::max(1e-3 * std::max(radius * radius, 1.0), 2e-6 * length * std::max(radius, 1.0));
@@ -1602,7 +1633,7 @@ int lbm_adjoint_backward(lbm_t *h, const double *seed, double *grad_state, doubl
         sp.body_prev = prev;
         sp.body_cur = cur;
         sp.body_next = scratch;
-        sp.tstep = dr.t_dev;
+        sp.tstep = dr.tstep + (j & 1);
         sp.parity = j & 1;
         // the body preparation only at the segment's first step: the later
         // states' geometry records come from the recomputation's own
@@ -1614,7 +1645,7 @@ int lbm_adjoint_backward(lbm_t *h, const double *seed, double *grad_state, doubl
         // as in the forward step
         CK(cudaEventRecord(fork, ms));
         CK(cudaStreamWaitEvent(ss, fork, 0));
-        if (lbm::needs_boundary_fix(dr)) lbm::launch_boundary_fix(dr, sp, ss);
+        lbm::launch_boundary_fix(dr, sp, ss);
         CK(cudaEventRecord(join, ss));
         CK(cudaStreamWaitEvent(ss2, fork, 0));
         lbm::launch_links(dr, sp, ss2);
@@ -1857,12 +1888,12 @@ struct lbm_ensemble_s {
     std::vector<lbm_t *> members;
     cudaStream_t stream = nullptr;          // the members' common stream
     cudaStream_t cap = nullptr;             // capture origin
-    cudaStream_t side = nullptr;            // batched mode: boundary cells, links and loads beside the bulk kernel
-    cudaEvent_t fork = nullptr, bjoin = nullptr;
+    cudaEvent_t fork = nullptr;
     // batched mode: the members split into ENS_LANES independent chains of
     // launches, each with its own capture and side streams
     cudaStream_t lcap[ENS_LANES] = {}, lside[ENS_LANES] = {}, lbulk[ENS_LANES] = {};
-    cudaEvent_t lfork[ENS_LANES] = {}, ljoin[ENS_LANES] = {}, ldone[ENS_LANES] = {}, lbdone[ENS_LANES] = {};
+    cudaEvent_t lfork[ENS_LANES] = {}, ljoin[ENS_LANES] = {}, ldone[ENS_LANES] = {};
+    cudaEvent_t lbdone[ENS_LANES][2] = {};  // by step parity: the lane's bulk kernel of step n done
     cudaEvent_t lstart = nullptr;
     std::vector<cudaEvent_t> join;          // one per member
     int mode = LBM_ENSEMBLE_BATCHED;
@@ -1894,18 +1925,16 @@ void ens_release(lbm_ensemble_t *e) {
     for (cudaEvent_t ev : e->join) cudaEventDestroy(ev);
     e->join.clear();
     if (e->fork) cudaEventDestroy(e->fork);
-    if (e->bjoin) cudaEventDestroy(e->bjoin);
     if (e->cap) cudaStreamDestroy(e->cap);
-    if (e->side) cudaStreamDestroy(e->side);
-    e->fork = e->bjoin = nullptr;
-    e->cap = e->side = nullptr;
+    e->fork = nullptr;
+    e->cap = nullptr;
     for (int l = 0; l < ENS_LANES; ++l) {
         for (cudaStream_t *st : {&e->lcap[l], &e->lside[l], &e->lbulk[l]})
             if (*st) cudaStreamDestroy(*st);
-        for (cudaEvent_t *ev : {&e->lfork[l], &e->ljoin[l], &e->ldone[l], &e->lbdone[l]})
+        for (cudaEvent_t *ev : {&e->lfork[l], &e->ljoin[l], &e->ldone[l], &e->lbdone[l][0], &e->lbdone[l][1]})
             if (*ev) cudaEventDestroy(*ev);
         e->lcap[l] = e->lside[l] = e->lbulk[l] = nullptr;
-        e->lfork[l] = e->ljoin[l] = e->ldone[l] = e->lbdone[l] = nullptr;
+        e->lfork[l] = e->ljoin[l] = e->ldone[l] = e->lbdone[l][0] = e->lbdone[l][1] = nullptr;
     }
     if (e->lstart) cudaEventDestroy(e->lstart);
     e->lstart = nullptr;
@@ -2003,14 +2032,14 @@ int ens_group_tables(lbm_ensemble_t *e, EnsGroup &g) {
     return LBM_OK;
 }
 
-// one batched step of every group: the kernels of enqueue_step, each as one
-// launch over the members of a group
-// one batched step of the groups of `lane` on the lane's streams (the bulk
-// kernel on `bulk` if not null, else on `main`); `remapped` (if not null) is
-// recorded once the step's remap is enqueued
-void ens_enqueue_batched(lbm_ensemble_t *e, std::vector<EnsGroup> &groups, int lane, int p, cudaStream_t main,
-                         cudaStream_t side, cudaEvent_t fork, cudaEvent_t join, cudaEvent_t remapped,
-                         cudaStream_t bulk = nullptr, cudaEvent_t bulk_done = nullptr) {
+// one batched step of the groups of `lane`: the kernels of enqueue_step, each as
+// one launch over the members of a group, in its order (the chain on lcap, links
+// and loads on lside, the bulk kernel on lbulk); `remapped` (if not null) is
+// recorded once the step's remap is enqueued, `first`: the first step of a capture
+void ens_enqueue_batched(lbm_ensemble_t *e, std::vector<EnsGroup> &groups, int lane, int p, bool first,
+                         cudaEvent_t remapped) {
+    const cudaStream_t main = e->lcap[lane], side = e->lside[lane], bulk = e->lbulk[lane];
+    const cudaEvent_t fork = e->lfork[lane], join = e->ljoin[lane];
     auto small = [&](int k, cudaStream_t st) {
         for (auto &g : groups) {
             if (g.lane != lane) continue;
@@ -2033,28 +2062,39 @@ void ens_enqueue_batched(lbm_ensemble_t *e, std::vector<EnsGroup> &groups, int l
     if (remapped) cudaEventRecord(remapped, main);
     cudaEventRecord(fork, main);
     cudaStreamWaitEvent(side, fork, 0);
-    cells(lbm::BK_BOUNDARY, side);
     small(lbm::BK_LINKS, side);
     small(lbm::BK_LOADS, side);
     cudaEventRecord(join, side);
-    if (bulk) {
+    if (!first) cudaStreamWaitEvent(main, e->lbdone[lane][p ^ 1], 0);
+    cells(lbm::BK_BOUNDARY, main);
+    cudaStreamWaitEvent(bulk, fork, 0);
+    cells(lbm::BK_BULK, bulk);
+    bool average = false, bodiless = false;
+    for (auto &g : groups)
+        if (g.lane == lane)
+            for (int i : g.members) {
+                average = average || e->members[i]->dv.avg_u;
+                bodiless = bodiless || nb(e->members[i]) == 0;
+            }
+    if (average) {
+        cudaEventRecord(fork, main);
         cudaStreamWaitEvent(bulk, fork, 0);
-        cells(lbm::BK_BULK, bulk);
-        cudaEventRecord(bulk_done, bulk);
-        cudaStreamWaitEvent(main, bulk_done, 0);
-    } else {
-        cells(lbm::BK_BULK, main);
+        for (auto &g : groups)
+            if (g.lane == lane)
+                for (int i : g.members)
+                    if (e->members[i]->dv.avg_u)
+                        lbm::launch_average(e->members[i]->dv, step_ptrs(e->members[i], p), bulk);
     }
+    cudaEventRecord(e->lbdone[lane][p], bulk);
     cudaStreamWaitEvent(main, join, 0);
     small(lbm::BK_FORCE, main);
-    for (auto &g : groups) {
-        if (g.lane != lane) continue;
-        for (int i : g.members) {
-            lbm_t *h = e->members[i];
-            const lbm::StepPtrs sp = step_ptrs(h, p);
-            if (nb(h) == 0) lbm::launch_tick(h->dv, sp, main);
-            if (h->dv.avg_u) lbm::launch_average(h->dv, sp, main);
-        }
+    if (bodiless) {
+        // a member without bodies advances its clock after its bulk kernel
+        cudaStreamWaitEvent(main, e->lbdone[lane][p], 0);
+        for (auto &g : groups)
+            if (g.lane == lane)
+                for (int i : g.members)
+                    if (nb(e->members[i]) == 0) lbm::launch_tick(e->members[i]->dv, step_ptrs(e->members[i], p), main);
     }
 }
 
@@ -2120,20 +2160,16 @@ int ens_graph(lbm_ensemble_t *e, const std::vector<int> &set, cudaGraphExec_t *o
     cudaGraph_t g = nullptr;
     cudaError_t err = cudaStreamBeginCapture(e->cap, cudaStreamCaptureModeThreadLocal);
     if (err == cudaSuccess) {
-        if (batched && lanes == 1) {
-            for (int k = 0; k < CHUNK_STEPS; ++k)
-                ens_enqueue_batched(e, eg.groups, 0, k & 1, e->cap, e->side, e->fork, e->bjoin, nullptr);
-        } else if (batched) {
+        if (batched) {
             cudaEventRecord(e->fork, e->cap);
             for (int l = 0; l < lanes; ++l) cudaStreamWaitEvent(e->lcap[l], e->fork, 0);
             for (int k = 0; k < CHUNK_STEPS; ++k)
                 for (int l = 0; l < lanes; ++l) {
                     if (k == 0 && l > 0) cudaStreamWaitEvent(e->lcap[l], e->lstart, 0);
-                    ens_enqueue_batched(e, eg.groups, l, k & 1, e->lcap[l], e->lside[l], e->lfork[l], e->ljoin[l],
-                                        k == 0 && l + 1 < lanes ? e->lstart : nullptr, e->lbulk[l],
-                                        e->lbdone[l]);
+                    ens_enqueue_batched(e, eg.groups, l, k & 1, k == 0, k == 0 && l + 1 < lanes ? e->lstart : nullptr);
                 }
             for (int l = 0; l < lanes; ++l) {
+                cudaStreamWaitEvent(e->lcap[l], e->lbdone[l][(CHUNK_STEPS - 1) & 1], 0);
                 cudaEventRecord(e->ldone[l], e->lcap[l]);
                 cudaStreamWaitEvent(e->cap, e->ldone[l], 0);
             }
@@ -2143,7 +2179,8 @@ int ens_graph(lbm_ensemble_t *e, const std::vector<int> &set, cudaGraphExec_t *o
                 lbm_t *h = e->members[i];
                 cudaStreamWaitEvent(h->cap, e->fork, 0);
                 for (int k = 0; k < CHUNK_STEPS; ++k)
-                    enqueue_step(h, k & 1, h->cap, nullptr, nullptr, true, false);
+                    enqueue_step(h, k & 1, h->cap, nullptr, nullptr, true, k == 0);
+                join_bulk(h, (CHUNK_STEPS - 1) & 1, h->cap);
                 cudaEventRecord(e->join[i], h->cap);
                 cudaStreamWaitEvent(e->cap, e->join[i], 0);
             }
@@ -2152,7 +2189,7 @@ int ens_graph(lbm_ensemble_t *e, const std::vector<int> &set, cudaGraphExec_t *o
     }
     cudaGraphExec_t x = nullptr;
     if (err == cudaSuccess)
-        err = cudaGraphInstantiate(&x, g, batched && lanes > 1 ? cudaGraphInstantiateFlagUseNodePriority : 0);
+        err = cudaGraphInstantiate(&x, g, cudaGraphInstantiateFlagUseNodePriority);
     if (g) cudaGraphDestroy(g);
     if (err != cudaSuccess) {
         for (auto &grp : eg.groups)
@@ -2185,9 +2222,7 @@ int lbm_ensemble_create(lbm_t *const *members, int n, lbm_ensemble_t **out) {
     e->members.assign(members, members + n);
     e->stream = members[0]->stream;
     cudaError_t err = cudaStreamCreateWithFlags(&e->cap, cudaStreamNonBlocking);
-    if (err == cudaSuccess) err = cudaStreamCreateWithFlags(&e->side, cudaStreamNonBlocking);
     if (err == cudaSuccess) err = cudaEventCreateWithFlags(&e->fork, cudaEventDisableTiming);
-    if (err == cudaSuccess) err = cudaEventCreateWithFlags(&e->bjoin, cudaEventDisableTiming);
     // lanes: the latency-bound kernels' streams at the greatest priority,
     // the bulk kernels' at the least, so that one lane's prep, remap and
     // force blocks are dispatched ahead of the other lane's pending bulk blocks
@@ -2197,7 +2232,7 @@ int lbm_ensemble_create(lbm_t *const *members, int n, lbm_ensemble_t **out) {
         err = cudaStreamCreateWithPriority(&e->lcap[l], cudaStreamNonBlocking, greatest);
         if (err == cudaSuccess) err = cudaStreamCreateWithPriority(&e->lside[l], cudaStreamNonBlocking, greatest);
         if (err == cudaSuccess) err = cudaStreamCreateWithPriority(&e->lbulk[l], cudaStreamNonBlocking, least);
-        for (cudaEvent_t *ev : {&e->lfork[l], &e->ljoin[l], &e->ldone[l], &e->lbdone[l]})
+        for (cudaEvent_t *ev : {&e->lfork[l], &e->ljoin[l], &e->ldone[l], &e->lbdone[l][0], &e->lbdone[l][1]})
             if (err == cudaSuccess) err = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
     }
     if (err == cudaSuccess) err = cudaEventCreateWithFlags(&e->lstart, cudaEventDisableTiming);

@@ -12,9 +12,9 @@
 //            all 19 b (f~_{-b}(x) where x - e_b lies beyond a no-slip wall,
 //            Eq. 4), LBGK relaxation to the second-order equilibrium with
 //            Guo's forcing, store; solid cells store deviation 0.
-//  boundary  only the listed fluid cells (F_NEAR or F_SOLID_PREV: they lie in
-//            the cubes around the bodies; the bulk kernel leaves them alone,
-//            so the two kernels may run concurrently):
+//  boundary  only the listed fluid cells (F_NEAR, F_SOLID_PREV or F_LINK: they
+//            lie in the cubes around the bodies; the bulk kernel leaves them
+//            alone, so the two kernels may run concurrently):
 //              - x was solid at n-1 (uncovered): f_b = f_eq(rho_avg, u_w(x)),
 //                rho_avg the mean density of the D3Q19 neighbours that are
 //                fluid in both epochs (1 if none), u_w at the state of step n;
@@ -983,7 +983,7 @@ template <typename R> __device__ __forceinline__ R lane_sum(R v) {
     return v;
 }
 
-// The cells the remap listed (fluid with F_NEAR or F_SOLID_PREV): refill,
+// The cells the remap listed (fluid with a flag of F_LISTED): refill,
 // bounce-back at walls and moving obstacles, then LBGK, a warp a cell with lane b
 // the direction b: the 19 pulls, wall velocities and relaxations run side by side
 // and the cell's sums by shuffles.  Latency-bound (some hundred cells a body): a
@@ -1114,7 +1114,7 @@ __device__ __forceinline__ void boundary_body(const Device &dv, const StepPtrs &
 }
 
 // grid of the boundary kernel: `turns` cells a warp for the cells a body of
-// half-width E usually lists (within ~1.2 cells of its surface: about 15 E^2 for
+// half-width E usually lists (within 1.5 cells of its surface: about 18 E^2 for
 // the bodies of the workloads), at most what the SMs hold at once; longer lists
 // take more turns.  A batched block pays its member lookup before its first cell
 // and runs beside other members' blocks (48 boxes, 32 steps: 23.4 ms with 4 cells a
@@ -1123,7 +1123,7 @@ int sm_count();
 constexpr int BOUNDARY_BATCH_TURNS = 4;
 int boundary_blocks(const Device &dv, int turns) {
     const long long E = (dv.remap_side - 1) / 2 - REMAP_MARGIN, per = BOUNDARY_WARPS * turns;
-    const long long blocks = ((long long)dv.nb * 15 * E * E + per - 1) / per;
+    const long long blocks = ((long long)dv.nb * 18 * E * E + per - 1) / per;
     return (int)std::min<long long>(std::max<long long>(blocks, 1), 4LL * sm_count());
 }
 
@@ -1620,10 +1620,6 @@ void launch_batch_cells(int k, int variant, const Batch &bt, unsigned blocks, in
     case 2: boundary_batch<__half><<<blocks, 32 * BOUNDARY_WARPS, 0, s>>>(bt); break;
     default: boundary_batch<__nv_bfloat16><<<blocks, 32 * BOUNDARY_WARPS, 0, s>>>(bt); break;
     }
-}
-
-bool needs_boundary_fix(const Device &dv) {
-    return dv.nb > 0;
 }
 
 }  // namespace lbm
