@@ -98,12 +98,12 @@ __global__ void init_flags_kernel(const Domain d, uint8_t *f0, uint8_t *f1, uint
 // neighbour's 1.42 cells, and the floor of the upper bound loses up to one.
 constexpr int STATIC_REACH = 4;
 
-// Axis a of a body's geometry record from that axis' centre coordinate,
-// velocity, angular velocity and the body x axis' component.  Every FP64
+// Axis a of a body's geometry record from that axis' centre coordinate and
+// velocity (geom_place), angular velocity and the body x axis' component
+// (geom_turn).  Every FP64
 // rounding is explicit, so a record made here and one made by the
 // rigid-body step's warp agree bit for bit.
-__device__ inline void geom_axis(const Domain &d, const BodyProps &p, int a, double Xa, double Va, double Wa,
-                                 double axa, BodyGeom &g) {
+__device__ inline void geom_place(const Domain &d, const BodyProps &p, int a, double Xa, double Va, BodyGeom &g) {
     const int n = a == 0 ? d.nx : (a == 1 ? d.ny : d.nz);
     const int per = a == 0 ? d.px : (a == 1 ? d.py : d.pz);
     const double inv = a == 0 ? d.inx : (a == 1 ? d.iny : d.inz);
@@ -117,8 +117,6 @@ __device__ inline void geom_axis(const Domain &d, const BodyProps &p, int a, dou
     g.cfd[a] = __dsub_rn(c, fc);
     g.cf[a] = (float)g.cfd[a];
     g.v[a] = (float)Va;
-    g.w[a] = (float)Wa;
-    g.ax[a] = (float)axa;
     int lo = (int)floor(__dsub_rn(Xa, p.reach)), hi = (int)floor(__dadd_rn(Xa, p.reach));
     int width = hi - lo + 1;
     int elo = lo - STATIC_REACH, ewidth = width + 2 * STATIC_REACH;
@@ -134,6 +132,11 @@ __device__ inline void geom_axis(const Domain &d, const BodyProps &p, int a, dou
     g.box[3 + a] = width;
     g.ebox[a] = elo;
     g.ebox[3 + a] = ewidth;
+}
+
+__device__ inline void geom_turn(int a, double Wa, double axa, BodyGeom &g) {
+    g.w[a] = (float)Wa;
+    g.ax[a] = (float)axa;
 }
 
 __device__ inline void geom_scalars(const BodyProps &p, BodyGeom &g) {
@@ -163,7 +166,8 @@ __device__ void make_geom(const Domain &d, const BodyProps &p, const BodyState &
                            __dmul_rn(2.0, __fma_rn(qx, qz, -__dmul_rn(w, qy)))};
     bool out = false;
     for (int a = 0; a < 3; ++a) {
-        geom_axis(d, p, a, s.X[a], s.V[a], s.W[a], axv[a], g);
+        geom_place(d, p, a, s.X[a], s.V[a], g);
+        geom_turn(a, s.W[a], axv[a], g);
         out = out || outside_walls(d, p, a, s.X[a], axv[a]);
     }
     geom_scalars(p, g);
@@ -637,7 +641,11 @@ template <> __device__ inline double load_dev<__nv_bfloat16>(const __nv_bfloat16
     return (double)__bfloat162float(*p);
 }
 
-constexpr int FORCE_THREADS = 256;
+constexpr int FORCE_THREADS = 256;                  // link threads of a force block ...
+constexpr int FORCE_BLOCK = FORCE_THREADS + 64;     // ... and the two warps of the rigid-body step
+
+// barrier of the link threads
+__device__ __forceinline__ void link_sync() { asm volatile("bar.sync 1, %0;" ::"n"(FORCE_THREADS) : "memory"); }
 constexpr int MAX_SEGMENTS = 1024;
 
 // minimum image of a cell difference o (|o| < n + 1) by integer compares
@@ -653,73 +661,155 @@ __device__ inline double wrap_near(double d, int n, int periodic) {
     return d > h ? d - n : (d < -h ? d + n : d);
 }
 
-// Rigid-body step (Algorithm 1, Eq. totalFSwimmer) of body b by one warp
-// (all 32 lanes call it).  An FP64 warp instruction costs the same however
-// many lanes it carries, so lanes hold components: six load components,
-// three axes, nine rotation-matrix entries, four quaternion components.
-// Per axis it adds, in order, the momentum-exchange sum, g times the
-// volume, the body's drive terms in term order and its springs in spring
-// order (body_loads' scratch), then advances by semi-implicit Euler
-// (dt = 1) in FP64.  It also writes the geometry record of the new state
-// into that state's slot, with its stamp, and checks the new state (walls,
-// finite, at most MAX_STEP per step).
-__device__ void integrate_body_warp(const Device &dv, const StepPtrs &sp, int b, int with_fluid) {
+// Rigid-body step (Algorithm 1, Eq. totalFSwimmer) of body b by two warps, the
+// translation by one and the rotation by the other.  An FP64 warp instruction
+// occupies its sub-partition for the same ~64 cycles however many lanes it
+// carries, so lanes hold components (six load components, three axes, nine
+// rotation-matrix entries, four quaternion components) and the two halves sit on
+// different sub-partitions.  Per axis it adds, in order, the momentum-exchange
+// sum, g times the volume, the body's drive terms in term order and its springs
+// in spring order (body_loads' scratch), then advances by semi-implicit Euler
+// (dt = 1) in FP64.  Both halves write their part of the geometry record of the
+// new state into that state's slot, with its stamp, and check the new state
+// (walls, finite, at most MAX_STEP per step).
+//
+// `wait()` separates what depends on the state of step n alone (loads, the
+// external force, R(q): done while the link sums are formed) from what needs the
+// hydrodynamic load; it returns false in a block that does not finish the body.
+// (128 x 64 x 64 channel, a step: 40.1 us with one warp doing it all after the
+// sums, 34.6 us so.)
+
+// the hydrodynamic load of step n: lane i < 6 component i of force and torque
+__device__ __forceinline__ double hydro_load(const Device &dv, const StepPtrs &sp, int b, int with_fluid,
+                                             const double (&c)[3]) {
     constexpr unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    const long long tstep = *dv.t_dev;
-    const BodyProps *pb = dv.props + b;
-    const double *st = reinterpret_cast<const double *>(sp.body_cur + b);       // X q V W
-    const int ax = lane < 3 ? lane : 0;
-
-    // external force on axis ax: g times the volume, then the body's drive
-    // terms in term order and its springs in spring order (loaded first, so
-    // that their chains of dependent loads overlap the ones below)
-    double Fext = dv.g[ax] * pb->volume;
-    if (lane < 3) {
-        for (int k = pb->drive_first; k < pb->drive_first + pb->drive_count; ++k) Fext += dv.drive_f[3 * k + ax];
-        for (int kk = pb->spring_first; kk < pb->spring_first + pb->spring_count; ++kk) {
-            const int k = dv.spring_list[kk];
-            const double f = dv.spring_f[3 * k + ax];
-            Fext += dv.springs[k].i == b ? f : -f;
-        }
-    }
-
-    // hydrodynamic load of step n, lane i < 6 component i
     double hyd = 0.0;
     if (with_fluid && dv.precision == 0) {
-        if (lane < 6)
-            for (int k = 0; k < FORCE_BLOCKS; ++k) hyd += __ldcg(dv.fpart + ((long long)b * FORCE_BLOCKS + k) * 6 + lane);
-    } else if (with_fluid) {
-        // F = S1 / 36 + Fv, T = (S2 - c x S1) / 36 + Tv - c x Fv with c the
-        // centre's position within its cell (the force kernel's terms)
-        double fv = 0.0;
-        int si = 0;
         if (lane < 6) {
-            fv = (double)__ldcg(dv.fx + b * 6 + lane) * (1.0 / (double)(1LL << FIX_BITS));
-            si = __ldcg(dv.fi + b * 6 + lane);
-            dv.fx[b * 6 + lane] = 0;
-            dv.fi[b * 6 + lane] = 0;
+            double v[FORCE_BLOCKS];
+#pragma unroll
+            for (int k = 0; k < FORCE_BLOCKS; ++k) v[k] = __ldcg(dv.fpart + ((long long)b * FORCE_BLOCKS + k) * 6 + lane);
+#pragma unroll
+            for (int k = 0; k < FORCE_BLOCKS; ++k) hyd += v[k];
+        }
+    } else if (with_fluid) {
+        // F = S1 / 36 + Fv, T = S2 / 36 + Tv - c x F with c the centre's
+        // position within its cell (the force kernel's terms)
+        if (lane < 6) {
+            const long long fx = __ldcg(dv.fx + b * 6 + lane);
+            const int si = __ldcg(dv.fi + b * 6 + lane);
+            hyd = fma((double)si, 1.0 / 36.0, (double)fx * (1.0 / (double)(1LL << FIX_BITS)));
         }
         const int i = lane % 3, j = (i + 1) % 3, k = (i + 2) % 3;
-        const double s1j = (double)__shfl_sync(FULL, si, j), s1k = (double)__shfl_sync(FULL, si, k);
-        const double fvj = __shfl_sync(FULL, fv, j), fvk = __shfl_sync(FULL, fv, k);
-        const double *c = dv.geom[sp.parity * dv.nb + b].cfd;
-        if (lane < 3) hyd = (double)si * (1.0 / 36.0) + fv;
-        else if (lane < 6)
-            hyd = ((double)si - (c[j] * s1k - c[k] * s1j)) * (1.0 / 36.0) + fv - (c[j] * fvk - c[k] * fvj);
+        const double fj = __shfl_sync(FULL, hyd, j), fk = __shfl_sync(FULL, hyd, k);
+        const double cj = j == 0 ? c[0] : (j == 1 ? c[1] : c[2]), ck = k == 0 ? c[0] : (k == 1 ? c[1] : c[2]);
+        if (lane >= 3) hyd = fma(ck, fj, fma(-cj, fk, hyd));
     }
+    return hyd;
+}
+
+// external force on axis ax: g times the volume, then the body's drive terms in
+// term order and its springs in spring order
+__device__ __forceinline__ double external_force(const Device &dv, const BodyProps *pb, int b, int ax) {
+    double F = dv.g[ax] * pb->volume;
+    const int d0 = pb->drive_first, d1 = d0 + pb->drive_count, s0 = pb->spring_first, s1 = s0 + pb->spring_count;
+    // the springs' chains of dependent loads start first
+    constexpr int AHEAD = 4;
+    double fs[AHEAD];
+#pragma unroll
+    for (int i = 0; i < AHEAD; ++i) {
+        fs[i] = 0.0;
+        if (s0 + i < s1) {
+            const int k = dv.spring_list[s0 + i];
+            const double f = dv.spring_f[3 * k + ax];
+            fs[i] = dv.springs[k].i == b ? f : -f;
+        }
+    }
+    for (int k = d0; k < d1; ++k) F += dv.drive_f[3 * k + ax];
+#pragma unroll
+    for (int i = 0; i < AHEAD; ++i)
+        if (s0 + i < s1) F += fs[i];
+    for (int kk = s0 + AHEAD; kk < s1; ++kk) {
+        const int k = dv.spring_list[kk];
+        const double f = dv.spring_f[3 * k + ax];
+        F += dv.springs[k].i == b ? f : -f;
+    }
+    return F;
+}
+
+// entries [o, o + n) of the 13 of a state, lane i < n entry o + i, into the new
+// state, its stamp and its tape and history entries
+__device__ __forceinline__ void put_state(const Device &dv, const StepPtrs &sp, int b, long long tstep,
+                                          const TapeCtl &tc, int o, int n, double v) {
+    const int lane = threadIdx.x & 31;
+    if (lane >= n) return;
+    reinterpret_cast<double *>(sp.body_next + b)[o + lane] = v;
+    reinterpret_cast<double *>(dv.gstamp + (sp.parity ^ 1) * dv.nb + b)[o + lane] = v;
+    const long long j = tstep - tc.t0;
+    if (tc.on && j >= 0 && j < tc.cap) tc.state[((j + 2) * dv.nb + b) * 13 + o + lane] = v;
+    if (dv.hist) dv.hist[((tstep % dv.hist_cap) * dv.nb + b) * 13 + o + lane] = v;
+}
+
+template <typename Wait>
+__device__ __forceinline__ void integrate_translation(const Device &dv, const StepPtrs &sp, int b, int with_fluid,
+                                                      Wait wait) {
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, ax = lane < 3 ? lane : 0;
+    const BodyProps *pb = dv.props + b;
+    const double *st = reinterpret_cast<const double *>(sp.body_cur + b);       // X q V W
+    const double X = st[ax], V = st[7 + ax], inv_m = pb->inv_m;
+    const long long tstep = *dv.t_dev;
+    const double prev = lane < 6 ? dv.fh[b * 6 + lane] : 0.0;
+    const TapeCtl tc = dv.tape ? *dv.tape : TapeCtl{};
+    const double Fext = external_force(dv, pb, b, ax);
+    const double *cg = dv.geom[sp.parity * dv.nb + b].cfd;
+    const double c[3] = {cg[0], cg[1], cg[2]};
+    if (!wait()) return;
+    const double hyd = hydro_load(dv, sp, b, with_fluid, c);
     double v = hyd;
     if (lane < 6) {
-        const double prev = dv.fh[b * 6 + lane];
         dv.fh[b * 6 + lane] = hyd;
         if (dv.avg_force && tstep > 0) v = 0.5 * (hyd + prev);
     }
+    const double Vn = V + (v + Fext) * inv_m;
+    const double Xn = X + Vn;
+    put_state(dv, sp, b, tstep, tc, 0, 3, Xn);
+    put_state(dv, sp, b, tstep, tc, 7, 3, Vn);
+    if (lane < 6) {
+        const long long j = tstep - tc.t0;
+        if (tc.on && j >= 0 && j < tc.cap) tc.force[(j * dv.nb + b) * 6 + lane] = hyd;
+    }
+    BodyGeom *g = dv.geom + (sp.parity ^ 1) * dv.nb + b;
+    if (lane < 3) geom_place(dv.dom, *pb, ax, Xn, Vn, *g);
+    if (lane == 0) geom_scalars(*pb, *g);
+    const bool finite = __all_sync(FULL, lane >= 3 || (isfinite(Xn) && isfinite(Vn)));
+    const bool fast = __any_sync(FULL, lane < 3 && fabs(Vn) > MAX_STEP);
+    if (lane == 0 && (!finite || fast)) atomicOr(dv.status, !finite ? ST_NAN : ST_UNSTABLE);
+}
 
-    // translation, lanes 0..2
-    const double F = v + Fext;
-    const double Vn = st[7 + ax] + F * pb->inv_m;
-    const double Xn = st[ax] + Vn;
-
+template <typename Wait>
+__device__ __forceinline__ void integrate_rotation(const Device &dv, const StepPtrs &sp, int b, int with_fluid,
+                                                   Wait wait) {
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, ax = lane < 3 ? lane : 0;
+    const BodyProps *pb = dv.props + b;
+    const double *st = reinterpret_cast<const double *>(sp.body_cur + b);       // X q V W
+    const double W = st[10 + ax], inv_I = pb->inv_inertia[ax];
+    const long long tstep = *dv.t_dev;
+    const double prev = lane < 6 ? dv.fh[b * 6 + lane] : 0.0;
+    const TapeCtl tc = dv.tape ? *dv.tape : TapeCtl{};
+    const double *cg = dv.geom[sp.parity * dv.nb + b].cfd;
+    const double c[3] = {cg[0], cg[1], cg[2]};
+    // with walls: the new position again, for the wall check of a capsule's ends
+    const bool walls = !(dv.dom.px && dv.dom.py && dv.dom.pz);
+    double X = 0.0, V = 0.0, inv_m = 0.0, Fext = 0.0;
+    if (walls) {
+        X = st[ax];
+        V = st[7 + ax];
+        inv_m = pb->inv_m;
+        Fext = external_force(dv, pb, b, ax);
+    }
     // R(q) of state n, entry (r, c) on lane 3 r + c < 9: 1 - 2 (a^2 + b^2)
     // on the diagonal, 2 (p q +- w u) off it
     const double qw = st[3], qv[3] = {st[4], st[5], st[6]};
@@ -739,15 +829,19 @@ __device__ void integrate_body_warp(const Device &dv, const StepPtrs &sp, int b,
         }
         Rrc = base + 2.0 * (A * Bq + Cq * D);
     }
-    // Omega += R diag(1/I) R^T T, lanes 0..2
-    const double T0 = __shfl_sync(FULL, v, 3), T1 = __shfl_sync(FULL, v, 4), T2 = __shfl_sync(FULL, v, 5);
     const double R0i = __shfl_sync(FULL, Rrc, ax), R1i = __shfl_sync(FULL, Rrc, 3 + ax),
                  R2i = __shfl_sync(FULL, Rrc, 6 + ax);
-    const double Tb = (R0i * T0 + R1i * T1 + R2i * T2) * pb->inv_inertia[ax];
-    const double Tb0 = __shfl_sync(FULL, Tb, 0), Tb1 = __shfl_sync(FULL, Tb, 1), Tb2 = __shfl_sync(FULL, Tb, 2);
     const double Ri0 = __shfl_sync(FULL, Rrc, 3 * ax), Ri1 = __shfl_sync(FULL, Rrc, 3 * ax + 1),
                  Ri2 = __shfl_sync(FULL, Rrc, 3 * ax + 2);
-    const double Wn = st[10 + ax] + (Ri0 * Tb0 + Ri1 * Tb1 + Ri2 * Tb2);
+    if (!wait()) return;
+    const double hyd = hydro_load(dv, sp, b, with_fluid, c);
+    double v = hyd;
+    if (dv.avg_force && tstep > 0) v = 0.5 * (hyd + prev);
+    // Omega += R diag(1/I) R^T T, lanes 0..2
+    const double T0 = __shfl_sync(FULL, v, 3), T1 = __shfl_sync(FULL, v, 4), T2 = __shfl_sync(FULL, v, 5);
+    const double Tb = (R0i * T0 + R1i * T1 + R2i * T2) * inv_I;
+    const double Tb0 = __shfl_sync(FULL, Tb, 0), Tb1 = __shfl_sync(FULL, Tb, 1), Tb2 = __shfl_sync(FULL, Tb, 2);
+    const double Wn = W + (Ri0 * Tb0 + Ri1 * Tb1 + Ri2 * Tb2);
 
     // q += 1/2 (0, Omega) (x) q, renormalised; lane 0 the scalar part,
     // lane 1 + i the vector component i
@@ -769,35 +863,11 @@ __device__ void integrate_body_warp(const Device &dv, const StepPtrs &sp, int b,
     sq += __shfl_xor_sync(FULL, sq, 1);
     sq += __shfl_xor_sync(FULL, sq, 2);
     const double qn = q4 * rsqrt(sq);
+    put_state(dv, sp, b, tstep, tc, 3, 4, qn);
+    put_state(dv, sp, b, tstep, tc, 10, 3, Wn);
 
-    // checks of state n+1
-    const bool finite = lane >= 3 || (isfinite(Xn) && isfinite(Vn) && isfinite(Wn));
-    const bool all_finite = __all_sync(FULL, finite);
-    const bool fast = __any_sync(FULL, lane < 3 && fabs(Vn) > MAX_STEP);
-
-    // the new state, its tape and history entries
-    auto put = [&](double *o) {
-        if (lane < 3) {
-            o[lane] = Xn;
-            o[7 + lane] = Vn;
-            o[10 + lane] = Wn;
-        }
-        if (lane < 4) o[3 + lane] = qn;
-    };
-    put(reinterpret_cast<double *>(sp.body_next + b));
-    if (dv.tape) {
-        const TapeCtl tc = *dv.tape;
-        const long long j = tstep - tc.t0;
-        if (tc.on && j >= 0 && j < tc.cap) {
-            put(tc.state + ((j + 2) * dv.nb + b) * 13);
-            if (lane < 6) tc.force[(j * dv.nb + b) * 6 + lane] = hyd;
-        }
-    }
-    if (dv.hist) put(dv.hist + ((tstep % dv.hist_cap) * dv.nb + b) * 13);
-
-    // the geometry record of state n+1 (its slot is the body buffer it was
-    // written to), lanes 0..2 an axis each; the body x axis is column 0 of R(q_{n+1})
-    const int slot = sp.parity ^ 1;
+    // the rotational part of the new state's geometry record; the body x axis is
+    // column 0 of R(q_{n+1})
     const double nw = __shfl_sync(FULL, qn, 0), nq[3] = {__shfl_sync(FULL, qn, 1), __shfl_sync(FULL, qn, 2),
                                                          __shfl_sync(FULL, qn, 3)};
     // column 0 of R: 1 - 2 (y^2 + z^2), 2 (x y + w z), 2 (x z - w y), one
@@ -808,16 +878,14 @@ __device__ void integrate_body_warp(const Device &dv, const StepPtrs &sp, int b,
         const double Cq = ax == 0 ? -nq[2] : (ax == 1 ? nw : -nw), D = ax == 0 ? nq[2] : (ax == 1 ? nq[2] : nq[1]);
         axa = (ax == 0 ? 1.0 : 0.0) + 2.0 * (A * B + Cq * D);
     }
-    BodyGeom *g = dv.geom + slot * dv.nb + b;
-    const bool out = lane < 3 && outside_walls(dv.dom, *pb, ax, Xn, axa);
-    if (lane < 3) geom_axis(dv.dom, *pb, ax, Xn, Vn, Wn, axa, *g);
-    if (lane == 0) geom_scalars(*pb, *g);
-    put(reinterpret_cast<double *>(dv.gstamp + slot * dv.nb + b));
-    const bool any_out = __any_sync(FULL, out);
-    if (lane == 0) {
-        if (!all_finite) atomicOr(dv.status, ST_NAN);
-        else if (fast) atomicOr(dv.status, ST_UNSTABLE);
-        if (any_out) atomicOr(dv.status, ST_OUTSIDE);
+    BodyGeom *g = dv.geom + (sp.parity ^ 1) * dv.nb + b;
+    if (lane < 3) geom_turn(ax, Wn, axa, *g);
+    const bool finite = __all_sync(FULL, lane >= 3 || isfinite(Wn));
+    if (lane == 0 && !finite) atomicOr(dv.status, ST_NAN);
+    if (walls) {
+        const double Xn = X + (V + (v + Fext) * inv_m);
+        const bool any_out = __any_sync(FULL, lane < 3 && outside_walls(dv.dom, *pb, ax, Xn, axa));
+        if (lane == 0 && any_out) atomicOr(dv.status, ST_OUTSIDE);
     }
 }
 
@@ -881,6 +949,37 @@ __device__ __forceinline__ void force_body(const Device &dv, const StepPtrs &sp,
     const long long C = d.C;
     const float s = dv.f16_inv_scale;
 
+    // the two warps past the link warps integrate the body in the block that
+    // finishes it; what they need of the state is loaded and formed meanwhile
+    __shared__ int last_of_body;
+    if (threadIdx.x >= FORCE_THREADS) {
+        auto wait = [&] {
+            __syncthreads();
+            return last_of_body != 0;
+        };
+        if (threadIdx.x < FORCE_THREADS + 32) integrate_translation(dv, sp, b, 1, wait);
+        else integrate_rotation(dv, sp, b, 1, wait);
+        if (!last_of_body) return;
+        asm volatile("bar.sync 2, 64;" ::: "memory");
+        if (threadIdx.x < FORCE_THREADS + 32) {
+            // the sums start the next step at zero
+            const int ln = threadIdx.x & 31;
+            if (sizeof(T) != 8 && ln < 6) {
+                dv.fx[b * 6 + ln] = 0;
+                dv.fi[b * 6 + ln] = 0;
+            }
+            if (ln == 0) {
+                dv.body_done[b] = 0u;
+                __threadfence();
+                if (atomicAdd(dv.blocks_done, 1u) == (unsigned)bk.gy - 1) {
+                    *dv.blocks_done = 0u;
+                    finish_step(dv, sp);
+                }
+            }
+        }
+        return;
+    }
+
     // exclusive prefix of the segment counts: thread t holds segments
     // [t per, (t+1) per), per <= 4 (side <= MAX_SEGMENTS), block scan
     __shared__ int prefix[MAX_SEGMENTS + 1];
@@ -903,7 +1002,7 @@ __device__ __forceinline__ void force_body(const Device &dv, const StepPtrs &sp,
             if (ln >= o) incl += v;
         }
         if (ln == 31) seg_warp[wp] = incl;
-        __syncthreads();
+        link_sync();
         int acc = incl - sum;
         for (int w = 0; w < wp; ++w) acc += seg_warp[w];
 #pragma unroll
@@ -914,7 +1013,7 @@ __device__ __forceinline__ void force_body(const Device &dv, const StepPtrs &sp,
         }
         if (threadIdx.x == FORCE_THREADS - 1) prefix[side] = acc;
     }
-    __syncthreads();
+    link_sync();
     const int total = prefix[side];
     const int chunk = (total + FORCE_BLOCKS - 1) / FORCE_BLOCKS;
     const int j0 = kb * chunk, j1 = min(total, j0 + chunk);
@@ -967,7 +1066,7 @@ __device__ __forceinline__ void force_body(const Device &dv, const StepPtrs &sp,
             for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
             if (lane == 0) part[warp][i] = v;
         }
-        __syncthreads();
+        link_sync();
         if (warp == 0) {
 #pragma unroll
             for (int i = 0; i < 6; ++i) {
@@ -1048,7 +1147,7 @@ __device__ __forceinline__ void force_body(const Device &dv, const StepPtrs &sp,
                 pi_[warp][i] = w;
             }
         }
-        __syncthreads();
+        link_sync();
         if (threadIdx.x < 6) {
             const int i = threadIdx.x;
             long long v = 0;
@@ -1059,40 +1158,27 @@ __device__ __forceinline__ void force_body(const Device &dv, const StepPtrs &sp,
             }
             if (v) atomicAdd(reinterpret_cast<unsigned long long *>(dv.fx + b * 6 + i), (unsigned long long)v);
             if (w) atomicAdd(dv.fi + b * 6 + i, w);
-            __threadfence();            // before the block counts itself done
         }
     }
-    // the last of body b's blocks integrates body b with its first warp
-    // (the drive and spring loads were evaluated beside the bulk kernel);
-    // the last body ends the step
-    __shared__ int last_of_body;
-    __syncthreads();
+    // the last of body b's blocks lets its integrating warps go on; the last body
+    // ends the step
+    link_sync();
     if (threadIdx.x == 0) {
         __threadfence();
         last_of_body = atomicAdd(dv.body_done + b, 1u) == (unsigned)bk.gx - 1;
+        __threadfence();
     }
     __syncthreads();
-    if (!last_of_body || threadIdx.x >= 32) return;
-    __threadfence();
-    integrate_body_warp(dv, sp, b, 1);
-    __syncwarp();
-    if (threadIdx.x != 0) return;
-    dv.body_done[b] = 0u;
-    __threadfence();
-    if (atomicAdd(dv.blocks_done, 1u) != (unsigned)bk.gy - 1) return;
-    __threadfence();
-    *dv.blocks_done = 0u;
-    finish_step(dv, sp);
 }
 
 template <typename T>
-__global__ void __launch_bounds__(FORCE_THREADS) force_kernel(const Device dv, const StepPtrs sp) {
+__global__ void __launch_bounds__(FORCE_BLOCK) force_kernel(const Device dv, const StepPtrs sp) {
     pdl_enter();
     force_body<T>(dv, sp, launch_blk());
 }
 
 template <typename T>
-__global__ void __launch_bounds__(FORCE_THREADS) force_batch(const Batch bt) {
+__global__ void __launch_bounds__(FORCE_BLOCK) force_batch(const Batch bt) {
     LBM_BATCH_MEMBER(bt);
     force_body<T>(sdv, ssp, sbk);
 }
@@ -1166,11 +1252,15 @@ __global__ void __launch_bounds__(512) near_tiles_kernel(const Device dv, const 
 }
 
 // the rigid-body step alone (bodies without fluid), one block: the loads,
-// then a warp a body
+// then two warps a body
 __global__ void __launch_bounds__(256) integrate_kernel(const Device dv, const StepPtrs sp, int with_fluid) {
     body_loads(dv, sp, threadIdx.x, threadIdx.x, blockDim.x);
     __syncthreads();
-    for (int b = threadIdx.x >> 5; b < dv.nb; b += blockDim.x >> 5) integrate_body_warp(dv, sp, b, with_fluid);
+    auto go = [] { return true; };
+    for (int i = threadIdx.x >> 5; i < 2 * dv.nb; i += blockDim.x >> 5) {
+        if (i & 1) integrate_rotation(dv, sp, i >> 1, with_fluid, go);
+        else integrate_translation(dv, sp, i >> 1, with_fluid, go);
+    }
     __syncthreads();
     if (threadIdx.x == 0) finish_step(dv, sp);
 }
@@ -1434,11 +1524,12 @@ void launch_remap(const Device &dv, const StepPtrs &sp, int init_mode, cudaStrea
 
 void launch_links(const Device &dv, const StepPtrs &sp, cudaStream_t s) {
     links_kernel<<<dim3(dv.link_side, dv.nb), 256, 0, s>>>(dv, sp);
-    loads_kernel<<<1, 64, 0, s>>>(dv, sp);
 }
 
+void launch_loads(const Device &dv, const StepPtrs &sp, cudaStream_t s) { loads_kernel<<<1, 64, 0, s>>>(dv, sp); }
+
 void launch_force(const Device &dv, const StepPtrs &sp, cudaStream_t s) {
-    const dim3 grid(FORCE_BLOCKS, dv.nb), block(FORCE_THREADS);
+    const dim3 grid(FORCE_BLOCKS, dv.nb), block(FORCE_BLOCK);
     const bool pdl = dv.pdl != 0;
     switch (dv.precision) {
     case 0: launch_kernel(pdl, force_kernel<double>, grid, block, 0, s, dv, sp); break;
@@ -1494,10 +1585,10 @@ void launch_batch_small(int k, const Batch &bt, unsigned blocks, int precision, 
     case BK_LOADS: loads_batch<<<blocks, 64, 0, s>>>(bt); break;
     case BK_FORCE:
         switch (precision) {
-        case 0: force_batch<double><<<blocks, FORCE_THREADS, 0, s>>>(bt); break;
-        case 1: force_batch<float><<<blocks, FORCE_THREADS, 0, s>>>(bt); break;
-        case 2: force_batch<__half><<<blocks, FORCE_THREADS, 0, s>>>(bt); break;
-        default: force_batch<__nv_bfloat16><<<blocks, FORCE_THREADS, 0, s>>>(bt); break;
+        case 0: force_batch<double><<<blocks, FORCE_BLOCK, 0, s>>>(bt); break;
+        case 1: force_batch<float><<<blocks, FORCE_BLOCK, 0, s>>>(bt); break;
+        case 2: force_batch<__half><<<blocks, FORCE_BLOCK, 0, s>>>(bt); break;
+        default: force_batch<__nv_bfloat16><<<blocks, FORCE_BLOCK, 0, s>>>(bt); break;
         }
         break;
     default: break;

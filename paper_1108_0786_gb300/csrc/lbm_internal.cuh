@@ -462,6 +462,7 @@ int list_variants(const Device &dv, int *vec, int *minb, int max);
 int default_vector_width(const Device &dv);
 void prepare_bulk_variants();           // host: shared-memory opt-in of the staged variants (once)
 void launch_links(const Device &dv, const StepPtrs &sp, cudaStream_t s);
+void launch_loads(const Device &dv, const StepPtrs &sp, cudaStream_t s);
 void launch_force(const Device &dv, const StepPtrs &sp, cudaStream_t s);
 void launch_integrate(const Device &dv, const StepPtrs &sp, int with_fluid, cudaStream_t s);
 void launch_tick(const Device &dv, const StepPtrs &sp, cudaStream_t s);

@@ -186,8 +186,8 @@ lbm::StepPtrs step_ptrs(lbm_t *h, int p, bool overlap = false) {
 // boundary cells and force + rigid-body step; the next step's chain follows at
 // once.  The bulk kernel runs on h->side beside it: the force sums read only
 // cells of the boundary kernel (F_LINK), so the chain of step n+1 needs nothing
-// of step n's bulk kernel until its boundary kernel.  The link lists and the
-// drive and spring loads run on h->side2 beside the boundary kernel.  What
+// of step n's bulk kernel until its boundary kernel.  The drive and spring loads
+// run on h->side2 beside the remap, the link lists beside the boundary kernel.  What
 // orders the shared buffers:
 //   bulk(n)      after remap(n) (flags n; the chain before it ends with
 //                boundary(n-1), the other writer of its sources) and, on its
@@ -213,6 +213,12 @@ void enqueue_step(lbm_t *h, int p, cudaStream_t s, cudaEvent_t *ev = nullptr, bo
         if (ev) cudaEventRecord(ev[2 * slot + 1], st);
         if (ran) ran[slot] = true;
     };
+    if (fork && bodies && fl) {
+        // the drive and spring loads need the states alone: beside the remap
+        cudaEventRecord(h->fork_ev, s);
+        cudaStreamWaitEvent(h->side2, h->fork_ev, 0);
+        lbm::launch_loads(h->dv, sp, h->side2);
+    }
     // captured steps leave the body preparation out (lbm_step runs it where needed)
     if (bodies && fl) run(LBM_KERNEL_REMAP, s, [&] { lbm::launch_remap(h->dv, sp, 0, s, !fork); });
     if (fork && bodies && fl) {
@@ -240,7 +246,10 @@ void enqueue_step(lbm_t *h, int p, cudaStream_t s, cudaEvent_t *ev = nullptr, bo
     if (fl) run(LBM_KERNEL_STREAM_COLLIDE, s, [&] { lbm::launch_stream_collide(h->dv, sp, s); });
     if (bodies && fl) {
         run(LBM_KERNEL_BOUNDARY, s, [&] { lbm::launch_boundary_fix(h->dv, sp, s); });
-        run(LBM_KERNEL_LINKS, s, [&] { lbm::launch_links(h->dv, sp, s); });
+        run(LBM_KERNEL_LINKS, s, [&] {
+            lbm::launch_links(h->dv, sp, s);
+            lbm::launch_loads(h->dv, sp, s);
+        });
     }
     if (bodies && fl) {
         // momentum exchange; the last block of each body runs its rigid-body step
@@ -283,6 +292,7 @@ void enqueue_overlapped(lbm_t *h, int p, cudaStream_t s, bool first) {
     // the chain
     lbm::launch_remap(h->dv, sp, 0, s);
     lbm::launch_links(h->dv, sp, s);
+    lbm::launch_loads(h->dv, sp, s);
     if (!first) cudaStreamWaitEvent(s, h->far_ev[q], 0);
     lbm::launch_boundary_fix(h->dv, sp, s);
     lbm::launch_near_bulk(h->dv, sp, s);
@@ -1649,6 +1659,7 @@ int lbm_adjoint_backward(lbm_t *h, const double *seed, double *grad_state, doubl
         CK(cudaEventRecord(join, ss));
         CK(cudaStreamWaitEvent(ss2, fork, 0));
         lbm::launch_links(dr, sp, ss2);
+        lbm::launch_loads(dr, sp, ss2);
         CK(cudaEventRecord(join2, ss2));
         lbm::launch_stream_collide(dr, sp, ms);
         if (copy_next && (rc3 = copy_slot(st, j + 1, ms))) return rc3;
@@ -2056,6 +2067,9 @@ void ens_enqueue_batched(lbm_ensemble_t *e, std::vector<EnsGroup> &groups, int l
             lbm::launch_batch_cells(k, e->variant[g.precision], b, g.blocks[k], g.precision, g.walls, st);
         }
     };
+    cudaEventRecord(fork, main);
+    cudaStreamWaitEvent(side, fork, 0);
+    small(lbm::BK_LOADS, side);
     // the batched remap takes its candidates from the body preparation
     small(lbm::BK_PREP, main);
     small(lbm::BK_REMAP, main);
@@ -2063,7 +2077,6 @@ void ens_enqueue_batched(lbm_ensemble_t *e, std::vector<EnsGroup> &groups, int l
     cudaEventRecord(fork, main);
     cudaStreamWaitEvent(side, fork, 0);
     small(lbm::BK_LINKS, side);
-    small(lbm::BK_LOADS, side);
     cudaEventRecord(join, side);
     if (!first) cudaStreamWaitEvent(main, e->lbdone[lane][p ^ 1], 0);
     cells(lbm::BK_BOUNDARY, main);
