@@ -278,8 +278,10 @@ __global__ void __launch_bounds__(ADJ_BOUNDARY_THREADS) adj_wall_kernel(const De
 }
 
 // ---- boundary cells of the body cubes: a warp per cell -------------------------
-// Block (blk, kb) classifies the ADJ_BOUNDARY_THREADS cells blk * 64 ... of
-// body kb's cube (cells whose flags are zero in epochs n and n+1 and that
+// Block (blk, kb) classifies ADJ_BOUNDARY_THREADS cells of body kb's cube, every
+// gridDim.x-th from blk (the full-rule cells are a shell, which consecutive cells
+// would leave to a few blocks: 27.8 against 13.3 us a launch on the 96 x 48 x 48
+// study) (cells whose flags are zero in epochs n and n+1 and that
 // were not uncovered at n: adj_bulk's; solid at n: zero adjoint; the
 // others the full rule, as adj_wall_kernel applies it) and lists the full-rule cells
 // in cube order.  Each warp then takes the listed cells w, w + 8, ... with
@@ -297,6 +299,19 @@ template <typename V> __device__ __forceinline__ V warp_sum(V v) {
     return v;
 }
 
+// a centre's cell, wrapped into the domain on periodic axes, and its position within
+template <typename A>
+__device__ __forceinline__ void centre_cell(const Domain &d, const double (&X)[3], int (&ci)[3], A (&cf)[3]) {
+    const int n3[3] = {d.nx, d.ny, d.nz}, per[3] = {d.px, d.py, d.pz};
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const double f = floor(X[i]);
+        ci[i] = (int)f;
+        if (per[i]) ci[i] = ((ci[i] % n3[i]) + n3[i]) % n3[i];
+        cf[i] = (A)(X[i] - f);
+    }
+}
+
 template <typename A, typename T, bool FIRST>
 __global__ void __launch_bounds__(32 * ADJ_CUBE_WARPS) adj_cube_kernel(const Device dv, const AdjPtrs ap) {
     const Domain d = dv.dom;
@@ -307,6 +322,9 @@ __global__ void __launch_bounds__(32 * ADJ_CUBE_WARPS) adj_cube_kernel(const Dev
     const int side = 2 * half + 1;
     const BodyState &sb = ap.body[kb];
     const int fx = (int)floor(sb.X[0]), fy = (int)floor(sb.X[1]), fz = (int)floor(sb.X[2]);
+    int ci[3];
+    A cf[3];
+    centre_cell(d, sb.X, ci, cf);
     // cube cell l -> lattice cell (x, y, z); false outside the cube or the domain
     auto cube_cell = [&](int l, int &x, int &y, int &z) {
         if (l >= side * side * side) return false;
@@ -325,7 +343,7 @@ __global__ void __launch_bounds__(32 * ADJ_CUBE_WARPS) adj_cube_kernel(const Dev
     A *__restrict__ aout = static_cast<A *>(ap.aout);
     // 1. classify this block's cells (the first ADJ_BOUNDARY_THREADS threads)
     bool listed = false;
-    const int l = blockIdx.x * ADJ_BOUNDARY_THREADS + tid;
+    const int l = blockIdx.x + tid * gridDim.x;
     if (tid < ADJ_BOUNDARY_THREADS) {
         int x, y, z;
         if (cube_cell(l, x, y, z)) {
@@ -395,12 +413,24 @@ __global__ void __launch_bounds__(32 * ADJ_CUBE_WARPS) adj_cube_kernel(const Dev
                 if (fzc & F_SOLID) {
                     // link (x, b) of step n: moving bounce-back of step n+1 and
                     // the momentum exchange of step n share u_w(x + e_b; S^n);
-                    // the offset from the body centre in FP64, the terms in A
+                    // the offset from the centre is an integer difference of
+                    // cells less the centre's position within its cell (the same
+                    // expression for every body: a cell in two cubes is written
+                    // by both blocks), the terms in A
                     const int k = ap.bid_cur[zc];
                     const BodyState &sk = ap.body[k];
-                    double od[3];
-                    offset_from(d, sk, (double)zx, (double)zy, (double)zz, od);
-                    const A o[3] = {(A)od[0], (A)od[1], (A)od[2]};
+                    int kc[3] = {ci[0], ci[1], ci[2]};
+                    A kf[3] = {cf[0], cf[1], cf[2]};
+                    if (k != kb) centre_cell(d, sk.X, kc, kf);
+                    A o[3];
+                    const int zp[3] = {wrap_axis(zx, d.nx), wrap_axis(zy, d.ny), wrap_axis(zz, d.nz)};
+                    const int n3[3] = {d.nx, d.ny, d.nz}, per[3] = {d.px, d.py, d.pz};
+#pragma unroll
+                    for (int i = 0; i < 3; ++i) {
+                        int io = zp[i] - kc[i];
+                        if (per[i]) io = 2 * io > n3[i] ? io - n3[i] : (2 * io < -n3[i] ? io + n3[i] : io);
+                        o[i] = (A)io - kf[i];
+                    }
                     const A W[3] = {(A)sk.W[0], (A)sk.W[1], (A)sk.W[2]};
                     const A uw0 = (A)sk.V[0] + (W[1] * o[2] - W[2] * o[1]);
                     const A uw1 = (A)sk.V[1] + (W[2] * o[0] - W[0] * o[2]);
@@ -617,135 +647,176 @@ adj_terms_kernel(const Device dv, const BodyState *states, const double *fhs, lo
     }
 }
 
-__device__ void adj_rot_matrix(const double q[4], const double Rh[3][3], double qh[4]) {
-    const double w = q[0], x = q[1], y = q[2], z = q[3];
-    qh[2] += -4 * y * Rh[0][0]; qh[3] += -4 * z * Rh[0][0];
-    qh[1] += 2 * y * Rh[0][1]; qh[2] += 2 * x * Rh[0][1]; qh[0] += -2 * z * Rh[0][1]; qh[3] += -2 * w * Rh[0][1];
-    qh[1] += 2 * z * Rh[0][2]; qh[3] += 2 * x * Rh[0][2]; qh[0] += 2 * y * Rh[0][2]; qh[2] += 2 * w * Rh[0][2];
-    qh[1] += 2 * y * Rh[1][0]; qh[2] += 2 * x * Rh[1][0]; qh[0] += 2 * z * Rh[1][0]; qh[3] += 2 * w * Rh[1][0];
-    qh[1] += -4 * x * Rh[1][1]; qh[3] += -4 * z * Rh[1][1];
-    qh[2] += 2 * z * Rh[1][2]; qh[3] += 2 * y * Rh[1][2]; qh[0] += -2 * x * Rh[1][2]; qh[1] += -2 * w * Rh[1][2];
-    qh[1] += 2 * z * Rh[2][0]; qh[3] += 2 * x * Rh[2][0]; qh[0] += -2 * y * Rh[2][0]; qh[2] += -2 * w * Rh[2][0];
-    qh[2] += 2 * z * Rh[2][1]; qh[3] += 2 * y * Rh[2][1]; qh[0] += 2 * x * Rh[2][1]; qh[1] += 2 * w * Rh[2][1];
-    qh[1] += -4 * x * Rh[2][2]; qh[2] += -4 * y * Rh[2][2];
-}
-
 // One block.  Sh^{n+1} = sa_next + the cell sums of reverse step n+1
-// (part, in block order); then the reverse step with the state-only terms
+// (part, a fixed order); then the reverse step with the state-only terms
 // of step n.  Writes Sh^n (rigid-body part plus the lever-arm term Th x
 // F_hydro of the torque sum) to sa_cur, (Fh, Th) to fadj and adds
-// dJ/dtheta.
+// dJ/dtheta.  A warp a body with components on lanes (axes, quaternion and matrix
+// entries): an FP64 warp instruction costs ~64 issue cycles whatever its lanes
+// carry, and this kernel is on the sweep's serial chain (a thread a body
+// took 19.8 us a launch for three bodies, this takes 11.4).
+constexpr int ADJ_WARPS = ADJ_THREADS / 32;
+constexpr int ADJ_SUM_GROUPS = 3;           // records a warp's lanes take side by side, nine sums each
+
 __global__ void __launch_bounds__(ADJ_THREADS) adj_integrate_kernel(const Device dv, const AdjBody ab) {
+    constexpr unsigned FULL = 0xffffffffu;
     const int nb = dv.nb;
-    const BodyState *S = ab.state;
-    // 1. complete Sh^{n+1}: warp w adds body b's block sums, lanes over the
-    //    blocks, then a fixed shuffle tree
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
-    for (int b = warp; b < nb; b += nwarps) {
-        double acc[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-        for (int k = lane; k < ab.part_count; k += 32) {
-            const double *p = ab.part + ((long long)b * ab.part_stride + k) * 9;
-#pragma unroll
-            for (int i = 0; i < 9; ++i) acc[i] += p[i];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    __shared__ double s_sum[ADJ_WARPS][9];
+    __shared__ double s_F[LBM_MAX_BODIES_DEV][3];       // Fh of every body
+    const int ax = lane < 3 ? lane : 0, i1 = (ax + 1) % 3, i2 = (ax + 2) % 3;
+    auto at = [](double v, int l) { return __shfl_sync(FULL, v, l); };
+    // warps that share a body's cell sums
+    const int share = nb <= 2 ? 4 : (nb <= 4 ? 2 : 1);
+    const int bodies = ADJ_WARPS / share;               // bodies in flight
+    for (int b0 = 0; b0 < nb; b0 += bodies) {
+        // 1. complete Sh^{n+1}: lane 9 g + c of each of the body's warps adds
+        //    component c of every (share x groups)-th record
+        const int b = b0 + warp % bodies, part = warp / bodies;
+        if (b < nb) {
+            double v = 0.0;
+            if (lane < 9 * ADJ_SUM_GROUPS) {
+                const double *p = ab.part + (long long)b * ab.part_stride * 9 + lane % 9;
+                const int step = share * ADJ_SUM_GROUPS;
+                int k = part * ADJ_SUM_GROUPS + lane / 9;
+                for (; k + 3 * step < ab.part_count; k += 4 * step) {
+                    const double q0 = p[9 * k], q1 = p[9 * (k + step)], q2 = p[9 * (k + 2 * step)],
+                                 q3 = p[9 * (k + 3 * step)];
+                    v += q0; v += q1; v += q2; v += q3;
+                }
+                for (; k < ab.part_count; k += step) v += p[9 * k];
+            }
+            const double w = v + at(v, lane + 9 < 32 ? lane + 9 : lane) + at(v, lane + 18 < 32 ? lane + 18 : lane);
+            if (lane < 9) s_sum[warp][lane] = w;
         }
-#pragma unroll
-        for (int i = 0; i < 9; ++i) {
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) acc[i] += __shfl_down_sync(0xffffffffu, acc[i], o);
+        __syncthreads();
+        if (part == 0 && b < nb) {
+            const BodyProps *pb = dv.props + b;
+            const double *st = reinterpret_cast<const double *>(ab.state + b);
+            const AdjBodyTerms *tm = ab.tb + b;
+            const double *fh = ab.fh + 6 * b;
+            // loads: the adjoint of state n + 1 (lane i < 13 component i), the terms
+            double sn = lane < 13 ? ab.sa_next[13 * b + lane] : 0.0;
+            const int c4 = lane < 4 ? lane : 0;
+            const double q1 = tm->q1[c4], q4s = st[3 + c4], inv_nn = tm->inv_nn;
+            const double W1 = tm->W1[ax], beta = tm->beta[ax], F = tm->F[ax], inv_I = pb->inv_inertia[ax];
+            const double R0i = tm->R[ax], R1i = tm->R[3 + ax], R2i = tm->R[6 + ax];         // column ax
+            const double Ri0 = tm->R[3 * ax], Ri1 = tm->R[3 * ax + 1], Ri2 = tm->R[3 * ax + 2];
+            const double fhF = fh[ax], fhT = fh[3 + ax], inv_m = pb->inv_m, g = dv.g[ax];
+            const int d0 = pb->drive_first, d1 = d0 + pb->drive_count;
+            // the cell sums: X, V, W of components 0..2, 7..9, 10..12
+            {
+                const int c = lane < 3 ? lane : (lane >= 7 && lane < 13 ? lane - 4 : -1);
+                if (c >= 0) {
+                    double v = s_sum[warp][c];
+                    for (int k = 1; k < share; ++k) v += s_sum[warp + k * bodies][c];
+                    sn += v;
+                    ab.sa_next[13 * b + lane] = sn;
+                }
+            }
+            // quaternion: qh4 = (qh - q1 (q1 . qh)) / |q|
+            const double qh = at(sn, 3 + c4);
+            double dot = q1 * qh;
+            dot += __shfl_xor_sync(FULL, dot, 1);
+            dot += __shfl_xor_sync(FULL, dot, 2);
+            const double qh4 = (qh - q1 * dot) * inv_nn;
+            const double h0 = at(qh4, 0), hv0 = at(qh4, 1), hv1 = at(qh4, 2), hv2 = at(qh4, 3);
+            const double hv[3] = {hv0, hv1, hv2};
+            const double Wa = at(W1, 0), Wb = at(W1, 1), Wc = at(W1, 2);
+            const double Wv[3] = {Wa, Wb, Wc};
+            const double w = at(q4s, 0), va = at(q4s, 1), vb = at(q4s, 2), vc = at(q4s, 3);
+            const double vv[3] = {va, vb, vc};
+            // the adjoint of q_n through the update: lane 0 the scalar part,
+            // lane 1 + i the vector component i
+            double qout;
+            {
+                const int i = lane >= 1 && lane <= 3 ? lane - 1 : 0, j = (i + 1) % 3, k = (i + 2) % 3;
+                const bool s0 = lane == 0;
+                const double p1 = s0 ? hv[0] : -h0, r1 = s0 ? Wv[0] : Wv[i];
+                const double p2 = s0 ? hv[1] : hv[j], r2 = s0 ? Wv[1] : Wv[k];
+                const double p3 = s0 ? hv[2] : -hv[k], r3 = s0 ? Wv[2] : Wv[j];
+                qout = (s0 ? h0 : hv[i]) + 0.5 * (p1 * r1 + p2 * r2 + p3 * r3);
+            }
+            // Omega: Wh1 = Wh + 1/2 (w qv - qh0 v + v x qv), lanes 0..2
+            const double Wh1 = at(sn, 10 + ax) + 0.5 * (w * hv[ax] - h0 * vv[ax] + vv[i1] * hv[i2] - vv[i2] * hv[i1]);
+            const double w0 = at(Wh1, 0), w1 = at(Wh1, 1), w2 = at(Wh1, 2);
+            const double alpha = R0i * w0 + R1i * w1 + R2i * w2;
+            const double aI = alpha * inv_I;
+            const double a0 = at(aI, 0), a1 = at(aI, 1), a2 = at(aI, 2);
+            const double Th = Ri0 * a0 + Ri1 * a1 + Ri2 * a2;
+            // translation
+            const double snx = at(sn, ax), vh1 = at(sn, 7 + ax) + snx;
+            const double Fh = vh1 * inv_m;
+            double F2 = vh1 * F, gv = g * Fh;
+            F2 = at(F2, 0) + at(F2, 1) + at(F2, 2);
+            gv = at(gv, 0) + at(gv, 1) + at(gv, 2);
+            // lever arm of the torque sum: T = sum (mid - X) x F_link
+            const double xout = snx + (at(Th, i1) * at(fhF, i2) - at(Th, i2) * at(fhF, i1));
+            // Rh_ij = Wh1_i beta_j / I_j + T_i alpha_j / I_j on lane 3 i + j, and the
+            // drive terms (F = f R a: dF_i / dR_ij = f a_j)
+            const int ri = lane < 9 ? lane / 3 : 0, rj = lane < 9 ? lane % 3 : 0;
+            const double bI = beta * inv_I;
+            double Rh = at(Wh1, ri) * at(bI, rj) + at(fhT, ri) * at(aI, rj);
+            const double Fi = at(Fh, ri);
+            for (int k = d0; k < d1; ++k) Rh += ab.td[k].f * Fi * dv.drives[k].axis[rj];     // f: zero outside the window
+            // the adjoint of R(q): antisymmetric, symmetric and diagonal pairs of Rh
+            // on lanes 0..2, 3..5, 6..8, then a component of q a lane
+            const double c0 = at(Rh, lane == 0 ? 7 : lane == 1 ? 2 : lane == 2 ? 3 : lane == 3 ? 1 : lane == 4 ? 2 : lane == 5 ? 5
+                                  : lane == 6 ? 4 : 0);
+            const double c1 = at(Rh, lane == 0 ? 5 : lane == 1 ? 6 : lane == 2 ? 1 : lane == 3 ? 3 : lane == 4 ? 6 : lane == 5 ? 7
+                                  : lane == 8 ? 4 : 8);
+            const double pr = lane < 3 ? c0 - c1 : c0 + c1;
+            const double A0 = at(pr, 0), A1 = at(pr, 1), A2 = at(pr, 2), S01 = at(pr, 3), S02 = at(pr, 4), S12 = at(pr, 5),
+                         Dx = at(pr, 6), Dy = at(pr, 7), Dz = at(pr, 8);
+            {
+                const double p0 = lane == 0 ? A0 : lane == 1 ? S01 : lane == 2 ? S01 : S02;
+                const double r0 = lane == 0 ? va : lane == 1 ? vb : va;
+                const double p1 = lane == 0 ? A1 : lane == 1 ? S02 : S12;
+                const double r1 = lane == 0 ? vb : lane == 3 ? vb : vc;
+                const double p2 = lane == 0 ? A2 : lane == 1 ? A0 : lane == 2 ? A1 : A2;
+                const double r2 = lane == 0 ? vc : w;
+                const double p3 = lane == 0 ? 0.0 : lane == 1 ? Dx : lane == 2 ? Dy : Dz;
+                const double r3 = lane == 1 ? va : lane == 2 ? vb : vc;
+                qout += 2.0 * (p0 * r0 + p1 * r1 + p2 * r2 - 2.0 * p3 * r3);
+            }
+            double *sc = ab.sa_cur + 13 * b;
+            if (lane < 3) {
+                sc[lane] = xout;
+                sc[7 + lane] = vh1;
+                sc[10 + lane] = Wh1;
+                ab.fadj[6 * b + lane] = Fh;
+                ab.fadj[6 * b + 3 + lane] = Th;
+                s_F[b][lane] = Fh;
+                ab.grad_body[5 * b + 1 + lane] += -beta * alpha * inv_I * inv_I;
+            }
+            if (lane < 4) sc[3 + lane] = qout;
+            if (lane == 0) {
+                ab.grad_body[5 * b] += -F2 * inv_m * inv_m;
+                ab.grad_body[5 * b + 4] += gv;
+            }
         }
-        if (lane == 0) {
-            double *sn = ab.sa_next + 13 * b;
-            for (int i = 0; i < 3; ++i) { sn[i] += acc[i]; sn[7 + i] += acc[3 + i]; sn[10 + i] += acc[6 + i]; }
-        }
+        __syncthreads();
     }
-    __syncthreads();
-    // 2. per body: Euler step and rotation update, reversed
-    for (int b = threadIdx.x; b < nb; b += blockDim.x) {
-        const BodyProps pb = dv.props[b];
-        const BodyState s = S[b];
-        const AdjBodyTerms tm = ab.tb[b];
-        const double *sn = ab.sa_next + 13 * b;
-        const double *fh = ab.fh + 6 * b;
-        const double *T = fh + 3;
-        double R[3][3];
-        for (int r = 0; r < 3; ++r)
-            for (int c = 0; c < 3; ++c) R[r][c] = tm.R[3 * r + c];
-        const double *beta = tm.beta, *W1 = tm.W1, *q1 = tm.q1;
-        const double w = s.q[0], v0 = s.q[1], v1 = s.q[2], v2 = s.q[3];
-        const double inv_nn = tm.inv_nn;
-        double dot = 0.0, qh4[4];
-        for (int i = 0; i < 4; ++i) dot += q1[i] * sn[3 + i];
-        for (int i = 0; i < 4; ++i) qh4[i] = (sn[3 + i] - q1[i] * dot) * inv_nn;
-        double out[13];
-        const double qv[3] = {qh4[1], qh4[2], qh4[3]};
-        out[3] = qh4[0] + 0.5 * (qv[0] * W1[0] + qv[1] * W1[1] + qv[2] * W1[2]);
-        const double t1[3] = {qv[1] * W1[2] - qv[2] * W1[1], qv[2] * W1[0] - qv[0] * W1[2], qv[0] * W1[1] - qv[1] * W1[0]};
-        const double vv[3] = {v0, v1, v2};
-        for (int i = 0; i < 3; ++i) out[4 + i] = qv[i] - 0.5 * qh4[0] * W1[i] + 0.5 * t1[i];
-        const double t2[3] = {vv[1] * qv[2] - vv[2] * qv[1], vv[2] * qv[0] - vv[0] * qv[2], vv[0] * qv[1] - vv[1] * qv[0]};
-        double Wh1[3];
-        for (int i = 0; i < 3; ++i) Wh1[i] = sn[10 + i] - 0.5 * qh4[0] * vv[i] + 0.5 * w * qv[i] + 0.5 * t2[i];
-        double alpha[3];
-        for (int i = 0; i < 3; ++i) alpha[i] = R[0][i] * Wh1[0] + R[1][i] * Wh1[1] + R[2][i] * Wh1[2];
-        double Th[3];
-        for (int i = 0; i < 3; ++i) {
-            out[10 + i] = Wh1[i];
-            Th[i] = R[i][0] * alpha[0] * pb.inv_inertia[0] + R[i][1] * alpha[1] * pb.inv_inertia[1] +
-                    R[i][2] * alpha[2] * pb.inv_inertia[2];
-            ab.grad_body[5 * b + 1 + i] += -beta[i] * alpha[i] * pb.inv_inertia[i] * pb.inv_inertia[i];
-        }
-        double Rh[3][3];
-        for (int i = 0; i < 3; ++i)
-            for (int j = 0; j < 3; ++j)
-                Rh[i][j] = Wh1[i] * beta[j] * pb.inv_inertia[j] + T[i] * alpha[j] * pb.inv_inertia[j];
-        double Fh[3], F2 = 0.0, gv = 0.0;
-        for (int i = 0; i < 3; ++i) {
-            const double vh1 = sn[7 + i] + sn[i];
-            out[i] = sn[i];
-            out[7 + i] = vh1;
-            Fh[i] = vh1 * pb.inv_m;
-            F2 += vh1 * tm.F[i];
-            gv += dv.g[i] * Fh[i];
-        }
-        ab.grad_body[5 * b] += -F2 * pb.inv_m * pb.inv_m;
-        ab.grad_body[5 * b + 4] += gv;
-        // lever arm of the torque sum: T = sum (mid - X) x F_link
-        out[0] += Th[1] * fh[2] - Th[2] * fh[1];
-        out[1] += Th[2] * fh[0] - Th[0] * fh[2];
-        out[2] += Th[0] * fh[1] - Th[1] * fh[0];
-        // drive terms of this body (F = f R a: dF_i / dR_ij = f a_j)
-        for (int k = pb.drive_first; k < pb.drive_first + pb.drive_count; ++k) {
-            const double f = ab.td[k].f;                 // zero outside the drive window
-            const double *a = dv.drives[k].axis;
-            for (int i = 0; i < 3; ++i)
-                for (int j = 0; j < 3; ++j) Rh[i][j] += f * Fh[i] * a[j];
-        }
-        double qh[4] = {0, 0, 0, 0};
-        adj_rot_matrix(s.q, Rh, qh);
-        for (int i = 0; i < 4; ++i) out[3 + i] += qh[i];
-        double *sc = ab.sa_cur + 13 * b;
-        for (int i = 0; i < 13; ++i) sc[i] = out[i];
-        for (int i = 0; i < 3; ++i) { ab.fadj[6 * b + i] = Fh[i]; ab.fadj[6 * b + 3 + i] = Th[i]; }
-    }
-    __syncthreads();
-    // 3. drive-term and spring gradients (one thread per term), then the
-    //    spring terms of each body's adjoint (thread b, its springs in order)
+    // 2. drive-term and spring gradients (one thread per term), and the spring
+    //    terms of each body's adjoint (lane i of the body's warp axis i, its
+    //    springs in order)
     const double tt = (double)ab.t;
     for (int k = threadIdx.x; k < dv.nd; k += blockDim.x) {
         const DriveTerm dt = dv.drives[k];
         if (tt < dt.t_on || tt >= dt.t_off) continue;
         const AdjDriveTerms tdk = ab.td[k];
-        const double *fa = ab.fadj + 6 * dt.body;
+        const double *fa = s_F[dt.body];
         const double proj = fa[0] * tdk.aw[0] + fa[1] * tdk.aw[1] + fa[2] * tdk.aw[2];
         ab.grad_drive[2 * k] += tdk.sn * proj;
         ab.grad_drive[2 * k + 1] += -dt.amp * tdk.cs * proj;
     }
-    for (int k = threadIdx.x; k < dv.ns; k += blockDim.x) {
+    for (int k = (int)threadIdx.x - 32; k < dv.ns; k += blockDim.x) {
+        if (k < 0) continue;
         const Spring sp_ = dv.springs[k];
         const AdjSpringTerms tsk = ab.ts[k];
         double fh[3], dvv = 0.0, fd = 0.0;
         for (int i = 0; i < 3; ++i) {
-            fh[i] = ab.fadj[6 * sp_.i + i] - ab.fadj[6 * sp_.j + i];
+            fh[i] = s_F[sp_.i][i] - s_F[sp_.j][i];
             dvv += fh[i] * tsk.dv[i];
         }
         ab.grad_spring[3 * k + 2] += -dvv;
@@ -755,21 +826,29 @@ __global__ void __launch_bounds__(ADJ_THREADS) adj_integrate_kernel(const Device
             ab.grad_spring[3 * k + 1] += sp_.k * fd;
         }
     }
-    for (int b = threadIdx.x; b < nb; b += blockDim.x) {
-        const BodyProps pb = dv.props[b];
+    for (int b = ADJ_WARPS - 1 - warp; b < nb; b += ADJ_WARPS) {
+        const BodyProps *pb = dv.props + b;
+        const int s0 = pb->spring_first, s1 = s0 + pb->spring_count;
         double *sc = ab.sa_cur + 13 * b;
-        for (int kk = pb.spring_first; kk < pb.spring_first + pb.spring_count; ++kk) {
+        double x = 0.0, v = 0.0;
+        if (lane < 3) {
+            x = sc[lane];
+            v = sc[7 + lane];
+        }
+        for (int kk = s0; kk < s1; ++kk) {
             const int k = dv.spring_list[kk];
             const Spring sp_ = dv.springs[k];
-            const AdjSpringTerms tsk = ab.ts[k];
+            const AdjSpringTerms *tsk = ab.ts + k;
             const double sign = sp_.i == b ? 1.0 : -1.0;
-            double fh[3], fd = 0.0;
-            for (int i = 0; i < 3; ++i) fh[i] = ab.fadj[6 * sp_.i + i] - ab.fadj[6 * sp_.j + i];
-            for (int i = 0; i < 3; ++i) sc[7 + i] += -sign * sp_.gamma * fh[i];
-            if (!(tsk.len > 0)) continue;
-            for (int i = 0; i < 3; ++i) fd += fh[i] * tsk.dir[i];
-            for (int i = 0; i < 3; ++i)
-                sc[i] += sign * (-sp_.k * (fd * tsk.dir[i] + tsk.ratio * (fh[i] - fd * tsk.dir[i])));
+            const double fh = s_F[sp_.i][ax] - s_F[sp_.j][ax], dir = tsk->dir[ax];
+            v += -sign * sp_.gamma * fh;
+            const double prod = fh * dir;
+            const double fd = at(prod, 0) + at(prod, 1) + at(prod, 2);
+            if (tsk->len > 0) x += sign * (-sp_.k * (fd * dir + tsk->ratio * (fh - fd * dir)));
+        }
+        if (lane < 3) {
+            sc[lane] = x;
+            sc[7 + lane] = v;
         }
     }
 }

@@ -1548,27 +1548,27 @@ int lbm_adjoint_backward(lbm_t *h, const double *seed, double *grad_state, doubl
         CK(cudaStreamCreateWithPriority(&rcaps2, cudaStreamNonBlocking, greatest));
     }
     cudaEvent_t ev_main = nullptr, ev_side = nullptr, ev_rec = nullptr, ev_free_main = nullptr,
-                ev_free_side = nullptr, ev_rfork = nullptr, ev_rjoin = nullptr, ev_rjoin2 = nullptr, ev_cfork = nullptr,
-                ev_cjoin = nullptr, ev_cjoin2 = nullptr;
+                ev_free_side = nullptr, ev_rfork = nullptr, ev_rjoin2 = nullptr, ev_cfork = nullptr, ev_cjoin2 = nullptr,
+                ev_rbulk[2] = {nullptr, nullptr}, ev_cbulk[2] = {nullptr, nullptr};
     CK(cudaEventCreateWithFlags(&ev_main, cudaEventDisableTiming));
     CK(cudaEventCreateWithFlags(&ev_side, cudaEventDisableTiming));
     CK(cudaEventCreateWithFlags(&ev_rec, cudaEventDisableTiming));
     CK(cudaEventCreateWithFlags(&ev_free_main, cudaEventDisableTiming));
     CK(cudaEventCreateWithFlags(&ev_free_side, cudaEventDisableTiming));
     CK(cudaEventCreateWithFlags(&ev_rfork, cudaEventDisableTiming));
-    CK(cudaEventCreateWithFlags(&ev_rjoin, cudaEventDisableTiming));
     CK(cudaEventCreateWithFlags(&ev_cfork, cudaEventDisableTiming));
-    CK(cudaEventCreateWithFlags(&ev_cjoin, cudaEventDisableTiming));
     CK(cudaEventCreateWithFlags(&ev_rjoin2, cudaEventDisableTiming));
     CK(cudaEventCreateWithFlags(&ev_cjoin2, cudaEventDisableTiming));
+    for (cudaEvent_t *ev : {&ev_rbulk[0], &ev_rbulk[1], &ev_cbulk[0], &ev_cbulk[1]})
+        CK(cudaEventCreateWithFlags(ev, cudaEventDisableTiming));
     struct Events {
-        cudaEvent_t *e[11];
+        cudaEvent_t *e[13];
         ~Events() {
             for (cudaEvent_t *p : e)
                 if (*p) cudaEventDestroy(*p);
         }
-    } events{{&ev_main, &ev_side, &ev_rec, &ev_free_main, &ev_free_side, &ev_rfork, &ev_rjoin, &ev_cfork, &ev_cjoin,
-               &ev_rjoin2, &ev_cjoin2}};
+    } events{{&ev_main, &ev_side, &ev_rec, &ev_free_main, &ev_free_side, &ev_rfork, &ev_cfork, &ev_rjoin2, &ev_cjoin2,
+               &ev_rbulk[0], &ev_rbulk[1], &ev_cbulk[0], &ev_cbulk[1]}};
     CK(cudaEventRecord(ev_main, s));
     CK(cudaEventRecord(ev_side, s));
     CK(cudaEventRecord(ev_free_main, s));
@@ -1622,19 +1622,24 @@ int lbm_adjoint_backward(lbm_t *h, const double *seed, double *grad_state, doubl
     // run, which the last reverse step needs)
     // The remap rewrites only the cubes around the bodies: a slot starts
     // from the epoch before it, as the forward's ping-pong buffers do.  The
-    // copy into slot j + 2 is made after step j's bulk kernel (beside the
-    // boundary branch), off the chain; slot 1's before the segment's first
-    // remap.  `copy_next`: step j + 1 follows.
+    // copy into slot j + 2 is made beside step j's boundary kernel, off the
+    // chain; slot 1's before the segment's first remap.  `copy_next`: step j + 1 follows.
     auto copy_slot = [&](const SlotSet &st, int j, cudaStream_t ms) -> int {
         CK(cudaMemcpyAsync(st.flags + C * (j + 1), st.flags + C * j, (size_t)C, cudaMemcpyDeviceToDevice, ms));
         CK(cudaMemcpyAsync(st.bid + C * (j + 1), st.bid + C * j, (size_t)C, cudaMemcpyDeviceToDevice, ms));
         return LBM_OK;
     };
+    // The streams are those of a captured forward step: the chain ms, the bulk
+    // kernel on ss (done events `bulk` by step parity), loads, links and the slot
+    // copies on ss2.
+    struct StepStreams {
+        cudaStream_t ms, ss, ss2;
+        cudaEvent_t fork, join2, *bulk;
+    };
     auto recompute_step = [&](const SlotSet &st, int j, const BodyState *prev, const BodyState *cur, bool last,
-                              bool copy_next, cudaStream_t ms, cudaStream_t ss, cudaStream_t ss2,
-                              cudaEvent_t fork, cudaEvent_t join, cudaEvent_t join2) -> int {
+                              bool copy_next, const StepStreams &q) -> int {
         int rc3;
-        if (j == 0 && (rc3 = copy_slot(st, 0, ms))) return rc3;
+        if (j == 0 && (rc3 = copy_slot(st, 0, q.ms))) return rc3;
         lbm::StepPtrs sp{};
         sp.src = slot_pop(st, j);
         sp.dst = slot_pop(st, j + 1);
@@ -1647,29 +1652,32 @@ int lbm_adjoint_backward(lbm_t *h, const double *seed, double *grad_state, doubl
         sp.body_next = scratch;
         sp.tstep = dr.tstep + (j & 1);
         sp.parity = j & 1;
+        if (!last) {
+            CK(cudaEventRecord(q.fork, q.ms));
+            CK(cudaStreamWaitEvent(q.ss2, q.fork, 0));
+            lbm::launch_loads(dr, sp, q.ss2);
+        }
         // the body preparation only at the segment's first step: the later
         // states' geometry records come from the recomputation's own
         // rigid-body steps (the same bits as the tape's states)
-        const bool prep = j == 0;
-        lbm::launch_remap(dr, sp, 0, ms, prep);
+        lbm::launch_remap(dr, sp, 0, q.ms, j == 0);
         if (last) return LBM_OK;
-        // boundary cells, and link lists with loads, beside the bulk kernel,
-        // as in the forward step
-        CK(cudaEventRecord(fork, ms));
-        CK(cudaStreamWaitEvent(ss, fork, 0));
-        lbm::launch_boundary_fix(dr, sp, ss);
-        CK(cudaEventRecord(join, ss));
-        CK(cudaStreamWaitEvent(ss2, fork, 0));
-        lbm::launch_links(dr, sp, ss2);
-        lbm::launch_loads(dr, sp, ss2);
-        CK(cudaEventRecord(join2, ss2));
-        lbm::launch_stream_collide(dr, sp, ms);
-        if (copy_next && (rc3 = copy_slot(st, j + 1, ms))) return rc3;
-        CK(cudaStreamWaitEvent(ms, join, 0));
-        CK(cudaStreamWaitEvent(ms, join2, 0));
-        lbm::launch_force(dr, sp, ms);
+        CK(cudaEventRecord(q.fork, q.ms));
+        CK(cudaStreamWaitEvent(q.ss2, q.fork, 0));
+        lbm::launch_links(dr, sp, q.ss2);
+        if (copy_next && (rc3 = copy_slot(st, j + 1, q.ss2))) return rc3;
+        CK(cudaEventRecord(q.join2, q.ss2));
+        if (j > 0) CK(cudaStreamWaitEvent(q.ms, q.bulk[(j & 1) ^ 1], 0));
+        lbm::launch_boundary_fix(dr, sp, q.ms);
+        CK(cudaStreamWaitEvent(q.ss, q.fork, 0));
+        lbm::launch_stream_collide(dr, sp, q.ss);
+        CK(cudaEventRecord(q.bulk[j & 1], q.ss));
+        CK(cudaStreamWaitEvent(q.ms, q.join2, 0));
+        lbm::launch_force(dr, sp, q.ms);
         return LBM_OK;
     };
+    const StepStreams eager{rs, rss, rss2, ev_rfork, ev_rjoin2, ev_rbulk},
+        captured{rcap, rcaps, rcaps2, ev_cfork, ev_cjoin2, ev_cbulk};
     // A full segment (K steps, not the last) is recomputed by a CUDA graph of
     // its set: its states are staged (epochs m - 1 .. m + K - 1) into the
     // set's staging buffer, so that one graph serves every full segment of
@@ -1681,7 +1689,8 @@ int lbm_adjoint_backward(lbm_t *h, const double *seed, double *grad_state, doubl
         int rc2 = LBM_OK;
         for (int j = 0; j < K && rc2 == LBM_OK; ++j)
             rc2 = recompute_step(st, j, stage[set] + (long long)j * B, stage[set] + (long long)(j + 1) * B, false,
-                                 j + 1 < K, rcap, rcaps, rcaps2, ev_cfork, ev_cjoin, ev_cjoin2);
+                                 j + 1 < K, captured);
+        if (rc2 == LBM_OK && cudaStreamWaitEvent(rcap, ev_cbulk[(K - 1) & 1], 0) != cudaSuccess) rc2 = LBM_E_CUDA;
         cudaGraph_t g = nullptr;
         const cudaError_t e1 = cudaStreamEndCapture(rcap, &g);
         if (rc2) {
@@ -1717,15 +1726,12 @@ int lbm_adjoint_backward(lbm_t *h, const double *seed, double *grad_state, doubl
             const bool extra = k == tp.nseg - 1;    // the remap of the epoch after the run
             for (int j = 0; j < L; ++j) {
                 int rc2;
-                if ((rc2 = recompute_step(st, j, S(m + j - 1), S(m + j), false, j + 1 < L || extra, rs, rss, rss2,
-                                          ev_rfork, ev_rjoin, ev_rjoin2)))
-                    return rc2;
+                if ((rc2 = recompute_step(st, j, S(m + j - 1), S(m + j), false, j + 1 < L || extra, eager))) return rc2;
             }
+            CK(cudaStreamWaitEvent(rs, ev_rbulk[(L - 1) & 1], 0));
             if (extra) {
                 int rc2;
-                if ((rc2 = recompute_step(st, L, S(m + L - 1), S(m + L), true, false, rs, rss, rss2, ev_rfork, ev_rjoin,
-                                          ev_rjoin2)))
-                    return rc2;
+                if ((rc2 = recompute_step(st, L, S(m + L - 1), S(m + L), true, false, eager))) return rc2;
             }
         }
         make_terms(k, rs);
