@@ -36,23 +36,43 @@ constexpr int ADJ_BOUNDARY_THREADS = 64;
 // no neighbour solid at n)
 constexpr uint8_t F_FULL_RULE = F_SOLID | F_SOLID_PREV | F_NEAR | F_WALL;
 
+// the collision's parameters in the adjoint's precision, rounded once on the host
+// (an FP64 conversion a thread would take the FP64 pipe's 64 cycles a warp)
+template <typename A> struct AdjParams;
+template <> struct AdjParams<double> {
+    __device__ static double omega(const Device &dv) { return dv.omega; }
+    __device__ static double guo(const Device &dv) { return 1.0 - 0.5 * dv.omega; }
+    __device__ static double g(const Device &dv, int i) { return dv.g[i]; }
+    __device__ static double half_g(const Device &dv, int i) { return 0.5 * dv.g[i]; }
+};
+template <> struct AdjParams<float> {
+    __device__ static float omega(const Device &dv) { return dv.omega_f; }
+    __device__ static float guo(const Device &dv) { return dv.guo_f; }
+    __device__ static float g(const Device &dv, int i) { return dv.g_f[i]; }
+    __device__ static float half_g(const Device &dv, int i) { return dv.gh_f[i]; }
+};
+
+// acc + s v for a component s of a direction
+template <typename A> __device__ __forceinline__ A plus(A acc, int s, A v) { return s > 0 ? acc + v : (s < 0 ? acc - v : acc); }
+
 // density and velocity of step n from the post-collision deviations:
 // rho = 1 + sum delta; the collision adds g to the momentum (Guo), so
 // rho u = sum e delta - g / 2
-template <typename A, typename T>
-__device__ inline void moments_post(const T *G, long long C, long long c, const Device &dv, A &rho, A (&u)[3]) {
+template <typename A>
+__device__ inline void moments_post(const A (&G)[Q], const Device &dv, A &rho, A (&u)[3]) {
     A r = 0, j0 = 0, j1 = 0, j2 = 0;
 #pragma unroll
     for (int b = 0; b < Q; ++b) {
-        const A v = (A)G[(long long)b * C + c];
-        r += v;
-        j0 += (A)ex(b) * v; j1 += (A)ey(b) * v; j2 += (A)ez(b) * v;
+        r += G[b];
+        j0 = plus(j0, ex(b), G[b]);
+        j1 = plus(j1, ey(b), G[b]);
+        j2 = plus(j2, ez(b), G[b]);
     }
     rho = (A)1 + r;
     const A ir = (A)1 / rho;
-    u[0] = (j0 - (A)(0.5 * dv.g[0])) * ir;
-    u[1] = (j1 - (A)(0.5 * dv.g[1])) * ir;
-    u[2] = (j2 - (A)(0.5 * dv.g[2])) * ir;
+    u[0] = (j0 - AdjParams<A>::half_g(dv, 0)) * ir;
+    u[1] = (j1 - AdjParams<A>::half_g(dv, 1)) * ir;
+    u[2] = (j2 - AdjParams<A>::half_g(dv, 2)) * ir;
 }
 
 // Transposed Jacobian of the LBGK collision with Guo's forcing at one cell:
@@ -60,35 +80,48 @@ __device__ inline void moments_post(const T *G, long long C, long long c, const 
 // of the pre-collision ones on exit.
 //   G_b = P_b - omega (P_b - feq_b(rho, u)) + (1 - omega / 2) w_b s_b(u)
 //   rho = sum P, u = (sum e P + g / 2) / rho, d u_i / d P_a = (e_ai - u_i) / rho
+// With t_b = w_b a_b the sums over b are t0 = sum t, sr = sum t feq / (w rho),
+// s_i = sum t (c e_i - 3 u_i) with c = 3 + 9 e.u, and f_i of the forcing.
 template <typename A>
 __device__ inline void collide_adjoint(A (&a)[Q], A rho, const A (&u)[3], const Device &dv) {
-    const A om = (A)dv.omega;
+    const A om = AdjParams<A>::omega(dv);
     const A uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-    A sr = 0, s0 = 0, s1 = 0, s2 = 0, f0 = 0, f1 = 0, f2 = 0;
+    const A g0 = AdjParams<A>::g(dv, 0), g1 = AdjParams<A>::g(dv, 1), g2 = AdjParams<A>::g(dv, 2);
+    const A rest = (A)1 - (A)1.5 * uu;
+    A t0 = 0, sr = 0, s0 = 0, s1 = 0, s2 = 0, f0 = 0, f1 = 0, f2 = 0;
 #pragma unroll
     for (int b = 0; b < Q; ++b) {
-        const A eu = (A)ex(b) * u[0] + (A)ey(b) * u[1] + (A)ez(b) * u[2];
-        const A wa = (A)wgt(b) * a[b];
-        sr += wa * ((A)1 + (A)3 * eu + (A)4.5 * eu * eu - (A)1.5 * uu);
-        const A c = (A)3 + (A)9 * eu;
-        s0 += wa * (c * (A)ex(b) - (A)3 * u[0]);
-        s1 += wa * (c * (A)ey(b) - (A)3 * u[1]);
-        s2 += wa * (c * (A)ez(b) - (A)3 * u[2]);
+        const A eu = plus(plus(plus((A)0, ex(b), u[0]), ey(b), u[1]), ez(b), u[2]);
+        const A t = (A)wgt(b) * a[b];
+        t0 += t;
+        sr += t * (eu * ((A)4.5 * eu + (A)3) + rest);
+        const A tc = t * ((A)9 * eu + (A)3);
+        s0 = plus(s0, ex(b), tc);
+        s1 = plus(s1, ey(b), tc);
+        s2 = plus(s2, ez(b), tc);
         if (dv.forced) {
-            const A eg = (A)(ex(b) * dv.g[0] + ey(b) * dv.g[1] + ez(b) * dv.g[2]);
-            f0 += wa * ((A)(-3.0 * dv.g[0]) + (A)9 * (A)ex(b) * eg);
-            f1 += wa * ((A)(-3.0 * dv.g[1]) + (A)9 * (A)ey(b) * eg);
-            f2 += wa * ((A)(-3.0 * dv.g[2]) + (A)9 * (A)ez(b) * eg);
+            const A te = t * plus(plus(plus((A)0, ex(b), g0), ey(b), g1), ez(b), g2);
+            f0 = plus(f0, ex(b), te);
+            f1 = plus(f1, ey(b), te);
+            f2 = plus(f2, ez(b), te);
         }
     }
-    const A kf = (A)1 - (A)0.5 * om;
+    s0 -= (A)3 * u[0] * t0;
+    s1 -= (A)3 * u[1] * t0;
+    s2 -= (A)3 * u[2] * t0;
+    const A kf = AdjParams<A>::guo(dv);
     const A ir = (A)1 / rho;
-    const A su0 = (om * rho * s0 + kf * f0) * ir, su1 = (om * rho * s1 + kf * f1) * ir,
-            su2 = (om * rho * s2 + kf * f2) * ir;
+    A su0 = om * s0, su1 = om * s1, su2 = om * s2;          // om rho s / rho
+    if (dv.forced) {
+        su0 += kf * ((A)9 * f0 - (A)3 * g0 * t0) * ir;
+        su1 += kf * ((A)9 * f1 - (A)3 * g1 * t0) * ir;
+        su2 += kf * ((A)9 * f2 - (A)3 * g2 * t0) * ir;
+    }
     const A base = om * sr - (su0 * u[0] + su1 * u[1] + su2 * u[2]);
+    const A om1 = (A)1 - om;
 #pragma unroll
     for (int b = 0; b < Q; ++b)
-        a[b] = ((A)1 - om) * a[b] + base + (A)ex(b) * su0 + (A)ey(b) * su1 + (A)ez(b) * su2;
+        a[b] = plus(plus(plus(om1 * a[b] + base, ex(b), su0), ey(b), su1), ez(b), su2);
 }
 
 // adjoint of the body-surface velocity u_w(p) = V + W x (p - X) for the
@@ -106,31 +139,44 @@ __device__ inline void adj_surface(const S W[3], const S o[3], const S uh[3], Ac
 }
 
 // ---- bulk cells: pure gather + transposed collision -------------------------
+// block `blk` of z-plane z: the plane's cells in row order, ADJ_THREADS a block
 template <typename A, typename T, bool FIRST>
-__global__ void __launch_bounds__(ADJ_THREADS) adj_bulk_kernel(const Device dv, const AdjPtrs ap) {
-    const Domain d = dv.dom;
-    const int x = blockIdx.x * blockDim.x + threadIdx.x;
-    const int y = blockIdx.y * blockDim.y + threadIdx.y;
-    const int z = blockIdx.z;
-    if (x >= d.nx || y >= d.ny) return;
-    const long long C = d.C;
-    const long long c = ((long long)z * d.ny + y) * d.nx + x;
-    if ((ap.flags_next[c] & F_FULL_RULE) || (ap.flags_cur[c] & F_SOLID_PREV)) return;   // a boundary cell
-    const A *__restrict__ ain = static_cast<const A *>(ap.ain);
-    A a[Q];
-#pragma unroll
-    for (int b = 0; b < Q; ++b) {
-        const int sx = wrap_axis(x + ex(b), d.nx), sy = wrap_axis(y + ey(b), d.ny), sz = wrap_axis(z + ez(b), d.nz);
-        a[b] = ain[(long long)b * C + ((long long)sz * d.ny + sy) * d.nx + sx];
+__device__ __forceinline__ void adj_bulk_cells(const Device &dv, const AdjPtrs &ap, int blk, int z) {
+    const Domain &d = dv.dom;
+    const unsigned nx = (unsigned)d.nx, q = (unsigned)blk * ADJ_THREADS + threadIdx.x;
+    if (q >= nx * (unsigned)d.ny) return;
+    unsigned r = __umulhi(q, ap.row_recip), xr = q - r * nx;         // row_recip: q / nx
+    if (xr >= nx) {
+        xr -= nx;
+        ++r;
     }
+    const int x = (int)xr, y = (int)r;
+    const long long C = d.C;
+    const unsigned c = ((unsigned)z * d.ny + y) * nx + xr;
+    const uint8_t fn = ap.flags_next[c], fc = ap.flags_cur[c];
+    const A *__restrict__ ain = static_cast<const A *>(ap.ain);
+    const T *__restrict__ G = static_cast<const T *>(ap.G);
+    A a[Q], g[Q];
+    // sources x + e (wrapped; a cell whose neighbour lies beyond a wall is not a bulk cell)
+    const int xs[3] = {x == 0 ? d.nx - 1 : x - 1, x, x == d.nx - 1 ? 0 : x + 1};
+    const int ys[3] = {y == 0 ? d.ny - 1 : y - 1, y, y == d.ny - 1 ? 0 : y + 1};
+    const int zs[3] = {z == 0 ? d.nz - 1 : z - 1, z, z == d.nz - 1 ? 0 : z + 1};
+#pragma unroll
+    for (int b = 0; b < Q; ++b)
+        a[b] = ain[b * C + (((unsigned)zs[1 + ez(b)] * d.ny + ys[1 + ey(b)]) * nx + xs[1 + ex(b)])];
+    if constexpr (!FIRST) {
+#pragma unroll
+        for (int b = 0; b < Q; ++b) g[b] = (A)G[b * C + c];
+    }
+    if ((fn & F_FULL_RULE) || (fc & F_SOLID_PREV)) return;           // the cube or wall kernel's
     if constexpr (!FIRST) {
         A rho, u[3];
-        moments_post<A, T>(static_cast<const T *>(ap.G), C, c, dv, rho, u);
+        moments_post<A>(g, dv, rho, u);
         collide_adjoint<A>(a, rho, u, dv);
     }
     A *__restrict__ aout = static_cast<A *>(ap.aout);
 #pragma unroll
-    for (int b = 0; b < Q; ++b) aout[(long long)b * C + c] = a[b];
+    for (int b = 0; b < Q; ++b) aout[b * C + c] = a[b];
 }
 
 // ---- wall-face cells: the full rule, a thread per cell -----------------------
@@ -173,8 +219,10 @@ __global__ void __launch_bounds__(ADJ_BOUNDARY_THREADS) adj_wall_kernel(const De
             const A *__restrict__ ain = static_cast<const A *>(ap.ain);
             const A *__restrict__ rin = static_cast<const A *>(ap.rin);
             const T *__restrict__ G = static_cast<const T *>(ap.G);
-            A rho, u[3];
-            moments_post<A, T>(G, C, c, dv, rho, u);
+            A rho, u[3], gv[Q];
+#pragma unroll
+            for (int b = 0; b < Q; ++b) gv[b] = (A)G[(long long)b * C + c];
+            moments_post<A>(gv, dv, rho, u);
             const bool fluid_next = !(fnext & F_SOLID);
             A own[Q], a[Q];
 #pragma unroll
@@ -293,6 +341,23 @@ __global__ void __launch_bounds__(ADJ_BOUNDARY_THREADS) adj_wall_kernel(const De
 // part[kb][blk] (the layout adj_integrate reads).
 constexpr int ADJ_CUBE_WARPS = 8;
 
+// the sums of v[0..3] over the warp, in every lane: halves exchange values (lane
+// bit 4: the first or last two, bit 3: one of them), then three butterfly steps
+template <typename V> __device__ __forceinline__ void warp_sum4(V (&v)[4]) {
+    constexpr unsigned FULL = 0xffffffffu;
+    const bool hi = threadIdx.x & 16, odd = threadIdx.x & 8;
+    const V k0 = hi ? v[2] : v[0], k1 = hi ? v[3] : v[1], o0 = hi ? v[0] : v[2], o1 = hi ? v[1] : v[3];
+    const V a0 = k0 + __shfl_xor_sync(FULL, o0, 16), a1 = k1 + __shfl_xor_sync(FULL, o1, 16);
+    V a = (odd ? a1 : a0) + __shfl_xor_sync(FULL, odd ? a0 : a1, 8);
+    a += __shfl_xor_sync(FULL, a, 4);
+    a += __shfl_xor_sync(FULL, a, 2);
+    a += __shfl_xor_sync(FULL, a, 1);
+    v[0] = __shfl_sync(FULL, a, 0);
+    v[1] = __shfl_sync(FULL, a, 8);
+    v[2] = __shfl_sync(FULL, a, 16);
+    v[3] = __shfl_sync(FULL, a, 24);
+}
+
 template <typename V> __device__ __forceinline__ V warp_sum(V v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -382,7 +447,13 @@ __global__ void __launch_bounds__(32 * ADJ_CUBE_WARPS) adj_cube_kernel(const Dev
     const A *__restrict__ ain = static_cast<const A *>(ap.ain);
     const A *__restrict__ rin = static_cast<const A *>(ap.rin);
     const T *__restrict__ G = static_cast<const T *>(ap.G);
-    A wsum[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};        // this warp's body-kb terms, cell by cell
+    A acc[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};         // this lane's body-kb terms over the warp's cells
+    // body kb's velocities and load adjoint in A, once a warp
+    const A V0[3] = {(A)sb.V[0], (A)sb.V[1], (A)sb.V[2]}, W0[3] = {(A)sb.W[0], (A)sb.W[1], (A)sb.W[2]};
+    A fa0[6] = {0, 0, 0, 0, 0, 0};
+    if constexpr (!FIRST)
+        for (int i = 0; i < 6; ++i) fa0[i] = (A)ap.fadj[6 * kb + i];
+    const A hg0 = AdjParams<A>::half_g(dv, 0), hg1 = AdjParams<A>::half_g(dv, 1), hg2 = AdjParams<A>::half_g(dv, 2);
     for (int e = warp; e < nlist; e += ADJ_CUBE_WARPS) {
         int x, y, z;
         cube_cell(list[e], x, y, z);
@@ -391,15 +462,14 @@ __global__ void __launch_bounds__(32 * ADJ_CUBE_WARPS) adj_cube_kernel(const Dev
         const bool fluid_next = !(fnext & F_SOLID);
         // density and velocity of step n from the post-collision populations
         const A gv = act ? (A)G[(long long)b * C + c] : (A)0;
-        const A rho = (A)1 + warp_sum(gv);
+        A m[4] = {gv, (A)bx * gv, (A)by * gv, (A)bz * gv};
+        warp_sum4(m);
+        const A rho = (A)1 + m[0];
         const A ir = (A)1 / rho;
-        const A u0 = (warp_sum((A)bx * gv) - (A)(0.5 * dv.g[0])) * ir;
-        const A u1 = (warp_sum((A)by * gv) - (A)(0.5 * dv.g[1])) * ir;
-        const A u2 = (warp_sum((A)bz * gv) - (A)(0.5 * dv.g[2])) * ir;
+        const A u0 = (m[1] - hg0) * ir, u1 = (m[2] - hg1) * ir, u2 = (m[3] - hg2) * ir;
         const A own = act ? ain[(long long)b * C + c] : (A)0;
         const A own_opp = __shfl_sync(0xffffffffu, own, ob);
         A a = own, crb = 0;
-        A acc[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
         if (act && b > 0) {
             const int zx = x + bx, zy = y + by, zz = z + bz;
             const bool wall = (!d.px && (zx < 0 || zx >= d.nx)) || (!d.py && (zy < 0 || zy >= d.ny)) ||
@@ -410,6 +480,8 @@ __global__ void __launch_bounds__(32 * ADJ_CUBE_WARPS) adj_cube_kernel(const Dev
                 const long long zc = ((long long)wrap_axis(zz, d.nz) * d.ny + wrap_axis(zy, d.ny)) * d.nx +
                                      wrap_axis(zx, d.nx);
                 const uint8_t fzc = ap.flags_cur[zc];
+                const int k = ap.bid_cur[zc];
+                const A pulled = ain[(long long)b * C + zc];
                 if (fzc & F_SOLID) {
                     // link (x, b) of step n: moving bounce-back of step n+1 and
                     // the momentum exchange of step n share u_w(x + e_b; S^n);
@@ -417,7 +489,6 @@ __global__ void __launch_bounds__(32 * ADJ_CUBE_WARPS) adj_cube_kernel(const Dev
                     // cells less the centre's position within its cell (the same
                     // expression for every body: a cell in two cubes is written
                     // by both blocks), the terms in A
-                    const int k = ap.bid_cur[zc];
                     const BodyState &sk = ap.body[k];
                     int kc[3] = {ci[0], ci[1], ci[2]};
                     A kf[3] = {cf[0], cf[1], cf[2]};
@@ -431,19 +502,26 @@ __global__ void __launch_bounds__(32 * ADJ_CUBE_WARPS) adj_cube_kernel(const Dev
                         if (per[i]) io = 2 * io > n3[i] ? io - n3[i] : (2 * io < -n3[i] ? io + n3[i] : io);
                         o[i] = (A)io - kf[i];
                     }
-                    const A W[3] = {(A)sk.W[0], (A)sk.W[1], (A)sk.W[2]};
-                    const A uw0 = (A)sk.V[0] + (W[1] * o[2] - W[2] * o[1]);
-                    const A uw1 = (A)sk.V[1] + (W[2] * o[0] - W[0] * o[2]);
-                    const A uw2 = (A)sk.V[2] + (W[0] * o[1] - W[1] * o[0]);
+                    A W[3] = {W0[0], W0[1], W0[2]}, V[3] = {V0[0], V0[1], V0[2]};
+                    A fa[6] = {fa0[0], fa0[1], fa0[2], fa0[3], fa0[4], fa0[5]};
+                    if (k != kb) {
+                        for (int i = 0; i < 3; ++i) {
+                            W[i] = (A)sk.W[i];
+                            V[i] = (A)sk.V[i];
+                        }
+                        if constexpr (!FIRST)
+                            for (int i = 0; i < 6; ++i) fa[i] = (A)ap.fadj[6 * k + i];
+                    }
+                    const A uw0 = V[0] + (W[1] * o[2] - W[2] * o[1]);
+                    const A uw1 = V[1] + (W[2] * o[0] - W[0] * o[2]);
+                    const A uw2 = V[2] + (W[0] * o[1] - W[1] * o[0]);
                     const A ua = -((A)bx * uw0 + (A)by * uw1 + (A)bz * uw2);     // e_-b . u_w
                     A mh = 0;
                     if constexpr (!FIRST) {
-                        const double *fa = ap.fadj + 6 * k;
                         // (mid - X) x e_b, mid = x + e_b / 2 = (x + e_b) - e_b / 2
                         const A m0 = o[0] - (A)(0.5 * bx), m1 = o[1] - (A)(0.5 * by), m2 = o[2] - (A)(0.5 * bz);
                         const A t0 = m1 * (A)bz - m2 * (A)by, t1 = m2 * (A)bx - m0 * (A)bz, t2 = m0 * (A)by - m1 * (A)bx;
-                        mh = (A)bx * (A)fa[0] + (A)by * (A)fa[1] + (A)bz * (A)fa[2] + t0 * (A)fa[3] + t1 * (A)fa[4] +
-                             t2 * (A)fa[5];
+                        mh = (A)bx * fa[0] + (A)by * fa[1] + (A)bz * fa[2] + t0 * fa[3] + t1 * fa[4] + t2 * fa[5];
                     }
                     const A wh = own_opp;
                     a = wh + (A)2 * mh;
@@ -456,7 +534,7 @@ __global__ void __launch_bounds__(32 * ADJ_CUBE_WARPS) adj_cube_kernel(const Dev
                     // z uncovered at n+1: x (fluid at n and n+1) fed its density
                     if (!(ap.flags_next[zc] & F_SOLID) && fluid_next) crb += rin[zc];
                 } else {
-                    a = ain[(long long)b * C + zc];
+                    a = pulled;
                 }
             }
         }
@@ -465,23 +543,25 @@ __global__ void __launch_bounds__(32 * ADJ_CUBE_WARPS) adj_cube_kernel(const Dev
             if (act) aout[(long long)b * C + c] = a;
         } else {
             // the transposed collision (collide_adjoint), its sums over the lanes
-            const A om = (A)dv.omega;
+            const A om = AdjParams<A>::omega(dv);
             const A uu = u0 * u0 + u1 * u1 + u2 * u2;
             const A eu = (A)bx * u0 + (A)by * u1 + (A)bz * u2;
             const A wa = act ? wb * a : (A)0;
             const A cc = (A)3 + (A)9 * eu;
-            const A sr = warp_sum(wa * ((A)1 + (A)3 * eu + (A)4.5 * eu * eu - (A)1.5 * uu));
-            const A s0 = warp_sum(wa * (cc * (A)bx - (A)3 * u0));
-            const A s1 = warp_sum(wa * (cc * (A)by - (A)3 * u1));
-            const A s2 = warp_sum(wa * (cc * (A)bz - (A)3 * u2));
+            A t4[4] = {wa * ((A)1 + (A)3 * eu + (A)4.5 * eu * eu - (A)1.5 * uu), wa * (cc * (A)bx - (A)3 * u0),
+                       wa * (cc * (A)by - (A)3 * u1), wa * (cc * (A)bz - (A)3 * u2)};
+            warp_sum4(t4);
+            const A sr = t4[0], s0 = t4[1], s1 = t4[2], s2 = t4[3];
             A f0 = 0, f1 = 0, f2 = 0;
             if (dv.forced) {
-                const A eg = (A)(bx * dv.g[0] + by * dv.g[1] + bz * dv.g[2]);
-                f0 = warp_sum(wa * ((A)(-3.0 * dv.g[0]) + (A)9 * (A)bx * eg));
-                f1 = warp_sum(wa * ((A)(-3.0 * dv.g[1]) + (A)9 * (A)by * eg));
-                f2 = warp_sum(wa * ((A)(-3.0 * dv.g[2]) + (A)9 * (A)bz * eg));
+                const A g0 = AdjParams<A>::g(dv, 0), g1 = AdjParams<A>::g(dv, 1), g2 = AdjParams<A>::g(dv, 2);
+                const A eg = (A)bx * g0 + (A)by * g1 + (A)bz * g2;
+                A f4[4] = {wa * ((A)9 * (A)bx * eg - (A)3 * g0), wa * ((A)9 * (A)by * eg - (A)3 * g1),
+                           wa * ((A)9 * (A)bz * eg - (A)3 * g2), (A)0};
+                warp_sum4(f4);
+                f0 = f4[0]; f1 = f4[1]; f2 = f4[2];
             }
-            const A kf = (A)1 - (A)0.5 * om;
+            const A kf = AdjParams<A>::guo(dv);
             const A su0 = (om * rho * s0 + kf * f0) * ir, su1 = (om * rho * s1 + kf * f1) * ir,
                     su2 = (om * rho * s2 + kf * f2) * ir;
             const A base = om * sr - (su0 * u0 + su1 * u1 + su2 * u2);
@@ -525,12 +605,13 @@ __global__ void __launch_bounds__(32 * ADJ_CUBE_WARPS) adj_cube_kernel(const Dev
             }
             if (lane == 0) static_cast<A *>(ap.rout)[c] = rh_out;
         }
-#pragma unroll
-        for (int i = 0; i < 9; ++i) wsum[i] += warp_sum(acc[i]);
     }
     // 3. the block's body-kb sums, warps in order
-    if (lane == 0)
-        for (int i = 0; i < 9; ++i) wacc[warp][i] = (double)wsum[i];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        const A v = warp_sum(acc[i]);
+        if (lane == 0) wacc[warp][i] = (double)v;
+    }
     __syncthreads();
     if (tid < 9) {
         double v = 0.0;
@@ -658,7 +739,7 @@ adj_terms_kernel(const Device dv, const BodyState *states, const double *fhs, lo
 constexpr int ADJ_WARPS = ADJ_THREADS / 32;
 constexpr int ADJ_SUM_GROUPS = 3;           // records a warp's lanes take side by side, nine sums each
 
-__global__ void __launch_bounds__(ADJ_THREADS) adj_integrate_kernel(const Device dv, const AdjBody ab) {
+__device__ __forceinline__ void adj_integrate(const Device &dv, const AdjBody &ab) {
     constexpr unsigned FULL = 0xffffffffu;
     const int nb = dv.nb;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -721,24 +802,24 @@ __global__ void __launch_bounds__(ADJ_THREADS) adj_integrate_kernel(const Device
             dot += __shfl_xor_sync(FULL, dot, 2);
             const double qh4 = (qh - q1 * dot) * inv_nn;
             const double h0 = at(qh4, 0), hv0 = at(qh4, 1), hv1 = at(qh4, 2), hv2 = at(qh4, 3);
-            const double hv[3] = {hv0, hv1, hv2};
+            auto hv = [&](int i) { return i == 0 ? hv0 : (i == 1 ? hv1 : hv2); };
             const double Wa = at(W1, 0), Wb = at(W1, 1), Wc = at(W1, 2);
-            const double Wv[3] = {Wa, Wb, Wc};
+            auto Wv = [&](int i) { return i == 0 ? Wa : (i == 1 ? Wb : Wc); };
             const double w = at(q4s, 0), va = at(q4s, 1), vb = at(q4s, 2), vc = at(q4s, 3);
-            const double vv[3] = {va, vb, vc};
+            auto vv = [&](int i) { return i == 0 ? va : (i == 1 ? vb : vc); };
             // the adjoint of q_n through the update: lane 0 the scalar part,
             // lane 1 + i the vector component i
             double qout;
             {
                 const int i = lane >= 1 && lane <= 3 ? lane - 1 : 0, j = (i + 1) % 3, k = (i + 2) % 3;
                 const bool s0 = lane == 0;
-                const double p1 = s0 ? hv[0] : -h0, r1 = s0 ? Wv[0] : Wv[i];
-                const double p2 = s0 ? hv[1] : hv[j], r2 = s0 ? Wv[1] : Wv[k];
-                const double p3 = s0 ? hv[2] : -hv[k], r3 = s0 ? Wv[2] : Wv[j];
-                qout = (s0 ? h0 : hv[i]) + 0.5 * (p1 * r1 + p2 * r2 + p3 * r3);
+                const double p1 = s0 ? hv(0) : -h0, r1 = s0 ? Wv(0) : Wv(i);
+                const double p2 = s0 ? hv(1) : hv(j), r2 = s0 ? Wv(1) : Wv(k);
+                const double p3 = s0 ? hv(2) : -hv(k), r3 = s0 ? Wv(2) : Wv(j);
+                qout = (s0 ? h0 : hv(i)) + 0.5 * (p1 * r1 + p2 * r2 + p3 * r3);
             }
             // Omega: Wh1 = Wh + 1/2 (w qv - qh0 v + v x qv), lanes 0..2
-            const double Wh1 = at(sn, 10 + ax) + 0.5 * (w * hv[ax] - h0 * vv[ax] + vv[i1] * hv[i2] - vv[i2] * hv[i1]);
+            const double Wh1 = at(sn, 10 + ax) + 0.5 * (w * hv(ax) - h0 * vv(ax) + vv(i1) * hv(i2) - vv(i2) * hv(i1));
             const double w0 = at(Wh1, 0), w1 = at(Wh1, 1), w2 = at(Wh1, 2);
             const double alpha = R0i * w0 + R1i * w1 + R2i * w2;
             const double aI = alpha * inv_I;
@@ -853,6 +934,28 @@ __global__ void __launch_bounds__(ADJ_THREADS) adj_integrate_kernel(const Device
     }
 }
 
+// The first launch of reverse step n: block (0, 0) the rigid-body step, the others
+// the bulk cells, which need neither its result nor each other's.  One launch
+// instead of two on two streams with events between them (96 x 48 x 48 study: a
+// launch takes 14.2 us, the rigid-body step alone 11.4 us).
+template <typename A, typename T, bool FIRST>
+__global__ void __launch_bounds__(ADJ_THREADS, sizeof(A) == 4 ? 3 : 2)
+adj_step_kernel(const Device dv, const AdjPtrs ap, const AdjBody ab, int body) {
+    int blk = blockIdx.x;
+    if (body) {
+        if (blk == 0) {
+            if (blockIdx.y == 0) adj_integrate(dv, ab);
+            return;
+        }
+        --blk;
+    }
+    adj_bulk_cells<A, T, FIRST>(dv, ap, blk, blockIdx.y);
+}
+
+__global__ void __launch_bounds__(ADJ_THREADS) adj_integrate_kernel(const Device dv, const AdjBody ab) {
+    adj_integrate(dv, ab);
+}
+
 // sa[b] += the cell sums part[b][0..count) (the last reverse step)
 __global__ void adj_reduce_kernel(int nb, const double *part, int stride, int count, double *sa) {
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
@@ -865,10 +968,12 @@ __global__ void adj_reduce_kernel(int nb, const double *part, int stride, int co
 }
 
 template <typename A, typename T, bool FIRST>
-void launch_bulk_cells(const Device &dv, const AdjPtrs &ap, cudaStream_t s) {
-    const dim3 blk(128, 2);
-    const dim3 grid((dv.dom.nx + 127) / 128, (dv.dom.ny + 1) / 2, dv.dom.nz);
-    adj_bulk_kernel<A, T, FIRST><<<grid, blk, 0, s>>>(dv, ap);
+void launch_step_cells(const Device &dv, const AdjPtrs &ptrs, const AdjBody *ab, cudaStream_t s) {
+    AdjPtrs ap = ptrs;
+    ap.row_recip = row_recip(dv.dom.nx);
+    const long long plane = (long long)dv.dom.nx * dv.dom.ny;
+    const dim3 grid((unsigned)((plane + ADJ_THREADS - 1) / ADJ_THREADS) + (ab ? 1 : 0), dv.dom.nz);
+    adj_step_kernel<A, T, FIRST><<<grid, ADJ_THREADS, 0, s>>>(dv, ap, ab ? *ab : AdjBody{}, ab ? 1 : 0);
 }
 
 template <typename A, typename T, bool FIRST>
@@ -903,13 +1008,13 @@ void launch_adj_terms(const Device &dv, const BodyState *states, const double *f
                                                                                                  tb, td, ts);
 }
 
-void launch_adj_bulk(const Device &dv, const AdjPtrs &ap, bool first, cudaStream_t s) {
+void launch_adj_step(const Device &dv, const AdjPtrs &ap, const AdjBody *ab, cudaStream_t s) {
     if (dv.precision == LBM_PREC_F64) {
-        if (first) launch_bulk_cells<double, double, true>(dv, ap, s);
-        else launch_bulk_cells<double, double, false>(dv, ap, s);
+        if (!ab) launch_step_cells<double, double, true>(dv, ap, ab, s);
+        else launch_step_cells<double, double, false>(dv, ap, ab, s);
     } else {
-        if (first) launch_bulk_cells<float, float, true>(dv, ap, s);
-        else launch_bulk_cells<float, float, false>(dv, ap, s);
+        if (!ab) launch_step_cells<float, float, true>(dv, ap, ab, s);
+        else launch_step_cells<float, float, false>(dv, ap, ab, s);
     }
 }
 

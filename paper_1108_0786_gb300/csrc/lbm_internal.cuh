@@ -405,6 +405,7 @@ struct AdjPtrs {
     const double *fadj;             // [nb][6] adjoint of force and torque of step n
     double *part;                   // [nb][part_stride][9] per-block body sums (X, V, W)
     int part_stride;
+    unsigned row_recip;             // row_recip of an x-row (the launch's)
 };
 
 // pointers of the reversed rigid-body step n (adjoint.cu)
@@ -495,7 +496,9 @@ void launch_adj_integrate(const Device &dv, const AdjBody &ab, cudaStream_t s);
 // (state t0 + j at states + j nb) and loads (fh + 6 j nb)
 void launch_adj_terms(const Device &dv, const BodyState *states, const double *fh, long long t0, int L,
                       AdjBodyTerms *tb, AdjDriveTerms *td, AdjSpringTerms *ts, cudaStream_t s);
-void launch_adj_bulk(const Device &dv, const AdjPtrs &ap, bool first, cudaStream_t s);
+// bulk cells and (ab) the rigid-body step of a reverse step; without ab the
+// first step's stream alone
+void launch_adj_step(const Device &dv, const AdjPtrs &ap, const AdjBody *ab, cudaStream_t s);
 void launch_adj_boundary(const Device &dv, const AdjPtrs &ap, bool first, cudaStream_t s);
 void launch_adj_reduce(const Device &dv, const double *part, int stride, int count, double *sa, cudaStream_t s);
 

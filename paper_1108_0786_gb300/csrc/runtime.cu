@@ -1456,17 +1456,18 @@ int lbm_adjoint_backward(lbm_t *h, const double *seed, double *grad_state, doubl
                 }
             for (cudaGraphExec_t &g : rgraph)
                 if (g) cudaGraphExecDestroy(g);
-            if (h->side) cudaStreamSynchronize(h->side);
             cudaStreamSynchronize(h->stream);
             free_list(h, list);
         }
     } guard{h, bk, rs, rss, rss2, rcap, rcaps, rcaps2, rgraph};
     // a slot set holds one segment's recomputed epochs: populations (slots
-    // 0..K), flags and body ids (slots 0..K+1)
+    // 0..K), flags and body ids (slots 0..K+1, an epoch's two maps side by side)
     struct SlotSet {
         void *pop = nullptr;
-        uint8_t *flags = nullptr, *bid = nullptr;
+        uint8_t *maps = nullptr;
     } sets[2];
+    auto slot_flags = [&](const SlotSet &st, int j) { return st.maps + 2 * C * j; };
+    auto slot_bid = [&](const SlotSet &st, int j) { return st.maps + 2 * C * j + C; };
     uint8_t *carry = nullptr;       // one set: the flags of epoch m + L kept from segment k + 1
     BodyState *stage[2] = {nullptr, nullptr};   // a full segment's states, epochs m - 1 .. m + K - 1
     void *A[2] = {nullptr, nullptr}, *R[2] = {nullptr, nullptr};
@@ -1507,8 +1508,7 @@ int lbm_adjoint_backward(lbm_t *h, const double *seed, double *grad_state, doubl
         for (int i = 0; i < nset; ++i) {
             if ((rc = alloc_list(h, bk, &stage[i], sizeof(BodyState) * B * (size_t)(K + 1)))) return rc;
             if ((rc = alloc_list(h, bk, &sets[i].pop, pop_sz * (K + 1)))) return rc;
-            if ((rc = alloc_list(h, bk, &sets[i].flags, (size_t)C * (K + 2)))) return rc;
-            if ((rc = alloc_list(h, bk, &sets[i].bid, (size_t)C * (K + 2)))) return rc;
+            if ((rc = alloc_list(h, bk, &sets[i].maps, 2 * (size_t)C * (K + 2)))) return rc;
         }
         if (nset == 1 && (rc = alloc_list(h, bk, &carry, (size_t)C))) return rc;
         for (int i = 0; i < 2; ++i) {
@@ -1531,10 +1531,7 @@ int lbm_adjoint_backward(lbm_t *h, const double *seed, double *grad_state, doubl
     }
     cudaStream_t s = h->stream;
     if ((rc = build_graphs(h))) return rc;        // creates the side stream
-    // the bulk part of each reverse step needs no body adjoint: it runs on
-    // the side stream, concurrently with the rigid-body and boundary parts;
-    // the recomputation runs on a stream of its own
-    cudaStream_t side = h->side;
+    // the recomputation runs on streams of its own
     if (fl) {
         CK(cudaStreamCreateWithFlags(&rs, cudaStreamNonBlocking));
         CK(cudaStreamCreateWithFlags(&rss, cudaStreamNonBlocking));
@@ -1547,32 +1544,26 @@ int lbm_adjoint_backward(lbm_t *h, const double *seed, double *grad_state, doubl
         CK(cudaStreamCreateWithPriority(&rcaps, cudaStreamNonBlocking, greatest));
         CK(cudaStreamCreateWithPriority(&rcaps2, cudaStreamNonBlocking, greatest));
     }
-    cudaEvent_t ev_main = nullptr, ev_side = nullptr, ev_rec = nullptr, ev_free_main = nullptr,
-                ev_free_side = nullptr, ev_rfork = nullptr, ev_rjoin2 = nullptr, ev_cfork = nullptr, ev_cjoin2 = nullptr,
+    cudaEvent_t ev_rec = nullptr, ev_free = nullptr, ev_rfork = nullptr, ev_rjoin2 = nullptr, ev_cfork = nullptr, ev_cjoin2 = nullptr,
+                ev_rcopy = nullptr, ev_ccopy = nullptr,
                 ev_rbulk[2] = {nullptr, nullptr}, ev_cbulk[2] = {nullptr, nullptr};
-    CK(cudaEventCreateWithFlags(&ev_main, cudaEventDisableTiming));
-    CK(cudaEventCreateWithFlags(&ev_side, cudaEventDisableTiming));
     CK(cudaEventCreateWithFlags(&ev_rec, cudaEventDisableTiming));
-    CK(cudaEventCreateWithFlags(&ev_free_main, cudaEventDisableTiming));
-    CK(cudaEventCreateWithFlags(&ev_free_side, cudaEventDisableTiming));
+    CK(cudaEventCreateWithFlags(&ev_free, cudaEventDisableTiming));
     CK(cudaEventCreateWithFlags(&ev_rfork, cudaEventDisableTiming));
     CK(cudaEventCreateWithFlags(&ev_cfork, cudaEventDisableTiming));
     CK(cudaEventCreateWithFlags(&ev_rjoin2, cudaEventDisableTiming));
     CK(cudaEventCreateWithFlags(&ev_cjoin2, cudaEventDisableTiming));
-    for (cudaEvent_t *ev : {&ev_rbulk[0], &ev_rbulk[1], &ev_cbulk[0], &ev_cbulk[1]})
+    for (cudaEvent_t *ev : {&ev_rcopy, &ev_ccopy, &ev_rbulk[0], &ev_rbulk[1], &ev_cbulk[0], &ev_cbulk[1]})
         CK(cudaEventCreateWithFlags(ev, cudaEventDisableTiming));
     struct Events {
-        cudaEvent_t *e[13];
+        cudaEvent_t *e[12];
         ~Events() {
             for (cudaEvent_t *p : e)
                 if (*p) cudaEventDestroy(*p);
         }
-    } events{{&ev_main, &ev_side, &ev_rec, &ev_free_main, &ev_free_side, &ev_rfork, &ev_cfork, &ev_rjoin2, &ev_cjoin2,
-               &ev_rbulk[0], &ev_rbulk[1], &ev_cbulk[0], &ev_cbulk[1]}};
-    CK(cudaEventRecord(ev_main, s));
-    CK(cudaEventRecord(ev_side, s));
-    CK(cudaEventRecord(ev_free_main, s));
-    CK(cudaEventRecord(ev_free_side, s));
+    } events{{&ev_rec, &ev_free, &ev_rfork, &ev_cfork, &ev_rjoin2, &ev_cjoin2,
+               &ev_rcopy, &ev_ccopy, &ev_rbulk[0], &ev_rbulk[1], &ev_cbulk[0], &ev_cbulk[1]}};
+    CK(cudaEventRecord(ev_free, s));
     double *gd = grads, *gs = grads + 2 * ND, *gb = grads + 2 * ND + 3 * NS;
     CK(cudaMemsetAsync(grads, 0, sizeof(double) * ngrad, s));
     CK(cudaMemsetAsync(part, 0, sizeof(double) * 9 * B * (size_t)stride, s));
@@ -1625,8 +1616,7 @@ int lbm_adjoint_backward(lbm_t *h, const double *seed, double *grad_state, doubl
     // copy into slot j + 2 is made beside step j's boundary kernel, off the
     // chain; slot 1's before the segment's first remap.  `copy_next`: step j + 1 follows.
     auto copy_slot = [&](const SlotSet &st, int j, cudaStream_t ms) -> int {
-        CK(cudaMemcpyAsync(st.flags + C * (j + 1), st.flags + C * j, (size_t)C, cudaMemcpyDeviceToDevice, ms));
-        CK(cudaMemcpyAsync(st.bid + C * (j + 1), st.bid + C * j, (size_t)C, cudaMemcpyDeviceToDevice, ms));
+        CK(cudaMemcpyAsync(slot_flags(st, j + 1), slot_flags(st, j), 2 * (size_t)C, cudaMemcpyDeviceToDevice, ms));
         return LBM_OK;
     };
     // The streams are those of a captured forward step: the chain ms, the bulk
@@ -1634,7 +1624,7 @@ int lbm_adjoint_backward(lbm_t *h, const double *seed, double *grad_state, doubl
     // copies on ss2.
     struct StepStreams {
         cudaStream_t ms, ss, ss2;
-        cudaEvent_t fork, join2, *bulk;
+        cudaEvent_t fork, join2, copied, *bulk;
     };
     auto recompute_step = [&](const SlotSet &st, int j, const BodyState *prev, const BodyState *cur, bool last,
                               bool copy_next, const StepStreams &q) -> int {
@@ -1643,10 +1633,10 @@ int lbm_adjoint_backward(lbm_t *h, const double *seed, double *grad_state, doubl
         lbm::StepPtrs sp{};
         sp.src = slot_pop(st, j);
         sp.dst = slot_pop(st, j + 1);
-        sp.flags_prev = st.flags + C * j;
-        sp.bid_prev = st.bid + C * j;
-        sp.flags_cur = st.flags + C * (j + 1);
-        sp.bid_cur = st.bid + C * (j + 1);
+        sp.flags_prev = slot_flags(st, j);
+        sp.bid_prev = slot_bid(st, j);
+        sp.flags_cur = slot_flags(st, j + 1);
+        sp.bid_cur = slot_bid(st, j + 1);
         sp.body_prev = prev;
         sp.body_cur = cur;
         sp.body_next = scratch;
@@ -1657,6 +1647,7 @@ int lbm_adjoint_backward(lbm_t *h, const double *seed, double *grad_state, doubl
             CK(cudaStreamWaitEvent(q.ss2, q.fork, 0));
             lbm::launch_loads(dr, sp, q.ss2);
         }
+        if (j > 0) CK(cudaStreamWaitEvent(q.ms, q.copied, 0));
         // the body preparation only at the segment's first step: the later
         // states' geometry records come from the recomputation's own
         // rigid-body steps (the same bits as the tape's states)
@@ -1665,8 +1656,9 @@ int lbm_adjoint_backward(lbm_t *h, const double *seed, double *grad_state, doubl
         CK(cudaEventRecord(q.fork, q.ms));
         CK(cudaStreamWaitEvent(q.ss2, q.fork, 0));
         lbm::launch_links(dr, sp, q.ss2);
-        if (copy_next && (rc3 = copy_slot(st, j + 1, q.ss2))) return rc3;
         CK(cudaEventRecord(q.join2, q.ss2));
+        if (copy_next && (rc3 = copy_slot(st, j + 1, q.ss2))) return rc3;
+        CK(cudaEventRecord(q.copied, q.ss2));
         if (j > 0) CK(cudaStreamWaitEvent(q.ms, q.bulk[(j & 1) ^ 1], 0));
         lbm::launch_boundary_fix(dr, sp, q.ms);
         CK(cudaStreamWaitEvent(q.ss, q.fork, 0));
@@ -1676,10 +1668,14 @@ int lbm_adjoint_backward(lbm_t *h, const double *seed, double *grad_state, doubl
         lbm::launch_force(dr, sp, q.ms);
         return LBM_OK;
     };
-    const StepStreams eager{rs, rss, rss2, ev_rfork, ev_rjoin2, ev_rbulk},
-        captured{rcap, rcaps, rcaps2, ev_cfork, ev_cjoin2, ev_cbulk};
-    // A full segment (K steps, not the last) is recomputed by a CUDA graph of
-    // its set: its states are staged (epochs m - 1 .. m + K - 1) into the
+    const StepStreams eager{rs, rss, rss2, ev_rfork, ev_rjoin2, ev_rcopy, ev_rbulk},
+        captured{rcap, rcaps, rcaps2, ev_cfork, ev_cjoin2, ev_ccopy, ev_cbulk};
+    // With enough segments a full one (K steps, not the last) is recomputed by a
+    // CUDA graph of its set: a graph costs the host about as much as launching its
+    // steps twice (~45 us a step to capture and instantiate, ~25 us to launch it
+    // kernel by kernel), so each set's is to be used at least four times.
+    const bool graphs = tp.nseg - 1 >= 4 * nset;
+    // The set's graph: its states are staged (epochs m - 1 .. m + K - 1) into the
     // set's staging buffer, so that one graph serves every full segment of
     // the set.
     auto full_graph = [&](int set) -> int {
@@ -1690,7 +1686,9 @@ int lbm_adjoint_backward(lbm_t *h, const double *seed, double *grad_state, doubl
         for (int j = 0; j < K && rc2 == LBM_OK; ++j)
             rc2 = recompute_step(st, j, stage[set] + (long long)j * B, stage[set] + (long long)(j + 1) * B, false,
                                  j + 1 < K, captured);
-        if (rc2 == LBM_OK && cudaStreamWaitEvent(rcap, ev_cbulk[(K - 1) & 1], 0) != cudaSuccess) rc2 = LBM_E_CUDA;
+        if (rc2 == LBM_OK && (cudaStreamWaitEvent(rcap, ev_cbulk[(K - 1) & 1], 0) != cudaSuccess ||
+                              cudaStreamWaitEvent(rcap, ev_ccopy, 0) != cudaSuccess))
+            rc2 = LBM_E_CUDA;
         cudaGraph_t g = nullptr;
         const cudaError_t e1 = cudaStreamEndCapture(rcap, &g);
         if (rc2) {
@@ -1709,14 +1707,14 @@ int lbm_adjoint_backward(lbm_t *h, const double *seed, double *grad_state, doubl
         const SlotSet &st = set_of(k);
         const int set = nset == 2 ? (k & 1) : 0;
         if (nset == 1 && k < tp.nseg - 1)       // epoch m + L, recomputed with segment k + 1
-            CK(cudaMemcpyAsync(carry, st.flags + C, (size_t)C, cudaMemcpyDeviceToDevice, rs));
+            CK(cudaMemcpyAsync(carry, slot_flags(st, 1), (size_t)C, cudaMemcpyDeviceToDevice, rs));
         CK(cudaMemcpyAsync(st.pop, static_cast<char *>(tp.ckpt_pop) + pop_sz * k, pop_sz,
                            cudaMemcpyDeviceToDevice, rs));
-        CK(cudaMemcpyAsync(st.flags, tp.ckpt_flags + C * k, (size_t)C, cudaMemcpyDeviceToDevice, rs));
-        CK(cudaMemcpyAsync(st.bid, tp.ckpt_bid + C * k, (size_t)C, cudaMemcpyDeviceToDevice, rs));
+        CK(cudaMemcpyAsync(slot_flags(st, 0), tp.ckpt_flags + C * k, (size_t)C, cudaMemcpyDeviceToDevice, rs));
+        CK(cudaMemcpyAsync(slot_bid(st, 0), tp.ckpt_bid + C * k, (size_t)C, cudaMemcpyDeviceToDevice, rs));
         CK(cudaMemcpyAsync(r_t, &m, sizeof m, cudaMemcpyHostToDevice, rs));
         CK(cudaMemcpyAsync(r_changed, ones, sizeof ones, cudaMemcpyHostToDevice, rs));
-        if (L == K && k < tp.nseg - 1) {
+        if (graphs && L == K && k < tp.nseg - 1) {
             int rc2;
             if ((rc2 = full_graph(set))) return rc2;
             CK(cudaMemcpyAsync(stage[set], S(m - 1), sizeof(BodyState) * B * (size_t)(K + 1),
@@ -1729,6 +1727,7 @@ int lbm_adjoint_backward(lbm_t *h, const double *seed, double *grad_state, doubl
                 if ((rc2 = recompute_step(st, j, S(m + j - 1), S(m + j), false, j + 1 < L || extra, eager))) return rc2;
             }
             CK(cudaStreamWaitEvent(rs, ev_rbulk[(L - 1) & 1], 0));
+            CK(cudaStreamWaitEvent(rs, ev_rcopy, 0));
             if (extra) {
                 int rc2;
                 if ((rc2 = recompute_step(st, L, S(m + L - 1), S(m + L), true, false, eager))) return rc2;
@@ -1741,12 +1740,11 @@ int lbm_adjoint_backward(lbm_t *h, const double *seed, double *grad_state, doubl
     };
     // segment k's slots are rewritten by the recomputation of segment k - 2
     // (two sets) or k - 1 (one set); it waits for the reverse steps that read
-    // them, ev_free_main / ev_free_side (the first reverse step of segment k
+    // them, ev_free (the first reverse step of segment k
     // - 1 reads slot 1 of segment k's set, the flags of epoch m + L, or with
     // one set their copy in carry)
     auto start_recompute = [&](int k) -> int {
-        CK(cudaStreamWaitEvent(rs, ev_free_main, 0));
-        CK(cudaStreamWaitEvent(rs, ev_free_side, 0));
+        CK(cudaStreamWaitEvent(rs, ev_free, 0));
         return recompute(k);
     };
     if (fl && (rc = start_recompute(tp.nseg - 1))) return rc;
@@ -1756,7 +1754,6 @@ int lbm_adjoint_backward(lbm_t *h, const double *seed, double *grad_state, doubl
         const SlotSet &st = set_of(k);
         if (fl) {
             CK(cudaStreamWaitEvent(s, ev_rec, 0));      // the segment's slots and terms are ready
-            CK(cudaEventRecord(ev_main, s));
         } else {
             make_terms(k, s);
         }
@@ -1779,15 +1776,16 @@ int lbm_adjoint_backward(lbm_t *h, const double *seed, double *grad_state, doubl
             ab.td = tset.td + (long long)j * ND;
             ab.ts = tset.ts + (long long)j * NS;
             ab.t = n;
-            lbm::launch_adj_integrate(dv, ab, s);
-            if (fl) {
+            if (!fl) {
+                lbm::launch_adj_integrate(dv, ab, s);
+            } else {
                 lbm::AdjPtrs ap{};
                 ap.G = slot_pop(st, j + 1);
-                ap.flags_cur = st.flags + C * (j + 1);
-                ap.bid_cur = st.bid + C * (j + 1);
-                ap.bid_prev = st.bid + C * j;
-                ap.flags_next = (j + 1 < L || k == tp.nseg - 1) ? st.flags + C * (j + 2)
-                                : nset == 2                    ? set_of(k + 1).flags + C
+                ap.flags_cur = slot_flags(st, j + 1);
+                ap.bid_cur = slot_bid(st, j + 1);
+                ap.bid_prev = slot_bid(st, j);
+                ap.flags_next = (j + 1 < L || k == tp.nseg - 1) ? slot_flags(st, j + 2)
+                                : nset == 2                    ? slot_flags(set_of(k + 1), 1)
                                                                : carry;
                 ap.ain = A[ai];
                 ap.rin = R[ai];
@@ -1797,17 +1795,14 @@ int lbm_adjoint_backward(lbm_t *h, const double *seed, double *grad_state, doubl
                 ap.fadj = fadj;
                 ap.part = part;
                 ap.part_stride = stride;
-                CK(cudaStreamWaitEvent(side, ev_main, 0));     // Ph^{n+1} of the boundary cells
-                lbm::launch_adj_bulk(dv, ap, false, side);
-                CK(cudaStreamWaitEvent(s, ev_side, 0));        // Ph^{n+1} of the bulk cells
-                CK(cudaEventRecord(ev_side, side));
+                // the rigid-body step with the bulk cells, then the boundary cells
+                // (which need its force and torque adjoints)
+                lbm::launch_adj_step(dv, ap, &ab, s);
                 lbm::launch_adj_boundary(dv, ap, false, s);
-                CK(cudaEventRecord(ev_main, s));
                 if (j == L - 1 && nset == 2) {
                     // segment k + 1's set (read up to here) is free for the
                     // recomputation of segment k - 1
-                    CK(cudaEventRecord(ev_free_main, s));
-                    CK(cudaEventRecord(ev_free_side, side));
+                    CK(cudaEventRecord(ev_free, s));
                     if (k > 0 && (rc = start_recompute(k - 1))) return rc;
                 }
                 ai ^= 1;
@@ -1815,25 +1810,23 @@ int lbm_adjoint_backward(lbm_t *h, const double *seed, double *grad_state, doubl
             cur ^= 1;
         }
         if (fl && nset == 1) {
-            CK(cudaEventRecord(ev_free_main, s));
-            CK(cudaEventRecord(ev_free_side, side));
+            CK(cudaEventRecord(ev_free, s));
             if (k > 0 && (rc = start_recompute(k - 1))) return rc;
         }
         CK(cudaGetLastError());
     }
     // sa[cur]: adjoint of state n0 without the cell sums of reverse step n0
     if (fl) {
-        CK(cudaStreamWaitEvent(s, ev_side, 0));
         lbm::launch_adj_reduce(dv, part, stride, stride, sa[cur], s);
         // the stream of step n0 itself: adjoint of the populations entering
         // the run and of the state n0 - 1 (its moving-wall velocities)
         CK(cudaMemsetAsync(fadj, 0, sizeof(double) * 6 * B, s));
         lbm::AdjPtrs ap{};
         ap.G = slot_pop(sets[0], 0);
-        ap.flags_cur = sets[0].flags;
-        ap.bid_cur = sets[0].bid;
-        ap.bid_prev = sets[0].bid;
-        ap.flags_next = sets[0].flags + C;
+        ap.flags_cur = slot_flags(sets[0], 0);
+        ap.bid_cur = slot_bid(sets[0], 0);
+        ap.bid_prev = slot_bid(sets[0], 0);
+        ap.flags_next = slot_flags(sets[0], 1);
         ap.ain = A[ai];
         ap.rin = R[ai];
         ap.aout = A[ai ^ 1];
@@ -1842,7 +1835,7 @@ int lbm_adjoint_backward(lbm_t *h, const double *seed, double *grad_state, doubl
         ap.fadj = fadj;
         ap.part = part;
         ap.part_stride = stride;
-        lbm::launch_adj_bulk(dv, ap, true, s);
+        lbm::launch_adj_step(dv, ap, nullptr, s);
         lbm::launch_adj_boundary(dv, ap, true, s);
         CK(cudaMemsetAsync(sa[cur ^ 1], 0, sizeof(double) * 13 * B, s));
         lbm::launch_adj_reduce(dv, part, stride, stride, sa[cur ^ 1], s);
