@@ -248,6 +248,20 @@ __device__ __forceinline__ void collide_f64(double (&f)[Q], const Device &dv) {
     }
     const double r3[2] = {3.0 * dv.ow[1] * rho, 3.0 * dv.ow[2] * rho};
     const double r45[2] = {1.5 * r3[0], 1.5 * r3[1]};
+    if (om1 == 0.0 && !forced) {
+        // tau = 1: the update is the equilibrium itself, the same bits without 18
+        // of the FMAs (0 f + a = a; a non-finite f makes every moment so)  203 x 149
+        // x 131 cells, 8 steps and the populations, 8.31 -> 7.17 ms
+#pragma unroll
+        for (int p = 0; p < Q / 2; ++p) {
+            const int b = 2 * p + 1, wc = p < 3 ? 0 : 1;
+            const double eu = edot(b, ux, uy, uz);
+            const double a = mad(r45[wc], p < 3 ? sq[p] : eu * eu, wc ? b2 : b1);
+            f[b] = mad(r3[wc], eu, a);
+            f[b + 1] = mad(-r3[wc], eu, a);
+        }
+        return;
+    }
 #pragma unroll
     for (int p = 0; p < Q / 2; ++p) {
         const int b = 2 * p + 1, wc = p < 3 ? 0 : 1;
