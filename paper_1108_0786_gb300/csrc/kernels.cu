@@ -358,7 +358,7 @@ __device__ __forceinline__ void remap_body(const Device &dv, const StepPtrs &sp,
     // tests sort them out): one round of loads less in a block's latency chain
     // (32^3 FP64 swimmer, a step: 45.1 -> 42.2 us with the narrower screen margin;
     // 128 x 64 x 64 channel 34.6 -> 33.7 us).
-    const bool all = SELF_CAND && dv.nb <= REMAP_STAGED;
+    const bool all = dv.nb <= REMAP_STAGED;
     if (all) {
         if (tid < dv.nb) cid[tid] = tid;
     } else if constexpr (SELF_CAND) {
@@ -624,6 +624,8 @@ __device__ __forceinline__ void links_body(const Device &dv, const StepPtrs &sp,
 __global__ void __launch_bounds__(256) links_kernel(const Device dv, const StepPtrs sp) { links_body(dv, sp, launch_blk()); }
 
 __global__ void __launch_bounds__(256) links_batch(const Batch bt) {
+    // nearly always there is nothing to rebuild: look before fetching the member
+    if (bt.dv[bt.member[blockIdx.x]].changed[bt.parity] == 0) return;
     LBM_BATCH_MEMBER(bt);
     links_body(sdv, ssp, sbk);
 }
@@ -1021,7 +1023,10 @@ __device__ __forceinline__ void force_body(const Device &dv, const StepPtrs &sp,
     }
     link_sync();
     const int total = prefix[side];
-    const int chunk = (total + FORCE_BLOCKS - 1) / FORCE_BLOCKS;
+    // FP64 partial sums are added in block order: the split is fixed.  The fixed-
+    // point sums of the other types take any number of blocks.
+    const int blocks = sizeof(T) == 8 ? FORCE_BLOCKS : bk.gx;
+    const int chunk = (total + blocks - 1) / blocks;
     const int j0 = kb * chunk, j1 = min(total, j0 + chunk);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 
@@ -1565,19 +1570,32 @@ int near_tile_cap(const Device &dv, int emax) {
     return (int)std::min<long long>((long long)dv.nb * per_body, near_tile_count(dv));
 }
 
-// the grids of launch_remap, launch_links and launch_force for one lattice
-void batch_grid_small(const Device &dv, int k, int g[3]) {
+// Force blocks a body in a batched launch over `members` lattices like dv: with
+// many bodies a block's member lookup and reductions cost more than its second
+// round of links (48 boxes of three bodies, two launches: boundary_batch_turns).
+// FP64 keeps its split, which the sums' order depends on.
+static int force_batch_blocks(const Device &dv, int members) {
+    const int bodies = members * dv.nb;
+    return dv.precision == 0 || bodies < 16 ? FORCE_BLOCKS : (bodies < 64 ? 2 : 1);
+}
+
+// the grids of launch_remap, launch_links and launch_force for one lattice of a
+// batched launch over `members` of them
+void batch_grid_small(const Device &dv, int k, int members, int g[3]) {
     g[0] = g[1] = g[2] = 0;
     if (dv.nb == 0) return;
     const int side = dv.remap_side;
     switch (k) {
-    case BK_PREP: case BK_LOADS: g[0] = g[1] = g[2] = 1; break;
+    // few bodies are all remap candidates, and states the host wrote are prepared
+    // before a batched run: nothing to prepare in its steps
+    case BK_PREP: g[0] = g[1] = g[2] = dv.nb > REMAP_STAGED ? 1 : 0; break;
+    case BK_LOADS: g[0] = g[1] = g[2] = 1; break;
     case BK_REMAP:
         g[0] = remap_blocks(side);
         g[1] = dv.nb; g[2] = 1;
         break;
     case BK_LINKS: g[0] = dv.link_side; g[1] = dv.nb; g[2] = 1; break;
-    case BK_FORCE: g[0] = FORCE_BLOCKS; g[1] = dv.nb; g[2] = 1; break;
+    case BK_FORCE: g[0] = force_batch_blocks(dv, members); g[1] = dv.nb; g[2] = 1; break;
     default: break;
     }
 }

@@ -483,9 +483,9 @@ void launch_average(const Device &dv, const StepPtrs &sp, cudaStream_t s);
 // zero when it does not run), and one launch of k over `blocks` flattened
 // blocks of the members of bt (all of storage `precision`); for BK_BULK,
 // `variant` indexes the batched bulk shapes (batch_bulk_shape)
-void batch_grid_small(const Device &dv, int k, int g[3]);                     // kernels.cu
+void batch_grid_small(const Device &dv, int k, int members, int g[3]);                     // kernels.cu
 void launch_batch_small(int k, const Batch &bt, unsigned blocks, int precision, cudaStream_t s);
-void batch_grid_cells(const Device &dv, int k, int variant, int g[3]);        // stream_collide.cu
+void batch_grid_cells(const Device &dv, int k, int variant, int members, int g[3]);        // stream_collide.cu
 void launch_batch_cells(int k, int variant, const Batch &bt, unsigned blocks, int precision, bool walls,
                         cudaStream_t s);     // walls: some member has a non-periodic axis
 // batched bulk shape i of a precision: its cells per thread, or 0 past the list

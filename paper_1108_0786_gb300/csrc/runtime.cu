@@ -2003,9 +2003,9 @@ int ens_group_tables(lbm_ensemble_t *e, EnsGroup &g) {
         for (int j = 0; j < M; ++j) {
             int gd[3];
             if (k == lbm::BK_BOUNDARY || k == lbm::BK_BULK)
-                lbm::batch_grid_cells(dvs[j], k, variant, gd);
+                lbm::batch_grid_cells(dvs[j], k, variant, M, gd);
             else
-                lbm::batch_grid_small(dvs[j], k, gd);
+                lbm::batch_grid_small(dvs[j], k, M, gd);
             first[j] = (int)total;
             for (int i = 0; i < 3; ++i) grid[3 * j + i] = gd[i];
             total += (long long)gd[0] * gd[1] * gd[2];
@@ -2301,7 +2301,7 @@ int lbm_ensemble_step(lbm_ensemble_t *e, const int *steps) {
     // state the host wrote prepares here
     for (int i = 0; i < n; ++i) {
         lbm_t *h = e->members[i];
-        if (left[i] > 0 && h->need_prep && nb(h) > 0 && fluid(h) && !overlapped(h)) {
+        if (left[i] > 0 && h->need_prep && nb(h) > 0 && fluid(h)) {
             lbm::launch_prep(h->dv, step_ptrs(h, (int)(h->steps & 1)), h->stream);
             h->need_prep = false;
         }

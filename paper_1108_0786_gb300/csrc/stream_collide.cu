@@ -250,7 +250,7 @@ __device__ __forceinline__ void collide_f64(double (&f)[Q], const Device &dv) {
     const double r45[2] = {1.5 * r3[0], 1.5 * r3[1]};
     if (om1 == 0.0 && !forced) {
         // tau = 1: the update is the equilibrium itself, the same bits without 18
-        // of the FMAs (0 f + a = a; a non-finite f makes every moment so)  203 x 149
+        // of the FMAs (0 f + a = a; a non-finite f makes every moment so): 203 x 149
         // x 131 cells, 8 steps and the populations, 8.31 -> 7.17 ms
 #pragma unroll
         for (int p = 0; p < Q / 2; ++p) {
@@ -1130,15 +1130,24 @@ __device__ __forceinline__ void boundary_body(const Device &dv, const StepPtrs &
 // grid of the boundary kernel: `turns` cells a warp for the cells a body of
 // half-width E usually lists (within 1.5 cells of its surface: about 18 E^2 for
 // the bodies of the workloads), at most what the SMs hold at once; longer lists
-// take more turns.  A batched block pays its member lookup before its first cell
-// and runs beside other members' blocks (48 boxes, 32 steps: 23.4 ms with 4 cells a
-// warp, 24.2 ms with one).
+// take more turns
 int sm_count();
-constexpr int BOUNDARY_BATCH_TURNS = 4;
+long long listed_cells(const Device &dv) {
+    const long long E = (dv.remap_side - 1) / 2 - REMAP_MARGIN;
+    return (long long)dv.nb * 18 * E * E;
+}
 int boundary_blocks(const Device &dv, int turns) {
-    const long long E = (dv.remap_side - 1) / 2 - REMAP_MARGIN, per = BOUNDARY_WARPS * turns;
-    const long long blocks = ((long long)dv.nb * 18 * E * E + per - 1) / per;
+    const long long per = BOUNDARY_WARPS * turns, blocks = (listed_cells(dv) + per - 1) / per;
     return (int)std::min<long long>(std::max<long long>(blocks, 1), 4LL * sm_count());
+}
+// turns of a batched launch over `members` lattices like dv: a block pays its
+// member lookup once for all its cells, so past about one wave of warps (5 blocks
+// an SM) each warp takes more of them (48 boxes in two launches, a step: 684 us
+// with 4 turns, 8 force blocks a body and the preparation kernel; 664 us with 2
+// force blocks and without it; 653 us with 8 turns and one force block)
+int boundary_batch_turns(const Device &dv, int members) {
+    const long long wave = 5LL * BOUNDARY_WARPS * sm_count();
+    return (int)std::min<long long>(std::max<long long>(members * listed_cells(dv) / wave, 1), 16);
 }
 
 template <typename T>
@@ -1603,11 +1612,11 @@ int batch_bulk_shape(int precision, int i) {
     return b ? b->vec : 0;
 }
 
-void batch_grid_cells(const Device &dv, int k, int variant, int g[3]) {
+void batch_grid_cells(const Device &dv, int k, int variant, int members, int g[3]) {
     g[0] = g[1] = g[2] = 0;
     const Domain &d = dv.dom;
     if (k == BK_BOUNDARY && dv.nb > 0) {
-        g[0] = boundary_blocks(dv, BOUNDARY_BATCH_TURNS);
+        g[0] = boundary_blocks(dv, boundary_batch_turns(dv, members));
         g[1] = g[2] = 1;
     } else if (k == BK_BULK) {
         const BatchShape *b = batch_shape(dv.precision, variant);
