@@ -668,8 +668,20 @@ __device__ __forceinline__ void bulk_body(const Device &dv, const StepPtrs &sp, 
         if constexpr (raw16) collide_lean<std::is_same<T, __half>::value>(g, dv);
         else collide<T>(g, dv);
         const bool solid = fl[i] & F_SOLID;
+        if constexpr (WALLS) {
 #pragma unroll
-        for (int b = 0; b < Q; ++b) f[b][i] = solid ? (Cd)0 : g[b];
+            for (int b = 0; b < Q; ++b) f[b][i] = solid ? (Cd)0 : g[b];
+        } else {
+            // few warps have a solid cell: a branch instead of 19 selects a cell
+            // (FP32, 512 x 256 x 256 cells: 794 -> 760 us, 24 bytes of spills for
+            // 40; the WALLS instance, with more registers held, is 2 % slower so)
+#pragma unroll
+            for (int b = 0; b < Q; ++b) f[b][i] = g[b];
+            if (solid) {
+#pragma unroll
+                for (int b = 0; b < Q; ++b) f[b][i] = (Cd)0;
+            }
+        }
     }
     // overlapped steps: a tile near a body is the near kernel's
     const bool far = !sp.far_skip || sp.far_skip[((long long)z * d.ny + y) * ((d.nx + TILE_X - 1) / TILE_X) +
@@ -1405,9 +1417,9 @@ struct Variant {
 };
 
 // the compiled variants of the bulk kernel; the first entry of a precision
-// and width is its default (FP32, two cells: 4 blocks an SM take 794 us on
+// and width is its default (FP32, two cells: 4 blocks an SM took 794 us on
 // 512 x 256 x 256 cells, 106 us on 204 x 148 x 132 and 20.0 us on 128 x 64 x 64,
-// against 833, 112 and 20.5 us without the register cap)
+// against 833, 112 and 20.5 us without the register cap; 760 and 100 us since)
 const Variant kVariants[] = {
     {0, 1, 1, launch_shape<double, 1, 1>},
     {0, 2, 1, launch_shape<double, 2, 1>},
