@@ -47,6 +47,8 @@ struct lbm_s {
     cudaEvent_t rd_ev[READS] = {};
     int *rd_status = nullptr;
     long long rd_seq = 0;
+    unsigned char *stage = nullptr;     // page-locked staging of the synchronising reads (read_stage)
+    int reads = 0;                      // synchronising reads so far, up to STAGE_AFTER
     // the reads run on a stream of their own beside the following step; a
     // step that overwrites a body buffer with a read pending waits for it
     cudaStream_t rd_stream = nullptr;
@@ -630,13 +632,52 @@ int check_status(lbm_t *h) {
     return status_error(h, st);
 }
 
-int sync_and_check(lbm_t *h) {
+// Host staging of the synchronising reads, page-locked: the status word, then up
+// to 13 doubles a body.  Null for a handle's first reads: allocating it costs about
+// as much as ten reads gain, so a handle that is read a few times does without.
+constexpr size_t STAGE_HEAD = 64;
+constexpr int STAGE_AFTER = 10;
+
+unsigned char *read_stage(lbm_t *h) {
+    if (!h->stage && h->reads < STAGE_AFTER && ++h->reads == STAGE_AFTER) {
+        void *p = nullptr;
+        if (cudaHostAlloc(&p, STAGE_HEAD + sizeof(BodyState) * std::max(nb(h), 1), cudaHostAllocDefault) != cudaSuccess) {
+            cudaGetLastError();         // refused: the reads go on without
+            p = nullptr;
+        }
+        h->stage = static_cast<unsigned char *>(p);
+    }
+    return h->stage;
+}
+
+// Wait for all enqueued work, return any latched device error and, without one,
+// copy `bytes` (at most a BodyState a body) from device memory `src` to `out`.
+// With the staging buffer both copies are enqueued before the one wait: a blocking
+// copy each is a round trip of its own (48^3 control step with its read of the body
+// states: 56.8 -> 44.9 us).
+int sync_and_read(lbm_t *h, const void *src, size_t bytes, void *out) {
     if (!h->ready) return LBM_OK;
+    unsigned char *stage = read_stage(h);
+    if (stage) {
+        CK(cudaMemcpyAsync(stage, h->dv.status, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+        if (bytes) CK(cudaMemcpyAsync(stage + STAGE_HEAD, src, bytes, cudaMemcpyDeviceToHost, h->stream));
+    }
     CK(cudaStreamSynchronize(h->stream));
     if (h->rd_stream) CK(cudaStreamSynchronize(h->rd_stream));
     CK(cudaGetLastError());
-    return check_status(h);
+    if (!stage) {
+        const int rc = check_status(h);
+        if (rc == LBM_OK && bytes) CK(cudaMemcpy(out, src, bytes, cudaMemcpyDeviceToHost));
+        return rc;
+    }
+    int st = 0;
+    std::memcpy(&st, stage, sizeof st);
+    const int rc = status_error(h, st);
+    if (rc == LBM_OK && bytes) std::memcpy(out, stage + STAGE_HEAD, bytes);
+    return rc;
 }
+
+int sync_and_check(lbm_t *h) { return sync_and_read(h, nullptr, 0, nullptr); }
 
 void release_device(lbm_t *h) {
     if (h->ready) cudaStreamSynchronize(h->stream);
@@ -653,6 +694,8 @@ void release_device(lbm_t *h) {
             cudaEventDestroy(ev);
             ev = nullptr;
         }
+    if (h->stage) cudaFreeHost(h->stage);
+    h->stage = nullptr;
     if (h->rd_status) cudaFreeHost(h->rd_status);
     h->rd_status = nullptr;
     for (int p = 0; p < 2; ++p)
@@ -1045,10 +1088,7 @@ int lbm_get_bodies(lbm_t *h, double *out) {
         std::memcpy(out, h->init_state.data(), sizeof(BodyState) * nb(h));
         return LBM_OK;
     }
-    int rc = sync_and_check(h);
-    if (rc) return rc;
-    if (nb(h)) CK(cudaMemcpy(out, h->bodies[h->steps & 1], sizeof(BodyState) * nb(h), cudaMemcpyDeviceToHost));
-    return LBM_OK;
+    return sync_and_read(h, h->bodies[h->steps & 1], sizeof(BodyState) * nb(h), out);
 }
 
 int lbm_get_bodies_async(lbm_t *h, double *out, long long *ticket) {
@@ -1096,10 +1136,7 @@ int lbm_get_forces(lbm_t *h, double *out) {
         std::memset(out, 0, sizeof(double) * 6 * nb(h));
         return LBM_OK;
     }
-    int rc = sync_and_check(h);
-    if (rc) return rc;
-    if (nb(h)) CK(cudaMemcpy(out, h->dv.fh, sizeof(double) * 6 * nb(h), cudaMemcpyDeviceToHost));
-    return LBM_OK;
+    return sync_and_read(h, h->dv.fh, sizeof(double) * 6 * nb(h), out);
 }
 
 static size_t field_elems(const lbm_t *h, int what) {
