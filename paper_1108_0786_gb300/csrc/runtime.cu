@@ -417,8 +417,8 @@ int ensure_device(lbm_t *h) {
     dv.link_side = 2 * (emax + 1) + 1;
     dv.seg_cap = dv.link_side * dv.link_side * 18;
     dv.hist_cap = h->hist_cap;
-    dv.vec = h->tune_vec ? h->tune_vec : lbm::default_vector_width(dv);
     dv.minb = h->tune_minb;
+    dv.vec = h->tune_vec ? h->tune_vec : lbm::default_vector_width(dv);
     dv.expire_waits = h->expire_waits;
 
     // per-body reciprocals and term lists (drive terms and springs keep

@@ -330,6 +330,10 @@ __device__ __forceinline__ float vscale_add(float a, float c, float b) { return 
 __device__ __forceinline__ F2 vscale_add(F2 a, float c, F2 b) {
     return pack2(__fmaf_rn(lo2(a), c, lo2(b)), __fmaf_rn(hi2(a), c, hi2(b)));
 }
+__device__ __forceinline__ float vmul_apart(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ F2 vmul_apart(F2 a, F2 b) {
+    return pack2(__fmul_rn(lo2(a), lo2(b)), __fmul_rn(hi2(a), hi2(b)));
+}
 __device__ __forceinline__ float vplus(float a, float c) { return __fadd_rn(a, c); }
 __device__ __forceinline__ F2 vplus(F2 a, float c) { return pack2(__fadd_rn(lo2(a), c), __fadd_rn(hi2(a), c)); }
 __device__ __forceinline__ float vrcp(float a) { return __frcp_rn(a); }
@@ -344,24 +348,32 @@ __device__ __forceinline__ R vdot(int b, R x, R y, R z) {
     return (ez(b) ? ez(b) : ey(b)) > 0 ? vadd(first, second) : vsub(first, second);
 }
 
-// LBGK (+ Guo) for 16-bit storage in the form with the fewest instructions
-// (these kernels are bound by instruction issue before HBM), for one cell
+// LBGK (+ Guo) for 16-bit storage in forms with few instructions, for one cell
 // (R = float) or two (R = F2) with the same bits.  Opposite directions
-// (b, b + 1) are paired: the moments come from pair sums and differences, and
+// (b, b + 1) are paired: the moments come from pair sums and differences.
+// BF16 (its rounding is stochastic, so only the size of an error counts):
 //   f~_b = ((1 - omega) f_b + a) +- C e.u,
 //   a = omega w (drho - 1.5 rho u.u + 4.5 rho (e.u)^2),  C = 3 omega w rho
 //   (+ (1 - omega/2) w (9 (e.u)(e.g) - 3 u.g +- 3 e.g) with forcing).
-// SCALED: the populations are k delta (k = f16_scale, a power of two) on entry
-// and exit, so the scale enters only rho, u and the per-cell constants, never a
-// population.  Use: rest(f_0), pair(f_b, f_b+1) for the nine pairs in order,
-// solve(), then relax0 and relax for the populations.
+// FP16 (SCALED: the populations are k delta, k = f16_scale, a power of two, on
+// entry and exit) rounds to nearest, and in a slow flow, whose populations
+// are a few units in the last place, exact results often lie half way between
+// two FP16 values.  There the weight comes last, on a sum of few bits, so that
+// FP32 gives the half-way value itself and the rounding to even is unbiased:
+//   f~_b = (1 - omega) f_b + omega w (a +- c),  c = 3 rho e.u,
+//   a = drho - 1.5 rho u.u + 4.5 rho (e.u)^2.
+// With BF16's form FP16's velocity field was 1.4 to 2 times as far from the
+// FP64 path (capsule swarms of 160 x 128 x 128 cells after 500 to 2000 steps),
+// with c and its sum in one rounding 1.1 times.
+// Use: rest(f_0), pair(f_b, f_b+1) for the nine pairs in order, solve(), then
+// relax0 and relax for the populations.
 template <typename R, bool SCALED>
 struct Lean {
     R s, jx, jy, jz;        // sum of delta, momentum; after solve(): u in jx, jy, jz
     R base;                 // k (drho - 1.5 rho u.u)
     R kr;                   // k rho
     R ug3;                  // -3 k u.g (forcing)
-    R b, A, C, N;           // a = A (e.u)^2 + b, C and -C of the weight class at hand
+    R b, A, C, N;           // BF16: a = A (e.u)^2 + b, C and -C of the weight class at hand; FP16: A, C without weight
 
     __device__ __forceinline__ void rest(R f0) { s = f0; }
     __device__ __forceinline__ void pair(int p, R f1, R f2) {
@@ -373,7 +385,7 @@ struct Lean {
         if (ez(b)) jz = p == 2 ? d : (ez(b) > 0 ? vadd(jz, d) : vsub(jz, d));
     }
     __device__ __forceinline__ void solve(const Device &dv) {
-        const float k = SCALED ? dv.f16_scale : 1.0f, ik = SCALED ? dv.f16_inv_scale : 1.0f;
+        const float k = SCALED ? dv.f16_scale : 1.0f;
         const bool forced = dv.forced;
         if (forced) {
             const float kh = 0.5f * k;
@@ -381,6 +393,7 @@ struct Lean {
             jy = vplus(jy, kh * dv.g_f[1]);
             jz = vplus(jz, kh * dv.g_f[2]);
         }
+        const float ik = SCALED ? dv.f16_inv_scale : 1.0f;
         const R rho = vplus(SCALED ? vscale(s, ik) : s, 1.0f);
         R inv = vrcp(rho);
         if (SCALED) inv = vscale(inv, ik);
@@ -390,11 +403,14 @@ struct Lean {
         const R usq = vfma(jx, jx, vfma(jy, jy, vmul(jz, jz)));
         kr = SCALED ? vscale(rho, k) : rho;
         base = vfma(vscale(kr, -1.5f), usq, s);
+        if constexpr (SCALED) {
+            A = vscale(kr, 4.5f);
+            C = vscale(kr, 3.0f);
+        }
         if (forced)
-            ug3 = vscale_add(jx, -3.0f * k * dv.g_f[0],
-                             vscale_add(jy, -3.0f * k * dv.g_f[1], vscale(jz, -3.0f * k * dv.g_f[2])));
+            ug3 = vscale(vscale_add(jx, dv.g_f[0], vscale_add(jy, dv.g_f[1], vscale(jz, dv.g_f[2]))), -3.0f * k);
     }
-    // the factors of weight class wc (1: axes, 2: diagonals)
+    // BF16: the factors of weight class wc (1: axes, 2: diagonals)
     __device__ __forceinline__ void weights(int wc, const Device &dv) {
         const float ow = dv.ow_f[wc];
         b = vscale(base, ow);
@@ -403,28 +419,45 @@ struct Lean {
         C = vscale(kr, 3.0f * ow);
         N = vscale(kr, -3.0f * ow);
     }
+    // TAU1 (both): omega = 1, the old populations have the factor 0 and are not read
+    template <bool TAU1 = false>
     __device__ __forceinline__ R relax0(R f0, const Device &dv) const {
-        R r = vscale_add(f0, dv.om1_f, vscale(base, dv.ow_f[0]));
+        R r = vscale(base, dv.ow_f[0]);
         if (dv.forced) r = vscale_add(ug3, dv.gw_f[0], r);
-        return r;
+        return TAU1 ? r : vscale_add(f0, dv.om1_f, r);
     }
-    // pair p; the weights of its class are set before the class's first pair
+    // pair p, in order (the weights of its class are set before the class's first pair)
+    template <bool TAU1 = false>
     __device__ __forceinline__ void relax(int p, R &f1, R &f2, const Device &dv) {
-        if (p == 0) weights(1, dv);
-        if (p == 3) weights(2, dv);
-        const int i = 2 * p + 1;
-        const R eu = vdot(i, jx, jy, jz), om1 = splat<R>(dv.om1_f);
-        R a = vfma(A, vmul(eu, eu), b);
-        if (dv.forced) {
-            const float k = SCALED ? dv.f16_scale : 1.0f;
-            const float eg = edot(i, dv.g_f[0], dv.g_f[1], dv.g_f[2]), gw = dv.gw_f[p < 3 ? 1 : 2];
-            a = vscale_add(eu, 9.0f * k * gw * eg, a);
-            const float c = 3.0f * k * gw * eg;
-            f1 = vplus(vfma(C, eu, vfma(f1, om1, a)), c);
-            f2 = vplus(vfma(N, eu, vfma(f2, om1, a)), -c);
+        const int i = 2 * p + 1, wc = p < 3 ? 1 : 2;
+        if constexpr (!SCALED) {
+            if (p == 0) weights(1, dv);
+            if (p == 3) weights(2, dv);
+        }
+        const R eu = vdot(i, jx, jy, jz);
+        R a = vfma(A, vmul(eu, eu), SCALED ? base : b);
+        if constexpr (SCALED) {
+            // scalar products: the assembler fuses a packed product with the sum after it
+            const R c = vmul_apart(C, eu);
+            R r1 = vscale(vadd(a, c), dv.ow_f[wc]), r2 = vscale(vsub(a, c), dv.ow_f[wc]);
+            if (dv.forced) {
+                const float k = dv.f16_scale, eg = edot(i, dv.g_f[0], dv.g_f[1], dv.g_f[2]), gw = dv.gw_f[wc];
+                const R g = vscale_add(vscale(eu, 9.0f * k), eg, ug3);
+                r1 = vscale_add(vplus(g, 3.0f * k * eg), gw, r1);
+                r2 = vscale_add(vplus(g, -3.0f * k * eg), gw, r2);
+            }
+            f1 = TAU1 ? r1 : vscale_add(f1, dv.om1_f, r1);
+            f2 = TAU1 ? r2 : vscale_add(f2, dv.om1_f, r2);
         } else {
-            f1 = vfma(C, eu, vfma(f1, om1, a));
-            f2 = vfma(N, eu, vfma(f2, om1, a));
+            const R om1 = splat<R>(dv.om1_f);
+            const float eg = edot(i, dv.g_f[0], dv.g_f[1], dv.g_f[2]), gw = dv.gw_f[wc];
+            if (dv.forced) a = vscale_add(eu, 9.0f * gw * eg, a);
+            f1 = vfma(C, eu, TAU1 ? a : vfma(f1, om1, a));
+            f2 = vfma(N, eu, TAU1 ? a : vfma(f2, om1, a));
+            if (dv.forced) {
+                f1 = vplus(f1, 3.0f * gw * eg);
+                f2 = vplus(f2, -3.0f * gw * eg);
+            }
         }
     }
 };
@@ -783,6 +816,17 @@ __device__ __forceinline__ void collide_words(unsigned (&w)[Q][V / 2], const uin
         const Dither d0 = dither_for<T>(c0 + 2 * j, sp.tstep), d1 = dither_for<T>(c0 + 2 * j + 1, sp.tstep);
         // solid cells store 0
         const unsigned keep = (fl[2 * j] & F_SOLID ? 0u : 0xffffu) | (fl[2 * j + 1] & F_SOLID ? 0u : 0xffff0000u);
+        if (dv.om1_f == 0.0f) {             // tau = 1: nothing to widen again
+            w[0][j] = narrow<T>(c.template relax0<true>(c.base, dv), d0, d1, 0) & keep;
+#pragma unroll
+            for (int p = 0; p < Q / 2; ++p) {
+                F2 f1, f2;
+                c.template relax<true>(p, f1, f2, dv);
+                w[2 * p + 1][j] = narrow<T>(f1, d0, d1, 2 * p + 1) & keep;
+                w[2 * p + 2][j] = narrow<T>(f2, d0, d1, 2 * p + 2) & keep;
+            }
+            continue;
+        }
         w[0][j] = narrow<T>(c.relax0(widen<T>(w[0][j]), dv), d0, d1, 0) & keep;
 #pragma unroll
         for (int p = 0; p < Q / 2; ++p) {
@@ -837,12 +881,16 @@ __device__ __forceinline__ void store_words(const unsigned (&w)[Q][V / 2], const
 // shuffled from the neighbouring lane).  The two cells of a word collide
 // together in packed FP32 arithmetic (Lean<F2>); the words are widened once for
 // the moments and again for the relaxation, so that only one pair's populations
-// are held in FP32 at a time.  Bound by instruction issue and, at 24 warps an SM,
-// by the bytes in flight: 512 x 256 x 256 cells take 428 us in FP16 (6.0 TB/s)
-// and 482 us in BF16 against 449 and 542 us with a cell at a time in scalar
+// are held in FP32 at a time, and at tau = 1, where they do not enter the
+// relaxation, not again at all.  All loads, the row ends' single cells included,
+// stand before the first shuffle: with each row end's load behind its
+// direction's shuffle the loads of several directions waited for one another
+// (issue slots 44 % used, FP16 four cells a thread 520 us).  Bound by the
+// bytes in flight and, in BF16 (the rounding), by instruction issue: 512 x 256 x
+// 256 cells at tau = 1 take 396 us in FP16 (6.5 TB/s) and 448 us in BF16, 428 and
+// 487 us at tau = 0.8, against 449 and 542 us with a cell at a time in scalar
 // arithmetic.  (Copying the sources ahead into shared memory with cp.async, two
-// stages at 16 warps an SM, took 525 and 549 us: the issue-bound part needs the
-// warps.)
+// stages at 16 warps an SM, took 525 and 549 us.)
 template <typename T, int V, bool WALLS>
 __device__ __forceinline__ void bulk16_body(const Device &dv, const StepPtrs &sp, const Blk &bk) {
     static_assert(sizeof(T) == 2 && V % 2 == 0, "two 16-bit cells a word");
@@ -875,7 +923,8 @@ __device__ __forceinline__ void bulk16_body(const Device &dv, const StepPtrs &sp
                                  {(cy + ym) * pitch, (cy + y) * pitch, (cy + yp) * pitch},
                                  {(zp * d.ny + ym) * pitch, (zp * d.ny + y) * pitch, (zp * d.ny + yp) * pitch}};
     const unsigned xl = 2u * (x0 == 0 ? d.nx - 1 : x0 - 1), xr = 2u * (x0 + V == d.nx ? 0 : x0 + V);
-    unsigned w[Q][W];
+    unsigned w[Q][W], edge[Q];
+    const bool e0 = lane == 0 || x0 == 0, e1 = lane == 31 || x0 + V == d.nx;
 #pragma unroll
     for (int b = 0; b < Q; ++b) {
         const bool own = WALLS && wr.beyond(b);
@@ -885,32 +934,35 @@ __device__ __forceinline__ void bulk16_body(const Device &dv, const StepPtrs &sp
             plane = reinterpret_cast<const char *>(src + (long long)opp(b) * C);
             row = rows[1][1];
         }
-        unsigned R[W];
-        {
-            const RawV r = __ldg(reinterpret_cast<const RawV *>(plane + (row + 2u * x0)));
-            memcpy(&R, &r, sizeof(R));
+        const RawV r = __ldg(reinterpret_cast<const RawV *>(plane + (row + 2u * x0)));
+        memcpy(&w[b], &r, sizeof(r));
+        edge[b] = 0;
+        if (ex(b) > 0 && e0) {
+            if (WALLS && wr.x && x0 == 0) edge[b] = (unsigned)src[(long long)opp(b) * C + c0];
+            else edge[b] = (unsigned)__ldg(reinterpret_cast<const unsigned short *>(plane + (row + xl)));
         }
-        if (ex(b) == 0) {
+        if (ex(b) < 0 && e1) {
+            if (WALLS && wr.x && x0 + V == d.nx) edge[b] = (unsigned)src[(long long)opp(b) * C + c0 + V - 1];
+            else edge[b] = (unsigned)__ldg(reinterpret_cast<const unsigned short *>(plane + (row + xr)));
+        }
+    }
 #pragma unroll
-            for (int j = 0; j < W; ++j) w[b][j] = R[j];
-        } else if (ex(b) > 0) {          // pull from x - 1: the left neighbour's last half-word first
-            unsigned lw = __shfl_up_sync(0xffffffffu, R[W - 1], 1);
-            if (lane == 0 || x0 == 0) {
-                if (WALLS && wr.x && x0 == 0) lw = (unsigned)src[(long long)opp(b) * C + c0] << 16;
-                else lw = (unsigned)__ldg(reinterpret_cast<const unsigned short *>(plane + (row + xl))) << 16;
-            }
-            w[b][0] = own ? R[0] : __byte_perm(lw, R[0], 0x5432);
+    for (int b = 0; b < Q; ++b) {
+        const bool own = WALLS && wr.beyond(b);
+        if (ex(b) > 0) {                 // pull from x - 1: the left neighbour's last half-word first
+            unsigned lw = __shfl_up_sync(0xffffffffu, w[b][W - 1], 1);
+            if (e0) lw = edge[b] << 16;
+            unsigned o[W];
 #pragma unroll
-            for (int j = 1; j < W; ++j) w[b][j] = own ? R[j] : __byte_perm(R[j - 1], R[j], 0x5432);
-        } else {                          // pull from x + 1: the right neighbour's first half-word last
-            unsigned rw = __shfl_down_sync(0xffffffffu, R[0], 1);
-            if (lane == 31 || x0 + V == d.nx) {
-                if (WALLS && wr.x && x0 + V == d.nx) rw = (unsigned)src[(long long)opp(b) * C + c0 + V - 1];
-                else rw = (unsigned)__ldg(reinterpret_cast<const unsigned short *>(plane + (row + xr)));
-            }
+            for (int j = 0; j < W; ++j) o[j] = own ? w[b][j] : __byte_perm(j ? w[b][j - 1] : lw, w[b][j], 0x5432);
 #pragma unroll
-            for (int j = 0; j < W - 1; ++j) w[b][j] = own ? R[j] : __byte_perm(R[j], R[j + 1], 0x5432);
-            w[b][W - 1] = own ? R[W - 1] : __byte_perm(R[W - 1], rw, 0x5432);
+            for (int j = 0; j < W; ++j) w[b][j] = o[j];
+        } else if (ex(b) < 0) {          // pull from x + 1: the right neighbour's first half-word last
+            unsigned rw = __shfl_down_sync(0xffffffffu, w[b][0], 1);
+            if (e1) rw = edge[b];
+#pragma unroll
+            for (int j = 0; j < W; ++j)
+                w[b][j] = own ? w[b][j] : __byte_perm(w[b][j], j + 1 < W ? w[b][j + 1 < W ? j + 1 : j] : rw, 0x5432);
         }
     }
 
@@ -1109,11 +1161,20 @@ __device__ __forceinline__ void boundary_body(const Device &dv, const StepPtrs &
         const Cd usq = mad(ux, ux, mad(uy, uy, uz * uz));
         const Cd base = mad((Cd)(-1.5) * rho, usq, mo.s);
         const Cd eu = signed_by(bx, ux) + signed_by(by, uy) + signed_by(bz, uz);
-        const Cd deq = w * mad(rho, mad((Cd)4.5 * eu, eu, (Cd)3 * eu), base);
-        Cd gt = 0;
+        Cd eg = 0, ug = 0, gt = 0;
         if (dv.forced) {
-            const Cd eg = signed_by(bx, gx) + signed_by(by, gy) + signed_by(bz, gz);
-            const Cd ug = mad(ux, gx, mad(uy, gy, uz * gz));
+            eg = signed_by(bx, gx) + signed_by(by, gy) + signed_by(bz, gz);
+            ug = mad(ux, gx, mad(uy, gy, uz * gz));
+        }
+        if constexpr (sizeof(T) == 2) {
+            // the weight last, as the bulk kernel's FP16 form (Lean)
+            const int wc = b == 0 ? 0 : (b < 7 ? 1 : 2);
+            Cd r = dv.ow_f[wc] * (mad((Cd)4.5 * rho, eu * eu, base) + (Cd)3 * rho * eu);
+            if (dv.forced) r = mad(dv.gw_f[wc], mad((Cd)9 * eu, eg, (Cd)(-3) * ug) + (Cd)3 * eg, r);
+            f = mad(dv.om1_f, f, r);
+        }
+        const Cd deq = w * mad(rho, mad((Cd)4.5 * eu, eu, (Cd)3 * eu), base);
+        if (dv.forced) {
             gt = (f32 ? (Cd)dv.guo_f : (Cd)(1.0 - 0.5 * dv.omega)) * w * mad((Cd)9 * eu, eg, (Cd)3 * (eg - ug));
         }
         const Cd om = f32 ? (Cd)dv.omega_f : (Cd)dv.omega;
@@ -1124,7 +1185,7 @@ __device__ __forceinline__ void boundary_body(const Device &dv, const StepPtrs &
             f += inc;
             if (b == 0) f -= dm.s;
             else if (b < 7) f += (Cd)0.5 * (signed_by(bx, gx - dm.x) + signed_by(by, gy - dm.y) + signed_by(bz, gz - dm.z));
-        } else {
+        } else if constexpr (sizeof(T) == 8) {
             f = mad(om, deq - f, f) + gt;
         }
         if (act) {
@@ -1427,19 +1488,19 @@ const Variant kVariants[] = {
     {1, 2, 1, launch_shape<float, 2, 1>},
     {1, 1, 1, launch_shape<float, 1, 1>},
     {1, 4, 1, launch_shape<float, 4, 1>},
-    {2, 4, 1, launch_shape<__half, 4, 1>},
     {2, 4, 2, launch_shape<__half, 4, 2>},
+    {2, 4, 1, launch_shape<__half, 4, 1>},
     {2, 4, 3, launch_shape<__half, 4, 3>},
-    {2, 8, 1, launch_shape<__half, 8, 1>},
     {2, 8, 2, launch_shape<__half, 8, 2>},
+    {2, 8, 1, launch_shape<__half, 8, 1>},
     {2, 2, 1, launch_shape<__half, 2, 1>},
     {2, 2, 4, launch_shape<__half, 2, 4>},
     {2, 1, 1, launch_shape<__half, 1, 1>},
-    {3, 4, 1, launch_shape<__nv_bfloat16, 4, 1>},
     {3, 4, 2, launch_shape<__nv_bfloat16, 4, 2>},
+    {3, 4, 1, launch_shape<__nv_bfloat16, 4, 1>},
     {3, 4, 3, launch_shape<__nv_bfloat16, 4, 3>},
-    {3, 8, 1, launch_shape<__nv_bfloat16, 8, 1>},
     {3, 8, 2, launch_shape<__nv_bfloat16, 8, 2>},
+    {3, 8, 1, launch_shape<__nv_bfloat16, 8, 1>},
     {3, 2, 1, launch_shape<__nv_bfloat16, 2, 1>},
     {3, 2, 4, launch_shape<__nv_bfloat16, 2, 4>},
     {3, 1, 1, launch_shape<__nv_bfloat16, 1, 1>},
@@ -1500,8 +1561,15 @@ void prepare_bulk_variants() {
     done = true;
 }
 
+// 16-bit storage takes 8 cells a thread (2 blocks an SM, the most bytes in flight)
+// where that leaves five or more waves of blocks, else 4 (FP16 396 against
+// 429 us on 512 x 256 x 256 cells, 58.9 against 61.7 us on 256 x 128 x 128, level on
+// 160 x 128 x 128, 19.8 against 19.4 us on 128 x 96 x 96; BF16 448 against 476,
+// 68.3 against 68.5, 48.4 against 47.1 and 23.1 against 22.0 us; 3 blocks an SM
+// of 4 cells spill: FP16 494 us).
 int default_vector_width(const Device &dv) {
-    const int pref = dv.precision == 0 ? 1 : (dv.precision == 1 ? 2 : 4);
+    const bool wide = dv.precision >= 2 && dv.minb == 0 && dv.dom.C >= 5LL * 2 * sm_count() * BULK_THREADS * 8;
+    const int pref = dv.precision == 0 ? 1 : (dv.precision == 1 ? 2 : (wide ? 8 : 4));
     for (int v = pref; v > 1; v >>= 1)
         if (dv.dom.nx % v == 0) return v;
     return 1;
@@ -1519,17 +1587,7 @@ int list_variants(const Device &dv, int *vec, int *minb, int max) {
 }
 
 void launch_stream_collide(const Device &dv, const StepPtrs &sp, cudaStream_t s) {
-    int minb = dv.minb;
-    if (minb == 0 && dv.precision >= 2 && dv.vec == 4) {
-        // 16-bit storage, four cells a thread: with 3 blocks an SM the registers
-        // spill a little, which pays once two or more waves of blocks overlap
-        // (FP16 428 against 526 us on 512 x 256 x 256 cells, 62 against 72 us on
-        // 204 x 148 x 132; on 128 x 64 x 64, one wave, 15.9 against 13.8 us)
-        const Domain &d = dv.dom;
-        const long long per_plane = (long long)(d.nx / 4) * d.ny;
-        minb = (per_plane + BULK_THREADS - 1) / BULK_THREADS * d.nz >= 2LL * 3 * sm_count() ? 3 : 2;
-    }
-    const Variant *v = find_variant(dv.precision, dv.vec, minb);
+    const Variant *v = find_variant(dv.precision, dv.vec, dv.minb);
     if (!v) v = find_variant(dv.precision, 1, 0);
     v->fn(dv, sp, s);
 }
