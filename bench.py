@@ -556,8 +556,9 @@ def ensemble_run(precision="f32", reference_edge=48):
     dt = time.perf_counter() - t0
     updates = sum(sc.cells * n for sc, n in zip(scs, steps))
     final = [lat.bodies() for lat in lats]
-    # per step and storage type: 8 kernels in each of the two chains (halves of the members)
-    launches = 8 * 16 * 2 * len({lat.precision for lat in lats})
+    # per step and storage type: 6 kernels (remap, links, loads, boundary, bulk, force; a member
+    # with more than 8 bodies adds the preparation) in each of the two chains (halves of the members)
+    launches = 6 * 16 * 2 * len({lat.precision for lat in lats})
     ens.close()
     for lat in lats:
         lat.close()

@@ -145,6 +145,33 @@ def test_batched_ensemble_of_mixed_members_equals_them_stepped_alone(gpu):
         lat.close()
 
 
+@pytest.mark.parametrize("precision", ["f32", "f64", "f16"])
+def test_large_batches_equal_members_stepped_alone(gpu, precision):
+    """24 boxes of three bodies in two launches (one force block a body for
+    32/16-bit storage, several cells a boundary warp), one of twelve bodies
+    (listed remap candidates) among them: the bits of each stepped alone."""
+    crowd = wl.Scenario("four swimmers", 48, 48, 48, 0.8)
+    for y, z in ((11.8, 12.1), (12.3, 36.2), (35.9, 11.7), (36.4, 35.8)):
+        wl.add_swimmer(crowd, (23.7, y, z), (1.0, 0.0, 0.0, 0.0), (wl.SPHERE,) * 3,
+                       3.0, 0.0, 12.0, 0.02, 0.01, 2e-3, 64.0, density=2.0)
+    scs = members(24, 48) + [crowd]
+    n = 19
+    lats = [lbm.from_scenario(sc, precision=precision) for sc in scs]
+    ens = lbm.Ensemble(lats)
+    ens.step(n)
+    ens.sync()
+    got = [(lat.bodies(), lat.pop()) for lat in lats]
+    ens.close()
+    for lat in lats:
+        lat.close()
+    for sc, (b, p) in zip(scs, got):
+        lat = lbm.from_scenario(sc, precision=precision)
+        lat.step(n)
+        assert np.array_equal(lat.bodies(), b)
+        assert np.array_equal(lat.pop(), p)
+        lat.close()
+
+
 def test_ensemble_autotune_keeps_the_bits(gpu):
     scs = members(4)
     alone = []
