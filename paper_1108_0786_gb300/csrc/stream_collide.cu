@@ -618,7 +618,7 @@ __device__ __forceinline__ WallRows wall_rows(const Domain &d, int y, int z) {
 // the boundary kernel
 __device__ __forceinline__ bool bulk_cell(uint8_t f) { return (f & F_SOLID) || !(f & F_LISTED); }
 
-template <typename T, int V, bool WALLS, bool TILE = false>
+template <typename T, int V, bool WALLS, bool TILE = false, bool AHEAD = false>
 __device__ __forceinline__ void bulk_body(const Device &dv, const StepPtrs &sp, const Blk &bk) {
     using Cd = typename Codec<T>::C;
     const Domain d = dv.dom;
@@ -661,32 +661,53 @@ __device__ __forceinline__ void bulk_body(const Device &dv, const StepPtrs &sp, 
     const unsigned rows[3][3] = {{(zm * d.ny + ym) * nxu, (zm * d.ny + y) * nxu, (zm * d.ny + yp) * nxu},
                                  {(z * d.ny + ym) * nxu, (z * d.ny + y) * nxu, (z * d.ny + yp) * nxu},
                                  {(zp * d.ny + ym) * nxu, (zp * d.ny + y) * nxu, (zp * d.ny + yp) * nxu}};
+    // AHEAD: all loads before the first shuffle, the row ends' single cells
+    // included: with each row end's load behind its direction's shuffle the loads
+    // of several directions wait for one another (FP32, 512 x 256 x 256 cells: 762 us in
+    // the then best shape, 746 us ahead; 100 x 100 x 200 with walls 69.9 and
+    // 58.7 us).  Not where the registers are short or the loads do not bound:
+    // the batched kernels (48 boxes of edge 48 to 96, a step: 636 us, 655 us ahead) and
+    // FP64 (a pass of the ragged swarm 7153 against 7294 us).
+    const bool e0 = lane == 0 || x0 == 0, e1 = lane == 31 || x0 + V == d.nx;
+    auto row_of = [&](int b) -> const T * {
+        if (WALLS && wr.beyond(b)) return src + (long long)opp(b) * C + rows[1][1];
+        return src + (long long)b * C + rows[1 - ez(b)][1 - ey(b)];
+    };
+    auto left_end = [&](int b) -> T {            // pull from x - 1
+        if (WALLS && wr.x && x0 == 0) return src[(long long)opp(b) * C + c0];
+        return row_of(b)[x0 == 0 ? d.nx - 1 : x0 - 1];
+    };
+    auto right_end = [&](int b) -> T {           // pull from x + 1
+        if (WALLS && wr.x && x0 + V == d.nx) return src[(long long)opp(b) * C + c0 + V - 1];
+        return row_of(b)[x0 + V == d.nx ? 0 : x0 + V];
+    };
+    T raw[Q][V], end[Q];
+    if constexpr (AHEAD) {
+#pragma unroll
+        for (int b = 0; b < Q; ++b) {
+            load_vec<T, V>(row_of(b) + (unsigned)x0, raw[b]);
+            if (ex(b) > 0 && e0) end[b] = left_end(b);
+            if (ex(b) < 0 && e1) end[b] = right_end(b);
+        }
+    }
     Cd f[Q][V];
 #pragma unroll
     for (int b = 0; b < Q; ++b) {
         const bool own = WALLS && wr.beyond(b);
-        const T *row = src + (long long)b * C + rows[1 - ez(b)][1 - ey(b)];
-        if (own) row = src + (long long)opp(b) * C + rows[1][1];
-        T A[V];
-        load_vec<T, V>(row + (unsigned)x0, A);
+        T (&A)[V] = raw[b];
+        if constexpr (!AHEAD) load_vec<T, V>(row_of(b) + (unsigned)x0, A);
         if (ex(b) == 0) {
 #pragma unroll
             for (int i = 0; i < V; ++i) f[b][i] = ld(A[i]);
-        } else if (ex(b) > 0) {          // pull from x - 1
+        } else if (ex(b) > 0) {
             T left = shfl(A[V - 1], 1, true);
-            if (lane == 0 || x0 == 0) {
-                if (WALLS && wr.x && x0 == 0) left = src[(long long)opp(b) * C + c0];
-                else left = row[x0 == 0 ? d.nx - 1 : x0 - 1];
-            }
+            if (e0) left = AHEAD ? end[b] : left_end(b);
             f[b][0] = ld(own ? A[0] : left);
 #pragma unroll
             for (int i = 1; i < V; ++i) f[b][i] = ld(own ? A[i] : A[i - 1]);
-        } else {                          // pull from x + 1
+        } else {
             T right = shfl(A[0], 1, false);
-            if (lane == 31 || x0 + V == d.nx) {
-                if (WALLS && wr.x && x0 + V == d.nx) right = src[(long long)opp(b) * C + c0 + V - 1];
-                else right = row[x0 + V == d.nx ? 0 : x0 + V];
-            }
+            if (e1) right = AHEAD ? end[b] : right_end(b);
 #pragma unroll
             for (int i = 0; i < V - 1; ++i) f[b][i] = ld(own ? A[i] : A[i + 1]);
             f[b][V - 1] = ld(own ? A[V - 1] : right);
@@ -756,7 +777,7 @@ template <typename T, int V, int MINB, bool WALLS>
 __global__ void __launch_bounds__(BULK_THREADS, MINB == 1 ? 0 : MINB)
 bulk_kernel(const Device dv, const StepPtrs sp) {
     pdl_enter();
-    bulk_body<T, V, WALLS>(dv, sp, launch_blk());
+    bulk_body<T, V, WALLS, false, sizeof(T) != 8>(dv, sp, launch_blk());
 }
 
 // a batched bulk block takes BATCH_PZ consecutive z-planes of its member:
@@ -1478,14 +1499,15 @@ struct Variant {
 };
 
 // the compiled variants of the bulk kernel; the first entry of a precision
-// and width is its default (FP32, two cells: 4 blocks an SM took 794 us on
-// 512 x 256 x 256 cells, 106 us on 204 x 148 x 132 and 20.0 us on 128 x 64 x 64,
-// against 833, 112 and 20.5 us without the register cap; 760 and 100 us since)
+// and width is its default (FP32, two cells: without a register cap 746 us on
+// 512 x 256 x 256 cells, 96 us on 204 x 148 x 132, 59 us on 100 x 100 x 200 with
+// walls and 19.6 us on 128 x 64 x 64, against 830, 108, 66 and 20.3 us capped for
+// 4 blocks an SM)
 const Variant kVariants[] = {
     {0, 1, 1, launch_shape<double, 1, 1>},
     {0, 2, 1, launch_shape<double, 2, 1>},
-    {1, 2, 4, launch_shape<float, 2, 4>},
     {1, 2, 1, launch_shape<float, 2, 1>},
+    {1, 2, 4, launch_shape<float, 2, 4>},
     {1, 1, 1, launch_shape<float, 1, 1>},
     {1, 4, 1, launch_shape<float, 4, 1>},
     {2, 4, 2, launch_shape<__half, 4, 2>},
