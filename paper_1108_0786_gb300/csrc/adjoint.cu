@@ -330,7 +330,7 @@ __global__ void __launch_bounds__(ADJ_BOUNDARY_THREADS) adj_wall_kernel(const De
 // gridDim.x-th from blk (the full-rule cells are a shell, which consecutive cells
 // would leave to a few blocks: 27.8 against 13.3 us a launch on the 96 x 48 x 48
 // study) (cells whose flags are zero in epochs n and n+1 and that
-// were not uncovered at n: adj_bulk's; solid at n: zero adjoint; the
+// were not uncovered at n: adj_bulk_cells'; solid at n: zero adjoint; the
 // others the full rule, as adj_wall_kernel applies it) and lists the full-rule cells
 // in cube order.  Each warp then takes the listed cells w, w + 8, ... with
 // lane b the direction b: the pull, wall and link terms of the 18
@@ -415,7 +415,7 @@ __global__ void __launch_bounds__(32 * ADJ_CUBE_WARPS) adj_cube_kernel(const Dev
             const long long c = ((long long)z * d.ny + y) * d.nx + x;
             const uint8_t fcur = ap.flags_cur[c], fnext = ap.flags_next[c];
             if (!(fnext & F_FULL_RULE) && !(fcur & F_SOLID_PREV)) {
-                // a bulk cell: adj_bulk's
+                // a bulk cell: adj_bulk_cells'
             } else if (fcur & F_SOLID) {            // obstacle at n: no adjoint
 #pragma unroll
                 for (int b = 0; b < Q; ++b) aout[(long long)b * C + c] = (A)0;

@@ -1,8 +1,9 @@
 // kernels.cu -- the per-body kernels of one coupled step and the field
 // export / import kernels:
 //   prep       per-body geometry records (remade only for states set from
-//              outside), remap candidate lists for the batched remap; a
-//              single lattice runs it only after the host wrote a state
+//              outside) and, for more than REMAP_STAGED bodies, the batched
+//              remap's candidate lists; steps of a single lattice and batched
+//              steps of few bodies run it only after the host wrote a state
 //   remap      map the bodies onto the lattice (Sec. 2.3), epoch flags, the
 //              boundary kernel's cell list
 //   links      per-body list of fluid->solid links (ballot + block scan)
@@ -12,7 +13,7 @@
 //              fixed-order reduction for FP64 storage, exact integer and
 //              fixed-point sums for 32/16-bit storage (deterministic both);
 //              the last block of each body runs its rigid-body time step
-//              (Algorithm 1) in FP64 on one warp
+//              (Algorithm 1) in FP64 on two warps (translation, rotation)
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
