@@ -127,6 +127,10 @@ __device__ inline void geom_place(const Domain &d, const BodyProps &p, int a, do
         if (elo < 0) elo += n;
         if (ewidth > n) ewidth = n;
     }
+    // a body's cube holds its grown box, also where X + reach rounds up to a cell
+    int ahead = elo - o;
+    if (per && ahead < 0) ahead += n;
+    ewidth = min(ewidth, 2 * half + 1 - ahead);
     g.box[a] = lo;
     g.box[3 + a] = width;
     g.ebox[a] = elo;
@@ -307,12 +311,14 @@ __device__ inline int wrap_up(int v, int n) { return v < n ? v : (v - n < n ? v 
 // overlapping cubes write identical values.  A cell tests only body b's
 // candidates, in body order (integer boxes, the FP32 screen, and the FP64
 // inside test only within the screen's margin).  Fluid cells flagged F_NEAR
-// F_SOLID_PREV or F_LINK are appended to the boundary kernel's list.
+// F_SOLID_PREV or F_LINK are appended to the boundary kernel's list, each once:
+// by the block row of the lowest-numbered body whose grown box holds the cell
+// (that body's cube covers it, and every cube that does has the body among its
+// candidates), so the list never exceeds C.
 constexpr int REMAP_THREADS = 256;
 constexpr int REMAP_R = 2;
 constexpr int REMAP_CELLS = REMAP_THREADS * REMAP_R;    // cube cells a block covers
 constexpr int REMAP_STAGED = 8;
-constexpr int REMAP_LIST_BUF = REMAP_CELLS;             // a block lists at most all of its cells
 
 // blocks a body of remap-cube side `side` takes
 inline int remap_blocks(int side) {
@@ -344,7 +350,7 @@ __device__ __forceinline__ void remap_body(const Device &dv, const StepPtrs &sp,
     }
     // this block's share of the boundary kernel's list, gathered in shared
     // memory and appended with one atomic at the end
-    __shared__ uint32_t lbuf[REMAP_LIST_BUF];
+    __shared__ uint32_t lbuf[REMAP_CELLS];
     __shared__ int lcount, lbase;
     const int org[3] = {geo[b].origin[0], geo[b].origin[1], geo[b].origin[2]};
     const int tid = threadIdx.x;
@@ -395,7 +401,7 @@ __device__ __forceinline__ void remap_body(const Device &dv, const StepPtrs &sp,
     // every lane runs each of its cells, so the ballots below see whole warps
         {
             int xr[REMAP_R], yr[REMAP_R], zr[REMAP_R], idr[REMAP_R];
-            bool linkr[REMAP_R];
+            bool linkr[REMAP_R], minr[REMAP_R];
             long long cr[REMAP_R];
             bool liver[REMAP_R];
 #pragma unroll
@@ -411,6 +417,7 @@ __device__ __forceinline__ void remap_body(const Device &dv, const StepPtrs &sp,
                 const int p3[3] = {x, y, z};
                 int id = NO_BODY;
                 bool reached = false;           // within STATIC_REACH cells of some body's box
+                bool mine = false;              // and of no lower-numbered body's than b: this block lists it
                 bool link = false;
                 for (int i = 0; i < ncand && live; ++i) {
                     const int kb = cid[i];
@@ -422,6 +429,7 @@ __device__ __forceinline__ void remap_body(const Device &dv, const StepPtrs &sp,
                         in = o >= 0 && o < g->ebox[3 + a];
                     }
                     if (!in) continue;
+                    if (!reached) mine = kb == b;
                     reached = true;
                     // the squared distance to the centre or axis in FP32: cells
                     // that may hold links, and the inside screen (cells within
@@ -443,6 +451,7 @@ __device__ __forceinline__ void remap_body(const Device &dv, const StepPtrs &sp,
                 zr[r] = z;
                 idr[r] = id;
                 linkr[r] = link;
+                minr[r] = mine;
                 cr[r] = ((long long)z * d.ny + y) * d.nx + x;
                 liver[r] = live && reached;
             }
@@ -498,31 +507,21 @@ __device__ __forceinline__ void remap_body(const Device &dv, const StepPtrs &sp,
                     sp.bid_cur[c] = (uint8_t)id;
                 }
                 // the boundary kernel's cells: a shared-memory atomic per warp
-                // (past the buffer, a global one)
-                const bool mine = live && !init_mode && !(flags & F_SOLID) && (flags & F_LISTED);
+                const bool mine = live && minr[r] && !init_mode && !(flags & F_SOLID) && (flags & F_LISTED);
                 const unsigned mb = __ballot_sync(0xffffffffu, mine);
                 if (mb) {
                     const int leader = __ffs(mb) - 1;
                     int base = 0;
                     if (lane == leader) base = atomicAdd(&lcount, __popc(mb));
                     base = __shfl_sync(0xffffffffu, base, leader);
-                    const int pos = base + __popc(mb & ((1u << lane) - 1u));
-                    if (mine) {
-                        if (pos < REMAP_LIST_BUF) {
-                            lbuf[pos] = (uint32_t)c;
-                        } else {
-                            const int g = atomicAdd(dv.bcount, 1);
-                            if (g < dv.blist_cap) dv.blist[g] = (uint32_t)c;
-                            else atomicOr(dv.status, ST_LINKS);
-                        }
-                    }
+                    if (mine) lbuf[base + __popc(mb & ((1u << lane) - 1u))] = (uint32_t)c;
                 }
             }
         }
     __syncthreads();
-    if (tid == 0) lbase = lcount ? atomicAdd(dv.bcount, min(lcount, REMAP_LIST_BUF)) : 0;
+    if (tid == 0) lbase = lcount ? atomicAdd(dv.bcount, lcount) : 0;
     __syncthreads();
-    const int nl = min(lcount, REMAP_LIST_BUF);
+    const int nl = lcount;
     for (int i = tid; i < nl; i += REMAP_THREADS) {
         if (lbase + i < dv.blist_cap) dv.blist[lbase + i] = lbuf[i];
         else atomicOr(dv.status, ST_LINKS);

@@ -256,8 +256,8 @@ struct Device {
     long long blist_cap;
     uint8_t *cand;          // [nb][nb]: body b's remap candidates in body order (BodyGeom::ncand of them)
     float *rho_near;        // [C] 32/16-bit storage: rho - 1 of each cell the boundary kernel collided this step
-    uint32_t *blist;        // cells the remap found fluid with F_NEAR or F_SOLID_PREV (the boundary kernel's)
-    int *bcount;            // entries in blist (a cell in two bodies' cubes may appear twice)
+    uint32_t *blist;        // cells the remap found fluid with a flag of F_LISTED (the boundary kernel's), each once
+    int *bcount;            // entries in blist
     double *drive_f;        // [nd][3] drive forces of the current step (integrator scratch)
     double *spring_f;       // [ns][3] spring forces on body i of each spring (integrator scratch)
     unsigned *blocks_done;  // bodies whose rigid-body step finished in the current step

@@ -465,12 +465,10 @@ int ensure_device(lbm_t *h) {
     if ((rc = alloc_into(h, &dv.geom, sizeof(lbm::BodyGeom) * 2 * std::max(B, 1)))) return rc;
     if ((rc = alloc_into(h, &dv.gstamp, sizeof(BodyState) * 2 * std::max(B, 1)))) return rc;
     {
-        // every cube cell is listed at most once per body cube, and a cell
-        // lies in few cubes: the smaller of the two bounds below (the
-        // remap checks the capacity and reports an overflow)
+        // every listed cell lies in a body's cube and is listed once (the
+        // remap checks the capacity all the same)
         const long long rs = dv.remap_side;
-        const long long cubes = (long long)B * rs * rs * rs, two_c = 2 * C + 1024;
-        const size_t cap = B > 0 && fluid(h) ? (size_t)std::min(cubes, two_c) : 1;
+        const size_t cap = B > 0 && fluid(h) ? (size_t)std::min((long long)B * rs * rs * rs, C) : 1;
         dv.blist_cap = h->list_cap_limit > 0 ? std::min((long long)cap, h->list_cap_limit) : (long long)cap;
         if ((rc = alloc_into(h, &dv.blist, sizeof(uint32_t) * cap))) return rc;
         if ((rc = alloc_into(h, &dv.cand, (size_t)std::max(B, 1) * std::max(B, 1)))) return rc;

@@ -1088,8 +1088,7 @@ template <typename R> __device__ __forceinline__ R lane_sum(R v) {
 // and the cell's sums by shuffles.  Latency-bound (some hundred cells a body): a
 // thread a cell walked ~250 dependent operations, in FP64 at 64 issue cycles
 // each.  (32^3 swimmer in FP64, a step: 93 -> 50 us, the kernel 70 us of it
-// before; 48^3 in FP32 with the body read: 69 -> 62 us a step.)  A cell listed twice (it lies in two bodies' cubes) is
-// computed twice with the same result.
+// before; 48^3 in FP32 with the body read: 69 -> 62 us a step.)
 constexpr int BOUNDARY_WARPS = 8;
 
 template <typename T>
