@@ -1571,8 +1571,11 @@ int near_tile_cap(const Device &dv, int emax) {
 }
 
 // Force blocks a body in a batched launch over `members` lattices like dv: with
-// many bodies a block's member lookup and reductions cost more than its second
-// round of links (48 boxes of three bodies, two launches: boundary_batch_turns).
+// many bodies a block's member lookup and reductions cost more than its further
+// rounds of links, also for large bodies (FP32, a step with this rule and with 8
+// blocks a body: 48 boxes of three spheres of radius 3 193 and 213 us, 8 boxes of
+// 27 of radius 5 192 and 211, 24 boxes of three of radius 10 648 and 655, 12 of
+// three of radius 12 506 and 508, 70 boxes of one of radius 12 394 and 401 us).
 // FP64 keeps its split, which the sums' order depends on.
 static int force_batch_blocks(const Device &dv, int members) {
     const int bodies = members * dv.nb;

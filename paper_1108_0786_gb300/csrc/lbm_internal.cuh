@@ -254,6 +254,7 @@ struct Device {
     BodyGeom *geom;         // [2][nb]: slot p holds the geometry of the state in body buffer p (parity)
     BodyState *gstamp;      // [2][nb]: the state each slot was made from (prep_kernel remakes on mismatch)
     long long blist_cap;
+    long long shell;        // cells within LINK_REACH of the bodies' surfaces, about the boundary list's length
     uint8_t *cand;          // [nb][nb]: body b's remap candidates in body order (BodyGeom::ncand of them)
     float *rho_near;        // [C] 32/16-bit storage: rho - 1 of each cell the boundary kernel collided this step
     uint32_t *blist;        // cells the remap found fluid with a flag of F_LISTED (the boundary kernel's), each once
@@ -485,9 +486,12 @@ void launch_average(const Device &dv, const StepPtrs &sp, cudaStream_t s);
 // `variant` indexes the batched bulk shapes (batch_bulk_shape)
 void batch_grid_small(const Device &dv, int k, int members, int g[3]);                     // kernels.cu
 void launch_batch_small(int k, const Batch &bt, unsigned blocks, int precision, cudaStream_t s);
-void batch_grid_cells(const Device &dv, int k, int variant, int members, int g[3]);        // stream_collide.cu
-void launch_batch_cells(int k, int variant, const Batch &bt, unsigned blocks, int precision, bool walls,
-                        cudaStream_t s);     // walls: some member has a non-periodic axis
+void batch_grid_cells(const Device &dv, int k, int variant, bool by_cell, int g[3]);      // stream_collide.cu
+// walls: some member has a non-periodic axis; by_cell: boundary_by_cell of the members' lists together
+void launch_batch_cells(int k, int variant, const Batch &bt, unsigned blocks, int precision, bool walls, bool by_cell,
+                        cudaStream_t s);
+// whether the boundary kernel takes a list of about `shell` cells a thread a cell (the same bits)
+bool boundary_by_cell(int precision, long long shell);
 // batched bulk shape i of a precision: its cells per thread, or 0 past the list
 int batch_bulk_shape(int precision, int i);
 int adjoint_part_stride(const Device &dv);

@@ -414,6 +414,12 @@ int ensure_device(lbm_t *h) {
     dv.f16_scale = h->precision == LBM_PREC_F16 ? 1024.0f : 1.0f;
     dv.f16_inv_scale = 1.0f / dv.f16_scale;
     dv.remap_side = 2 * (emax + lbm::REMAP_MARGIN) + 1;
+    double shell = 0.0;
+    for (const auto &p : h->props) {
+        const double R = p.r + lbm::LINK_REACH;
+        shell += 4.0 / 3.0 * M_PI * (R * R * R - p.r * p.r * p.r) + M_PI * (R * R - p.r * p.r) * p.l;
+    }
+    dv.shell = (long long)std::min(shell, (double)C);
     dv.link_side = 2 * (emax + 1) + 1;
     dv.seg_cap = dv.link_side * dv.link_side * 18;
     dv.hist_cap = h->hist_cap;
@@ -1916,6 +1922,7 @@ int lbm_adjoint_backward(lbm_t *h, const double *seed, double *grad_state, doubl
 struct EnsGroup {
     int precision = 1;
     bool walls = false;                     // some member has a non-periodic axis
+    bool by_cell = false;                   // the boundary kernel a thread a cell (boundary_by_cell)
     int lane = 0;                           // batched mode: the chain of launches the group is in
     std::vector<int> members;               // ensemble indices
     void *mem = nullptr;                    // the tables, one allocation (first member's allocator)
@@ -2026,6 +2033,9 @@ int ens_group_tables(lbm_ensemble_t *e, EnsGroup &g) {
         sps[j].row_recip = sps[M + j].row_recip = lbm::row_recip(h->nx / lbm::batch_bulk_shape(g.precision, variant));
     }
     if (M > 65535) return ens_fail(e, LBM_E_ARG, "more than 65535 members of one precision");
+    long long shell = 0;
+    for (const lbm::Device &dv : dvs) shell += dv.shell;
+    g.by_cell = lbm::boundary_by_cell(g.precision, shell);
     std::vector<int> tab;                   // per kernel: first[M + 1], grid[3 M]
     std::vector<size_t> off(lbm::BK_COUNT);
     std::vector<unsigned short> owner;      // per kernel, per flattened block: its member
@@ -2038,7 +2048,7 @@ int ens_group_tables(lbm_ensemble_t *e, EnsGroup &g) {
         for (int j = 0; j < M; ++j) {
             int gd[3];
             if (k == lbm::BK_BOUNDARY || k == lbm::BK_BULK)
-                lbm::batch_grid_cells(dvs[j], k, variant, M, gd);
+                lbm::batch_grid_cells(dvs[j], k, variant, g.by_cell, gd);
             else
                 lbm::batch_grid_small(dvs[j], k, M, gd);
             first[j] = (int)total;
@@ -2100,7 +2110,7 @@ void ens_enqueue_batched(lbm_ensemble_t *e, std::vector<EnsGroup> &groups, int l
             if (g.lane != lane) continue;
             lbm::Batch b = g.bt[k];
             b.parity = p;
-            lbm::launch_batch_cells(k, e->variant[g.precision], b, g.blocks[k], g.precision, g.walls, st);
+            lbm::launch_batch_cells(k, e->variant[g.precision], b, g.blocks[k], g.precision, g.walls, g.by_cell, st);
         }
     };
     cudaEventRecord(fork, main);
@@ -2436,10 +2446,10 @@ int lbm_ensemble_autotune(lbm_ensemble_t *e, int trials, int *cells_per_thread) 
             // the populations of every member's next step, which that step rewrites in full
             lbm::Batch b = g.bt[lbm::BK_BULK];
             b.parity = p;
-            lbm::launch_batch_cells(lbm::BK_BULK, v, b, g.blocks[lbm::BK_BULK], prec, g.walls, e->stream);
+            lbm::launch_batch_cells(lbm::BK_BULK, v, b, g.blocks[lbm::BK_BULK], prec, g.walls, g.by_cell, e->stream);
             cudaEventRecord(e0, e->stream);
             for (int t = 0; t < trials; ++t)
-                lbm::launch_batch_cells(lbm::BK_BULK, v, b, g.blocks[lbm::BK_BULK], prec, g.walls, e->stream);
+                lbm::launch_batch_cells(lbm::BK_BULK, v, b, g.blocks[lbm::BK_BULK], prec, g.walls, g.by_cell, e->stream);
             cudaEventRecord(e1, e->stream);
             cudaError_t err = cudaEventSynchronize(e1);
             float ms = 0.0f;

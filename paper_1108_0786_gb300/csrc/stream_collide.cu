@@ -1082,6 +1082,47 @@ template <typename R> __device__ __forceinline__ R lane_sum(R v) {
     return v;
 }
 
+// LBGK (+ Guo) of a listed cell from the moments of its populations, in the forms
+// of the bulk kernels but for the order of the sums; boundary_warp and
+// boundary_cell share it, so that a cell gets the same value from either
+template <typename Cd> struct Listed { Cd gx, gy, gz, rho, ux, uy, uz, base, ug; };
+template <typename Cd>
+__device__ __forceinline__ Listed<Cd> listed_cell(const Device &dv, const Moments<Cd> &mo) {
+    const bool f32 = sizeof(Cd) == 4;
+    Listed<Cd> c;
+    c.gx = f32 ? (Cd)dv.g_f[0] : (Cd)dv.g[0];
+    c.gy = f32 ? (Cd)dv.g_f[1] : (Cd)dv.g[1];
+    c.gz = f32 ? (Cd)dv.g_f[2] : (Cd)dv.g[2];
+    c.rho = (Cd)1 + mo.s;
+    const Cd inv = (Cd)1 / c.rho;
+    c.ux = mad((Cd)0.5, c.gx, mo.x) * inv;
+    c.uy = mad((Cd)0.5, c.gy, mo.y) * inv;
+    c.uz = mad((Cd)0.5, c.gz, mo.z) * inv;
+    const Cd usq = mad(c.ux, c.ux, mad(c.uy, c.uy, c.uz * c.uz));
+    c.base = mad((Cd)(-1.5) * c.rho, usq, mo.s);
+    c.ug = dv.forced ? mad(c.ux, c.gx, mad(c.uy, c.gy, c.uz * c.gz)) : (Cd)0;
+    return c;
+}
+// population f of weight w (class wc) relaxed, FP32: its increment
+template <typename T, typename Cd>
+__device__ __forceinline__ Cd listed_relax(const Device &dv, const Listed<Cd> &c, Cd f, Cd w, int wc, Cd eu, Cd eg) {
+    if constexpr (sizeof(T) == 2) {
+        // the weight last, as the bulk kernel's FP16 form (Lean)
+        Cd r = dv.ow_f[wc] * (mad((Cd)4.5 * c.rho, eu * eu, c.base) + (Cd)3 * c.rho * eu);
+        if (dv.forced) r = mad(dv.gw_f[wc], mad((Cd)9 * eu, eg, (Cd)(-3) * c.ug) + (Cd)3 * eg, r);
+        return mad(dv.om1_f, f, r);
+    } else {
+        const bool f32 = sizeof(Cd) == 4;
+        const Cd deq = w * mad(c.rho, mad((Cd)4.5 * eu, eu, (Cd)3 * eu), c.base);
+        Cd gt = 0;
+        if (dv.forced)
+            gt = (f32 ? (Cd)dv.guo_f : (Cd)(1.0 - 0.5 * dv.omega)) * w * mad((Cd)9 * eu, eg, (Cd)3 * (eg - c.ug));
+        const Cd om = f32 ? (Cd)dv.omega_f : (Cd)dv.omega;
+        if constexpr (std::is_same<T, float>::value) return mad(om, deq - f, gt);
+        else return dv.forced ? mad(om, deq - f, f) + gt : mad(om, deq - f, f);
+    }
+}
+
 // The cells the remap listed (fluid with a flag of F_LISTED): refill,
 // bounce-back at walls and moving obstacles, then LBGK, a warp a cell with lane b
 // the direction b: the 19 pulls, wall velocities and relaxations run side by side
@@ -1091,156 +1132,280 @@ template <typename R> __device__ __forceinline__ R lane_sum(R v) {
 // before; 48^3 in FP32 with the body read: 69 -> 62 us a step.)
 constexpr int BOUNDARY_WARPS = 8;
 
+// a lane's direction
+struct LaneDir {
+    bool act;                       // lanes past the last direction hold none
+    int b, x, y, z, ob;             // direction, its components, its reverse
+    LaneFactors sg;
+};
+__device__ __forceinline__ LaneDir lane_dir(int lane) {
+    LaneDir l;
+    l.act = lane < Q;
+    l.b = l.act ? lane : 0;
+    l.x = lane_component(0, l.b);
+    l.y = lane_component(1, l.b);
+    l.z = lane_component(2, l.b);
+    l.ob = l.b == 0 ? 0 : ((l.b & 1) ? l.b + 1 : l.b - 1);
+    l.sg = lane_factors(lane);
+    return l;
+}
+
+// listed cell cl by one warp
 template <typename T>
-__device__ __forceinline__ void boundary_body(const Device &dv, const StepPtrs &sp, const Blk &bk) {
+__device__ __forceinline__ void boundary_warp(const Device &dv, const StepPtrs &sp, unsigned cl, int lane, const LaneDir &ld) {
     using Cd = typename Codec<T>::C;
     constexpr unsigned FULL = 0xffffffffu;
     const Domain &d = dv.dom;
-    const int lane = threadIdx.x & 31;
-    int l = bk.x * BOUNDARY_WARPS + (threadIdx.x >> 5);
-    // the count may pass the capacity after an overflow (reported as an error): never read past it
-    const int listed = (int)min((long long)*dv.bcount, dv.blist_cap);
-    if (l >= listed) return;
-    const bool act = lane < Q;
-    const int b = act ? lane : 0;
-    const int bx = lane_component(0, b), by = lane_component(1, b), bz = lane_component(2, b);
-    const int ob = b == 0 ? 0 : ((b & 1) ? b + 1 : b - 1);
+    const bool act = ld.act;
+    const int b = ld.b, bx = ld.x, by = ld.y, bz = ld.z;
     const Cd w = b == 0 ? (Cd)wgt(0) : (b < 7 ? (Cd)wgt(1) : (Cd)wgt(7));
-    const LaneFactors sg = lane_factors(lane);
     const long long C = d.C;
     const T *__restrict__ src = static_cast<const T *>(sp.src);
     T *__restrict__ dst = static_cast<T *>(sp.dst);
     const float s = dv.f16_inv_scale;
-    const bool f32 = sizeof(Cd) == 4;
-    const Cd gx = f32 ? (Cd)dv.g_f[0] : (Cd)dv.g[0], gy = f32 ? (Cd)dv.g_f[1] : (Cd)dv.g[1],
-             gz = f32 ? (Cd)dv.g_f[2] : (Cd)dv.g[2];
-    for (; l < listed; l += bk.gx * BOUNDARY_WARPS) {
-        const unsigned cl = dv.blist[l];          // C < 2^31: 32-bit division
-        const unsigned nxu = (unsigned)d.nx, nyu = (unsigned)d.ny;
-        const unsigned row = cl / nxu, zu = row / nyu;
-        const int x = (int)(cl - row * nxu), y = (int)(row - zu * nyu), z = (int)zu;
-        const uint8_t fc = sp.flags_cur[cl];
-        Cd f = 0;
-        if (fc & F_SOLID_PREV) {
-            // uncovered cell: f = f_eq(rho_avg, u_w(x)) with the state of step n;
-            // rho_avg over the D3Q19 neighbours fluid in both epochs (1 if none),
-            // as deviations (small numbers: no 1 + drho is rounded), lane a the
-            // neighbour x + e_a
-            const int nx_ = x + bx, ny_ = y + by, nz_ = z + bz;
-            const bool in = act && b > 0 &&
-                            !((!d.px && (nx_ < 0 || nx_ >= d.nx)) || (!d.py && (ny_ < 0 || ny_ >= d.ny)) ||
-                              (!d.pz && (nz_ < 0 || nz_ >= d.nz)));
-            const long long nc = ((long long)wrap_axis(nz_, d.nz) * d.ny + wrap_axis(ny_, d.ny)) * d.nx +
-                                 wrap_axis(nx_, d.nx);
-            Cd drho = 0;
+    const unsigned nxu = (unsigned)d.nx, nyu = (unsigned)d.ny;      // C < 2^31: 32-bit division
+    const unsigned row = cl / nxu, zu = row / nyu;
+    const int x = (int)(cl - row * nxu), y = (int)(row - zu * nyu), z = (int)zu;
+    const uint8_t fc = sp.flags_cur[cl];
+    Cd f = 0;
+    if (fc & F_SOLID_PREV) {
+        // uncovered cell: f = f_eq(rho_avg, u_w(x)) with the state of step n;
+        // rho_avg over the D3Q19 neighbours fluid in both epochs (1 if none),
+        // as deviations (small numbers: no 1 + drho is rounded), lane a the
+        // neighbour x + e_a
+        const int nx_ = x + bx, ny_ = y + by, nz_ = z + bz;
+        const bool in = act && b > 0 &&
+                        !((!d.px && (nx_ < 0 || nx_ >= d.nx)) || (!d.py && (ny_ < 0 || ny_ >= d.ny)) ||
+                          (!d.pz && (nz_ < 0 || nz_ >= d.nz)));
+        const long long nc = ((long long)wrap_axis(nz_, d.nz) * d.ny + wrap_axis(ny_, d.ny)) * d.nx +
+                             wrap_axis(nx_, d.nx);
+        Cd drho = 0;
 #pragma unroll
-            for (int q = 0; q < Q; ++q) drho += Codec<T>::ld(src[q * C + nc], s);
-            const bool ok = in && !(sp.flags_cur[nc] & (F_SOLID | F_SOLID_PREV));
-            const int cnt = __popc(__ballot_sync(FULL, ok));
-            const Cd sum = lane_sum(ok ? drho : (Cd)0);
-            drho = cnt ? sum / (Cd)cnt : (Cd)0;
-            const Cd rho = (Cd)1 + drho;
-            const int k = sp.bid_prev[cl];
+        for (int q = 0; q < Q; ++q) drho += Codec<T>::ld(src[q * C + nc], s);
+        const bool ok = in && !(sp.flags_cur[nc] & (F_SOLID | F_SOLID_PREV));
+        const int cnt = __popc(__ballot_sync(FULL, ok));
+        const Cd sum = lane_sum(ok ? drho : (Cd)0);
+        drho = cnt ? sum / (Cd)cnt : (Cd)0;
+        const Cd rho = (Cd)1 + drho;
+        const int k = sp.bid_prev[cl];
+        Cd u[3] = {0, 0, 0};
+        if (k != NO_BODY) wall_velocity(d, dv.geom[sp.parity * dv.nb + k], sp.body_cur[k], x, y, z, u);
+        const Cd uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+        const Cd eu = signed_by(bx, u[0]) + signed_by(by, u[1]) + signed_by(bz, u[2]);
+        f = w * drho + w * rho * ((Cd)3 * eu + (Cd)4.5 * eu * eu - (Cd)1.5 * uu);
+        if (!act) f = 0;
+    } else {
+        // bounce-back at walls (Eq. 4) and at obstacles of step n-1
+        const int sx = x - bx, sy = y - by, sz = z - bz;
+        const bool wall = (!d.px && (sx < 0 || sx >= d.nx)) || (!d.py && (sy < 0 || sy >= d.ny)) ||
+                          (!d.pz && (sz < 0 || sz >= d.nz));
+        const long long sc = ((long long)wrap_axis(sz, d.nz) * d.ny + wrap_axis(sy, d.ny)) * d.nx +
+                             wrap_axis(sx, d.nx);
+        const uint8_t fp = sp.flags_prev[sc];
+        const int k = sp.bid_prev[sc];
+        const Cd own = act ? Codec<T>::ld(src[(long long)b * C + cl], s) : (Cd)0;
+        const Cd pulled = Codec<T>::ld(src[(long long)b * C + sc], s);
+        const Cd rho_x = (Cd)1 + lane_sum(own);
+        const Cd own_opp = __shfl_sync(FULL, own, ld.ob);
+        f = pulled;
+        if (wall) {
+            f = own_opp;                                                 // Eq. 4
+        } else if (fp & F_SOLID) {
             Cd u[3] = {0, 0, 0};
-            if (k != NO_BODY) wall_velocity(d, dv.geom[sp.parity * dv.nb + k], sp.body_cur[k], x, y, z, u);
-            const Cd uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+            if (k != NO_BODY) wall_velocity(d, dv.geom[(sp.parity ^ 1) * dv.nb + k], sp.body_prev[k], sx, sy, sz, u);
             const Cd eu = signed_by(bx, u[0]) + signed_by(by, u[1]) + signed_by(bz, u[2]);
-            f = w * drho + w * rho * ((Cd)3 * eu + (Cd)4.5 * eu * eu - (Cd)1.5 * uu);
-            if (!act) f = 0;
+            f = own_opp + (Cd)6 * w * rho_x * eu;                        // moving wall
+        }
+        if (!act) f = 0;
+    }
+    const Moments<Cd> mo = lane_moments(f, lane, ld.sg);
+    if constexpr (sizeof(T) != 8)
+        if (lane == 0) dv.rho_near[cl] = mo.s;      // rho - 1 for the momentum exchange
+    const Listed<Cd> c = listed_cell(dv, mo);
+    const Cd eu = signed_by(bx, c.ux) + signed_by(by, c.uy) + signed_by(bz, c.uz);
+    const Cd eg = dv.forced ? signed_by(bx, c.gx) + signed_by(by, c.gy) + signed_by(bz, c.gz) : (Cd)0;
+    const Cd v = listed_relax<T>(dv, c, f, w, b == 0 ? 0 : (b < 7 ? 1 : 2), eu, eg);
+    if constexpr (std::is_same<T, float>::value) {
+        // the increments' mass and momentum are moved to 0 and g (collide_f32)
+        const Moments<Cd> dm = lane_moments(act ? v : (Cd)0, lane, ld.sg);
+        f += v;
+        if (b == 0) f -= dm.s;
+        else if (b < 7)
+            f += (Cd)0.5 * (signed_by(bx, c.gx - dm.x) + signed_by(by, c.gy - dm.y) + signed_by(bz, c.gz - dm.z));
+    } else {
+        f = v;
+    }
+    if (act) {
+        T out;
+        if constexpr (std::is_same<T, __nv_bfloat16>::value) {
+            out = __ushort_as_bfloat16((unsigned short)(bf16_sr_add(f, bf16_dither_word(cl, *sp.tstep, b >> 2), b) >> 16));
         } else {
-            // bounce-back at walls (Eq. 4) and at obstacles of step n-1
-            const int sx = x - bx, sy = y - by, sz = z - bz;
-            const bool wall = (!d.px && (sx < 0 || sx >= d.nx)) || (!d.py && (sy < 0 || sy >= d.ny)) ||
-                              (!d.pz && (sz < 0 || sz >= d.nz));
-            const long long sc = ((long long)wrap_axis(sz, d.nz) * d.ny + wrap_axis(sy, d.ny)) * d.nx +
-                                 wrap_axis(sx, d.nx);
-            const uint8_t fp = sp.flags_prev[sc];
-            const int k = sp.bid_prev[sc];
-            const Cd own = act ? Codec<T>::ld(src[(long long)b * C + cl], s) : (Cd)0;
-            const Cd pulled = Codec<T>::ld(src[(long long)b * C + sc], s);
-            const Cd rho_x = (Cd)1 + lane_sum(own);
-            const Cd own_opp = __shfl_sync(FULL, own, ob);
-            f = pulled;
-            if (wall) {
-                f = own_opp;                                                 // Eq. 4
-            } else if (fp & F_SOLID) {
-                Cd u[3] = {0, 0, 0};
-                if (k != NO_BODY) wall_velocity(d, dv.geom[(sp.parity ^ 1) * dv.nb + k], sp.body_prev[k], sx, sy, sz, u);
-                const Cd eu = signed_by(bx, u[0]) + signed_by(by, u[1]) + signed_by(bz, u[2]);
-                f = own_opp + (Cd)6 * w * rho_x * eu;                        // moving wall
-            }
-            if (!act) f = 0;
+            out = Codec<T>::st(f, dv.f16_scale);
         }
-        // LBGK (+ Guo), the bulk kernels' update with the sums over the lanes
-        const Moments<Cd> mo = lane_moments(f, lane, sg);
-        if constexpr (sizeof(T) != 8)
-            if (lane == 0) dv.rho_near[cl] = mo.s;      // rho - 1 for the momentum exchange
-        const Cd rho = (Cd)1 + mo.s;
-        const Cd inv = (Cd)1 / rho;
-        const Cd ux = mad((Cd)0.5, gx, mo.x) * inv, uy = mad((Cd)0.5, gy, mo.y) * inv, uz = mad((Cd)0.5, gz, mo.z) * inv;
-        const Cd usq = mad(ux, ux, mad(uy, uy, uz * uz));
-        const Cd base = mad((Cd)(-1.5) * rho, usq, mo.s);
-        const Cd eu = signed_by(bx, ux) + signed_by(by, uy) + signed_by(bz, uz);
-        Cd eg = 0, ug = 0, gt = 0;
-        if (dv.forced) {
-            eg = signed_by(bx, gx) + signed_by(by, gy) + signed_by(bz, gz);
-            ug = mad(ux, gx, mad(uy, gy, uz * gz));
-        }
-        if constexpr (sizeof(T) == 2) {
-            // the weight last, as the bulk kernel's FP16 form (Lean)
-            const int wc = b == 0 ? 0 : (b < 7 ? 1 : 2);
-            Cd r = dv.ow_f[wc] * (mad((Cd)4.5 * rho, eu * eu, base) + (Cd)3 * rho * eu);
-            if (dv.forced) r = mad(dv.gw_f[wc], mad((Cd)9 * eu, eg, (Cd)(-3) * ug) + (Cd)3 * eg, r);
-            f = mad(dv.om1_f, f, r);
-        }
-        const Cd deq = w * mad(rho, mad((Cd)4.5 * eu, eu, (Cd)3 * eu), base);
-        if (dv.forced) {
-            gt = (f32 ? (Cd)dv.guo_f : (Cd)(1.0 - 0.5 * dv.omega)) * w * mad((Cd)9 * eu, eg, (Cd)3 * (eg - ug));
-        }
-        const Cd om = f32 ? (Cd)dv.omega_f : (Cd)dv.omega;
-        if constexpr (std::is_same<T, float>::value) {
-            // the increments' mass and momentum are moved to 0 and g (collide_f32)
-            const Cd inc = act ? mad(om, deq - f, gt) : (Cd)0;
-            const Moments<Cd> dm = lane_moments(inc, lane, sg);
-            f += inc;
-            if (b == 0) f -= dm.s;
-            else if (b < 7) f += (Cd)0.5 * (signed_by(bx, gx - dm.x) + signed_by(by, gy - dm.y) + signed_by(bz, gz - dm.z));
-        } else if constexpr (sizeof(T) == 8) {
-            f = mad(om, deq - f, f) + gt;
-        }
-        if (act) {
-            T out;
-            if constexpr (std::is_same<T, __nv_bfloat16>::value) {
-                out = __ushort_as_bfloat16((unsigned short)(bf16_sr_add(f, bf16_dither_word(cl, *sp.tstep, b >> 2), b) >> 16));
-            } else {
-                out = Codec<T>::st(f, dv.f16_scale);
-            }
-            dst[(long long)b * C + cl] = out;
-        }
+        dst[(long long)b * C + cl] = out;
     }
 }
 
-// grid of the boundary kernel: `turns` cells a warp for the cells a body of
-// half-width E usually lists (within 1.5 cells of its surface: about 18 E^2 for
-// the bodies of the workloads), at most what the SMs hold at once; longer lists
-// take more turns
+template <typename T>
+__device__ __forceinline__ void boundary_body(const Device &dv, const StepPtrs &sp, const Blk &bk) {
+    const int lane = threadIdx.x & 31;
+    // the count may pass the capacity after an overflow (reported as an error): never read past it
+    const int listed = (int)min((long long)*dv.bcount, dv.blist_cap);
+    int l = bk.x * BOUNDARY_WARPS + (threadIdx.x >> 5);
+    if (l >= listed) return;
+    const LaneDir ld = lane_dir(lane);
+    for (; l < listed; l += bk.gx * BOUNDARY_WARPS) boundary_warp<T>(dv, sp, dv.blist[l], lane, ld);
+}
+
+// lane_sum and lane_moments of the populations of one thread, in their order
+template <typename R> __device__ __forceinline__ R tree_sum(const R (&v)[Q]) {
+    R a[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) a[i] = i + 16 < Q ? v[i] + v[i + 16] : v[i];
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+        for (int i = 0; i < o; ++i) a[i] = a[i] + a[i + o];
+    return a[0];
+}
+template <typename R> __device__ __forceinline__ Moments<R> tree_moments(const R (&f)[Q]) {
+    R out[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        R p[8];
+        bool any[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            any[i] = false;
+            p[i] = 0;
+#pragma unroll
+            for (int b = i; b < Q; b += 8) {
+                const int e = q == 0 ? 1 : (q == 1 ? ex(b) : (q == 2 ? ey(b) : ez(b)));
+                if (e == 0) continue;
+                const R v = e > 0 ? f[b] : -f[b];
+                p[i] = any[i] ? p[i] + v : v;
+                any[i] = true;
+            }
+        }
+#pragma unroll
+        for (int o = 1; o < 8; o <<= 1)
+#pragma unroll
+            for (int i = 0; i < 8; i += 2 * o) {
+                if (any[i] && any[i + o]) p[i] = p[i] + p[i + o];
+                else if (any[i + o]) p[i] = p[i + o];
+                any[i] = any[i] || any[i + o];
+            }
+        out[q] = p[0];
+    }
+    return Moments<R>{out[0], out[1], out[2], out[3]};
+}
+
+// Listed cell cl (not uncovered) by one thread: boundary_warp's operations in its
+// order, without the additions of zeros, so the same value.
+template <typename T>
+__device__ __forceinline__ void boundary_cell(const Device &dv, const StepPtrs &sp, unsigned cl) {
+    using Cd = typename Codec<T>::C;
+    const Domain &d = dv.dom;
+    const long long C = d.C;
+    const T *__restrict__ src = static_cast<const T *>(sp.src);
+    T *__restrict__ dst = static_cast<T *>(sp.dst);
+    const float s = dv.f16_inv_scale;
+    const unsigned nxu = (unsigned)d.nx, nyu = (unsigned)d.ny;
+    const unsigned row = cl / nxu, zu = row / nyu;
+    const int x = (int)(cl - row * nxu), y = (int)(row - zu * nyu), z = (int)zu;
+    // the source of a direction with component e: [1 - e]
+    const int xs[3] = {x == 0 ? d.nx - 1 : x - 1, x, x == d.nx - 1 ? 0 : x + 1};
+    const int ys[3] = {y == 0 ? d.ny - 1 : y - 1, y, y == d.ny - 1 ? 0 : y + 1};
+    const int zs[3] = {z == 0 ? d.nz - 1 : z - 1, z, z == d.nz - 1 ? 0 : z + 1};
+    const bool xw[3] = {!d.px && x == 0, false, !d.px && x == d.nx - 1}, yw[3] = {!d.py && y == 0, false, !d.py && y == d.ny - 1},
+               zw[3] = {!d.pz && z == 0, false, !d.pz && z == d.nz - 1};
+    auto source = [&](int b) { return ((unsigned)zs[1 - ez(b)] * nyu + ys[1 - ey(b)]) * nxu + xs[1 - ex(b)]; };
+    auto beyond = [&](int b) { return xw[1 - ex(b)] || yw[1 - ey(b)] || zw[1 - ez(b)]; };
+    Cd f[Q];
+    unsigned walls = 0, solid = 0;
+#pragma unroll
+    for (int b = 0; b < Q; ++b) {
+        const unsigned sc = source(b);
+        f[b] = Codec<T>::ld(src[(long long)b * C + sc], s);
+        if (b > 0 && beyond(b)) walls |= 1u << b;
+        else if (sp.flags_prev[sc] & F_SOLID) solid |= 1u << b;
+    }
+    if (walls | solid) {
+        Cd own[Q];
+#pragma unroll
+        for (int b = 0; b < Q; ++b) own[b] = Codec<T>::ld(src[(long long)b * C + cl], s);
+        const Cd rho_x = (Cd)1 + tree_sum(own);
+#pragma unroll
+        for (int b = 0; b < Q; ++b) {
+            if (walls >> b & 1u) {
+                f[b] = own[opp(b)];                                      // Eq. 4
+            } else if (solid >> b & 1u) {
+                const int k = sp.bid_prev[source(b)];
+                Cd u[3] = {0, 0, 0};
+                if (k != NO_BODY)
+                    wall_velocity(d, dv.geom[(sp.parity ^ 1) * dv.nb + k], sp.body_prev[k], x - ex(b), y - ey(b), z - ez(b), u);
+                const Cd w = (Cd)wgt(b);
+                f[b] = own[opp(b)] + (Cd)6 * w * rho_x * edot(b, u[0], u[1], u[2]);      // moving wall
+            }
+        }
+    }
+    const Moments<Cd> mo = tree_moments(f);
+    if constexpr (sizeof(T) != 8) dv.rho_near[cl] = mo.s;
+    const Listed<Cd> c = listed_cell(dv, mo);
+    Cd v[Q];
+#pragma unroll
+    for (int b = 0; b < Q; ++b)
+        v[b] = listed_relax<T>(dv, c, f[b], (Cd)wgt(b), b == 0 ? 0 : (b < 7 ? 1 : 2), edot(b, c.ux, c.uy, c.uz),
+                               dv.forced ? edot(b, c.gx, c.gy, c.gz) : (Cd)0);
+    if constexpr (std::is_same<T, float>::value) {
+        const Moments<Cd> dm = tree_moments(v);
+#pragma unroll
+        for (int b = 0; b < Q; ++b) {
+            v[b] = f[b] + v[b];
+            if (b == 0) v[b] -= dm.s;
+            else if (b < 7) v[b] += (Cd)0.5 * edot(b, c.gx - dm.x, c.gy - dm.y, c.gz - dm.z);
+        }
+    }
+    const Dither dz = dither_for<T>(cl, sp.tstep);
+#pragma unroll
+    for (int b = 0; b < Q; ++b) {
+        T out;
+        if constexpr (std::is_same<T, __nv_bfloat16>::value) out = store16<T>(v[b], dz, b);
+        else out = Codec<T>::st(v[b], dv.f16_scale);
+        dst[(long long)b * C + cl] = out;
+    }
+}
+
+// The boundary kernel of long lists: a thread a cell, the uncovered cells (few)
+// by their warp.  A warp a cell keeps a short list's latency low, but costs
+// instruction issue (FP64: its pipe) for 32 lanes and a cell at a time.
+constexpr int BOUNDARY_THREADS = 128;
+
+template <typename T>
+__device__ __forceinline__ void boundary_cells_body(const Device &dv, const StepPtrs &sp, const Blk &bk) {
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int listed = (int)min((long long)*dv.bcount, dv.blist_cap);
+    const LaneDir ld = lane_dir(lane);
+    for (long long l0 = (long long)bk.x * BOUNDARY_THREADS + (threadIdx.x & ~31u); l0 < listed;
+         l0 += (long long)bk.gx * BOUNDARY_THREADS) {
+        const bool have = l0 + lane < listed;
+        const unsigned cl = have ? dv.blist[l0 + lane] : 0u;
+        const bool uncovered = have && (sp.flags_cur[cl] & F_SOLID_PREV);
+        unsigned rest = __ballot_sync(FULL, uncovered);
+        if (have && !uncovered) boundary_cell<T>(dv, sp, cl);
+        __syncwarp();
+        for (; rest; rest &= rest - 1) boundary_warp<T>(dv, sp, __shfl_sync(FULL, cl, __ffs(rest) - 1), lane, ld);
+    }
+}
+
+// grid of the boundary kernels: a warp or a thread for each cell of the expected
+// list and an eighth to spare, at most what the SMs hold at once (a warp a cell)
+// or about four waves; longer lists take turns
 int sm_count();
-long long listed_cells(const Device &dv) {
-    const long long E = (dv.remap_side - 1) / 2 - REMAP_MARGIN;
-    return (long long)dv.nb * 18 * E * E;
-}
-int boundary_blocks(const Device &dv, int turns) {
-    const long long per = BOUNDARY_WARPS * turns, blocks = (listed_cells(dv) + per - 1) / per;
-    return (int)std::min<long long>(std::max<long long>(blocks, 1), 4LL * sm_count());
-}
-// turns of a batched launch over `members` lattices like dv: a block pays its
-// member lookup once for all its cells, so past about one wave of warps (5 blocks
-// an SM) each warp takes more of them (48 boxes in two launches, a step: 684 us
-// with 4 turns, 8 force blocks a body and the preparation kernel; 664 us with 2
-// force blocks and without it; 653 us with 8 turns and one force block)
-int boundary_batch_turns(const Device &dv, int members) {
-    const long long wave = 5LL * BOUNDARY_WARPS * sm_count();
-    return (int)std::min<long long>(std::max<long long>(members * listed_cells(dv) / wave, 1), 16);
+int boundary_blocks(const Device &dv, bool by_cell) {
+    const long long cells = dv.shell + dv.shell / 8, per = by_cell ? BOUNDARY_THREADS : BOUNDARY_WARPS;
+    return (int)std::min<long long>(std::max<long long>((cells + per - 1) / per, 1), (by_cell ? 16LL : 4LL) * sm_count());
 }
 
 template <typename T>
@@ -1252,6 +1417,17 @@ template <typename T>
 __global__ void __launch_bounds__(32 * BOUNDARY_WARPS) boundary_batch(const Batch bt) {
     LBM_BATCH_MEMBER(bt);
     boundary_body<T>(sdv, ssp, sbk);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(BOUNDARY_THREADS) boundary_cells_kernel(const Device dv, const StepPtrs sp) {
+    boundary_cells_body<T>(dv, sp, launch_blk());
+}
+
+template <typename T>
+__global__ void __launch_bounds__(BOUNDARY_THREADS) boundary_cells_batch(const Batch bt) {
+    LBM_BATCH_MEMBER(bt);
+    boundary_cells_body<T>(sdv, ssp, sbk);
 }
 
 // ---- TMA row-staged variant ---------------------------------------------------
@@ -1548,10 +1724,21 @@ const Variant *find_variant(int precision, int vec, int minb) {
 template <typename T>
 void launch_boundary(const Device &dv, const StepPtrs &sp, cudaStream_t s) {
     // the list's length is on the device: blocks past it return at once
-    boundary_kernel<T><<<boundary_blocks(dv, 1), 32 * BOUNDARY_WARPS, 0, s>>>(dv, sp);
+    if (boundary_by_cell(dv.precision, dv.shell))
+        boundary_cells_kernel<T><<<boundary_blocks(dv, true), BOUNDARY_THREADS, 0, s>>>(dv, sp);
+    else
+        boundary_kernel<T><<<boundary_blocks(dv, false), 32 * BOUNDARY_WARPS, 0, s>>>(dv, sp);
 }
 
 }  // namespace
+
+// The two kernels take the same time at lists of about 5,000 cells in FP64 (33 us)
+// and 10,000 to 17,000 in the other types (16 to 18 us); past that a warp a cell
+// falls behind (spheres of radius 4 and 8 in 192^3 cells, a warp and a thread a
+// cell: 10,291 cells FP64 53 and 33 us, FP32 16.3 and 17.8; 34,720 cells 151 and
+// 52, 34.7 and 20.4, FP16 28.0 and 18.3; 367,462 cells 1503 and 375, 283 and 114,
+// 220 and 90 us).
+bool boundary_by_cell(int precision, long long shell) { return shell >= (precision == 0 ? 6000 : 15000); }
 
 bool valid_vector_width(const Device &dv, int v) {
     if (v == -1) {
@@ -1703,11 +1890,11 @@ int batch_bulk_shape(int precision, int i) {
     return b ? b->vec : 0;
 }
 
-void batch_grid_cells(const Device &dv, int k, int variant, int members, int g[3]) {
+void batch_grid_cells(const Device &dv, int k, int variant, bool by_cell, int g[3]) {
     g[0] = g[1] = g[2] = 0;
     const Domain &d = dv.dom;
     if (k == BK_BOUNDARY && dv.nb > 0) {
-        g[0] = boundary_blocks(dv, boundary_batch_turns(dv, members));
+        g[0] = boundary_blocks(dv, by_cell);
         g[1] = g[2] = 1;
     } else if (k == BK_BULK) {
         const BatchShape *b = batch_shape(dv.precision, variant);
@@ -1720,7 +1907,13 @@ void batch_grid_cells(const Device &dv, int k, int variant, int members, int g[3
     }
 }
 
-void launch_batch_cells(int k, int variant, const Batch &bt, unsigned blocks, int precision, bool walls,
+template <typename T>
+static void launch_boundary_batch(const Batch &bt, unsigned blocks, bool by_cell, cudaStream_t s) {
+    if (by_cell) boundary_cells_batch<T><<<blocks, BOUNDARY_THREADS, 0, s>>>(bt);
+    else boundary_batch<T><<<blocks, 32 * BOUNDARY_WARPS, 0, s>>>(bt);
+}
+
+void launch_batch_cells(int k, int variant, const Batch &bt, unsigned blocks, int precision, bool walls, bool by_cell,
                         cudaStream_t s) {
     if (blocks == 0) return;
     if (k == BK_BULK) {
@@ -1729,10 +1922,10 @@ void launch_batch_cells(int k, int variant, const Batch &bt, unsigned blocks, in
         return;
     }
     switch (precision) {
-    case 0: boundary_batch<double><<<blocks, 32 * BOUNDARY_WARPS, 0, s>>>(bt); break;
-    case 1: boundary_batch<float><<<blocks, 32 * BOUNDARY_WARPS, 0, s>>>(bt); break;
-    case 2: boundary_batch<__half><<<blocks, 32 * BOUNDARY_WARPS, 0, s>>>(bt); break;
-    default: boundary_batch<__nv_bfloat16><<<blocks, 32 * BOUNDARY_WARPS, 0, s>>>(bt); break;
+    case 0: launch_boundary_batch<double>(bt, blocks, by_cell, s); break;
+    case 1: launch_boundary_batch<float>(bt, blocks, by_cell, s); break;
+    case 2: launch_boundary_batch<__half>(bt, blocks, by_cell, s); break;
+    default: launch_boundary_batch<__nv_bfloat16>(bt, blocks, by_cell, s); break;
     }
 }
 

@@ -1,7 +1,9 @@
-"""Many bodies whose remap cubes overlap: rods packed side by side in a small
-box.  Every fluid cell near a body is listed once for the boundary kernel, so
-the list holds however many cubes cover a cell, and FP64 storage matches the
-oracle at the parity bars (populations 1e-12, positions 1e-10 relative)."""
+"""Many bodies: rods whose remap cubes overlap (every fluid cell near a body is
+listed once for the boundary kernel, so the list holds however many cubes cover
+a cell), and lists long enough for the boundary kernel to take a thread a cell.
+FP64 storage matches the oracle at the parity bars (populations 1e-12, positions
+1e-10 relative); a lattice gives the same bits whichever way its list is taken
+(alone a warp a cell, in an ensemble a thread a cell)."""
 import numpy as np
 import pytest
 
@@ -97,3 +99,61 @@ def test_list_holds_each_cell_once():
     lat.step(16)
     lat.sync()
     lat.close()
+
+
+def suspension(bodies, bc, seed=0):
+    """Spheres of radius 3 on a loose grid of 44 x 40 x 48 cells, fast enough to
+    cover and uncover cells."""
+    sc = wl.Scenario("suspension", 44, 40, 48, 0.8, bc=bc, g=(2e-6, -1e-6, 3e-6))
+    rng = wl.SplitMix64(77 + seed)
+    sites = [(i, j, k) for k in range(4) for j in range(3) for i in range(4)]
+    for s in sites[:bodies]:
+        pos = tuple((v + 0.5) * p + rng.uniform(-0.4, 0.4) for v, p in zip(s, (11, 13, 12)))
+        sc.bodies.append(wl.Body(wl.SPHERE, 3.0, 0.0, 2.0 * wl.sphere_volume(3.0), pos))
+    return sc
+
+
+def swept(sim, sc):
+    for b in range(len(sc.bodies)):
+        s = sim.bodies()[b].copy()
+        s[7:10] = (0.04 * (1 - b % 3), 0.03 * (b % 2), -0.03 + 0.015 * (b % 5))
+        s[10:13] = (0.01, -0.005 * (b % 3), 0.0)
+        sim.set_body_state(b, s)
+
+
+@pytest.mark.parametrize("bc", [7, wl.PERIODIC_X, 0])
+def test_long_list_matches_the_oracle(bc):
+    sc = suspension(36, bc)                     # about 9,600 cells listed
+    gpu, ref = lbm.from_scenario(sc, precision="f64"), oracle.from_scenario(sc)
+    for sim in (gpu, ref):
+        swept(sim, sc)
+    for _ in range(4):
+        gpu.step(4)
+        ref.step(4)
+        assert np.array_equal(gpu.flags(), ref.flags())
+        assert np.abs(gpu.pop() - ref.pop()).max() < 1e-12
+        fr = ref.forces()
+        assert np.abs(gpu.forces() - fr).max() < 1e-12 + 1e-10 * np.abs(fr).max()
+    gpu.close()
+
+
+@pytest.mark.parametrize("bc", [7, wl.PERIODIC_Z])
+@pytest.mark.parametrize("precision", ["f64", "f32", "f16", "bf16"])
+def test_bits_of_a_warp_and_a_thread_a_cell(precision, bc):
+    n = 18 if precision == "f64" else 36        # about 4,800 and 9,600 cells a lattice
+    scs = [suspension(n, bc, k) for k in range(6)]
+    lats = [lbm.from_scenario(sc, precision=precision) for sc in scs]
+    for m, sc in zip(lats, scs):
+        swept(m, sc)
+    ens = lbm.Ensemble(lats)
+    ens.step(16)                                # in two launches: 14,400 and 28,900 cells each
+    ens.sync()
+    for m, sc in zip(lats, scs):
+        lat = lbm.from_scenario(sc, precision=precision)
+        swept(lat, sc)
+        lat.step(16)
+        assert np.array_equal(m.bodies(), lat.bodies()) and np.array_equal(m.pop(), lat.pop())
+        lat.close()
+    ens.close()
+    for m in lats:
+        m.close()
