@@ -728,29 +728,36 @@ adj_terms_kernel(const Device dv, const BodyState *states, const double *fhs, lo
     }
 }
 
-// One block.  Sh^{n+1} = sa_next + the cell sums of reverse step n+1
-// (part, a fixed order); then the reverse step with the state-only terms
+// Sh^{n+1} = sa_next + the cell sums of reverse step n+1 (part, a fixed order); then the reverse step with the state-only terms
 // of step n.  Writes Sh^n (rigid-body part plus the lever-arm term Th x
 // F_hydro of the torque sum) to sa_cur, (Fh, Th) to fadj and adds
 // dJ/dtheta.  A warp a body with components on lanes (axes, quaternion and matrix
 // entries): an FP64 warp instruction costs ~64 issue cycles whatever its lanes
 // carry, and this kernel is on the sweep's serial chain (a thread a body
-// took 19.8 us a launch for three bodies, this takes 11.4).
+// took 19.8 us a launch for three bodies, this takes 11.4).  Past eight bodies the
+// bodies are dealt to several blocks, and the last of them to finish (ab.done)
+// does the drive terms and springs.  In one block the bodies' rounds of eight cost
+// more than the thread-a-body form from about 100 bodies on; a reverse step of 100
+// and 200 spheres of radius 3 (FP32, 96^3 and 120 x 96 x 96 cells) took 363 and
+// 662 us so, 351 and 584 us with a thread a body, 266 and 454 us with blocks.
 constexpr int ADJ_WARPS = ADJ_THREADS / 32;
+constexpr int ADJ_AXIS_GROUPS = 32 / 3;     // bodies a warp takes side by side, three axes each
+__host__ __device__ inline int adj_integrate_blocks(int nb) { return (nb + ADJ_WARPS - 1) / ADJ_WARPS; }
 constexpr int ADJ_SUM_GROUPS = 3;           // records a warp's lanes take side by side, nine sums each
 
-__device__ __forceinline__ void adj_integrate(const Device &dv, const AdjBody &ab) {
+__device__ __forceinline__ void adj_integrate(const Device &dv, const AdjBody &ab, int blk, int blocks) {
     constexpr unsigned FULL = 0xffffffffu;
     const int nb = dv.nb;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     __shared__ double s_sum[ADJ_WARPS][9];
     __shared__ double s_F[LBM_MAX_BODIES_DEV][3];       // Fh of every body
+    __shared__ int s_last;
     const int ax = lane < 3 ? lane : 0, i1 = (ax + 1) % 3, i2 = (ax + 2) % 3;
     auto at = [](double v, int l) { return __shfl_sync(FULL, v, l); };
     // warps that share a body's cell sums
     const int share = nb <= 2 ? 4 : (nb <= 4 ? 2 : 1);
     const int bodies = ADJ_WARPS / share;               // bodies in flight
-    for (int b0 = 0; b0 < nb; b0 += bodies) {
+    for (int b0 = blk * bodies; b0 < nb; b0 += blocks * bodies) {
         // 1. complete Sh^{n+1}: lane 9 g + c of each of the body's warps adds
         //    component c of every (share x groups)-th record
         const int b = b0 + warp % bodies, part = warp / bodies;
@@ -878,8 +885,20 @@ __device__ __forceinline__ void adj_integrate(const Device &dv, const AdjBody &a
         }
         __syncthreads();
     }
+    if (blocks > 1) {
+        if (threadIdx.x == 0) {
+            __threadfence();
+            s_last = atomicAdd(ab.done, 1u) == (unsigned)blocks - 1;
+            if (s_last) *ab.done = 0u;
+            __threadfence();
+        }
+        __syncthreads();
+        if (!s_last) return;
+        for (int i = threadIdx.x; i < 3 * nb; i += ADJ_THREADS) s_F[i / 3][i % 3] = __ldcg(ab.fadj + 6 * (i / 3) + i % 3);
+        __syncthreads();
+    }
     // 2. drive-term and spring gradients (one thread per term), and the spring
-    //    terms of each body's adjoint (lane i of the body's warp axis i, its
+    //    terms of each body's adjoint (three lanes a body, an axis each, its
     //    springs in order)
     const double tt = (double)ab.t;
     for (int k = threadIdx.x; k < dv.nd; k += blockDim.x) {
@@ -907,34 +926,50 @@ __device__ __forceinline__ void adj_integrate(const Device &dv, const AdjBody &a
             ab.grad_spring[3 * k + 1] += sp_.k * fd;
         }
     }
-    for (int b = ADJ_WARPS - 1 - warp; b < nb; b += ADJ_WARPS) {
-        const BodyProps *pb = dv.props + b;
-        const int s0 = pb->spring_first, s1 = s0 + pb->spring_count;
-        double *sc = ab.sa_cur + 13 * b;
+    const int grp = lane / 3, axis = lane % 3;
+    for (int b0 = (ADJ_WARPS - 1 - warp) * ADJ_AXIS_GROUPS; b0 < nb; b0 += ADJ_WARPS * ADJ_AXIS_GROUPS) {
+        const int b = b0 + grp;
+        const bool on = grp < ADJ_AXIS_GROUPS && b < nb;
+        const BodyProps *pb = dv.props + (on ? b : 0);
+        const int s0 = pb->spring_first, count = on ? pb->spring_count : 0;
+        int most = count;
+        for (int o = 16; o > 0; o >>= 1) most = max(most, __shfl_xor_sync(FULL, most, o));
+        double *sc = ab.sa_cur + 13 * (on ? b : 0);
         double x = 0.0, v = 0.0;
-        if (lane < 3) {
-            x = sc[lane];
-            v = sc[7 + lane];
+        if (on) {
+            x = __ldcg(sc + axis);
+            v = __ldcg(sc + 7 + axis);
         }
-        for (int kk = s0; kk < s1; ++kk) {
-            const int k = dv.spring_list[kk];
-            const Spring sp_ = dv.springs[k];
-            const AdjSpringTerms *tsk = ab.ts + k;
-            const double sign = sp_.i == b ? 1.0 : -1.0;
-            const double fh = s_F[sp_.i][ax] - s_F[sp_.j][ax], dir = tsk->dir[ax];
-            v += -sign * sp_.gamma * fh;
+        for (int i = 0; i < most; ++i) {
+            const bool has = i < count;
+            double sign = 0.0, fh = 0.0, dir = 0.0, k = 0.0, ratio = 0.0, gamma = 0.0, len = 0.0;
+            if (has) {
+                const int j = dv.spring_list[s0 + i];
+                const Spring sp_ = dv.springs[j];
+                const AdjSpringTerms *tsk = ab.ts + j;
+                sign = sp_.i == b ? 1.0 : -1.0;
+                fh = s_F[sp_.i][axis] - s_F[sp_.j][axis];
+                dir = tsk->dir[axis];
+                k = sp_.k;
+                gamma = sp_.gamma;
+                ratio = tsk->ratio;
+                len = tsk->len;
+            }
             const double prod = fh * dir;
-            const double fd = at(prod, 0) + at(prod, 1) + at(prod, 2);
-            if (tsk->len > 0) x += sign * (-sp_.k * (fd * dir + tsk->ratio * (fh - fd * dir)));
+            const double fd = at(prod, 3 * grp) + at(prod, 3 * grp + 1) + at(prod, 3 * grp + 2);
+            if (has) {
+                v += -sign * gamma * fh;
+                if (len > 0) x += sign * (-k * (fd * dir + ratio * (fh - fd * dir)));
+            }
         }
-        if (lane < 3) {
-            sc[lane] = x;
-            sc[7 + lane] = v;
+        if (on) {
+            sc[axis] = x;
+            sc[7 + axis] = v;
         }
     }
 }
 
-// The first launch of reverse step n: block (0, 0) the rigid-body step, the others
+// The first launch of reverse step n: blocks (0, y) the rigid-body step, the others
 // the bulk cells, which need neither its result nor each other's.  One launch
 // instead of two on two streams with events between them (96 x 48 x 48 study: a
 // launch takes 14.2 us, the rigid-body step alone 11.4 us).
@@ -944,7 +979,8 @@ adj_step_kernel(const Device dv, const AdjPtrs ap, const AdjBody ab, int body) {
     int blk = blockIdx.x;
     if (body) {
         if (blk == 0) {
-            if (blockIdx.y == 0) adj_integrate(dv, ab);
+            const int blocks = min(adj_integrate_blocks(dv.nb), (int)gridDim.y);
+            if ((int)blockIdx.y < blocks) adj_integrate(dv, ab, blockIdx.y, blocks);
             return;
         }
         --blk;
@@ -953,7 +989,7 @@ adj_step_kernel(const Device dv, const AdjPtrs ap, const AdjBody ab, int body) {
 }
 
 __global__ void __launch_bounds__(ADJ_THREADS) adj_integrate_kernel(const Device dv, const AdjBody ab) {
-    adj_integrate(dv, ab);
+    adj_integrate(dv, ab, blockIdx.x, gridDim.x);
 }
 
 // sa[b] += the cell sums part[b][0..count) (the last reverse step)
@@ -997,7 +1033,7 @@ int adjoint_part_stride(const Device &dv) {
 }
 
 void launch_adj_integrate(const Device &dv, const AdjBody &ab, cudaStream_t s) {
-    adj_integrate_kernel<<<1, ADJ_THREADS, 0, s>>>(dv, ab);
+    adj_integrate_kernel<<<adj_integrate_blocks(dv.nb), ADJ_THREADS, 0, s>>>(dv, ab);
 }
 
 void launch_adj_terms(const Device &dv, const BodyState *states, const double *fh, long long t0, int L,

@@ -446,6 +446,7 @@ struct AdjBody {
     int part_stride, part_count;
     double *grad_drive, *grad_spring, *grad_body;   // [nd][2], [ns][3], [nb][5] (added to)
     long long t;                    // step n
+    unsigned *done;                 // blocks of the step that have finished their bodies (zero between steps)
 };
 
 // ---- launch wrappers (kernels.cu / stream_collide.cu / adjoint.cu) ---------

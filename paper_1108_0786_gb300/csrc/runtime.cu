@@ -1531,7 +1531,7 @@ int lbm_adjoint_backward(lbm_t *h, const double *seed, double *grad_state, doubl
     if ((rc = alloc_list(h, bk, &fadj, sizeof(double) * 6 * B))) return rc;
     if ((rc = alloc_list(h, bk, &part, sizeof(double) * 9 * B * (size_t)stride))) return rc;
     const size_t ngrad = 2 * (size_t)ND + 3 * (size_t)NS + 5 * (size_t)B;
-    if ((rc = alloc_list(h, bk, &grads, sizeof(double) * ngrad))) return rc;
+    if ((rc = alloc_list(h, bk, &grads, sizeof(double) * (ngrad + 1)))) return rc;     // and AdjBody::done
     int nset = 0;
     if (fl) {
         // two sets let segment k - 1 be recomputed while segment k is
@@ -1606,7 +1606,7 @@ int lbm_adjoint_backward(lbm_t *h, const double *seed, double *grad_state, doubl
                &ev_rcopy, &ev_ccopy, &ev_rbulk[0], &ev_rbulk[1], &ev_cbulk[0], &ev_cbulk[1]}};
     CK(cudaEventRecord(ev_free, s));
     double *gd = grads, *gs = grads + 2 * ND, *gb = grads + 2 * ND + 3 * NS;
-    CK(cudaMemsetAsync(grads, 0, sizeof(double) * ngrad, s));
+    CK(cudaMemsetAsync(grads, 0, sizeof(double) * (ngrad + 1), s));
     CK(cudaMemsetAsync(part, 0, sizeof(double) * 9 * B * (size_t)stride, s));
     CK(cudaMemcpyAsync(sa[0], seed, sizeof(double) * 13 * B, cudaMemcpyHostToDevice, s));
     int cur = 0;                    // sa[cur]: adjoint of state n + 1
@@ -1817,6 +1817,7 @@ int lbm_adjoint_backward(lbm_t *h, const double *seed, double *grad_state, doubl
             ab.td = tset.td + (long long)j * ND;
             ab.ts = tset.ts + (long long)j * NS;
             ab.t = n;
+            ab.done = reinterpret_cast<unsigned *>(grads + ngrad);
             if (!fl) {
                 lbm::launch_adj_integrate(dv, ab, s);
             } else {
