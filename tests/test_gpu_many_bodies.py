@@ -65,3 +65,16 @@ def test_gradients_of_many_bodies(bodies, options):
     np.testing.assert_allclose(final, ref_run.bodies(), rtol=1e-10, atol=1e-12)
     for k in ("state", "prev", "drive", "spring", "body"):
         assert np.abs(got[k] - ref[k]).max() <= 1e-9 * max(np.abs(ref[k]).max(), 1e-300), k
+
+
+@pytest.mark.parametrize("bodies", [4, 5, 24, 254])
+def test_rigid_bodies_without_fluid(bodies):
+    """Every body steps once a step and the clock advances once."""
+    sc = chain(bodies)
+    lat, ref = (moving(lbm.from_scenario(sc, precision="f64", options=lbm.OPT_NO_FLUID)),
+                moving(oracle.from_scenario(sc, lbm.OPT_NO_FLUID)))
+    for n in (1, 3, 40):
+        lat.step(n)
+        ref.step(n)
+        np.testing.assert_allclose(lat.bodies(), ref.bodies(), rtol=1e-10, atol=1e-12)
+    lat.close()
