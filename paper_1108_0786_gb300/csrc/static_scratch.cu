@@ -93,14 +93,19 @@ cudaError_t partials_address(double **out) {
 // its cells twice and add their links twice).
 inline int scan_extent(int side, int n, int periodic) { return periodic && n < side ? n : side; }
 
-// minimum image of a distance i / 2 - f with i an integer number of half cells
-// and f in [0, 1): twice the integer part, wrapped into [-n, n) less 2 f
-__device__ __forceinline__ int near_half(int i2, int n, int periodic, float f2) {
+// minimum image of a distance i / 2 - f with i an integer number of half cells,
+// f in [0, 1) and k = ceil(2 f): twice the integer part, so that i / 2 - f lies in
+// [-n / 2, n / 2).  A distance within n + 1 of zero needs one period, on an axis of
+// one cell up to two.
+__device__ __forceinline__ int near_half(int i2, int n, int periodic, int k) {
     if (!periodic) return i2;
-    if ((float)(i2 - n) >= f2) return i2 - 2 * n;
-    if ((float)(i2 + n) < f2) return i2 + 2 * n;
-    return i2;
+    if (i2 - n >= k) return i2 - 2 * n;
+    if (i2 + n < k) i2 += 2 * n;
+    return i2 + n < k ? i2 + 2 * n : i2;
 }
+
+// exponent bits all set: an infinity or NaN (integer operations, not the FP64 pipe)
+__device__ __forceinline__ bool non_finite(double v) { return (__double2hiint(v) & 0x7ff00000) == 0x7ff00000; }
 
 // Block (k, b): cells k*256 .. of the box of extents (sx, sy, sz) that
 // starts at floor(X_b) - hw (the cube of side 2 hw + 1 around floor(X_b),
@@ -125,13 +130,13 @@ static_partials_kernel(const double *__restrict__ pop, const uint8_t *__restrict
     // the centre wrapped into the domain: its cell and the position within it
     int corner[3], ci[3];
     double cf[3];
-    float cf2[3];
+    int cf2[3];                 // ceil(2 cf)
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         const double X = sb[a], fx = floor(X);
         corner[a] = (int)fx - hw;
         cf[a] = X - fx;
-        cf2[a] = 2.0f * (float)cf[a];
+        cf2[a] = (cf[a] > 0.0) + (cf[a] > 0.5);
         ci[a] = (int)fx;
         if (per[a]) {
             ci[a] %= n3[a];
@@ -195,6 +200,8 @@ static_partials_kernel(const double *__restrict__ pop, const uint8_t *__restrict
     double acc[6] = {0, 0, 0, 0, 0, 0};
     if ((int)threadIdx.x < total) {
         const double V[3] = {sb[7], sb[8], sb[9]}, W[3] = {sb[10], sb[11], sb[12]};
+        bool odd = false;
+        for (int i = 0; i < 3; ++i) odd = odd || non_finite(V[i]) || non_finite(W[i]) || non_finite(cf[i]);
         for (int j = threadIdx.x; j < total; j += NA_THREADS) {
             const int t = s_link[j] >> 5, a = s_link[j] & 31;
             const int c = s_cell[t];
@@ -219,6 +226,18 @@ static_partials_kernel(const double *__restrict__ pop, const uint8_t *__restrict
             const double eu = -(by(e[0], u0) + by(e[1], u1) + by(e[2], u2));
             const double w6 = a < 7 ? 6.0 * wgt(1) : 6.0 * wgt(7);
             const double mag = 2.0 * ga + w6 * rho * eu;
+            if (odd || non_finite(mag)) {
+                // Eq. hydroF with its zero components multiplied out: 0 * inf is no 0
+                const double m = 2.0 * ga - w6 * rho * (e[0] * u0 + e[1] * u1 + e[2] * u2);
+                const double fl[3] = {e[0] * m, e[1] * m, e[2] * m};
+                acc[0] += fl[0];
+                acc[1] += fl[1];
+                acc[2] += fl[2];
+                acc[3] += om[1] * fl[2] - om[2] * fl[1];
+                acc[4] += om[2] * fl[0] - om[0] * fl[2];
+                acc[5] += om[0] * fl[1] - om[1] * fl[0];
+                continue;
+            }
             acc[0] += by(e[0], mag);
             acc[1] += by(e[1], mag);
             acc[2] += by(e[2], mag);
