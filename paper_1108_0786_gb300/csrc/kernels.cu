@@ -1290,31 +1290,56 @@ __global__ void __launch_bounds__(64 * INTEGRATE_BODIES) integrate_kernel(const 
 
 // ---- field export / import -----------------------------------------------
 
-// The value of a float expansion hi + lo under additions: TwoSum (Knuth; Moller)
-// keeps each addition's rounding error in lo, so that a sum of 19 FP32 values
-// carries about 48 bits without the FP64 pipe (2 results a cycle an SM here,
-// against 128 FP32 ones).  Infinities and NaN do not survive it (inf - inf):
-// callers check the result.
+// The rounding error of s = a + b: TwoSum (Knuth; Moller), so that a + b = s + e exactly.
+// Infinities and NaN do not survive it (inf - inf): callers check the result.
+__device__ __forceinline__ float sum_error(float a, float b, float s) {
+    const float t = s - a;
+    return (a - (s - t)) + (b - t);
+}
+
+// Sums of 19 FP32 values as float expansions, without the FP64 pipe (2 results a
+// cycle an SM here, against 128 FP32 ones).  FloatSum (hi + lo) is off by at most
+// 190 2^-48 of the values' absolute sum S, enough beside 1 in a density; FloatSum3
+// by less than 2^-60 S, which also leaves a small difference of large values its digits.
 struct FloatSum {
     float hi, lo;
     __device__ __forceinline__ void add(float v) {
-        const float s = hi + v, t = s - hi;
-        lo += (hi - (s - t)) + (v - t);
+        const float s = hi + v;
+        lo += sum_error(hi, v, s);
         hi = s;
+    }
+};
+struct FloatSum3 {
+    float a, b, c;
+    __device__ __forceinline__ void add_low(float v) {      // a value of the size of a's rounding errors
+        const float s = b + v;
+        c += sum_error(b, v, s);
+        b = s;
+    }
+    __device__ __forceinline__ void add(float v) {
+        const float s = a + v;
+        add_low(sum_error(a, v, s));
+        a = s;
+    }
+    // the sum as hi + lo, lo at most half an ulp of hi (to 2^-48 of the sum)
+    __device__ __forceinline__ FloatSum two() const {
+        const float h = a + b, l = sum_error(a, b, h);
+        const float l2 = l + c, m = sum_error(l, c, l2);
+        const float g = h + l2;
+        return FloatSum{g, sum_error(h, l2, g) + m};
     }
 };
 
 // w_a + delta as stored in O.  FP32 output of 32/16-bit storage adds the two
 // parts of w_a (FP32 value and remainder) with one TwoSum: the FP64 sum rounded
-// to FP32, but for ties that the remainder's own rounding (2^-24 of an ulp)
-// decides.
+// to FP32, but within 2^-23 of an ulp of a tie, where the rounding of the
+// remainders decides (a branch to FP64 there costs what FP64 for all does).
 template <typename O, typename T>
 __device__ __forceinline__ O pop_value(double w, float wh, float wl, const T *v, float scale) {
     if constexpr (sizeof(O) == 4 && sizeof(T) <= 4) {
         const float x = load_dev_f<T>(v, scale);
-        const float s = wh + x, t = s - wh;
-        const float e = (wh - (s - t)) + (x - t);
-        return fabsf(s) < INFINITY ? s + (e + wl) : s;
+        const float s = wh + x;
+        return fabsf(s) < INFINITY ? s + (sum_error(wh, x, s) + wl) : s;
     } else {
         return (O)(w + load_dev<T>(v, scale));
     }
@@ -1392,9 +1417,11 @@ __device__ __forceinline__ void moments_f64(const T (&v)[Q], float scale, double
 
 // Density (U = false) or velocity (U = true) of each cell, one thread a cell,
 // all 19 loads issued before the sums.  FP32 output of 32/16-bit storage sums in
-// float expansions and divides with one correction step, so that the result is
-// rounded about once, as from FP64 sums; FP64 storage and FP64 output sum in
-// FP64.  A cell whose sums are not finite takes the FP64 path.
+// float expansions and divides with one correction step: the exact value rounded
+// once, to 2^-20 of an ulp, as from FP64 sums (one FP32 remainder of a two-part
+// momentum was up to 7e-4 of an ulp further off where forces cancel it).  FP64
+// storage and FP64 output sum in FP64, as does a cell whose sums are not finite.
+// (128^3 cells from FP32, velocity: 48 us, FP64 sums 480 us, two-part sums 41 us.)
 template <typename T, typename O, bool U>
 __global__ void __launch_bounds__(EXPORT_THREADS)
 export_moments_kernel(const Device dv, const T *__restrict__ pop, const uint8_t *__restrict__ flags, int mask_solid,
@@ -1416,17 +1443,12 @@ export_moments_kernel(const Device dv, const T *__restrict__ pop, const uint8_t 
         return;
     }
     if constexpr (sizeof(O) == 4 && sizeof(T) <= 4) {
-        FloatSum s{0.0f, 0.0f}, j[3] = {{0.0f, 0.0f}, {0.0f, 0.0f}, {0.0f, 0.0f}};
+        float x[Q];
 #pragma unroll
-        for (int a = 0; a < Q; ++a) {
-            const float x = load_dev_f<T>(&v[a], scale);
-            s.add(x);
-            if constexpr (U) {
-                if (ex(a)) j[0].add(ex(a) > 0 ? x : -x);
-                if (ey(a)) j[1].add(ey(a) > 0 ? x : -x);
-                if (ez(a)) j[2].add(ez(a) > 0 ? x : -x);
-            }
-        }
+        for (int a = 0; a < Q; ++a) x[a] = load_dev_f<T>(&v[a], scale);
+        FloatSum s{x[0], 0.0f};
+#pragma unroll
+        for (int a = 1; a < Q; ++a) s.add(x[a]);
         FloatSum rho{1.0f, s.lo};
         rho.add(s.hi);
         if constexpr (!U) {
@@ -1436,22 +1458,43 @@ export_moments_kernel(const Device dv, const T *__restrict__ pop, const uint8_t 
                 return;
             }
         } else {
+            // momentum by pairs of opposite directions: x_a - x_a+1 = dh + dl
+            FloatSum3 j[3];
+#pragma unroll
+            for (int p = 0; p < Q / 2; ++p) {
+                const int a = 2 * p + 1;
+                const float dh = x[a] - x[a + 1], dl = sum_error(x[a], -x[a + 1], dh);
+#pragma unroll
+                for (int i = 0; i < 3; ++i) {
+                    const int e = i == 0 ? ex(a) : (i == 1 ? ey(a) : ez(a));
+                    if (e == 0) continue;
+                    if (p == i) {
+                        j[i] = FloatSum3{dh, dl, 0.0f};
+                    } else {
+                        j[i].add(e > 0 ? dh : -dh);
+                        j[i].add_low(e > 0 ? dl : -dl);
+                    }
+                }
+            }
             const float inv = 1.0f / rho.hi;
             float q[3];
             bool finite = true;
 #pragma unroll
             for (int i = 0; i < 3; ++i) {
-                const float gh = dv.gh_f[i], gl = dv.gl_f[i];           // g / 2 in two parts
-                j[i].lo -= gl;
+                const float gh = dv.gh_f[i];            // g / 2 in three parts
                 j[i].add(-gh);
-                const float n = j[i].hi + j[i].lo, nl = (j[i].hi - n) + j[i].lo;
-                const float q0 = n * inv;
-                const float r = fmaf(-q0, rho.hi, n) + fmaf(-q0, rho.lo, nl);
-                q[i] = fmaf(r, inv, q0);
+                j[i].add_low(-dv.gl_f[i]);
+                j[i].c -= dv.gr_f[i];
+                // scaled, so that the remainders of the smallest momenta do not underflow
+                FloatSum n = j[i].two();
+                n.hi *= 0x1p48f;
+                n.lo *= 0x1p48f;
+                const float q0 = n.hi * inv;
+                q[i] = fmaf(fmaf(-q0, rho.hi, n.hi) + fmaf(-q0, rho.lo, n.lo), inv, q0);
                 finite = finite && fabsf(q[i]) < INFINITY;
             }
             if (finite) {
-                for (int i = 0; i < 3; ++i) out[i * C + c] = q[i];
+                for (int i = 0; i < 3; ++i) out[i * C + c] = q[i] * 0x1p-48f;
                 return;
             }
         }

@@ -238,7 +238,7 @@ struct Device {
     double tau, omega, g[3];
     float omega_f, guo_f, g_f[3];   // omega, 1 - omega / 2 and g rounded to FP32 once (the FP32 collision's)
     float om1_f, ow_f[3], gw_f[3];  // 1 - omega; omega w and (1 - omega / 2) w per weight class (rest, axis, diagonal)
-    float gh_f[3], gl_f[3];         // g / 2 as an FP32 value and its remainder
+    float gh_f[3], gl_f[3], gr_f[3];        // g / 2 as the sum of three FP32 values
     double om1, ow[3], gw[3];       // the same in FP64: 1 - omega, omega w and (1 - omega / 2) w per weight class
     int forced;
     int avg_force;          // the rigid-body step uses the mean load of steps n and n-1

@@ -397,6 +397,7 @@ int ensure_device(lbm_t *h) {
         dv.g_f[i] = (float)dv.g[i];
         dv.gh_f[i] = (float)(0.5 * dv.g[i]);
         dv.gl_f[i] = (float)(0.5 * dv.g[i] - (double)dv.gh_f[i]);
+        dv.gr_f[i] = (float)(0.5 * dv.g[i] - (double)dv.gh_f[i] - (double)dv.gl_f[i]);
     }
     dv.om1 = 1.0 - dv.omega;
     dv.om1_f = (float)dv.om1;
