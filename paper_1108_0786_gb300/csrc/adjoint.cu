@@ -42,14 +42,16 @@ template <typename A> struct AdjParams;
 template <> struct AdjParams<double> {
     __device__ static double omega(const Device &dv) { return dv.omega; }
     __device__ static double guo(const Device &dv) { return 1.0 - 0.5 * dv.omega; }
-    __device__ static double g(const Device &dv, int i) { return dv.g[i]; }
     __device__ static double half_g(const Device &dv, int i) { return 0.5 * dv.g[i]; }
+    __device__ static double g3(const Device &dv, int i) { return 3.0 * dv.g[i]; }
+    __device__ static double eg(const Device &dv, int b) { return ex(b) * dv.g[0] + ey(b) * dv.g[1] + ez(b) * dv.g[2]; }
 };
 template <> struct AdjParams<float> {
     __device__ static float omega(const Device &dv) { return dv.omega_f; }
     __device__ static float guo(const Device &dv) { return dv.guo_f; }
-    __device__ static float g(const Device &dv, int i) { return dv.g_f[i]; }
     __device__ static float half_g(const Device &dv, int i) { return dv.gh_f[i]; }
+    __device__ static float g3(const Device &dv, int i) { return dv.g3_f[i]; }
+    __device__ static float eg(const Device &dv, int b) { return dv.eg_f[b]; }
 };
 
 // acc + s v for a component s of a direction
@@ -86,7 +88,6 @@ template <typename A>
 __device__ inline void collide_adjoint(A (&a)[Q], A rho, const A (&u)[3], const Device &dv) {
     const A om = AdjParams<A>::omega(dv);
     const A uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
-    const A g0 = AdjParams<A>::g(dv, 0), g1 = AdjParams<A>::g(dv, 1), g2 = AdjParams<A>::g(dv, 2);
     const A rest = (A)1 - (A)1.5 * uu;
     A t0 = 0, sr = 0, s0 = 0, s1 = 0, s2 = 0, f0 = 0, f1 = 0, f2 = 0;
 #pragma unroll
@@ -100,7 +101,7 @@ __device__ inline void collide_adjoint(A (&a)[Q], A rho, const A (&u)[3], const 
         s1 = plus(s1, ey(b), tc);
         s2 = plus(s2, ez(b), tc);
         if (dv.forced) {
-            const A te = t * plus(plus(plus((A)0, ex(b), g0), ey(b), g1), ez(b), g2);
+            const A te = t * AdjParams<A>::eg(dv, b);
             f0 = plus(f0, ex(b), te);
             f1 = plus(f1, ey(b), te);
             f2 = plus(f2, ez(b), te);
@@ -113,9 +114,9 @@ __device__ inline void collide_adjoint(A (&a)[Q], A rho, const A (&u)[3], const 
     const A ir = (A)1 / rho;
     A su0 = om * s0, su1 = om * s1, su2 = om * s2;          // om rho s / rho
     if (dv.forced) {
-        su0 += kf * ((A)9 * f0 - (A)3 * g0 * t0) * ir;
-        su1 += kf * ((A)9 * f1 - (A)3 * g1 * t0) * ir;
-        su2 += kf * ((A)9 * f2 - (A)3 * g2 * t0) * ir;
+        su0 += kf * ((A)9 * f0 - AdjParams<A>::g3(dv, 0) * t0) * ir;
+        su1 += kf * ((A)9 * f1 - AdjParams<A>::g3(dv, 1) * t0) * ir;
+        su2 += kf * ((A)9 * f2 - AdjParams<A>::g3(dv, 2) * t0) * ir;
     }
     const A base = om * sr - (su0 * u[0] + su1 * u[1] + su2 * u[2]);
     const A om1 = (A)1 - om;
@@ -364,17 +365,27 @@ template <typename V> __device__ __forceinline__ V warp_sum(V v) {
     return v;
 }
 
-// a centre's cell, wrapped into the domain on periodic axes, and its position within
+// a centre's cell, wrapped into the domain on periodic axes, and its position
+// within it, as a value in A and the rest
 template <typename A>
-__device__ __forceinline__ void centre_cell(const Domain &d, const double (&X)[3], int (&ci)[3], A (&cf)[3]) {
+__device__ __forceinline__ void centre_cell(const Domain &d, const double (&X)[3], int (&ci)[3], A (&cf)[3], A (&cr)[3]) {
     const int n3[3] = {d.nx, d.ny, d.nz}, per[3] = {d.px, d.py, d.pz};
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
         const double f = floor(X[i]);
         ci[i] = (int)f;
         if (per[i]) ci[i] = ((ci[i] % n3[i]) + n3[i]) % n3[i];
-        cf[i] = (A)(X[i] - f);
+        const double in = X[i] - f;
+        cf[i] = (A)in;
+        cr[i] = (A)(in - (double)cf[i]);
     }
+}
+
+// i - (c + r) rounded once to A: the difference's own rounding error (TwoSum) joins the rest
+template <typename A> __device__ __forceinline__ A cell_offset(int i, A c, A r) {
+    if constexpr (sizeof(A) == 8) return (A)i - c;
+    const A a = (A)i, s = a - c, t = s - a;
+    return s + (((a - (s - t)) - (c + t)) - r);
 }
 
 template <typename A, typename T, bool FIRST>
@@ -388,8 +399,8 @@ __global__ void __launch_bounds__(32 * ADJ_CUBE_WARPS) adj_cube_kernel(const Dev
     const BodyState &sb = ap.body[kb];
     const int fx = (int)floor(sb.X[0]), fy = (int)floor(sb.X[1]), fz = (int)floor(sb.X[2]);
     int ci[3];
-    A cf[3];
-    centre_cell(d, sb.X, ci, cf);
+    A cf[3], cr[3];
+    centre_cell(d, sb.X, ci, cf, cr);
     // cube cell l -> lattice cell (x, y, z); false outside the cube or the domain
     auto cube_cell = [&](int l, int &x, int &y, int &z) {
         if (l >= side * side * side) return false;
@@ -453,6 +464,8 @@ __global__ void __launch_bounds__(32 * ADJ_CUBE_WARPS) adj_cube_kernel(const Dev
     A fa0[6] = {0, 0, 0, 0, 0, 0};
     if constexpr (!FIRST)
         for (int i = 0; i < 6; ++i) fa0[i] = (A)ap.fadj[6 * kb + i];
+    const A eg = dv.forced ? AdjParams<A>::eg(dv, b) : (A)0;
+    const A g30 = AdjParams<A>::g3(dv, 0), g31 = AdjParams<A>::g3(dv, 1), g32 = AdjParams<A>::g3(dv, 2);
     const A hg0 = AdjParams<A>::half_g(dv, 0), hg1 = AdjParams<A>::half_g(dv, 1), hg2 = AdjParams<A>::half_g(dv, 2);
     for (int e = warp; e < nlist; e += ADJ_CUBE_WARPS) {
         int x, y, z;
@@ -486,13 +499,13 @@ __global__ void __launch_bounds__(32 * ADJ_CUBE_WARPS) adj_cube_kernel(const Dev
                     // link (x, b) of step n: moving bounce-back of step n+1 and
                     // the momentum exchange of step n share u_w(x + e_b; S^n);
                     // the offset from the centre is an integer difference of
-                    // cells less the centre's position within its cell (the same
+                    // cells less the centre's position within its cell, rounded once (the same
                     // expression for every body: a cell in two cubes is written
                     // by both blocks), the terms in A
                     const BodyState &sk = ap.body[k];
                     int kc[3] = {ci[0], ci[1], ci[2]};
-                    A kf[3] = {cf[0], cf[1], cf[2]};
-                    if (k != kb) centre_cell(d, sk.X, kc, kf);
+                    A kf[3] = {cf[0], cf[1], cf[2]}, kr[3] = {cr[0], cr[1], cr[2]};
+                    if (k != kb) centre_cell(d, sk.X, kc, kf, kr);
                     A o[3];
                     const int zp[3] = {wrap_axis(zx, d.nx), wrap_axis(zy, d.ny), wrap_axis(zz, d.nz)};
                     const int n3[3] = {d.nx, d.ny, d.nz}, per[3] = {d.px, d.py, d.pz};
@@ -500,7 +513,7 @@ __global__ void __launch_bounds__(32 * ADJ_CUBE_WARPS) adj_cube_kernel(const Dev
                     for (int i = 0; i < 3; ++i) {
                         int io = zp[i] - kc[i];
                         if (per[i]) io = 2 * io > n3[i] ? io - n3[i] : (2 * io < -n3[i] ? io + n3[i] : io);
-                        o[i] = (A)io - kf[i];
+                        o[i] = cell_offset(io, kf[i], kr[i]);
                     }
                     A W[3] = {W0[0], W0[1], W0[2]}, V[3] = {V0[0], V0[1], V0[2]};
                     A fa[6] = {fa0[0], fa0[1], fa0[2], fa0[3], fa0[4], fa0[5]};
@@ -554,10 +567,7 @@ __global__ void __launch_bounds__(32 * ADJ_CUBE_WARPS) adj_cube_kernel(const Dev
             const A sr = t4[0], s0 = t4[1], s1 = t4[2], s2 = t4[3];
             A f0 = 0, f1 = 0, f2 = 0;
             if (dv.forced) {
-                const A g0 = AdjParams<A>::g(dv, 0), g1 = AdjParams<A>::g(dv, 1), g2 = AdjParams<A>::g(dv, 2);
-                const A eg = (A)bx * g0 + (A)by * g1 + (A)bz * g2;
-                A f4[4] = {wa * ((A)9 * (A)bx * eg - (A)3 * g0), wa * ((A)9 * (A)by * eg - (A)3 * g1),
-                           wa * ((A)9 * (A)bz * eg - (A)3 * g2), (A)0};
+                A f4[4] = {wa * ((A)9 * (A)bx * eg - g30), wa * ((A)9 * (A)by * eg - g31), wa * ((A)9 * (A)bz * eg - g32), (A)0};
                 warp_sum4(f4);
                 f0 = f4[0]; f1 = f4[1]; f2 = f4[2];
             }

@@ -238,8 +238,9 @@ struct Device {
     double tau, omega, g[3];
     float omega_f, guo_f, g_f[3];   // omega, 1 - omega / 2 and g rounded to FP32 once (the FP32 collision's)
     float om1_f, ow_f[3], gw_f[3];  // 1 - omega; omega w and (1 - omega / 2) w per weight class (rest, axis, diagonal)
+    double om1, ow[3], gw[3];       // the same in FP64
     float gh_f[3], gl_f[3], gr_f[3];        // g / 2 as the sum of three FP32 values
-    double om1, ow[3], gw[3];       // the same in FP64: 1 - omega, omega w and (1 - omega / 2) w per weight class
+    float g3_f[3], eg_f[Q];         // 3 g and e_a . g, formed in FP64 and rounded once (the reverse sweep's)
     int forced;
     int avg_force;          // the rigid-body step uses the mean load of steps n and n-1
     float f16_scale, f16_inv_scale;

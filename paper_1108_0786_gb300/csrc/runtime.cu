@@ -398,7 +398,10 @@ int ensure_device(lbm_t *h) {
         dv.gh_f[i] = (float)(0.5 * dv.g[i]);
         dv.gl_f[i] = (float)(0.5 * dv.g[i] - (double)dv.gh_f[i]);
         dv.gr_f[i] = (float)(0.5 * dv.g[i] - (double)dv.gh_f[i] - (double)dv.gl_f[i]);
+        dv.g3_f[i] = (float)(3.0 * dv.g[i]);
     }
+    for (int a = 0; a < lbm::Q; ++a)
+        dv.eg_f[a] = (float)(lbm::ex(a) * dv.g[0] + lbm::ey(a) * dv.g[1] + lbm::ez(a) * dv.g[2]);
     dv.om1 = 1.0 - dv.omega;
     dv.om1_f = (float)dv.om1;
     {
