@@ -137,7 +137,10 @@ int lbm_set_allocator(lbm_t *h, lbm_alloc_fn alloc_fn, lbm_free_fn free_fn, void
 
 /* CUDA stream (a cudaStream_t) on which all work is enqueued; NULL is the
  * legacy default stream.  The device is the current device at the first
- * device allocation. */
+ * device allocation.  A step graph's bulk kernel runs at the stream's priority
+ * and the short kernels beside it one step above (both at the greatest where
+ * that is the stream's); after a change to a stream of another priority the next
+ * step waits for the device and captures the graphs anew. */
 int lbm_set_stream(lbm_t *h, void *stream);
 
 /* Add a rigid body (Sec. 2.2, 3.1-3.2): sphere of `radius` (length 0) or
@@ -199,7 +202,12 @@ int lbm_set_fields(lbm_t *h, int what, const void *host_in, int dtype);
  * synchronisation).  Returns launch errors only. */
 int lbm_step(lbm_t *h, int n);
 
-/* Wait for all enqueued work and return any latched device error. */
+/* Wait for all enqueued work and return any latched device error.  A handle's
+ * tenth synchronising read (lbm_sync, lbm_get_bodies, lbm_get_forces and the
+ * other calls that synchronise) allocates page-locked host memory once, 64 bytes
+ * and 104 for each body, through which that read and the later ones take one
+ * round trip to the device instead of two; it is kept until lbm_destroy, and
+ * where it is refused the reads go on without it. */
 int lbm_sync(lbm_t *h);
 
 /* Time average of the velocity field (Sec. 6, Fig. 13: the flow around one

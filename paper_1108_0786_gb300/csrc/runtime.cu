@@ -62,6 +62,8 @@ struct lbm_s {
     bool ready = false, graphs_ready = false;
     int device = 0;
     cudaStream_t stream = nullptr, cap = nullptr, side = nullptr;
+    bool new_stream = false;            // lbm_set_stream since the step graphs' priorities were looked up
+    int priority = 0;                   // the stream's priority then
     cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
     // a third branch of the step graphs: the link lists and loads beside the
     // boundary kernel (a small lattice's bulk kernel is shorter than both)
@@ -560,23 +562,53 @@ int ensure_device(lbm_t *h) {
     return LBM_OK;
 }
 
+// Node priorities of a step graph launched on a stream of priority p: the bulk
+// kernel keeps p and the chain goes one step above, so that against the caller's
+// other streams a lattice stands where its stream does.  Where p is the greatest
+// already both keep it, or, if `lower`, the bulk kernel goes one step below.
+struct ChainPriority {
+    int chain, bulk;
+};
+cudaError_t chain_priority(cudaStream_t s, bool lower, int &p, ChainPriority &out) {
+    int least = 0, greatest = 0;
+    cudaError_t e = cudaStreamGetPriority(s, &p);
+    if (e == cudaSuccess) e = cudaDeviceGetStreamPriorityRange(&least, &greatest);
+    out.chain = std::max(p - 1, greatest);
+    out.bulk = out.chain == p && lower ? std::min(p + 1, least) : p;
+    return e;
+}
+
 int build_graphs(lbm_t *h) {
+    if (h->graphs_ready && h->new_stream) {
+        int p = 0;
+        CK(cudaStreamGetPriority(h->stream, &p));
+        if (p != h->priority) {
+            // the graphs' nodes carry priorities: capture them anew, once nothing runs
+            CK(cudaDeviceSynchronize());
+            drop_graphs(h);
+            for (cudaStream_t *st : {&h->cap, &h->side, &h->side2, &h->far}) {
+                if (*st) cudaStreamDestroy(*st);
+                *st = nullptr;
+            }
+        }
+    }
+    h->new_stream = false;
     if (h->graphs_ready) return LBM_OK;
     // the chain (captured on cap) takes precedence over the bulk kernel beside
     // it, so that its short kernels start as soon as SMs free
     const bool ov = h->dv.overlap != 0, chain = nb(h) > 0 && fluid(h);
-    int least = 0, greatest = 0;
-    CK(cudaDeviceGetStreamPriorityRange(&least, &greatest));
-    if (!h->cap) CK(cudaStreamCreateWithPriority(&h->cap, cudaStreamNonBlocking, chain ? greatest : 0));
-    if (!h->side) CK(cudaStreamCreateWithPriority(&h->side, cudaStreamNonBlocking, least));
+    ChainPriority pr;
+    CK(chain_priority(h->stream, ov, h->priority, pr));
+    if (!h->cap) CK(cudaStreamCreateWithPriority(&h->cap, cudaStreamNonBlocking, chain ? pr.chain : pr.bulk));
+    if (!h->side) CK(cudaStreamCreateWithPriority(&h->side, cudaStreamNonBlocking, pr.bulk));
     if (!h->fork_ev) CK(cudaEventCreateWithFlags(&h->fork_ev, cudaEventDisableTiming));
     if (!h->join_ev) CK(cudaEventCreateWithFlags(&h->join_ev, cudaEventDisableTiming));
-    if (!h->side2) CK(cudaStreamCreateWithPriority(&h->side2, cudaStreamNonBlocking, chain ? greatest : 0));
+    if (!h->side2) CK(cudaStreamCreateWithPriority(&h->side2, cudaStreamNonBlocking, chain ? pr.chain : pr.bulk));
     if (!h->join2_ev) CK(cudaEventCreateWithFlags(&h->join2_ev, cudaEventDisableTiming));
     for (cudaEvent_t &ev : h->bulk_ev)
         if (!ev) CK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
     if (ov) {
-        if (!h->far) CK(cudaStreamCreateWithPriority(&h->far, cudaStreamNonBlocking, least));
+        if (!h->far) CK(cudaStreamCreateWithPriority(&h->far, cudaStreamNonBlocking, pr.bulk));
         for (int i = 0; i < 2; ++i) {
             if (!h->far_ev[i]) CK(cudaEventCreateWithFlags(&h->far_ev[i], cudaEventDisableTiming));
             if (!h->near_ev[i]) CK(cudaEventCreateWithFlags(&h->near_ev[i], cudaEventDisableTiming));
@@ -795,6 +827,7 @@ int lbm_set_allocator(lbm_t *h, lbm_alloc_fn a, lbm_free_fn f, void *ctx) {
 int lbm_set_stream(lbm_t *h, void *stream) {
     if (!h) return LBM_E_ARG;
     h->stream = static_cast<cudaStream_t>(stream);
+    h->new_stream = true;
     return LBM_OK;
 }
 
@@ -2287,15 +2320,16 @@ int lbm_ensemble_create(lbm_t *const *members, int n, lbm_ensemble_t **out) {
     e->stream = members[0]->stream;
     cudaError_t err = cudaStreamCreateWithFlags(&e->cap, cudaStreamNonBlocking);
     if (err == cudaSuccess) err = cudaEventCreateWithFlags(&e->fork, cudaEventDisableTiming);
-    // lanes: the latency-bound kernels' streams at the greatest priority,
-    // the bulk kernels' at the least, so that one lane's prep, remap and
+    // lanes: the latency-bound kernels' streams at a greater priority than
+    // the bulk kernels', so that one lane's prep, remap and
     // force blocks are dispatched ahead of the other lane's pending bulk blocks
-    int least = 0, greatest = 0;
-    if (err == cudaSuccess) err = cudaDeviceGetStreamPriorityRange(&least, &greatest);
+    int priority = 0;
+    ChainPriority pr{};
+    if (err == cudaSuccess) err = chain_priority(e->stream, true, priority, pr);
     for (int l = 0; l < ENS_LANES && err == cudaSuccess; ++l) {
-        err = cudaStreamCreateWithPriority(&e->lcap[l], cudaStreamNonBlocking, greatest);
-        if (err == cudaSuccess) err = cudaStreamCreateWithPriority(&e->lside[l], cudaStreamNonBlocking, greatest);
-        if (err == cudaSuccess) err = cudaStreamCreateWithPriority(&e->lbulk[l], cudaStreamNonBlocking, least);
+        err = cudaStreamCreateWithPriority(&e->lcap[l], cudaStreamNonBlocking, pr.chain);
+        if (err == cudaSuccess) err = cudaStreamCreateWithPriority(&e->lside[l], cudaStreamNonBlocking, pr.chain);
+        if (err == cudaSuccess) err = cudaStreamCreateWithPriority(&e->lbulk[l], cudaStreamNonBlocking, pr.bulk);
         for (cudaEvent_t *ev : {&e->lfork[l], &e->ljoin[l], &e->ldone[l], &e->lbdone[l][0], &e->lbdone[l][1]})
             if (err == cudaSuccess) err = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
     }
