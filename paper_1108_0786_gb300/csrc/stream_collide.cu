@@ -350,21 +350,22 @@ __device__ __forceinline__ R vdot(int b, R x, R y, R z) {
 
 // LBGK (+ Guo) for 16-bit storage in forms with few instructions, for one cell
 // (R = float) or two (R = F2) with the same bits.  Opposite directions
-// (b, b + 1) are paired: the moments come from pair sums and differences.
-// BF16 (its rounding is stochastic, so only the size of an error counts):
-//   f~_b = ((1 - omega) f_b + a) +- C e.u,
-//   a = omega w (drho - 1.5 rho u.u + 4.5 rho (e.u)^2),  C = 3 omega w rho
-//   (+ (1 - omega/2) w (9 (e.u)(e.g) - 3 u.g +- 3 e.g) with forcing).
-// FP16 (SCALED: the populations are k delta, k = f16_scale, a power of two, on
-// entry and exit) rounds to nearest, and in a slow flow, whose populations
-// are a few units in the last place, exact results often lie half way between
-// two FP16 values.  There the weight comes last, on a sum of few bits, so that
-// FP32 gives the half-way value itself and the rounding to even is unbiased:
+// (b, b + 1) are paired: the moments come from pair sums and differences.  The
+// weight comes last:
 //   f~_b = (1 - omega) f_b + omega w (a +- c),  c = 3 rho e.u,
-//   a = drho - 1.5 rho u.u + 4.5 rho (e.u)^2.
-// With BF16's form FP16's velocity field was 1.4 to 2 times as far from the
-// FP64 path (capsule swarms of 160 x 128 x 128 cells after 500 to 2000 steps),
-// with c and its sum in one rounding 1.1 times.
+//   a = drho - 1.5 rho u.u + 4.5 rho (e.u)^2
+//   (+ (1 - omega/2) w (9 (e.u)(e.g) - 3 u.g +- 3 e.g) with forcing).
+// With the weight folded into per-cell factors (3 omega w rho, ...) the factors'
+// roundings are the same in every step and cell of a slow flow (rho has few
+// values near 1), a momentum source of up to 6e-8 a step: the channel swimmer's
+// displacement in BF16 was 1.25 +- 0.03 times as far from the FP64 path (64
+// offsets, 4000 steps), though BF16's rounding is stochastic.  FP16 (SCALED: the
+// populations are k delta, k = f16_scale, a power of two, on entry and exit)
+// rounds to nearest, and in a slow flow, whose populations are a few units in the
+// last place, exact results often lie half way between two FP16 values; with c
+// and its sum rounded apart FP32 gives the half-way value itself and the rounding
+// to even is unbiased (one rounding: 1.1 times the error of the velocity field;
+// folded weights: 1.4 to 2 times).
 // Use: rest(f_0), pair(f_b, f_b+1) for the nine pairs in order, solve(), then
 // relax0 and relax for the populations.
 template <typename R, bool SCALED>
@@ -373,7 +374,7 @@ struct Lean {
     R base;                 // k (drho - 1.5 rho u.u)
     R kr;                   // k rho
     R ug3;                  // -3 k u.g (forcing)
-    R b, A, C, N;           // BF16: a = A (e.u)^2 + b, C and -C of the weight class at hand; FP16: A, C without weight
+    R A, C;                 // a = A (e.u)^2 + base, c = C e.u, C = 3 k rho
 
     __device__ __forceinline__ void rest(R f0) { s = f0; }
     __device__ __forceinline__ void pair(int p, R f1, R f2) {
@@ -403,61 +404,50 @@ struct Lean {
         const R usq = vfma(jx, jx, vfma(jy, jy, vmul(jz, jz)));
         kr = SCALED ? vscale(rho, k) : rho;
         base = vfma(vscale(kr, -1.5f), usq, s);
-        if constexpr (SCALED) {
-            A = vscale(kr, 4.5f);
-            C = vscale(kr, 3.0f);
-        }
+        A = vscale(kr, 4.5f);
+        C = vscale(kr, 3.0f);
         if (forced)
             ug3 = vscale(vscale_add(jx, dv.g_f[0], vscale_add(jy, dv.g_f[1], vscale(jz, dv.g_f[2]))), -3.0f * k);
     }
-    // BF16: the factors of weight class wc (1: axes, 2: diagonals)
-    __device__ __forceinline__ void weights(int wc, const Device &dv) {
-        const float ow = dv.ow_f[wc];
-        b = vscale(base, ow);
-        if (dv.forced) b = vscale_add(ug3, dv.gw_f[wc], b);
-        A = vscale(kr, 4.5f * ow);
-        C = vscale(kr, 3.0f * ow);
-        N = vscale(kr, -3.0f * ow);
-    }
-    // TAU1 (both): omega = 1, the old populations have the factor 0 and are not read
+    // TAU1: omega = 1, the old populations have the factor 0 and are not read
     template <bool TAU1 = false>
     __device__ __forceinline__ R relax0(R f0, const Device &dv) const {
         R r = vscale(base, dv.ow_f[0]);
         if (dv.forced) r = vscale_add(ug3, dv.gw_f[0], r);
         return TAU1 ? r : vscale_add(f0, dv.om1_f, r);
     }
-    // pair p, in order (the weights of its class are set before the class's first pair)
     template <bool TAU1 = false>
-    __device__ __forceinline__ void relax(int p, R &f1, R &f2, const Device &dv) {
+    __device__ __forceinline__ void relax(int p, R &f1, R &f2, const Device &dv) const {
         const int i = 2 * p + 1, wc = p < 3 ? 1 : 2;
-        if constexpr (!SCALED) {
-            if (p == 0) weights(1, dv);
-            if (p == 3) weights(2, dv);
-        }
         const R eu = vdot(i, jx, jy, jz);
-        R a = vfma(A, vmul(eu, eu), SCALED ? base : b);
+        const R a = vfma(A, vmul(eu, eu), base);
+        // scalar products: the assembler fuses a packed product with the sum after it
+        const R c = vmul_apart(C, eu);
+        R r1, r2;
         if constexpr (SCALED) {
-            // scalar products: the assembler fuses a packed product with the sum after it
-            const R c = vmul_apart(C, eu);
-            R r1 = vscale(vadd(a, c), dv.ow_f[wc]), r2 = vscale(vsub(a, c), dv.ow_f[wc]);
-            if (dv.forced) {
-                const float k = dv.f16_scale, eg = edot(i, dv.g_f[0], dv.g_f[1], dv.g_f[2]), gw = dv.gw_f[wc];
-                const R g = vscale_add(vscale(eu, 9.0f * k), eg, ug3);
-                r1 = vscale_add(vplus(g, 3.0f * k * eg), gw, r1);
-                r2 = vscale_add(vplus(g, -3.0f * k * eg), gw, r2);
-            }
-            f1 = TAU1 ? r1 : vscale_add(f1, dv.om1_f, r1);
-            f2 = TAU1 ? r2 : vscale_add(f2, dv.om1_f, r2);
+            r1 = vscale(vadd(a, c), dv.ow_f[wc]);
+            r2 = vscale(vsub(a, c), dv.ow_f[wc]);
+        } else {
+            const R ow = splat<R>(dv.ow_f[wc]);
+            r1 = vmul(vadd(a, c), ow);
+            r2 = vmul(vsub(a, c), ow);
+        }
+        if (dv.forced) {
+            const float k = SCALED ? dv.f16_scale : 1.0f, eg = edot(i, dv.g_f[0], dv.g_f[1], dv.g_f[2]), gw = dv.gw_f[wc];
+            const R g = vscale_add(vscale(eu, 9.0f * k), eg, ug3);
+            r1 = vscale_add(vplus(g, 3.0f * k * eg), gw, r1);
+            r2 = vscale_add(vplus(g, -3.0f * k * eg), gw, r2);
+        }
+        if constexpr (TAU1) {
+            f1 = r1;
+            f2 = r2;
+        } else if constexpr (SCALED) {
+            f1 = vscale_add(f1, dv.om1_f, r1);
+            f2 = vscale_add(f2, dv.om1_f, r2);
         } else {
             const R om1 = splat<R>(dv.om1_f);
-            const float eg = edot(i, dv.g_f[0], dv.g_f[1], dv.g_f[2]), gw = dv.gw_f[wc];
-            if (dv.forced) a = vscale_add(eu, 9.0f * gw * eg, a);
-            f1 = vfma(C, eu, TAU1 ? a : vfma(f1, om1, a));
-            f2 = vfma(N, eu, TAU1 ? a : vfma(f2, om1, a));
-            if (dv.forced) {
-                f1 = vplus(f1, 3.0f * gw * eg);
-                f2 = vplus(f2, -3.0f * gw * eg);
-            }
+            f1 = vfma(f1, om1, r1);
+            f2 = vfma(f2, om1, r2);
         }
     }
 };
@@ -908,8 +898,8 @@ __device__ __forceinline__ void store_words(const unsigned (&w)[Q][V / 2], const
 // direction's shuffle the loads of several directions waited for one another
 // (issue slots 44 % used, FP16 four cells a thread 520 us).  Bound by the
 // bytes in flight and, in BF16 (the rounding), by instruction issue: 512 x 256 x
-// 256 cells at tau = 1 take 396 us in FP16 (6.5 TB/s) and 448 us in BF16, 428 and
-// 487 us at tau = 0.8, against 449 and 542 us with a cell at a time in scalar
+// 256 cells at tau = 1 take 396 us in FP16 (6.5 TB/s) and 441 us in BF16, 429 and
+// 486 us at tau = 0.8, against 449 and 542 us with a cell at a time in scalar
 // arithmetic.  (Copying the sources ahead into shared memory with cp.async, two
 // stages at 16 warps an SM, took 525 and 549 us.)
 template <typename T, int V, bool WALLS>
