@@ -19,8 +19,8 @@ LIB = os.path.join(OUT_DIR, "liblbm.so")
 HEADER = os.path.join(ROOT, "include", "lbm.h")
 SOURCES = ["stream_collide.cu", "kernels.cu", "runtime.cu", "static_scratch.cu", "adjoint.cu"]
 # the cell kernels are compiled without implicit multiply-add contraction: a
-# cell's arithmetic then rounds the same in every kernel that runs it (launch
-# shapes, batched ensembles, the boundary kernel); the wanted FMAs are explicit
+# cell's arithmetic then rounds the same in every launch shape, in batched
+# ensembles and in either boundary kernel; the wanted FMAs are explicit
 NO_CONTRACT = {"stream_collide.cu"}
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",

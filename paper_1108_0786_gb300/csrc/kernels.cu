@@ -116,13 +116,9 @@ __device__ inline void geom_place(const Domain &d, const BodyProps &p, int a, do
     g.cfd[a] = __dsub_rn(c, fc);
     g.cf[a] = (float)g.cfd[a];
     g.v[a] = (float)Va;
-    int lo = (int)floor(__dsub_rn(Xa, p.reach)), hi = (int)floor(__dadd_rn(Xa, p.reach));
-    int width = hi - lo + 1;
-    int elo = lo - STATIC_REACH, ewidth = width + 2 * STATIC_REACH;
+    const int lo = (int)floor(__dsub_rn(Xa, p.reach)), hi = (int)floor(__dadd_rn(Xa, p.reach));
+    int elo = lo - STATIC_REACH, ewidth = hi - lo + 1 + 2 * STATIC_REACH;
     if (per) {
-        lo %= n;
-        if (lo < 0) lo += n;
-        if (width > n) width = n;
         elo %= n;
         if (elo < 0) elo += n;
         if (ewidth > n) ewidth = n;
@@ -131,8 +127,6 @@ __device__ inline void geom_place(const Domain &d, const BodyProps &p, int a, do
     int ahead = elo - o;
     if (per && ahead < 0) ahead += n;
     ewidth = min(ewidth, 2 * half + 1 - ahead);
-    g.box[a] = lo;
-    g.box[3 + a] = width;
     g.ebox[a] = elo;
     g.ebox[3 + a] = ewidth;
 }
@@ -363,8 +357,7 @@ __device__ __forceinline__ void remap_body(const Device &dv, const StepPtrs &sp,
     // first REMAP_STAGED records are staged in shared memory.
     // With at most REMAP_STAGED bodies every body is a candidate (the cells' box
     // tests sort them out): one round of loads less in a block's latency chain
-    // (32^3 FP64 swimmer, a step: 45.1 -> 42.2 us with the narrower screen margin;
-    // 128 x 64 x 64 channel 34.6 -> 33.7 us).
+    // (0.9 us of a 128 x 64 x 64 channel step).
     const bool all = dv.nb <= REMAP_STAGED;
     if (all) {
         if (tid < dv.nb) cid[tid] = tid;
@@ -926,8 +919,8 @@ __device__ inline long long to_fixed(float v) {
 //   F = sum e_a [2 f~_a(x_f) + 6 w_a rho(x_f) e_-a . u_w(x_f + e_a)],
 //   T = sum (x_f + e_a / 2 - X) x F_link
 // with f~ of step n (dst) and the body state of step n.  The last of body
-// b's blocks to finish runs body b's rigid-body step on its first warp; the
-// last body to finish ends the step (clock, change flag).
+// b's blocks to finish runs body b's rigid-body step on the two warps past its
+// link warps; the last body to finish ends the step (clock, change flag).
 //
 // FP64 storage: every term in FP64; each block reduces with warp shuffles
 // in a fixed order and writes its partial sums, which the rigid-body step

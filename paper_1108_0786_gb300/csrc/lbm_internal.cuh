@@ -128,8 +128,7 @@ struct BodyGeom {
     int shape;
     int side;               // edge of the remap cube, 2 (E + REMAP_MARGIN) + 1
     int ncand;              // state n: bodies whose grown box meets this body's remap cube (cand list; the batched remap's)
-    int box[6];             // per axis: lower corner (wrapped) and width of [floor(X - reach), floor(X + reach)]
-    int ebox[6];            // the same grown by STATIC_REACH cells
+    int ebox[6];            // per axis: lower corner (wrapped) and width of [floor(X - reach), floor(X + reach)] grown by STATIC_REACH cells
     double cfd[3];          // the position within the cell in FP64
 };
 
@@ -170,16 +169,6 @@ __device__ inline void offset_from(const Domain &d, const BodyState &b, double p
     o[0] = min_image(px - b.X[0], d.nx, d.inx, d.px);
     o[1] = min_image(py - b.X[1], d.ny, d.iny, d.py);
     o[2] = min_image(pz - b.X[2], d.nz, d.inz, d.pz);
-}
-
-// velocity of the body surface at lattice point p: V + Omega x (p - X)
-__device__ inline void surface_velocity(const Domain &d, const BodyState &b, double px, double py,
-                                        double pz, double u[3]) {
-    double o[3];
-    offset_from(d, b, px, py, pz, o);
-    u[0] = b.V[0] + (b.W[1] * o[2] - b.W[2] * o[1]);
-    u[1] = b.V[1] + (b.W[2] * o[0] - b.W[0] * o[2]);
-    u[2] = b.V[2] + (b.W[0] * o[1] - b.W[1] * o[0]);
 }
 
 // Recording of a forward run for the reverse sweep: when `on`, the rigid-body
@@ -225,8 +214,9 @@ inline unsigned row_recip(int n) { return n > 1 ? (unsigned)((1ULL << 32) / (uns
 // step n-1 and the remap of step n.  An option (LBM_OPT_OVERLAP), not the
 // default: the bulk kernel needs nearly every SM's memory parallelism to
 // hold HBM at its peak, so short kernels that share the SMs with it slow it
-// by about as much as their own time (measured on the 33.5 M-cell capsule
-// swarm: 0.889 ms a step overlapped against 0.872 ms serial).
+// by about as much as their own time, while the ordinary step graph already runs
+// the chain beside the bulk kernel (33.5 M-cell capsule swarm: 0.849 ms a step
+// overlapped against 0.771 ms).
 constexpr int TILE_X = 64;
 
 struct Device {

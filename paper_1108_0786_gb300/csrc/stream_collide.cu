@@ -22,18 +22,18 @@
 //                no-slip wall, f_b = f~_{-b}(x) (Eq. 4); if y was solid at
 //                n-1, f_b = f~_{-b}(x) + 6 w_b rho(x) e_b . u_w(y) with rho(x)
 //                the density of x at n-1 and u_w at the state of step n-1;
-//            then the same LBGK collision.
+//            then the same LBGK collision (sums in another order).
 //
 // Populations are stored as deviations delta = f - w from the rest
 // equilibrium (16-bit formats: FP16 scaled by 2^10, BF16 unscaled), so the
 // small velocity signal survives FP32 and 16-bit storage; the collision runs
 // in FP64 for FP64 storage and in FP32 otherwise.
 //
-// Memory access of the bulk kernel: thread (tx, ty) of block (bx, by, z)
-// handles V consecutive cells of row (y, z); each population is fetched as
-// one aligned V-wide vector, and the +-1 x shift of the pull is completed
-// with a warp shuffle from the neighbouring lane (a scalar load at row and
-// warp ends).  Every population byte is read once and written once.
+// Memory access of the bulk kernel: a thread handles V consecutive cells of a
+// row, the V-cell groups of a z-plane dealt to the threads in row order; each
+// population is fetched as one aligned V-wide vector, and the +-1 x shift of the
+// pull is completed with a warp shuffle from the neighbouring lane (a scalar load
+// at row and warp ends).  Every population byte is read once and written once.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
@@ -108,9 +108,11 @@ __device__ __forceinline__ T shfl(T v, int delta, bool up) {
 }
 
 // explicit fused multiply-adds: this file is compiled without implicit
-// contraction (-fmad=false), so every kernel that runs a cell's arithmetic --
-// any launch shape, the batched ensemble kernels, the boundary kernel --
-// rounds it identically, and the FMAs the collision wants are spelled out
+// contraction (-fmad=false), so the bulk kernel's launch shapes, its batched form
+// and the near kernel round a cell's arithmetic identically, and so do the two
+// boundary kernels (whose sums run in another order than the bulk kernel's: which
+// cells are listed depends on the bodies alone); the FMAs the collision wants are
+// spelled out
 __device__ __forceinline__ float mad(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double mad(double a, double b, double c) { return __fma_rn(a, b, c); }
 
@@ -211,9 +213,10 @@ __device__ __forceinline__ void collide_f32(float (&f)[Q], const Device &dv) {
 // takes two FMAs:
 //   f~ = ((1 - omega) f + a) +- C e.u,  a = omega w (drho - 1.5 rho u.u + 4.5 rho (e.u)^2),
 //   C = 3 omega w rho  (+ (1 - omega/2) w (9 (e.u)(e.g) - 3 u.g +- 3 e.g) with forcing).
-// 130 FP64 instructions a cell against 240 with each direction on its own: the
-// bulk kernel takes 1205 us a launch on 203 x 149 x 131 cells (1957 before),
-// its FP64 pipe 87 % busy.
+// 130 FP64 instructions a cell (112 at tau = 1) against 240 with each direction on
+// its own: a launch on 203 x 149 x 131 cells takes 977 us (842 at tau = 1, 1337
+// with a body force).  Against 64-bit-mantissa arithmetic a collision's error is
+// 0.7 to 0.9 times that of the plain form for tau in 0.51 .. 2.
 __device__ __forceinline__ void collide_f64(double (&f)[Q], const Device &dv) {
     double d[Q / 2];
     double s = f[0];
@@ -250,8 +253,7 @@ __device__ __forceinline__ void collide_f64(double (&f)[Q], const Device &dv) {
     const double r45[2] = {1.5 * r3[0], 1.5 * r3[1]};
     if (om1 == 0.0 && !forced) {
         // tau = 1: the update is the equilibrium itself, the same bits without 18
-        // of the FMAs (0 f + a = a; a non-finite f makes every moment so): 203 x 149
-        // x 131 cells, 8 steps and the populations, 8.31 -> 7.17 ms
+        // of the FMAs (0 f + a = a; a non-finite f makes every moment so)
 #pragma unroll
         for (int p = 0; p < Q / 2; ++p) {
             const int b = 2 * p + 1, wc = p < 3 ? 0 : 1;
@@ -464,12 +466,12 @@ __device__ __forceinline__ void collide_lean(float (&f)[Q], const Device &dv) {
     for (int p = 0; p < Q / 2; ++p) c.relax(p, f[2 * p + 1], f[2 * p + 2], dv);
 }
 
-// the collision of storage type T on its deviations, unscaled
+// the collision of storage type T on its values as loaded (raw_ld for 16-bit storage)
 template <typename T, typename Cd>
 __device__ __forceinline__ void collide(Cd (&f)[Q], const Device &dv) {
     if constexpr (std::is_same<T, double>::value) collide_f64(f, dv);
     else if constexpr (std::is_same<T, float>::value) collide_f32(f, dv);
-    else collide_lean<false>(f, dv);
+    else collide_lean<std::is_same<T, __half>::value>(f, dv);
 }
 
 // 16-bit storage without a per-population scale: FP16 keeps k delta, so the
@@ -564,8 +566,8 @@ template <typename T> __device__ __forceinline__ Dither dither_for(long long c, 
 // a block, so that no lane idles at the end of a row whatever nx is.  A warp's
 // lanes may cross a row end, where the loads of a row's first and last cell
 // take over from the shuffles.  (Blocks of 32 or 128 groups of one row left 21 %
-// of the FP64 kernel's lanes idle at nx = 203: 1205 -> 955 us a launch on
-// 203 x 149 x 131 cells; 22 % of the FP32 kernel's at nx = 100.)
+// of the FP64 kernel's lanes idle at nx = 203, which cost 26 % of its time, and
+// 22 % of the FP32 kernel's at nx = 100.)
 constexpr int BULK_THREADS = 256;
 
 __device__ __forceinline__ void plane_group(const Blk &bk, int nxq, int ny, unsigned recip, int &xq, int &y,
@@ -709,8 +711,7 @@ __device__ __forceinline__ void bulk_body(const Device &dv, const StepPtrs &sp, 
         Cd g[Q];
 #pragma unroll
         for (int b = 0; b < Q; ++b) g[b] = f[b][i];
-        if constexpr (raw16) collide_lean<std::is_same<T, __half>::value>(g, dv);
-        else collide<T>(g, dv);
+        collide<T>(g, dv);
         const bool solid = fl[i] & F_SOLID;
         if constexpr (WALLS) {
 #pragma unroll
@@ -895,8 +896,8 @@ __device__ __forceinline__ void store_words(const unsigned (&w)[Q][V / 2], const
 // are held in FP32 at a time, and at tau = 1, where they do not enter the
 // relaxation, not again at all.  All loads, the row ends' single cells included,
 // stand before the first shuffle: with each row end's load behind its
-// direction's shuffle the loads of several directions waited for one another
-// (issue slots 44 % used, FP16 four cells a thread 520 us).  Bound by the
+// direction's shuffle the loads of several directions wait for one another (four
+// cells a thread, FP16: 520 us, 429 ahead).  Bound by the
 // bytes in flight and, in BF16 (the rounding), by instruction issue: 512 x 256 x
 // 256 cells at tau = 1 take 396 us in FP16 (6.5 TB/s) and 441 us in BF16, 429 and
 // 486 us at tau = 0.8, against 449 and 542 us with a cell at a time in scalar
@@ -1571,13 +1572,12 @@ __global__ void __launch_bounds__(TMA_THREADS, MINB) bulk_tma_kernel(const Devic
                     if constexpr (sizeof(T) == 2) f[b] = raw_ld<T>(v);
                     else f[b] = Codec<T>::ld(v, inv_scale);
                 }
+                collide<T>(f, dv);
                 if constexpr (sizeof(T) == 2) {
-                    collide_lean<std::is_same<T, __half>::value>(f, dv);
                     const Dither dz = dither_for<T>(c0 + x, sp.tstep);
 #pragma unroll
                     for (int b = 0; b < Q; ++b) dst[(long long)b * C + c0 + x] = store16<T>(f[b], dz, b);
                 } else {
-                    collide<T>(f, dv);
 #pragma unroll
                     for (int b = 0; b < Q; ++b) dst[(long long)b * C + c0 + x] = Codec<T>::st(f[b], scale);
                 }
