@@ -1961,6 +1961,7 @@ struct EnsGroup {
     int precision = 1;
     bool walls = false;                     // some member has a non-periodic axis
     bool by_cell = false;                   // the boundary kernel a thread a cell (boundary_by_cell)
+    int variant = 0;                        // batched bulk shape, which the tables are made for
     int lane = 0;                           // batched mode: the chain of launches the group is in
     std::vector<int> members;               // ensemble indices
     void *mem = nullptr;                    // the tables, one allocation (first member's allocator)
@@ -1989,7 +1990,7 @@ struct lbm_ensemble_s {
     cudaEvent_t lstart = nullptr;
     std::vector<cudaEvent_t> join;          // one per member
     int mode = LBM_ENSEMBLE_BATCHED;
-    int variant[4] = {-1, -1, -1, -1};      // batched bulk shape per precision (-1: the default)
+    int variant[4] = {-1, -1, -1, -1};      // autotuned bulk shape per precision (-1: a group's default)
     // one graph per set of members advanced together (CHUNK_STEPS steps)
     std::vector<EnsGraph> graphs;
     std::vector<unsigned> gens;             // the members' graph generations the cached graphs were built at
@@ -2059,7 +2060,7 @@ int ens_variant(const lbm_ensemble_t *e, int precision, const std::vector<int> &
 int ens_group_tables(lbm_ensemble_t *e, EnsGroup &g) {
     const int M = (int)g.members.size();
     lbm_t *h0 = e->members[g.members[0]];
-    const int variant = ens_variant(e, g.precision, g.members);
+    const int variant = g.variant = ens_variant(e, g.precision, g.members);
     std::vector<lbm::Device> dvs(M);
     std::vector<lbm::StepPtrs> sps(2 * M);
     for (int j = 0; j < M; ++j) {
@@ -2123,7 +2124,6 @@ int ens_group_tables(lbm_ensemble_t *e, EnsGroup &g) {
         b.members = M;
         b.parity = 0;
     }
-    e->variant[g.precision] = variant;
     return LBM_OK;
 }
 
@@ -2148,7 +2148,7 @@ void ens_enqueue_batched(lbm_ensemble_t *e, std::vector<EnsGroup> &groups, int l
             if (g.lane != lane) continue;
             lbm::Batch b = g.bt[k];
             b.parity = p;
-            lbm::launch_batch_cells(k, e->variant[g.precision], b, g.blocks[k], g.precision, g.walls, g.by_cell, st);
+            lbm::launch_batch_cells(k, g.variant, b, g.blocks[k], g.precision, g.walls, g.by_cell, st);
         }
     };
     cudaEventRecord(fork, main);
